@@ -333,7 +333,7 @@ struct ibem_handle {
     double* d_hsy = nullptr;        // Helmholtz: split-layout output [2R][N]
     bool far_on_the_fly = false;    // Helmholtz FP64 coupling generated on the fly (stored K too large)
     double far_diam = 0.0;          // bound on the distance of two points of a far block (cluster balls)
-    float4* d_gen_pts = nullptr;    // double-float point tables [C][q2][2] of the generated coupling
+    float4* d_gen_pts = nullptr;    // double-float point tables [C][2][q2] of the generated coupling
     float4* d_gen_trig = nullptr;   // e^{i j 2 pi / 2048} as double-float pairs
     float4* d_gen_x = nullptr;      // moments, chunked double-float complex [nch][C][q2][RC]
     size_t gen_x_bytes = 0;
