@@ -98,7 +98,7 @@ void free_handle(ibem_handle* h) {
                     h->d_pairs_by_cls[1], h->d_pairs_by_cls[2], h->d_pairs_by_cls[3], h->d_pairs_by_cls[4],
                     h->d_near, h->d_near32, h->d_far_ptr, h->d_far_src, h->d_far_tgt, h->d_K, h->d_Kdf, h->d_xh2, h->d_far_rows,
                     h->d_xs, h->d_ys, h->d_xh, h->d_yh, h->d_xs32, h->d_ys32, h->d_yh32, h->d_src32, h->d_diag,
-                    h->d_solver, h->d_red, h->d_status, h->d_Kc, h->d_xh4, h->d_hsx, h->d_hsy,
+                    h->d_solver, h->d_red, h->d_status, h->d_Kc, h->d_xh4, h->d_hcol, h->d_hsx, h->d_hsy,
                     h->d_bj_ptr, h->d_bj_off, h->d_bj_dofs, h->d_bj_inv, h->d_up_ptr, h->d_up_src,
                     h->d_up_tgt, h->d_up_rows, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->d_mr, h->d_Mf, h->d_Sf,
                     h->d_gen_pts, h->d_gen_trig, h->d_gen_x, h->d_Kbf, h->d_graded_pairs, h->d_graded_tab,
@@ -128,6 +128,13 @@ ibem_status plan_error_status(const std::string& msg) {
         if (msg.find(key) != std::string::npos) return IBEM_ERR_GEOMETRY;
     return IBEM_ERR_ARG;
 }
+
+// Which of the two mirrored far blocks (sigma, tau), (tau, sigma) a symmetric
+// coupling stores: the one whose row has the smaller id if the ids' sum is odd,
+// the larger id if it is even, so that every row owns about half of its far
+// list.  (With sigma < tau throughout the first rows own all of theirs, the last
+// none; one CTA works on a row, so the longest row bounds a small tree's time.)
+bool half_owner(int64_t sigma, int64_t tau) { return (((sigma + tau) & 1) != 0) == (sigma < tau); }
 
 // the FP64 operator needs stored coupling matrices for Laplace (Helmholtz can
 // generate them on the fly)
@@ -363,7 +370,6 @@ ibem_status ibem_create(const ibem_patch* patches, int npatch, const ibem_params
     std::vector<int32_t> ftgt(P.n_far);
     for (int64_t c = 0; c < P.C; ++c) {
         if (P.far_ptr[c + 1] > P.far_ptr[c]) h->far_rows.push_back((int32_t)c);
-        if (P.far_ptr[c + 1] - P.far_ptr[c] > h->max_far_row) h->max_far_row = (int)(P.far_ptr[c + 1] - P.far_ptr[c]);
         for (int64_t k = P.far_ptr[c]; k < P.far_ptr[c + 1]; ++k) ftgt[k] = (int32_t)c;
     }
     TRY(upload(&h->d_far_ptr, P.far_ptr, st), "upload far ptr");
@@ -384,7 +390,7 @@ ibem_status ibem_create(const ibem_patch* patches, int npatch, const ibem_params
         std::vector<int32_t> usrc, utgt;
         for (int64_t c = 0; c < P.C; ++c) {
             for (int64_t k = P.far_ptr[c]; k < P.far_ptr[c + 1]; ++k)
-                if (P.far_src[k] > c) {
+                if (half_owner(c, P.far_src[k])) {
                     usrc.push_back(P.far_src[k]);
                     utgt.push_back((int32_t)c);
                 }
@@ -456,10 +462,10 @@ ibem_status ibem_get_info(const ibem_handle* h, ibem_info* info) {
     info->n_near_singular[2] = P.n_cls[CLS_VERTEX];
     info->n_near_singular[3] = P.n_cls[CLS_SUBDIV];
     info->bytes_near = P.n_near * (int64_t)P.nb * P.nb * (h->helm ? 16 : 8);
-    // the FP64 coupling matrices actually stored: upper half in double-float
-    // (Laplace), every far block natively (Laplace) or in double-float (Helmholtz)
+    // the FP64 coupling matrices actually stored: upper half in double-float, or
+    // every far block natively (Laplace)
     const int64_t per = (int64_t)h->kpt * 4 * P.q2;
-    info->bytes_far = h->d_Kdf ? h->n_up * per * 8 : (h->d_K ? P.n_far * per * 8 : (h->d_Kc ? P.n_far * per * 16 : 0));
+    info->bytes_far = h->d_Kdf ? h->n_up * per * 8 : (h->d_K ? P.n_far * per * 8 : (h->d_Kc ? h->n_up * per * 16 : 0));
     info->assembled = h->assembled ? 1 : 0;
     info->max_gauss_order = P.max_order;
     info->n_near_graded = P.n_graded;
@@ -498,14 +504,17 @@ ibem_status ibem_assemble(ibem_handle* h) {
         if (!h->d_near32 && (e = cudaMalloc(&h->d_near32, nn * sizeof(float))))
             return cuda_fail(h, e, "alloc near blocks fp32");
         if (P.n_far > 0 && h->helm) {
-            // stored complex coupling (16 B per entry) if it fits in half of the free memory
+            // stored complex coupling (16 B per entry, one of two mirrored blocks) if the full
+            // list would fit in half of the free memory (the column shares and moments
+            // of an application take the rest)
             size_t nk = (size_t)P.n_far * h->kpt * 4 * P.q2;
+            size_t nku = (size_t)(h->n_up > 0 ? h->n_up : 1) * h->kpt * 4 * P.q2;
             size_t free_b = 0, total_b = 0;
             cudaMemGetInfo(&free_b, &total_b);
             h->far_on_the_fly = P.prm.fp64_coupling != IBEM_COUPLING_DF || nk * sizeof(float4) > free_b / 2;
             if (P.prm.fp64_coupling == IBEM_COUPLING_FP32_ONLY) h->far_on_the_fly = true;
             if (!h->far_on_the_fly)
-                if ((e = cudaMalloc(&h->d_Kc, nk * sizeof(float4)))) return cuda_fail(h, e, "alloc coupling matrices");
+                if ((e = cudaMalloc(&h->d_Kc, nku * sizeof(float4)))) return cuda_fail(h, e, "alloc coupling matrices");
         } else if (P.n_far > 0 && P.prm.fp64_coupling != IBEM_COUPLING_NONE &&
                    P.prm.fp64_coupling != IBEM_COUPLING_FP32_ONLY) {   // Laplace (GENERATE: as DF)
             size_t nk = (size_t)P.n_far * h->kpt * 4 * P.q2;
@@ -525,8 +534,6 @@ ibem_status ibem_assemble(ibem_handle* h) {
         if ((e = launch_far_assembly(h))) return cuda_fail(h, e, "far assembly");
     }
     if ((e = cudaStreamSynchronize(h->stream))) return cuda_fail(h, e, "assemble sync");
-    // work vectors sized before assembly lack the stored coupling's moment buffer
-    if (h->d_Kc && !h->d_xh4) h->ws_nrhs = 0;
     if (!h->d_bj_inv) {
         std::string msg;
         if ((e = build_block_jacobi(h, &msg))) return msg.empty() ? cuda_fail(h, e, "block-Jacobi") : fail(h, IBEM_ERR_BREAKDOWN, msg);

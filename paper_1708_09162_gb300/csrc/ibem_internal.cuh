@@ -327,8 +327,10 @@ struct ibem_handle {
     double* d_K = nullptr;          // [n_far][kpt][4 q2]: entry (a, b = s + 4k) at [k][4a + s] (native)
     float2* d_Kdf = nullptr;        // same layout, (hi, lo) float pairs (double-float coupling)
     float2* d_xh2 = nullptr;        // forward moments split into (hi, lo) float pairs
-    float4* d_Kc = nullptr;         // Helmholtz: double-float complex coupling (re_hi, re_lo, im_hi, im_lo)
-    float4* d_xh4 = nullptr;        // Helmholtz: forward moments as double-float complex
+    float4* d_Kc = nullptr;         // Helmholtz: double-float complex coupling (re_hi, re_lo, im_hi, im_lo), one of two mirrored blocks
+    float4* d_xh4 = nullptr;        // Helmholtz: forward moments as double-float complex, one pass of right-hand sides
+    float4* d_hcol = nullptr;       // Helmholtz: column shares of the stored blocks, one pass
+    int hdf_rhs = 0;                // right-hand sides d_xh4 and d_hcol are sized for
     double* d_hsx = nullptr;        // Helmholtz: split-layout input  [2R][max(N, nq)]
     double* d_hsy = nullptr;        // Helmholtz: split-layout output [2R][N]
     bool far_on_the_fly = false;    // Helmholtz FP64 coupling generated on the fly (stored K too large)
@@ -340,8 +342,7 @@ struct ibem_handle {
     int kpt = 0;
     int df_nst = 0;   // ring depth of the double-float coupling (autotuned at assembly; 0 = default)
     std::vector<int32_t> far_rows;  // target clusters with a non-empty far list
-    int max_far_row = 0;            // longest far list
-    // upper half of the far field (source id > target id), used with symmetric storage
+    // half of the far field, one of every two mirrored blocks, used with symmetric storage
     std::vector<int32_t> up_rows;
     int max_up_row = 0;
     int64_t n_up = 0;
@@ -498,6 +499,8 @@ cudaError_t launch_coupling_gen(ibem_handle* h, int R);
 // The same coupling contracted on the tensor cores in BF16 digit slices (q = 8).
 bool sliced_supported(const ibem_handle* h);
 cudaError_t launch_coupling_sliced(ibem_handle* h, int R);
+// Helmholtz coupling from stored double-float matrices (kernels_helm_df.cu).
+cudaError_t launch_helm_coupling_df(ibem_handle* h, int R);
 // Double-float coupling launcher and the autotuner of its ring depth (kernels_apply.cu).
 cudaError_t launch_coupling_df(ibem_handle* h, int R, int nst);
 cudaError_t tune_coupling_df(ibem_handle* h);

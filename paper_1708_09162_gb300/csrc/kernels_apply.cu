@@ -268,7 +268,7 @@ __device__ inline bool mbar_wait(uint64_t* bar, unsigned parity, long long limit
 
 // Laplace coupling matrices are symmetric, K_{tau sigma} = K_{sigma tau}^T (the
 // kernel and the product of surface measures are symmetric and evaluated
-// identically), so only the blocks with sigma < tau are stored.  The CTA of
+// identically), so only one of the two is stored (half_owner).  The CTA of
 // row sigma streams them once and uses each twice: rows give
 // y^_sigma = sum K x^_tau (register accumulation, stored at the end), columns
 // give the block's share K^T x^_sigma of y^_tau (reduced across the 4 lanes
@@ -411,7 +411,7 @@ __global__ void coupling_df_kernel(const int32_t* __restrict__ rows, const int64
     if (active && s == 0) yh[(r * C + sigma) * q2 + a] = acc;
 }
 
-// y^_tau += sum over the stored blocks (sigma, tau), sigma < tau, of their column
+// y^_tau += sum over the stored blocks (sigma, tau) of their column
 // shares, in the order of the transposed list.
 __global__ void column_gather_kernel(int R, int64_t C, int q2, const int64_t* __restrict__ tptr,
                                      const int32_t* __restrict__ tblk, const float2* __restrict__ colpart,
@@ -600,9 +600,8 @@ cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
     if (nrhs <= h->ws_nrhs) return cudaSuccess;
     Plan& P = h->P;
     if (h->helm) {
-        cudaFree(h->d_hsx); cudaFree(h->d_hsy); cudaFree(h->d_xh4);
+        cudaFree(h->d_hsx); cudaFree(h->d_hsy);
         h->d_hsx = h->d_hsy = nullptr;
-        h->d_xh4 = nullptr;
     }
     cudaFree(h->d_xs); cudaFree(h->d_ys); cudaFree(h->d_xh); cudaFree(h->d_yh);
     cudaFree(h->d_xs32); cudaFree(h->d_src32); cudaFree(h->d_xh2);
@@ -633,9 +632,6 @@ cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
         size_t n = (size_t)(P.N > P.nq ? P.N : P.nq);
         if ((e = cudaMalloc(&h->d_hsx, (size_t)nrhs * n * sizeof(double)))) return e;
         if ((e = cudaMalloc(&h->d_hsy, (size_t)nrhs * P.N * sizeof(double)))) return e;
-        // double-float moments of the stored coupling only (none when it is generated)
-        if (h->d_Kc && (e = cudaMalloc(&h->d_xh4, (size_t)(nrhs / 2 + 1) * P.C * ((P.q2 + 1) & ~1) * sizeof(float4) + 32)))
-            return e;
     }
     h->ws_nrhs = nrhs;
     return cudaSuccess;

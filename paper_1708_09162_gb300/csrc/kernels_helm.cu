@@ -10,9 +10,10 @@
 // parts.
 //
 // Near blocks: [n_near][nb][nb] double2 (re, im).  Coupling matrices of the
-// FP64 operator: stored as double-float complex (re_hi, re_lo, im_hi, im_lo),
-// layout [n_far][kpt][4 q2] like the Laplace case, or - when they would not fit
-// in the memory budget - generated on the fly in FP64.
+// FP64 operator: one of two mirrored blocks stored as double-float complex (re_hi,
+// re_lo, im_hi, im_lo), layout [n_up][kpt][4 q2] like the Laplace case
+// (kernels_helm_df.cu), or - when they would not fit in the memory budget -
+// generated on the fly.
 #include "ibem_internal.cuh"
 
 namespace ibem {
@@ -316,157 +317,6 @@ __global__ void helm_far_assemble_kernel(int64_t n_far, const int32_t* __restric
     }
     float rh = (float)vr, ih = (float)vi;
     K[idx] = make_float4(rh, (float)(vr - (double)rh), ih, (float)(vi - (double)ih));
-}
-
-// split moments of the 2R real "right-hand sides" into double-float complex
-// (re_hi, re_lo, im_hi, im_lo) rows of q2p entries (q2p even: 32-byte rows)
-__global__ void helm_split_kernel(int R, int64_t C, int q2, int q2p, const double* __restrict__ xh,
-                                  float4* __restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)R * C * q2p) return;
-    int64_t r = i / (C * q2p);
-    int64_t rem = i % (C * q2p);
-    int64_t c = rem / q2p;
-    int a = (int)(rem % q2p);
-    double vr = 0.0, vi = 0.0;
-    if (a < q2) {
-        vr = xh[((2 * r) * C + c) * q2 + a];
-        vi = xh[((2 * r + 1) * C + c) * q2 + a];
-    }
-    float rh = (float)vr, ih = (float)vi;
-    out[i] = make_float4(rh, (float)(vr - (double)rh), ih, (float)(vi - (double)ih));
-}
-
-// double-float helpers: exact product a*b = p + e; acc (hi, lo) += (p, e)
-__device__ inline void df_mac(float ah, float al, float bh, float bl, float& hi, float& lo) {
-    float p = ah * bh;
-    float e = fmaf(ah, bh, -p);
-    e = fmaf(ah, bl, e);
-    e = fmaf(al, bh, e);
-    float t = hi + p;
-    float z = t - hi;
-    float err = (hi - (t - z)) + (p - z);
-    hi = t;
-    lo += err + e;
-}
-
-__device__ inline unsigned hsmem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ inline void hmbar_init(uint64_t* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(hsmem(bar)), "r"(count) : "memory");
-}
-__device__ inline void hmbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(hsmem(bar)), "r"(bytes) : "memory");
-}
-__device__ inline void hbulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     hsmem(dst)),
-                 "l"(src), "r"(bytes), "r"(hsmem(bar))
-                 : "memory");
-}
-__device__ inline bool hmbar_wait(uint64_t* bar, unsigned parity, long long limit) {
-    for (long long it = 0; it < limit; ++it) {
-        unsigned ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(hsmem(bar)), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-// Streaming complex coupling, FP64-accurate (double-float), same pipeline as
-// the Laplace kernel: one CTA per target cluster, NST stages of (K block,
-// source moments) filled by cp.async.bulk, bounded mbarrier waits.
-template <int KPT, int NST>
-__global__ void helm_coupling_df_kernel(const int32_t* __restrict__ rows, const int64_t* __restrict__ fptr,
-                                        const int32_t* __restrict__ fsrc, const float4* __restrict__ K, int q2,
-                                        int q2p, int maxrow, int64_t C, const float4* __restrict__ xh,
-                                        double* __restrict__ yh, long long wait_limit, int* __restrict__ status) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-    int32_t* srcs = reinterpret_cast<int32_t*>(smem + 128);
-    const int stride = 4 * q2;
-    const int belems = KPT * stride;
-    const int selems = belems + q2p;
-    float4* stage = reinterpret_cast<float4*>(smem + 128 + (((size_t)maxrow * 4 + 15) / 16) * 16);
-    const unsigned kbytes = (unsigned)belems * 16u, xbytes = (unsigned)q2p * 16u;
-    const int sigma = rows[blockIdx.x];
-    const int64_t r = blockIdx.y;
-    const int t = threadIdx.x, s = t & 3, a = t >> 2;
-    const bool active = t < stride;
-    const int64_t b0 = fptr[sigma];
-    const int n = (int)(fptr[sigma + 1] - b0);
-    const float4* xr = xh + r * C * q2p;
-    for (int j = t; j < n; j += blockDim.x) srcs[j] = fsrc[b0 + j];
-    if (t == 0) {
-        for (int i = 0; i < NST; ++i) hmbar_init(&full[i], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-    if (t == 0) {
-        for (int i = 0; i < NST && i < n; ++i) {
-            float4* dst = stage + (size_t)i * selems;
-            hmbar_expect_tx(&full[i], kbytes + xbytes);
-            hbulk_load(dst, K + (b0 + i) * (int64_t)belems, kbytes, &full[i]);
-            hbulk_load(dst + belems, xr + (int64_t)srcs[i] * q2p, xbytes, &full[i]);
-        }
-    }
-    double accr = 0.0, acci = 0.0;
-    int i = 0;
-    bool failed = false;
-    for (; i < n; ++i) {
-        const int st = i % NST;
-        const bool ok = hmbar_wait(&full[st], (unsigned)((i / NST) & 1), wait_limit);
-        if (ok && active) {
-            const float4* Kb = stage + (size_t)st * selems + t;
-            const float4* xt = stage + (size_t)st * selems + belems;
-            float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-#pragma unroll
-            for (int kk = 0; kk < KPT; ++kk) {
-                int b = s + 4 * kk;
-                if (b < q2) {
-                    float4 kv = Kb[kk * stride];
-                    float4 x = xt[b];
-                    // (Kr + i Ki)(xr + i xi) = (Kr xr - Ki xi) + i (Kr xi + Ki xr)
-                    df_mac(kv.x, kv.y, x.x, x.y, rh, rl);
-                    df_mac(-kv.z, -kv.w, x.z, x.w, rh, rl);
-                    df_mac(kv.x, kv.y, x.z, x.w, ih, il);
-                    df_mac(kv.z, kv.w, x.x, x.y, ih, il);
-                }
-            }
-            accr += (double)rh + (double)rl;
-            acci += (double)ih + (double)il;
-        }
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        if (t == 0 && i + NST < n) {
-            float4* dst = stage + (size_t)st * selems;
-            hmbar_expect_tx(&full[st], kbytes + xbytes);
-            hbulk_load(dst, K + (b0 + i + NST) * (int64_t)belems, kbytes, &full[st]);
-            hbulk_load(dst + belems, xr + (int64_t)srcs[i + NST] * q2p, xbytes, &full[st]);
-        }
-    }
-    if (failed) {
-        if (t == 0) {
-            atomicOr(status, 1);
-            for (int j = i; j < n && j < i + NST; ++j) hmbar_wait(&full[j % NST], (unsigned)((j / NST) & 1), 1LL << 24);
-        }
-        __syncthreads();
-        return;
-    }
-    accr += __shfl_xor_sync(0xffffffffu, accr, 1);
-    accr += __shfl_xor_sync(0xffffffffu, accr, 2);
-    acci += __shfl_xor_sync(0xffffffffu, acci, 1);
-    acci += __shfl_xor_sync(0xffffffffu, acci, 2);
-    if (active && s == 0) {
-        yh[((2 * r) * C + sigma) * q2 + a] = accr;
-        yh[((2 * r + 1) * C + sigma) * q2 + a] = acci;
-    }
 }
 
 // Complex coupling generated on the fly in FP64 (when the stored matrices would
@@ -828,8 +678,9 @@ cudaError_t helm_launch_near_assembly(ibem_handle* h) {
 cudaError_t helm_launch_far_assembly(ibem_handle* h) {
     Plan& P = h->P;
     if (P.n_far == 0 || !h->d_Kc) return cudaSuccess;
-    int64_t total = P.n_far * (int64_t)h->kpt * 4 * P.q2;
-    helm_far_assemble_kernel<<<nblk(total, 256), 256, 0, h->stream>>>(P.n_far, h->d_far_tgt, h->d_far_src, h->d_igeo,
+    int64_t total = h->n_up * (int64_t)h->kpt * 4 * P.q2;   // one of two mirrored blocks
+    if (total == 0) return cudaSuccess;
+    helm_far_assemble_kernel<<<nblk(total, 256), 256, 0, h->stream>>>(h->n_up, h->d_up_tgt, h->d_up_src, h->d_igeo,
                                                                       P.q2, h->kpt, P.prm.kappa, h->d_Kc);
     return cudaGetLastError();
 }
@@ -881,37 +732,7 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
                     h->launches += 2;
                 }
             } else if (h->d_Kc) {
-                const int q2p = (q2 + 1) & ~1;
-                helm_split_kernel<<<nblk((int64_t)R * P.C * q2p, T), T, 0, st>>>(R, P.C, q2, q2p, h->d_xh, h->d_xh4);
-                int threads = ((4 * q2 + 31) / 32) * 32;
-                dim3 grid(nrows, R);
-                const size_t sbytes = ((size_t)h->kpt * 4 * q2 + q2p) * sizeof(float4);
-                const size_t head = 128 + (((size_t)h->max_far_row * 4 + 15) / 16) * 16;
-#define IBEM_HDF_LAUNCH(K_, N_)                                                                                   \
-    {                                                                                                             \
-        size_t sm = head + (size_t)(N_)*sbytes;                                                                   \
-        if ((e = cudaFuncSetAttribute(helm_coupling_df_kernel<K_, N_>,                                           \
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))                     \
-            return e;                                                                                             \
-        helm_coupling_df_kernel<K_, N_><<<grid, threads, sm, st>>>(h->d_far_rows, h->d_far_ptr, h->d_far_src,    \
-                                                                   h->d_Kc, q2, q2p, h->max_far_row, P.C,         \
-                                                                   h->d_xh4, h->d_yh, h->wait_limit, h->d_status); \
-    }                                                                                                             \
-    break;
-                switch (h->kpt) {
-                    case 1: IBEM_HDF_LAUNCH(1, 8)
-                    case 3: IBEM_HDF_LAUNCH(3, 6)
-                    case 4: IBEM_HDF_LAUNCH(4, 4)
-                    case 7: IBEM_HDF_LAUNCH(7, 3)
-                    case 9: IBEM_HDF_LAUNCH(9, 2)
-                    case 13: IBEM_HDF_LAUNCH(13, 2)
-                    case 16: IBEM_HDF_LAUNCH(16, 2)
-                    case 21: IBEM_HDF_LAUNCH(21, 1)
-                    case 25: IBEM_HDF_LAUNCH(25, 1)
-                    default: return cudaErrorInvalidValue;
-                }
-#undef IBEM_HDF_LAUNCH
-                h->launches += 2;
+                if ((e = launch_helm_coupling_df(h, R))) return e;
             } else if (P.prm.fp64_coupling == IBEM_COUPLING_SLICED && sliced_supported(h)) {
                 if ((e = launch_coupling_sliced(h, R))) return e;
             } else if (P.prm.fp64_coupling != IBEM_COUPLING_NATIVE && gen_supported(h)) {
