@@ -8,6 +8,7 @@
 
 #include <algorithm>
 
+#include "fp64_eval.cuh"
 #include "ibem_internal.cuh"
 
 using namespace ibem;
@@ -93,7 +94,7 @@ std::vector<double> bezier_extraction(int p, int m) {
 
 void free_handle(ibem_handle* h) {
     void* ptrs[] = {h->d_patches, h->d_knots, h->d_cpw, h->d_ext, h->d_qgeo, h->d_igeo, h->d_igeo32, h->d_phi,
-                    h->d_phi_sub, h->d_rule[0], h->d_rule[1], h->d_rule[2], h->d_M, h->d_S, h->d_balls, h->d_mu1d, h->d_mu1d_off, h->d_near_ptr,
+                    h->d_phi_sub, h->d_rule[0], h->d_rule[1], h->d_rule[2], h->d_trig64, h->d_M, h->d_S, h->d_balls, h->d_mu1d, h->d_mu1d_off, h->d_near_ptr,
                     h->d_near_src, h->d_near_tgt, h->d_near_cls, h->d_near_orient, h->d_pairs_by_cls[0],
                     h->d_pairs_by_cls[1], h->d_pairs_by_cls[2], h->d_pairs_by_cls[3], h->d_pairs_by_cls[4],
                     h->d_near, h->d_near32, h->d_far_ptr, h->d_far_src, h->d_far_tgt, h->d_K, h->d_Kdf, h->d_xh2, h->d_far_rows,
@@ -255,6 +256,10 @@ ibem_status ibem_create(const ibem_patch* patches, int npatch, const ibem_params
     TRY(upload(&h->d_cpw, P.cpw, st), "upload control points");
     std::vector<double> ext = bezier_extraction(P.p, P.m);
     TRY(upload(&h->d_ext, ext, st), "upload extraction");
+    {
+        const std::vector<double> trig = trig64_table();
+        TRY(upload(reinterpret_cast<double**>(&h->d_trig64), trig, st), "upload trig table");
+    }
 
     // Bernstein products at the regular and the subdivided Gauss points
     std::vector<double> gx, gw;

@@ -293,6 +293,7 @@ struct ibem_handle {
     double* d_phi_sub = nullptr;    // [4][Q*Q][nb] at the 2x2-subdivided Gauss points
     double* d_rule[3] = {nullptr, nullptr, nullptr};  // singular rules, SoA [5][n]
     int rule_n[3] = {0, 0, 0};
+    double2* d_trig64 = nullptr;    // cos and sin table of the FP64 evaluation (fp64_eval.cuh)
     double* d_M = nullptr;          // [q][pp] 1D leaf moments int L_a B_i (times h)
     double* d_S = nullptr;          // [2][q][q] 1D M2M: S_c[a][b] = L_a((c + z_b) / 2)
     float* d_Mf = nullptr;          // FP32 copies of M and S for the FP32 many-right-hand-side path
@@ -474,9 +475,11 @@ cudaError_t apply_operator(ibem_handle* h, const double* x, double* y, int nrhs,
 cudaError_t launch_rhs(ibem_handle* h, const double* g, int nrhs, double* b);
 cudaError_t launch_potential(ibem_handle* h, const double* w, int nrhs, const double* pts,
                              int64_t npts, double* u);
+// direct potential of several densities, split layout (kernels_potential.cu)
+cudaError_t launch_potential_multi(ibem_handle* h, const double* w, int nrhs, const double* pts, int64_t npts,
+                                   double* u);
 // the direct Laplace potential on caller-provided work space (ws: ndof_super
-// doubles, srcs: E Q^2 sources); used by launch_potential and the
-// allocation-free entry point
+// doubles, srcs: E Q^2 sources); used by the allocation-free entry point
 cudaError_t launch_potential_ws(ibem_handle* h, const double* w, int nrhs, const double* pts, int64_t npts,
                                 double* u, double* ws, double4_32a* srcs);
 cudaError_t launch_near_diagonal(ibem_handle* h, double* diag);

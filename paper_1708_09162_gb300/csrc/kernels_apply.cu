@@ -916,7 +916,8 @@ __global__ void potential_kernel(int64_t npts, const double* __restrict__ pts, i
 // Direct Laplace potential on caller-provided work space: ws holds the lifted
 // density of one right-hand side (ndof_super doubles), srcs the Gauss-point
 // sources (E Q^2); u is cleared and accumulated with atomics over chunks of
-// sources.  Shared by ibem_potential and the allocation-free entry point.
+// sources.  The allocation-free entry point's form: one density at a time, in
+// fixed work space (ibem_potential: kernels_potential.cu).
 cudaError_t launch_potential_ws(ibem_handle* h, const double* w, int nrhs, const double* pts, int64_t npts,
                                 double* u, double* ws, double4_32a* srcs) {
     Plan& P = h->P;
@@ -944,18 +945,9 @@ cudaError_t launch_potential_ws(ibem_handle* h, const double* w, int nrhs, const
 
 cudaError_t launch_potential(ibem_handle* h, const double* w, int nrhs, const double* pts, int64_t npts,
                              double* u) {
-    Plan& P = h->P;
-    cudaError_t e;
-    if (h->helm) {
-        if ((e = ensure_workspace(h, 2 * nrhs))) return e;
-        return helm_launch_potential(h, w, nrhs, pts, npts, u, h->d_hsx);
-    }
-    if ((e = ensure_workspace(h, 1))) return e;
-    double4_32a* srcs = nullptr;
-    if ((e = cudaMallocAsync(&srcs, (size_t)P.E * P.Q * P.Q * sizeof(double4_32a), h->stream))) return e;
-    e = launch_potential_ws(h, w, nrhs, pts, npts, u, h->d_xs, srcs);
-    cudaFreeAsync(srcs, h->stream);
-    return e;
+    if (!h->helm) return launch_potential_multi(h, w, nrhs, pts, npts, u);
+    cudaError_t e = ensure_workspace(h, 2 * nrhs);
+    return e ? e : helm_launch_potential(h, w, nrhs, pts, npts, u, h->d_hsx);
 }
 
 }  // namespace ibem
