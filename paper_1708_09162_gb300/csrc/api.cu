@@ -94,7 +94,7 @@ std::vector<double> bezier_extraction(int p, int m) {
 
 void free_handle(ibem_handle* h) {
     void* ptrs[] = {h->d_patches, h->d_knots, h->d_cpw, h->d_ext, h->d_qgeo, h->d_igeo, h->d_igeo32, h->d_phi,
-                    h->d_phi_sub, h->d_rule[0], h->d_rule[1], h->d_rule[2], h->d_trig64, h->d_M, h->d_S, h->d_balls, h->d_mu1d, h->d_mu1d_off, h->d_near_ptr,
+                    h->d_phi_sub, h->d_gauss, h->d_trig64, h->d_M, h->d_S, h->d_balls, h->d_mu1d, h->d_mu1d_off, h->d_near_ptr,
                     h->d_near_src, h->d_near_tgt, h->d_near_cls, h->d_near_orient, h->d_pairs_by_cls[0],
                     h->d_pairs_by_cls[1], h->d_pairs_by_cls[2], h->d_pairs_by_cls[3], h->d_pairs_by_cls[4],
                     h->d_near, h->d_near32, h->d_far_ptr, h->d_far_src, h->d_far_tgt, h->d_K, h->d_Kdf, h->d_xh2, h->d_far_rows,
@@ -282,12 +282,13 @@ ibem_status ibem_create(const ibem_patch* patches, int npatch, const ibem_params
         }
     TRY(upload(&h->d_phi, phi, st), "upload phi");
     TRY(upload(&h->d_phi_sub, phis, st), "upload phi_sub");
-    for (int c = 0; c < 3; ++c) {
-        if (P.n_cls[c] == 0) continue;
-        std::vector<double> soa;
-        singular_rule(c, P.Qs, soa);
-        h->rule_n[c] = (int)(soa.size() / 5);
-        TRY(upload(&h->d_rule[c], soa, st), "upload singular rule");
+    {
+        std::vector<double> rules(gx), nx, nw;
+        rules.insert(rules.end(), gw.begin(), gw.end());
+        gauss_legendre(P.Qs, nx, nw);
+        rules.insert(rules.end(), nx.begin(), nx.end());
+        rules.insert(rules.end(), nw.begin(), nw.end());
+        TRY(upload(&h->d_gauss, rules, st), "upload Gauss rules");
     }
 
     // FMM transfer matrices (1D): leaf moments and M2M re-expansion
@@ -328,7 +329,9 @@ ibem_status ibem_create(const ibem_patch* patches, int npatch, const ibem_params
             const int c = P.near_cls[k];
             if ((c == CLS_REGULAR || c == CLS_SUBDIV) && P.near_order[k] != P.Q)
                 bygrade[(c == CLS_SUBDIV) * (IBEM_MAX_GAUSS + 1) + P.near_order[k]].push_back((int32_t)k);
-            else
+            else if (t <= P.near_src[k] || ((c == CLS_REGULAR || c == CLS_SUBDIV) &&
+                                            near_streamed(P.Q, P.nb, h->helm, c == CLS_SUBDIV)))
+                // mirrored pairs are formed together, except by the streaming kernel
                 bycls[c].push_back((int32_t)k);
         }
     // graded groups: pairs, Gauss rule and Bernstein products at that order

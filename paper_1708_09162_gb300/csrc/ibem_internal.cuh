@@ -260,8 +260,6 @@ void chebyshev_nodes(int q, std::vector<double>& z);
 void lagrange_values(const std::vector<double>& z, double x, double* L);
 void element_of(const Plan& P, int64_t e, int* patch, int* ix, int* iy);
 void cluster_of(const Plan& P, int64_t c, int* patch, int* level, int* ix, int* iy);
-// Canonical rules (x1, x2, y1, y2, w) of the touching classes, SoA [5][n].
-void singular_rule(int cls, int n, std::vector<double>& soa);
 
 }  // namespace ibem
 
@@ -291,8 +289,7 @@ struct ibem_handle {
     float* d_igeo32 = nullptr;      // same in FP32
     double* d_phi = nullptr;        // [Q*Q][nb] Bernstein products at the regular Gauss points
     double* d_phi_sub = nullptr;    // [4][Q*Q][nb] at the 2x2-subdivided Gauss points
-    double* d_rule[3] = {nullptr, nullptr, nullptr};  // singular rules, SoA [5][n]
-    int rule_n[3] = {0, 0, 0};
+    double* d_gauss = nullptr;      // 1D Gauss rules: nodes and weights [2][Q] of the regular, then [2][Qs] of the Duffy rules
     double2* d_trig64 = nullptr;    // cos and sin table of the FP64 evaluation (fp64_eval.cuh)
     double* d_M = nullptr;          // [q][pp] 1D leaf moments int L_a B_i (times h)
     double* d_S = nullptr;          // [2][q][q] 1D M2M: S_c[a][b] = L_a((c + z_b) / 2)
@@ -306,7 +303,7 @@ struct ibem_handle {
     int32_t* d_near_cls = nullptr;
     int32_t* d_near_orient = nullptr;
     int32_t* d_pairs_by_cls[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    int64_t n_list[5] = {0, 0, 0, 0, 0};   // lengths of d_pairs_by_cls (graded pairs excluded)
+    int64_t n_list[5] = {0, 0, 0, 0, 0};   // lengths of d_pairs_by_cls (graded pairs excluded; one of two mirrored pairs unless streamed)
     // graded near pairs (order != Q): one group per (class, order), its pairs
     // contiguous in d_graded_pairs, its rule (nodes, weights) and Bernstein
     // table ([1 or 4][n^2][nb]) at tab_off in d_graded_tab
@@ -455,13 +452,14 @@ cudaError_t helm_launch_potential(ibem_handle* h, const double* w, int nrhs, con
                                   double* u, double* wsplit);
 __global__ void helm_split_vec_kernel(int R, int64_t n, const double* __restrict__ in, double* __restrict__ out);
 __global__ void helm_join_vec_kernel(int R, int64_t n, const double* __restrict__ in, double* __restrict__ out);
-// near-field assembly (kernels_setup.cu): the streaming form of the regular and
-// subdivided pairs, used where the shared-matrix form needs more than
-// IBEM_MAX_SMEM_BYTES (near_shared_bytes) of shared memory
+// near-field assembly: product and Duffy rules (kernels_near.cu) ...
+bool near_streamed(int Q, int nb, bool cplx, bool subdiv);
+cudaError_t launch_near_blocks(ibem_handle* h, bool cplx, double kappa, double* blocks);
+// ... and the streaming form of the regular and subdivided pairs for high orders
+// (kernels_setup.cu)
 cudaError_t launch_near_stream(ibem_handle* h, int cls, bool cplx, double kappa, double* blocks);
 // the graded pairs (orders != Q), one streaming launch per (class, order) group
 cudaError_t launch_near_graded(ibem_handle* h, bool cplx, double kappa, double* blocks);
-size_t near_shared_bytes(int Q, int nb, bool cplx, bool subdiv);
 // potential_fmm.cu
 cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, const double* pts, int64_t npts,
                                  double* u, int64_t* n_far_terms, int64_t* n_near_terms);

@@ -14,22 +14,12 @@
 // re_lo, im_hi, im_lo), layout [n_up][kpt][4 q2] like the Laplace case
 // (kernels_helm_df.cu), or - when they would not fit in the memory budget -
 // generated on the fly.
+#include "fp64_eval.cuh"
 #include "ibem_internal.cuh"
 
 namespace ibem {
 
 static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
-
-__constant__ double c_hgx[IBEM_MAX_GAUSS], c_hgw[IBEM_MAX_GAUSS];
-
-__device__ inline void helm_elem(int64_t e, int ne1, int* patch, int* ix, int* iy) {
-    int64_t per = (int64_t)ne1 * ne1;
-    *patch = (int)(e / per);
-    uint32_t x, y;
-    morton2_inv((uint32_t)(e % per), &x, &y);
-    *ix = (int)x;
-    *iy = (int)y;
-}
 
 // exp(i kappa r) / (4 pi r) * w
 __device__ inline void helm_kernel64(double kappa, double r, double w, double* re, double* im) {
@@ -40,211 +30,7 @@ __device__ inline void helm_kernel64(double kappa, double r, double w, double* r
     *im = f * s;
 }
 
-// ---- near field assembly -------------------------------------------------------
-// Regular pairs: one CTA per pair; shared XA[QQ][4], XB[QQ][4], Gre, Gim [QQ][QQ],
-// Hre, Him [QQ][nb].
-__global__ void helm_near_regular_kernel(const int32_t* __restrict__ list, const int32_t* __restrict__ tgt,
-                                         const int32_t* __restrict__ src, const double* __restrict__ qgeo,
-                                         const double* __restrict__ phi, int QQ, int nb, double kappa,
-                                         double2* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    double* XA = sm;
-    double* XB = XA + 4 * QQ;
-    double* Gr = XB + 4 * QQ;
-    double* Gi = Gr + QQ * QQ;
-    double* Hr = Gi + QQ * QQ;
-    double* Hi = Hr + QQ * nb;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    for (int i = threadIdx.x; i < 4 * QQ; i += blockDim.x) {
-        XA[i] = qgeo[4 * QQ * t + i];
-        XB[i] = qgeo[4 * QQ * s + i];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < QQ * QQ; i += blockDim.x) {
-        int a = i / QQ, b = i % QQ;
-        double d0 = XA[4 * a] - XB[4 * b], d1 = XA[4 * a + 1] - XB[4 * b + 1], d2 = XA[4 * a + 2] - XB[4 * b + 2];
-        helm_kernel64(kappa, sqrt(d0 * d0 + d1 * d1 + d2 * d2), XA[4 * a + 3] * XB[4 * b + 3], &Gr[i], &Gi[i]);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < QQ * nb; i += blockDim.x) {
-        int a = i / nb, j = i % nb;
-        double vr = 0.0, vi = 0.0;
-        for (int b = 0; b < QQ; ++b) {
-            double p = phi[b * nb + j];
-            vr += Gr[a * QQ + b] * p;
-            vi += Gi[a * QQ + b] * p;
-        }
-        Hr[i] = vr;
-        Hi[i] = vi;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
-        int r = i / nb, j = i % nb;
-        double vr = 0.0, vi = 0.0;
-        for (int a = 0; a < QQ; ++a) {
-            double p = phi[a * nb + r];
-            vr += p * Hr[a * nb + j];
-            vi += p * Hi[a * nb + j];
-        }
-        blocks[k * nb * nb + i] = make_double2(vr, vi);
-    }
-}
-
-// Subdivided pairs: 2 x 2 sub-squares of both elements, geometry on the fly.
-__global__ void helm_near_subdiv_kernel(GeomView g, const int32_t* __restrict__ list, const int32_t* __restrict__ tgt,
-                                        const int32_t* __restrict__ src, const double* __restrict__ phi_sub, int Q,
-                                        int nb, int ne1, double kappa, double2* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    int QQ = Q * Q;
-    double* XA = sm;
-    double* XB = XA + 16 * QQ;
-    double* Gr = XB + 16 * QQ;
-    double* Gi = Gr + QQ * QQ;
-    double* Hr = Gi + QQ * QQ;
-    double* Hi = Hr + QQ * nb;
-    double* ar = Hi + QQ * nb;
-    double* ai = ar + nb * nb;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    double h = 1.0 / ne1;
-    for (int i = threadIdx.x; i < 8 * QQ; i += blockDim.x) {
-        int which = i / (4 * QQ);
-        int r = i % (4 * QQ);
-        int sub = r / QQ, gq = r % QQ;
-        int patch, ix, iy;
-        helm_elem(which ? s : t, ne1, &patch, &ix, &iy);
-        double su = 0.5 * (sub & 1) + 0.5 * c_hgx[gq % Q];
-        double sv = 0.5 * (sub >> 1) + 0.5 * c_hgx[gq / Q];
-        double F[3], Fu[3], Fv[3];
-        eval_patch(g, patch, (ix + su) * h, (iy + sv) * h, F, Fu, Fv);
-        double* o = (which ? XB : XA) + 4 * r;
-        o[0] = F[0]; o[1] = F[1]; o[2] = F[2];
-        o[3] = 0.25 * c_hgw[gq % Q] * c_hgw[gq / Q] * surface_measure(Fu, Fv) * h * h;
-    }
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) { ar[i] = 0.0; ai[i] = 0.0; }
-    __syncthreads();
-    for (int sa = 0; sa < 4; ++sa)
-        for (int sb = 0; sb < 4; ++sb) {
-            const double* A = XA + 4 * QQ * sa;
-            const double* B = XB + 4 * QQ * sb;
-            for (int i = threadIdx.x; i < QQ * QQ; i += blockDim.x) {
-                int a = i / QQ, b = i % QQ;
-                double d0 = A[4 * a] - B[4 * b], d1 = A[4 * a + 1] - B[4 * b + 1], d2 = A[4 * a + 2] - B[4 * b + 2];
-                helm_kernel64(kappa, sqrt(d0 * d0 + d1 * d1 + d2 * d2), A[4 * a + 3] * B[4 * b + 3], &Gr[i], &Gi[i]);
-            }
-            __syncthreads();
-            const double* pb = phi_sub + (size_t)sb * QQ * nb;
-            for (int i = threadIdx.x; i < QQ * nb; i += blockDim.x) {
-                int a = i / nb, j = i % nb;
-                double vr = 0.0, vi = 0.0;
-                for (int b = 0; b < QQ; ++b) {
-                    double p = pb[b * nb + j];
-                    vr += Gr[a * QQ + b] * p;
-                    vi += Gi[a * QQ + b] * p;
-                }
-                Hr[i] = vr;
-                Hi[i] = vi;
-            }
-            __syncthreads();
-            const double* pa = phi_sub + (size_t)sa * QQ * nb;
-            for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
-                int r = i / nb, j = i % nb;
-                double vr = 0.0, vi = 0.0;
-                for (int a = 0; a < QQ; ++a) {
-                    double p = pa[a * nb + r];
-                    vr += p * Hr[a * nb + j];
-                    vi += p * Hi[a * nb + j];
-                }
-                ar[i] += vr;
-                ai[i] += vi;
-            }
-            __syncthreads();
-        }
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) blocks[k * nb * nb + i] = make_double2(ar[i], ai[i]);
-}
-
-// Touching pairs: the Duffy-type rules mapped through the canonical orientation.
-// Shared: SAr[nb][CH], SAi[nb][CH], SB[nb][CH].
-__global__ void helm_near_singular_kernel(GeomView g, const int32_t* __restrict__ list,
-                                          const int32_t* __restrict__ tgt, const int32_t* __restrict__ src,
-                                          const int32_t* __restrict__ orient, const double* __restrict__ rule,
-                                          int npts, int p, int ne1, double kappa, double2* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    const int CH = blockDim.x;
-    const int pp = p + 1, nb = pp * pp;
-    double* SAr = sm;
-    double* SAi = SAr + nb * CH;
-    double* SB = SAi + nb * CH;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    int ka = orient[k] >> 3, kb = orient[k] & 7;
-    int pa, ixa, iya, pb, ixb, iyb;
-    helm_elem(t, ne1, &pa, &ixa, &iya);
-    helm_elem(s, ne1, &pb, &ixb, &iyb);
-    double h = 1.0 / ne1;
-    const double scale = h * h * h * h;
-    double accr[5] = {0, 0, 0, 0, 0}, acci[5] = {0, 0, 0, 0, 0};
-    for (int base = 0; base < npts; base += CH) {
-        int ip = base + threadIdx.x;
-        if (ip < npts) {
-            double x1 = rule[ip], x2 = rule[npts + ip], y1 = rule[2 * npts + ip], y2 = rule[3 * npts + ip];
-            double w = rule[4 * npts + ip];
-            double xa, ya, xb, yb;
-            dihedral(ka, x1, x2, &xa, &ya);
-            dihedral(kb, y1, y2, &xb, &yb);
-            double FA[3], FB[3], Fu[3], Fv[3];
-            eval_patch(g, pa, (ixa + xa) * h, (iya + ya) * h, FA, Fu, Fv);
-            double kA = surface_measure(Fu, Fv);
-            eval_patch(g, pb, (ixb + xb) * h, (iyb + yb) * h, FB, Fu, Fv);
-            double kB = surface_measure(Fu, Fv);
-            double d0 = FA[0] - FB[0], d1 = FA[1] - FB[1], d2 = FA[2] - FB[2];
-            double vr, vi;
-            helm_kernel64(kappa, sqrt(d0 * d0 + d1 * d1 + d2 * d2), w * scale * kA * kB, &vr, &vi);
-            double bxu[IBEM_MAX_P + 1], bxv[IBEM_MAX_P + 1], byu[IBEM_MAX_P + 1], byv[IBEM_MAX_P + 1];
-            bernstein(p, xa, bxu);
-            bernstein(p, ya, bxv);
-            bernstein(p, xb, byu);
-            bernstein(p, yb, byv);
-            for (int iv = 0; iv < pp; ++iv)
-                for (int iu = 0; iu < pp; ++iu) {
-                    double ba = bxu[iu] * bxv[iv];
-                    SAr[(iv * pp + iu) * CH + threadIdx.x] = vr * ba;
-                    SAi[(iv * pp + iu) * CH + threadIdx.x] = vi * ba;
-                    SB[(iv * pp + iu) * CH + threadIdx.x] = byu[iu] * byv[iv];
-                }
-        } else {
-            for (int i = 0; i < nb; ++i) {
-                SAr[i * CH + threadIdx.x] = 0.0;
-                SAi[i * CH + threadIdx.x] = 0.0;
-                SB[i * CH + threadIdx.x] = 0.0;
-            }
-        }
-        __syncthreads();
-        for (int r = 0; r < 5; ++r) {
-            int e = threadIdx.x + r * CH;
-            if (e < nb * nb) {
-                int i = e / nb, j = e % nb;
-                const double* ar = SAr + i * CH;
-                const double* ai = SAi + i * CH;
-                const double* b = SB + j * CH;
-                double vr = 0.0, vi = 0.0;
-                for (int c = 0; c < CH; ++c) {
-                    vr += ar[c] * b[c];
-                    vi += ai[c] * b[c];
-                }
-                accr[r] += vr;
-                acci[r] += vi;
-            }
-        }
-        __syncthreads();
-    }
-    for (int r = 0; r < 5; ++r) {
-        int e = threadIdx.x + r * CH;
-        if (e < nb * nb) blocks[k * nb * nb + e] = make_double2(accr[r], acci[r]);
-    }
-}
-
+// ---- near field: FP32 copy and diagonal --------------------------------------------
 __global__ void helm_to_float_kernel(const double2* __restrict__ in, float2* __restrict__ out, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = make_float2((float)in[i].x, (float)in[i].y);
@@ -300,7 +86,8 @@ __global__ void helm_near_diag_kernel(int64_t N, int p, int ne1, const int64_t* 
 // ---- coupling matrices (stored, double-float complex) ------------------------------
 __global__ void helm_far_assemble_kernel(int64_t n_far, const int32_t* __restrict__ ftgt,
                                          const int32_t* __restrict__ fsrc, const double* __restrict__ igeo, int q2,
-                                         int kpt, double kappa, float4* __restrict__ K) {
+                                         int kpt, double kappa, const double2* __restrict__ trig,
+                                         float4* __restrict__ K) {
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t per = (int64_t)kpt * 4 * q2;
     if (idx >= n_far * per) return;
@@ -313,7 +100,7 @@ __global__ void helm_far_assemble_kernel(int64_t n_far, const int32_t* __restric
         const double* A = igeo + 4 * ((int64_t)ftgt[blk] * q2 + a);
         const double* B = igeo + 4 * ((int64_t)fsrc[blk] * q2 + b);
         double d0 = A[0] - B[0], d1 = A[1] - B[1], d2 = A[2] - B[2];
-        helm_kernel64(kappa, sqrt(d0 * d0 + d1 * d1 + d2 * d2), A[3] * B[3], &vr, &vi);
+        green64<true>(d0 * d0 + d1 * d1 + d2 * d2, kappa, A[3] * B[3] * (1.0 / (4.0 * IBEM_PI)), trig, &vr, &vi);
     }
     float rh = (float)vr, ih = (float)vi;
     K[idx] = make_float4(rh, (float)(vr - (double)rh), ih, (float)(vi - (double)ih));
@@ -565,42 +352,17 @@ __global__ void helm_join_vec_kernel(int R, int64_t n, const double* __restrict_
 // ---- host launchers ----------------------------------------------------------------------
 cudaError_t helm_launch_near_assembly(ibem_handle* h) {
     Plan& P = h->P;
-    GeomView g{h->d_patches, h->d_knots, h->d_cpw};
-    int QQ = P.Q * P.Q, nb = P.nb;
-    double kappa = P.prm.kappa;
+    const int nb = P.nb;
+    const double kappa = P.prm.kappa;
     cudaError_t e;
-    std::vector<double> gx, gw;
-    gauss_legendre(P.Q, gx, gw);
-    if ((e = cudaMemcpyToSymbolAsync(c_hgx, gx.data(), P.Q * sizeof(double), 0, cudaMemcpyHostToDevice, h->stream))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_hgw, gw.data(), P.Q * sizeof(double), 0, cudaMemcpyHostToDevice, h->stream))) return e;
     double2* blocks = reinterpret_cast<double2*>(h->d_near);
     for (int cls : {CLS_REGULAR, CLS_SUBDIV}) {
-        if (h->n_list[cls] > 0 && near_shared_bytes(P.Q, nb, true, cls == CLS_SUBDIV) > IBEM_MAX_SMEM_BYTES &&
+        if (h->n_list[cls] > 0 && near_streamed(P.Q, nb, true, cls == CLS_SUBDIV) &&
             (e = launch_near_stream(h, cls, true, kappa, h->d_near)))
             return e;
     }
     if ((e = launch_near_graded(h, true, kappa, h->d_near))) return e;
-    if (h->n_list[CLS_REGULAR] > 0 && near_shared_bytes(P.Q, nb, true, false) <= IBEM_MAX_SMEM_BYTES) {
-        size_t sm = (size_t)(8 * QQ + 2 * QQ * QQ + 2 * QQ * nb) * sizeof(double);
-        if ((e = cudaFuncSetAttribute(helm_near_regular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        helm_near_regular_kernel<<<(unsigned)h->n_list[CLS_REGULAR], 128, sm, h->stream>>>(
-            h->d_pairs_by_cls[CLS_REGULAR], h->d_near_tgt, h->d_near_src, h->d_qgeo, h->d_phi, QQ, nb, kappa, blocks);
-    }
-    if (h->n_list[CLS_SUBDIV] > 0 && near_shared_bytes(P.Q, nb, true, true) <= IBEM_MAX_SMEM_BYTES) {
-        size_t sm = (size_t)(32 * QQ + 2 * QQ * QQ + 2 * QQ * nb + 2 * nb * nb) * sizeof(double);
-        if ((e = cudaFuncSetAttribute(helm_near_subdiv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        helm_near_subdiv_kernel<<<(unsigned)h->n_list[CLS_SUBDIV], 128, sm, h->stream>>>(
-            g, h->d_pairs_by_cls[CLS_SUBDIV], h->d_near_tgt, h->d_near_src, h->d_phi_sub, P.Q, nb, P.ne1, kappa, blocks);
-    }
-    for (int c = 0; c < 3; ++c) {
-        if (h->n_list[c] == 0) continue;
-        const int CH = 128;
-        size_t sm = (size_t)3 * nb * CH * sizeof(double);
-        if ((e = cudaFuncSetAttribute(helm_near_singular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        helm_near_singular_kernel<<<(unsigned)h->n_list[c], CH, sm, h->stream>>>(
-            g, h->d_pairs_by_cls[c], h->d_near_tgt, h->d_near_src, h->d_near_orient, h->d_rule[c], h->rule_n[c], P.p,
-            P.ne1, kappa, blocks);
-    }
+    if ((e = launch_near_blocks(h, true, kappa, h->d_near))) return e;
     if ((e = cudaGetLastError())) return e;
     int64_t nn = P.n_near * nb * nb;
     helm_to_float_kernel<<<nblk(nn, 256), 256, 0, h->stream>>>(blocks, reinterpret_cast<float2*>(h->d_near32), nn);
@@ -615,7 +377,7 @@ cudaError_t helm_launch_far_assembly(ibem_handle* h) {
     int64_t total = h->n_up * (int64_t)h->kpt * 4 * P.q2;   // one of two mirrored blocks
     if (total == 0) return cudaSuccess;
     helm_far_assemble_kernel<<<nblk(total, 256), 256, 0, h->stream>>>(h->n_up, h->d_up_tgt, h->d_up_src, h->d_igeo,
-                                                                      P.q2, h->kpt, P.prm.kappa, h->d_Kc);
+                                                                      P.q2, h->kpt, P.prm.kappa, h->d_trig64, h->d_Kc);
     return cudaGetLastError();
 }
 

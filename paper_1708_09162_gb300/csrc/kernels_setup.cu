@@ -2,14 +2,8 @@
 // points, near-field Galerkin blocks in the Bernstein superspace, FMM coupling
 // matrices, the Jacobi diagonal.
 //
-// Near field (Sec. 3.2, Sec. 4.3, Sec. 4 item 4): for a near element pair
-// (t, s) the block
-//     B[i][j] = int_t int_s k(x) k(y) u*(F(x), F(y)) B_i(x) B_j(y) dy dx
-// of the (p+1)^2 Bernstein products B_i on each element.  Regular pairs use an
-// n x n Gauss rule per element (B = Phi^T G Phi with G[a][b] the weighted
-// kernel at Gauss point pairs), subdivided pairs the same on 2 x 2 sub-squares,
-// touching pairs the Duffy-type rules of the identical / common-edge /
-// common-vertex classes mapped through the pair's canonical orientation.
+// Near field: kernels_near.cu; here the streaming form of regular and subdivided
+// pairs for high Gauss orders and graded orders.
 //
 // Coupling (Sec. 4.2): K[a][b] = k(z_a) k(z_b) u*(F(z_a), F(z_b)) at the tensor
 // Chebyshev points of the target and source cluster, stored FP64 in the layout
@@ -82,121 +76,15 @@ __global__ void igeo_kernel(GeomView g, int64_t C, int m, int q, double* igeo, f
     o32[0] = (float)F[0]; o32[1] = (float)F[1]; o32[2] = (float)F[2]; o32[3] = (float)k;
 }
 
-// ---- near field: regular pairs --------------------------------------------
-// One CTA per pair.  Shared: XA[QQ][4], XB[QQ][4], G[QQ][QQ], H[QQ][nb].
-__global__ void near_regular_kernel(const int32_t* __restrict__ list, int64_t n,
-                                    const int32_t* __restrict__ tgt, const int32_t* __restrict__ src,
-                                    const double* __restrict__ qgeo, const double* __restrict__ phi,
-                                    int QQ, int nb, double* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    double* XA = sm;
-    double* XB = XA + 4 * QQ;
-    double* G = XB + 4 * QQ;
-    double* H = G + QQ * QQ;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    for (int i = threadIdx.x; i < 4 * QQ; i += blockDim.x) {
-        XA[i] = qgeo[4 * QQ * t + i];
-        XB[i] = qgeo[4 * QQ * s + i];
-    }
-    __syncthreads();
-    const double inv4pi = 1.0 / (4.0 * IBEM_PI);
-    for (int i = threadIdx.x; i < QQ * QQ; i += blockDim.x) {
-        int a = i / QQ, b = i % QQ;
-        double d0 = XA[4 * a] - XB[4 * b], d1 = XA[4 * a + 1] - XB[4 * b + 1], d2 = XA[4 * a + 2] - XB[4 * b + 2];
-        double r = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-        G[i] = XA[4 * a + 3] * XB[4 * b + 3] * inv4pi / r;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < QQ * nb; i += blockDim.x) {
-        int a = i / nb, j = i % nb;
-        double acc = 0.0;
-        for (int b = 0; b < QQ; ++b) acc += G[a * QQ + b] * phi[b * nb + j];
-        H[i] = acc;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
-        int r = i / nb, j = i % nb;
-        double acc = 0.0;
-        for (int a = 0; a < QQ; ++a) acc += phi[a * nb + r] * H[a * nb + j];
-        blocks[k * nb * nb + i] = acc;
-    }
-}
-
-// ---- near field: subdivided pairs (2 x 2 sub-squares of both elements) ------
-// Shared: XA[4][QQ][4], XB[4][QQ][4], G[QQ][QQ], H[QQ][nb], acc[nb][nb].
-__global__ void near_subdiv_kernel(GeomView g, const int32_t* __restrict__ list, int64_t n,
-                                   const int32_t* __restrict__ tgt, const int32_t* __restrict__ src,
-                                   const double* __restrict__ phi_sub, int Q, int nb, int ne1,
-                                   double* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    int QQ = Q * Q;
-    double* XA = sm;
-    double* XB = XA + 16 * QQ;
-    double* G = XB + 16 * QQ;
-    double* H = G + QQ * QQ;
-    double* acc = H + QQ * nb;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    double h = 1.0 / ne1;
-    for (int i = threadIdx.x; i < 8 * QQ; i += blockDim.x) {
-        int which = i / (4 * QQ);      // 0: target, 1: source
-        int r = i % (4 * QQ);
-        int sub = r / QQ, gq = r % QQ;
-        int patch, ix, iy;
-        dev_element_of(which ? s : t, ne1, &patch, &ix, &iy);
-        double su = 0.5 * (sub & 1) + 0.5 * c_gx[gq % Q];
-        double sv = 0.5 * (sub >> 1) + 0.5 * c_gx[gq / Q];
-        double F[3], Fu[3], Fv[3];
-        eval_patch(g, patch, (ix + su) * h, (iy + sv) * h, F, Fu, Fv);
-        double* o = (which ? XB : XA) + 4 * r;
-        o[0] = F[0]; o[1] = F[1]; o[2] = F[2];
-        o[3] = 0.25 * c_gw[gq % Q] * c_gw[gq / Q] * surface_measure(Fu, Fv) * h * h;
-    }
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) acc[i] = 0.0;
-    __syncthreads();
-    const double inv4pi = 1.0 / (4.0 * IBEM_PI);
-    for (int sa = 0; sa < 4; ++sa)
-        for (int sb = 0; sb < 4; ++sb) {
-            const double* A = XA + 4 * QQ * sa;
-            const double* B = XB + 4 * QQ * sb;
-            for (int i = threadIdx.x; i < QQ * QQ; i += blockDim.x) {
-                int a = i / QQ, b = i % QQ;
-                double d0 = A[4 * a] - B[4 * b], d1 = A[4 * a + 1] - B[4 * b + 1], d2 = A[4 * a + 2] - B[4 * b + 2];
-                G[i] = A[4 * a + 3] * B[4 * b + 3] * inv4pi / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-            }
-            __syncthreads();
-            const double* pb = phi_sub + (size_t)sb * QQ * nb;
-            for (int i = threadIdx.x; i < QQ * nb; i += blockDim.x) {
-                int a = i / nb, j = i % nb;
-                double v = 0.0;
-                for (int b = 0; b < QQ; ++b) v += G[a * QQ + b] * pb[b * nb + j];
-                H[i] = v;
-            }
-            __syncthreads();
-            const double* pa = phi_sub + (size_t)sa * QQ * nb;
-            for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) {
-                int r = i / nb, j = i % nb;
-                double v = 0.0;
-                for (int a = 0; a < QQ; ++a) v += pa[a * nb + r] * H[a * nb + j];
-                acc[i] += v;
-            }
-            __syncthreads();
-        }
-    for (int i = threadIdx.x; i < nb * nb; i += blockDim.x) blocks[k * nb * nb + i] = acc[i];
-}
-
 // ---- near field: regular and subdivided pairs, streaming form -------------
-// For Gauss orders whose Q^2 x Q^2 kernel matrix does not fit in shared memory
-// (the forms above keep it there).  One CTA of NS_T threads per pair; for each
+// For Gauss orders above those of near_product_kernel (near_streamed).  One CTA of NS_T threads per pair; for each
 // pair of point sets (the elements themselves, or each of the 2 x 2 x 2 x 2
 // sub-square pairs) the CTA walks the target points in chunks of NS_T: thread t
 // forms H[a][j] = sum_b G(a, b) phi_B[b][j] for its target point a in
 // registers (G = w_a w_b u*(x_a, y_b), complex for Helmholtz), the chunk is
 // stored in shared memory, and the block entries B[r][j] += sum_a phi_A[a][r]
 // H[a][j] are accumulated by their owning threads (entry e = t + NS_T i).
-// The same sums as the shared-matrix forms, in the same order over b for each
-// H[a][j]; the sum over a runs chunk by chunk.  Shared: XA[QQ][4], XB[QQ][4],
+// The sum over a runs chunk by chunk.  Shared: XA[QQ][4], XB[QQ][4],
 // H[NS_T][NB] (real and imaginary parts for Helmholtz).
 constexpr int NS_T = 128;
 
@@ -411,85 +299,6 @@ cudaError_t launch_near_stream(ibem_handle* h, int cls, bool cplx, double kappa,
     return cplx ? launch_near_stream_t<true>(h, cls, kappa, blocks) : launch_near_stream_t<false>(h, cls, kappa, blocks);
 }
 
-size_t near_shared_bytes(int Q, int nb, bool cplx, bool subdiv) {
-    const size_t QQ = (size_t)Q * Q, cw = cplx ? 2 : 1;
-    return (subdiv ? 32 * QQ + cw * QQ * QQ + cw * QQ * nb + cw * nb * nb : 8 * QQ + cw * QQ * QQ + cw * QQ * nb) *
-           sizeof(double);
-}
-
-// ---- near field: touching pairs (Duffy-type rules) -------------------------
-// The rule's canonical points (x^, y^) are mapped by rho_{kA} and rho_{kB} into
-// the element-local squares.  Points are processed in chunks of blockDim.x.
-// Shared: SA[nb][CH], SB[nb][CH].
-__global__ void near_singular_kernel(GeomView g, const int32_t* __restrict__ list, int64_t n,
-                                     const int32_t* __restrict__ tgt, const int32_t* __restrict__ src,
-                                     const int32_t* __restrict__ orient, const double* __restrict__ rule,
-                                     int npts, int p, int ne1, double* __restrict__ blocks) {
-    extern __shared__ double sm[];
-    const int CH = blockDim.x;
-    const int pp = p + 1, nb = pp * pp;
-    double* SA = sm;
-    double* SB = SA + nb * CH;
-    int64_t k = list[blockIdx.x];
-    int64_t t = tgt[k], s = src[k];
-    int ka = orient[k] >> 3, kb = orient[k] & 7;
-    int pa, ixa, iya, pb, ixb, iyb;
-    dev_element_of(t, ne1, &pa, &ixa, &iya);
-    dev_element_of(s, ne1, &pb, &ixb, &iyb);
-    double h = 1.0 / ne1;
-    const double scale = h * h * h * h / (4.0 * IBEM_PI);
-    double acc[5] = {0, 0, 0, 0, 0};   // nb * nb <= 625 <= 5 * 128 entries per thread
-    for (int base = 0; base < npts; base += CH) {
-        int ip = base + threadIdx.x;
-        if (ip < npts) {
-            double x1 = rule[ip], x2 = rule[npts + ip], y1 = rule[2 * npts + ip], y2 = rule[3 * npts + ip];
-            double w = rule[4 * npts + ip];
-            double xa, ya, xb, yb;
-            dihedral(ka, x1, x2, &xa, &ya);
-            dihedral(kb, y1, y2, &xb, &yb);
-            double FA[3], FB[3], Fu[3], Fv[3];
-            eval_patch(g, pa, (ixa + xa) * h, (iya + ya) * h, FA, Fu, Fv);
-            double kA = surface_measure(Fu, Fv);
-            eval_patch(g, pb, (ixb + xb) * h, (iyb + yb) * h, FB, Fu, Fv);
-            double kB = surface_measure(Fu, Fv);
-            double d0 = FA[0] - FB[0], d1 = FA[1] - FB[1], d2 = FA[2] - FB[2];
-            double val = w * scale * kA * kB / sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-            double bxu[IBEM_MAX_P + 1], bxv[IBEM_MAX_P + 1], byu[IBEM_MAX_P + 1], byv[IBEM_MAX_P + 1];
-            bernstein(p, xa, bxu);
-            bernstein(p, ya, bxv);
-            bernstein(p, xb, byu);
-            bernstein(p, yb, byv);
-            for (int iv = 0; iv < pp; ++iv)
-                for (int iu = 0; iu < pp; ++iu) {
-                    SA[(iv * pp + iu) * CH + threadIdx.x] = val * bxu[iu] * bxv[iv];
-                    SB[(iv * pp + iu) * CH + threadIdx.x] = byu[iu] * byv[iv];
-                }
-        } else {
-            for (int i = 0; i < nb; ++i) {
-                SA[i * CH + threadIdx.x] = 0.0;
-                SB[i * CH + threadIdx.x] = 0.0;
-            }
-        }
-        __syncthreads();
-        for (int r = 0; r < 5; ++r) {
-            int e = threadIdx.x + r * CH;
-            if (e < nb * nb) {
-                int i = e / nb, j = e % nb;
-                const double* a = SA + i * CH;
-                const double* b = SB + j * CH;
-                double v = 0.0;
-                for (int c = 0; c < CH; ++c) v += a[c] * b[c];
-                acc[r] += v;
-            }
-        }
-        __syncthreads();
-    }
-    for (int r = 0; r < 5; ++r) {
-        int e = threadIdx.x + r * CH;
-        if (e < nb * nb) blocks[k * nb * nb + e] = acc[r];
-    }
-}
-
 // ---- far field: coupling matrices -----------------------------------------
 // Stored as doubles (native) or as float pairs hi = fl(K), lo = fl(K - hi).
 __global__ void far_assemble_kernel(int64_t n_far, const int32_t* __restrict__ ftgt,
@@ -594,49 +403,15 @@ cudaError_t launch_geometry_tables(ibem_handle* h) {
 
 cudaError_t launch_near_assembly(ibem_handle* h) {
     Plan& P = h->P;
-    GeomView g{h->d_patches, h->d_knots, h->d_cpw};
-    int QQ = P.Q * P.Q, nb = P.nb;
+    const int nb = P.nb;
     cudaError_t e;
-    // the Gauss rule is module-wide: load this handle's before the subdivided pairs use it
-    {
-        std::vector<double> gx, gw;
-        gauss_legendre(P.Q, gx, gw);
-        if ((e = cudaMemcpyToSymbolAsync(c_gx, gx.data(), P.Q * sizeof(double), 0, cudaMemcpyHostToDevice,
-                                         h->stream)) ||
-            (e = cudaMemcpyToSymbolAsync(c_gw, gw.data(), P.Q * sizeof(double), 0, cudaMemcpyHostToDevice,
-                                         h->stream)))
-            return e;
-    }
     for (int cls : {CLS_REGULAR, CLS_SUBDIV}) {
-        if (h->n_list[cls] > 0 && near_shared_bytes(P.Q, nb, false, cls == CLS_SUBDIV) > IBEM_MAX_SMEM_BYTES &&
+        if (h->n_list[cls] > 0 && near_streamed(P.Q, nb, false, cls == CLS_SUBDIV) &&
             (e = launch_near_stream(h, cls, false, 0.0, h->d_near)))
             return e;
     }
     if ((e = launch_near_graded(h, false, 0.0, h->d_near))) return e;
-    // regular
-    if (h->n_list[CLS_REGULAR] > 0 && near_shared_bytes(P.Q, nb, false, false) <= IBEM_MAX_SMEM_BYTES) {
-        size_t sm = (size_t)(8 * QQ + QQ * QQ + QQ * nb) * sizeof(double);
-        if ((e = cudaFuncSetAttribute(near_regular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        near_regular_kernel<<<(unsigned)h->n_list[CLS_REGULAR], 128, sm, h->stream>>>(
-            h->d_pairs_by_cls[CLS_REGULAR], h->n_list[CLS_REGULAR], h->d_near_tgt, h->d_near_src, h->d_qgeo,
-            h->d_phi, QQ, nb, h->d_near);
-    }
-    if (h->n_list[CLS_SUBDIV] > 0 && near_shared_bytes(P.Q, nb, false, true) <= IBEM_MAX_SMEM_BYTES) {
-        size_t sm = (size_t)(32 * QQ + QQ * QQ + QQ * nb + nb * nb) * sizeof(double);
-        if ((e = cudaFuncSetAttribute(near_subdiv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        near_subdiv_kernel<<<(unsigned)h->n_list[CLS_SUBDIV], 128, sm, h->stream>>>(
-            g, h->d_pairs_by_cls[CLS_SUBDIV], h->n_list[CLS_SUBDIV], h->d_near_tgt, h->d_near_src, h->d_phi_sub,
-            P.Q, nb, P.ne1, h->d_near);
-    }
-    for (int c = 0; c < 3; ++c) {
-        if (h->n_list[c] == 0) continue;
-        const int CH = 128;
-        size_t sm = (size_t)2 * nb * CH * sizeof(double);
-        if ((e = cudaFuncSetAttribute(near_singular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-        near_singular_kernel<<<(unsigned)h->n_list[c], CH, sm, h->stream>>>(
-            g, h->d_pairs_by_cls[c], h->n_list[c], h->d_near_tgt, h->d_near_src, h->d_near_orient, h->d_rule[c],
-            h->rule_n[c], P.p, P.ne1, h->d_near);
-    }
+    if ((e = launch_near_blocks(h, false, 0.0, h->d_near))) return e;
     if ((e = cudaGetLastError())) return e;
     int64_t nn = P.n_near * nb * nb;
     to_float_kernel<<<nblk(nn, 256), 256, 0, h->stream>>>(h->d_near, h->d_near32, nn);

@@ -106,72 +106,6 @@ static int64_t cluster_id(const Plan& P, int patch, int level, int ix, int iy) {
     return P.level_off[level] + (int64_t)patch * ((int64_t)1 << (2 * level)) + morton2(ix, iy);
 }
 
-void singular_rule(int cls, int n, std::vector<double>& soa) {
-    std::vector<double> g, w;
-    gauss_legendre(n, g, w);
-    std::vector<double> X1, X2, Y1, Y2, W;
-    auto split = [](double z, double s, int o, double* x, double* y) {
-        double a = (1.0 - z) * s;
-        if (o == 0) { *x = a; *y = a + z; } else { *x = a + z; *y = a; }
-    };
-    for (int i0 = 0; i0 < n; ++i0)
-        for (int i1 = 0; i1 < n; ++i1)
-            for (int i2 = 0; i2 < n; ++i2)
-                for (int i3 = 0; i3 < n; ++i3) {
-                    double xi = g[i0], e1 = g[i1], e2 = g[i2], e3 = g[i3];
-                    double Wq = w[i0] * w[i1] * w[i2] * w[i3];
-                    if (cls == CLS_IDENTICAL) {
-                        // e1 = eta, e2 = s1, e3 = s2
-                        for (int tri = 0; tri < 2; ++tri) {
-                            double z1 = tri == 0 ? xi : xi * e1;
-                            double z2 = tri == 0 ? xi * e1 : xi;
-                            for (int o1 = 0; o1 < 2; ++o1)
-                                for (int o2 = 0; o2 < 2; ++o2) {
-                                    double x1, y1, x2, y2;
-                                    split(z1, e2, o1, &x1, &y1);
-                                    split(z2, e3, o2, &x2, &y2);
-                                    X1.push_back(x1); X2.push_back(x2);
-                                    Y1.push_back(y1); Y2.push_back(y2);
-                                    W.push_back(Wq * xi * (1.0 - z1) * (1.0 - z2));
-                                }
-                        }
-                    } else if (cls == CLS_EDGE) {
-                        // pyramids of the cube (x1, y1, z); e3 = s along the edge
-                        for (int pyr = 0; pyr < 3; ++pyr) {
-                            double x1, y1, z;
-                            if (pyr == 0) { x1 = xi; y1 = xi * e1; z = xi * e2; }
-                            else if (pyr == 1) { x1 = xi * e1; y1 = xi; z = xi * e2; }
-                            else { x1 = xi * e1; y1 = xi * e2; z = xi; }
-                            for (int o = 0; o < 2; ++o) {
-                                double x2, y2;
-                                split(z, e3, o, &x2, &y2);
-                                X1.push_back(x1); X2.push_back(x2);
-                                Y1.push_back(y1); Y2.push_back(y2);
-                                W.push_back(Wq * xi * xi * (1.0 - z));
-                            }
-                        }
-                    } else {
-                        // pyramids of the 4-cube (x1, x2, y1, y2)
-                        for (int pyr = 0; pyr < 4; ++pyr) {
-                            double c[4];
-                            double rest[3] = {xi * e1, xi * e2, xi * e3};
-                            int k = 0;
-                            for (int d = 0; d < 4; ++d) c[d] = (d == pyr) ? xi : rest[k++];
-                            X1.push_back(c[0]); X2.push_back(c[1]);
-                            Y1.push_back(c[2]); Y2.push_back(c[3]);
-                            W.push_back(Wq * xi * xi * xi);
-                        }
-                    }
-                }
-    size_t np = W.size();
-    soa.resize(5 * np);
-    std::copy(X1.begin(), X1.end(), soa.begin());
-    std::copy(X2.begin(), X2.end(), soa.begin() + np);
-    std::copy(Y1.begin(), Y1.end(), soa.begin() + 2 * np);
-    std::copy(Y2.begin(), Y2.end(), soa.begin() + 3 * np);
-    std::copy(W.begin(), W.end(), soa.begin() + 4 * np);
-}
-
 namespace {
 
 struct Ball { double c[3]; double r; };
