@@ -16,7 +16,7 @@
 //
 // Kernels: inference in BF16 (the preconditioner, ibem_cnn_forward) runs all
 // four layers on the tensor cores (tcgen05 implicit GEMM, conv_tc_kernel).
-// Training and the FP32 mode use one tiled direct convolution (16 x 16 output
+// Training and the FP32 mode use one tiled direct convolution (12 x 36 output
 // pixels of one image and 16 output channels per CTA, input halo tile and
 // weights staged in shared memory, FP32 FMA) for the forward pass and, with
 // flipped transposed weights and the ReLU mask fused, the input gradient; the
@@ -63,7 +63,7 @@ struct ibem_cnn {
     void* d_wtc = nullptr;       // BF16 tensor-core weight tiles of the four layers
     size_t wtc_bytes = 0;
     int* d_status = nullptr;     // device-side wait status of the tensor-core layers
-    double* d_red = nullptr;     // [0] loss, [1] |s|^2, [2] loss sum of an epoch
+    double* d_red = nullptr;     // [0] loss, [1] |s|^2, [2] loss sum of an epoch, [8..] partial sums of the loss
     int coarse = 1;              // coarsening factor f of the preconditioner's images (1: the fine grid)
     float* d_cimg = nullptr;     // coarse images of the preconditioner
     size_t cimg_floats = 0;
@@ -75,9 +75,16 @@ namespace ibem {
 
 namespace {
 
-constexpr int TS = 16;        // output tile side
-constexpr int CIB = 8;        // input channels per shared-memory stage
-constexpr int WG_ITEMS = 256; // CTAs along the pixel axis of the weight gradient
+// Tiles of the FMA kernels, in pixels.  The images have 2^m + p pixels a side: 12 x
+// 36 (and 12 x 18) leaves 6 to 12% of a tile outside the image at 34, 66 and 130,
+// 16 x 16 between 23% and 99%.
+constexpr int TY = 12, TX = 36;
+constexpr int CT_T = TY * TX / 2;   // threads of the convolution: two pixels each
+constexpr int CIB = 8;              // input channels per shared-memory stage
+constexpr int GX = 18;              // width of the weight gradient's tile (height TY)
+constexpr int GP = TY * GX;
+constexpr int WG_ITEMS = 304;       // CTAs along the pixel axis of the weight gradient: two per SM
+constexpr int LOSS_CTAS = 152;
 
 inline unsigned cblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -92,33 +99,36 @@ __device__ inline float wq(float w, int bf) { return bf ? __bfloat162float(__flo
 // out[b][co][y][x] = bias[co] + sum_ci sum_k w[co][ci][k] in[b][ci][y + dy - 1][x + dx - 1]
 // (k = 3 dy + dx), then ReLU if relu, then zeroed where mask[b][co][y][x] <= 0
 // if mask is given.  Grid: (tiles of the image, ceil(Cout / COB), B).
+// Bound: FP32 FMA.  A thread holds two pixels, 18 columns apart, of COB channels, so
+// that one read of a tap's weights from shared memory serves 2 COB FMA (with one
+// pixel the reads took longer than the FMA): 96 images of 34 x 34, the four
+// forward layers 232 us instead of 421, the three input gradients 226 instead of 390.
 template <typename TI, typename TO, typename TM, int COB>
-__global__ void __launch_bounds__(256) conv_tile_kernel(const TI* __restrict__ in, int Cin, int H, int W,
-                                                        const float* __restrict__ w,
-                                                        const float* __restrict__ bias, int Cout, int relu, int bf,
-                                                        const TM* __restrict__ mask, TO* __restrict__ out) {
-    __shared__ float s_in[CIB][TS + 2][TS + 2];
+__global__ void __launch_bounds__(CT_T) conv_tile_kernel(const TI* __restrict__ in, int Cin, int H, int W,
+                                                         const float* __restrict__ w,
+                                                         const float* __restrict__ bias, int Cout, int relu, int bf,
+                                                         const TM* __restrict__ mask, TO* __restrict__ out) {
+    __shared__ float s_in[CIB][TY + 2][TX + 2];
     __shared__ __align__(16) float s_w[CIB][9][COB];
-    const int tiles_x = (W + TS - 1) / TS;
-    const int ty0 = (blockIdx.x / tiles_x) * TS, tx0 = (blockIdx.x % tiles_x) * TS;
+    const int tiles_x = (W + TX - 1) / TX;
+    const int ty0 = (blockIdx.x / tiles_x) * TY, tx0 = (blockIdx.x % tiles_x) * TX;
     const int co0 = blockIdx.y * COB;
     const int64_t b = blockIdx.z;
-    const int t = threadIdx.x, py = t / TS, px = t % TS;
-    const int y = ty0 + py, x = tx0 + px;
+    const int t = threadIdx.x, py = t / (TX / 2), px = t % (TX / 2);
     const int64_t HW = (int64_t)H * W;
-    float acc[COB];
+    float acc[2][COB];
 #pragma unroll
-    for (int c = 0; c < COB; ++c) acc[c] = (bias && co0 + c < Cout) ? bias[co0 + c] : 0.0f;
+    for (int c = 0; c < COB; ++c) acc[0][c] = acc[1][c] = (bias && co0 + c < Cout) ? bias[co0 + c] : 0.0f;
     for (int ci0 = 0; ci0 < Cin; ci0 += CIB) {
-        for (int i = t; i < CIB * (TS + 2) * (TS + 2); i += 256) {
-            const int c = i / ((TS + 2) * (TS + 2)), r = i % ((TS + 2) * (TS + 2));
-            const int yy = ty0 - 1 + r / (TS + 2), xx = tx0 - 1 + r % (TS + 2);
+        for (int i = t; i < CIB * (TY + 2) * (TX + 2); i += CT_T) {
+            const int c = i / ((TY + 2) * (TX + 2)), r = i % ((TY + 2) * (TX + 2));
+            const int yy = ty0 - 1 + r / (TX + 2), xx = tx0 - 1 + r % (TX + 2);
             float v = 0.0f;
             if (ci0 + c < Cin && yy >= 0 && yy < H && xx >= 0 && xx < W)
                 v = ld_act(in, (b * Cin + ci0 + c) * HW + (int64_t)yy * W + xx);
-            s_in[c][r / (TS + 2)][r % (TS + 2)] = v;
+            s_in[c][r / (TX + 2)][r % (TX + 2)] = v;
         }
-        for (int i = t; i < CIB * 9 * COB; i += 256) {
+        for (int i = t; i < CIB * 9 * COB; i += CT_T) {
             const int co = i % COB, k = (i / COB) % 9, c = i / (9 * COB);
             float v = 0.0f;
             if (ci0 + c < Cin && co0 + co < Cout) v = wq(w[((int64_t)(co0 + co) * Cin + ci0 + c) * 9 + k], bf);
@@ -127,25 +137,33 @@ __global__ void __launch_bounds__(256) conv_tile_kernel(const TI* __restrict__ i
         __syncthreads();
         const int cmax = min(CIB, Cin - ci0);
         for (int c = 0; c < cmax; ++c) {
-            float v[9];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) v[k] = s_in[c][py + k / 3][px + k % 3];
+            for (int k = 0; k < 9; ++k) {
+                const float v0 = s_in[c][py + k / 3][px + k % 3], v1 = s_in[c][py + k / 3][px + TX / 2 + k % 3];
 #pragma unroll
-            for (int k = 0; k < 9; ++k)
-#pragma unroll
-                for (int co = 0; co < COB; ++co) acc[co] = fmaf(s_w[c][k][co], v[k], acc[co]);
+                for (int co = 0; co < COB; ++co) {
+                    const float wv = s_w[c][k][co];
+                    acc[0][co] = fmaf(wv, v0, acc[0][co]);
+                    acc[1][co] = fmaf(wv, v1, acc[1][co]);
+                }
+            }
         }
         __syncthreads();
     }
-    if (y >= H || x >= W) return;
+    const int y = ty0 + py;
 #pragma unroll
-    for (int co = 0; co < COB; ++co) {
-        if (co0 + co >= Cout) break;
-        float r = acc[co];
-        if (relu && r < 0.0f) r = 0.0f;
-        const int64_t o = (b * Cout + co0 + co) * HW + (int64_t)y * W + x;
-        if (mask && !(ld_act(mask, o) > 0.0f)) r = 0.0f;
-        st_act(out, o, r);
+    for (int q = 0; q < 2; ++q) {
+        const int x = tx0 + px + q * (TX / 2);
+        if (y >= H || x >= W) continue;
+#pragma unroll
+        for (int co = 0; co < COB; ++co) {
+            if (co0 + co >= Cout) break;
+            float r = acc[q][co];
+            if (relu && r < 0.0f) r = 0.0f;
+            const int64_t o = (b * Cout + co0 + co) * HW + (int64_t)y * W + x;
+            if (mask && !(ld_act(mask, o) > 0.0f)) r = 0.0f;
+            st_act(out, o, r);
+        }
     }
 }
 
@@ -385,120 +403,150 @@ __global__ void flip_weights_kernel(const float* __restrict__ w, int Cin, int Co
     wt[i] = wq(w[((int64_t)co * Cin + ci) * 9 + (8 - k)], bf);
 }
 
-// Partial weight gradients: CTA (x, y) sums, over its range of (image, tile)
-// items, g[b][co][pix] * in[b][ci][pix + tap] for co < Cout (<= 32), the 8
-// input channels of chunk y and the 9 taps; thread = (ci within chunk, co).
+// Partial weight and bias gradients: a CTA sums, over its range of (image, tile) items,
+// g[b][co][pix] * in[b][ci][pix + tap] for all co < Cout, ci < Cin (<= 32 each) and the 9
+// taps, and g[b][co][pix].  Thread = (ci, 4 channels co): per pixel one 16-byte read of
+// g (shared by the 32 values of ci) and three new input values feed 36 FMA, so
+// the FMA pipe bounds it (9 FMA per four reads before: 458 us for the four layers of
+// 96 images of 34 x 34, and 484 us for the bias sums in kernels of their own; now
+// 274 us for both).  part: [rows][Cout * Cin * 9 + Cout].
 template <typename T>
 __global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict__ g, const T* __restrict__ in, int B,
                                                          int Cin, int H, int W, int Cout, int items_per_cta,
                                                          float* __restrict__ part) {
-    __shared__ float s_g[32][TS * TS + 1];
-    __shared__ float s_in[CIB][TS + 2][TS + 2];
-    const int tiles_x = (W + TS - 1) / TS, tiles = tiles_x * ((H + TS - 1) / TS);
+    extern __shared__ __align__(16) float wg_sm[];
+    float4* s_g = reinterpret_cast<float4*>(wg_sm);                    // [GP][8]: 4 channels each
+    float* s_in = wg_sm + GP * 32;                                     // [32][TY + 2][GX + 2]
+    constexpr int RW = GX + 2, PL = (TY + 2) * RW + 1;                 // odd plane stride: no bank conflicts over ci
+    const int tiles_x = (W + GX - 1) / GX, tiles = tiles_x * ((H + TY - 1) / TY);
     const int64_t HW = (int64_t)H * W;
-    const int t = threadIdx.x, co = t % 32, c = t / 32;
-    const int ci0 = blockIdx.y * CIB;
+    const int t = threadIdx.x, cq = t & 7, ci = t >> 3;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
     const int64_t it1 = min((int64_t)B * tiles, it0 + items_per_cta);
-    float acc[9];
+    float acc[4][9], bsum[4];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
+    for (int c = 0; c < 4; ++c) {
+        bsum[c] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[c][k] = 0.0f;
+    }
+    const bool wact = ci < Cin && 4 * cq < Cout;
     for (int64_t item = it0; item < it1; ++item) {
         const int64_t b = item / tiles;
         const int tile = (int)(item % tiles);
-        const int ty0 = (tile / tiles_x) * TS, tx0 = (tile % tiles_x) * TS;
-        for (int i = t; i < Cout * TS * TS; i += 256) {
-            const int o = i / (TS * TS), pix = i % (TS * TS);
-            const int yy = ty0 + pix / TS, xx = tx0 + pix % TS;
-            s_g[o][pix] = (yy < H && xx < W) ? g[(b * Cout + o) * HW + (int64_t)yy * W + xx] : 0.0f;
+        const int ty0 = (tile / tiles_x) * TY, tx0 = (tile % tiles_x) * GX;
+        for (int i = t; i < 32 * GP; i += 256) {
+            const int o = i / GP, pix = i - o * GP, yy = ty0 + pix / GX, xx = tx0 + pix % GX;
+            reinterpret_cast<float*>(s_g)[pix * 32 + o] =
+                (o < Cout && yy < H && xx < W) ? g[(b * Cout + o) * HW + (int64_t)yy * W + xx] : 0.0f;
         }
-        for (int i = t; i < CIB * (TS + 2) * (TS + 2); i += 256) {
-            const int cc = i / ((TS + 2) * (TS + 2)), r = i % ((TS + 2) * (TS + 2));
-            const int yy = ty0 - 1 + r / (TS + 2), xx = tx0 - 1 + r % (TS + 2);
+        for (int i = t; i < Cin * (TY + 2) * RW; i += 256) {
+            const int c = i / ((TY + 2) * RW), r = i - c * (TY + 2) * RW;
+            const int yy = ty0 - 1 + r / RW, xx = tx0 - 1 + r % RW;
             float v = 0.0f;
-            if (ci0 + cc < Cin && yy >= 0 && yy < H && xx >= 0 && xx < W)
-                v = ld_act(in, (b * Cin + ci0 + cc) * HW + (int64_t)yy * W + xx);
-            s_in[cc][r / (TS + 2)][r % (TS + 2)] = v;
+            if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = ld_act(in, (b * Cin + c) * HW + (int64_t)yy * W + xx);
+            s_in[c * PL + r] = v;
         }
         __syncthreads();
-        if (co < Cout && ci0 + c < Cin) {
-            for (int py = 0; py < TS; ++py) {
+        if (wact) {
+            const float* base = s_in + ci * PL;
+            for (int py = 0; py < TY; ++py) {
                 // 3 x 3 window slid along the row: three new values per pixel
                 float w0[3], w1[3];
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
-                    w0[dy] = s_in[c][py + dy][0];
-                    w1[dy] = s_in[c][py + dy][1];
+                    w0[dy] = base[(py + dy) * RW];
+                    w1[dy] = base[(py + dy) * RW + 1];
                 }
-                for (int px = 0; px < TS; ++px) {
-                    float w2[3];
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) w2[dy] = s_in[c][py + dy][px + 2];
-                    const float gv = s_g[co][py * TS + px];
+#pragma unroll 6
+                for (int px = 0; px < GX; ++px) {
+                    const float4 gv = s_g[(py * GX + px) * 8 + cq];
+                    const float gc[4] = {gv.x, gv.y, gv.z, gv.w};
 #pragma unroll
                     for (int dy = 0; dy < 3; ++dy) {
-                        acc[dy * 3 + 0] = fmaf(gv, w0[dy], acc[dy * 3 + 0]);
-                        acc[dy * 3 + 1] = fmaf(gv, w1[dy], acc[dy * 3 + 1]);
-                        acc[dy * 3 + 2] = fmaf(gv, w2[dy], acc[dy * 3 + 2]);
+                        const float w2 = base[(py + dy) * RW + px + 2];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            acc[c][dy * 3 + 0] = fmaf(gc[c], w0[dy], acc[c][dy * 3 + 0]);
+                            acc[c][dy * 3 + 1] = fmaf(gc[c], w1[dy], acc[c][dy * 3 + 1]);
+                            acc[c][dy * 3 + 2] = fmaf(gc[c], w2, acc[c][dy * 3 + 2]);
+                        }
                         w0[dy] = w1[dy];
-                        w1[dy] = w2[dy];
+                        w1[dy] = w2;
                     }
+                    if (ci == 0)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) bsum[c] += gc[c];
                 }
             }
         }
         __syncthreads();
     }
-    if (co < Cout && ci0 + c < Cin) {
-        float* dst = part + (int64_t)blockIdx.x * Cout * Cin * 9 + ((int64_t)co * Cin + ci0 + c) * 9;
+    if (wact) {
+        float* dst = part + (int64_t)blockIdx.x * (Cout * Cin * 9 + Cout);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dst[k] = acc[k];
+        for (int c = 0; c < 4; ++c) {
+            const int co = 4 * cq + c;
+            if (co >= Cout) break;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) dst[((int64_t)co * Cin + ci) * 9 + k] = acc[c][k];
+            if (ci == 0) dst[Cout * Cin * 9 + co] = bsum[c];
+        }
     }
 }
+constexpr size_t WG_SMEM = ((size_t)GP * 32 + (size_t)32 * ((TY + 2) * (GX + 2) + 1)) * sizeof(float);
 
-// gw[i] = sum over rows r (in order) of part[r][i]
-__global__ void sum_rows_kernel(const float* __restrict__ part, int rows, int n, float* __restrict__ gw) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// out[i] = sum over rows r of part[r][i]: a CTA takes 32 columns, its 8 warps every
+// eighth row each, combined in order; columns below nw go to gw, the others to gb
+__global__ void __launch_bounds__(256) sum_rows_kernel(const float* __restrict__ part, int rows, int n, int nw,
+                                                       float* __restrict__ gw, float* __restrict__ gb) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     float s = 0.0f;
-    for (int r = 0; r < rows; ++r) s += part[(int64_t)r * n + i];
-    gw[i] = s;
-}
-
-// gb[co] = sum over b and pixels of g[b][co][.]; one CTA per channel
-__global__ void bias_grad_kernel(const float* __restrict__ g, int B, int Cout, int64_t HW, float* __restrict__ gb) {
-    __shared__ float red[256];
-    const int co = blockIdx.x;
-    float s = 0.0f;
-    for (int64_t i = threadIdx.x; i < (int64_t)B * HW; i += blockDim.x) s += g[((i / HW) * Cout + co) * HW + i % HW];
-    red[threadIdx.x] = s;
+    if (i < n)
+#pragma unroll 4
+        for (int r = wid; r < rows; r += 8) s += part[(int64_t)r * n + i];
+    red[wid][lane] = s;
     __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-        __syncthreads();
+    if (wid == 0 && i < n) {
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v += red[k][lane];
+        if (i < nw) gw[i] = v;
+        else gb[i - nw] = v;
     }
-    if (threadIdx.x == 0) gb[co] = red[0];
 }
 
-// g = (out - target) / B; loss[0] = 1/(2B) sum (out - target)^2; loss[2] += B * loss[0]
+// g = (out - target) / B and the CTAs' partial sums of (out - target)^2; loss_sum_kernel
+// then gives loss[0] = 1/(2B) sum (out - target)^2 and loss[2] += B * loss[0]
 template <typename T>
-__global__ void loss_kernel(int64_t n, int B, const T* __restrict__ out, const float* __restrict__ target,
-                            float* __restrict__ g, double* __restrict__ loss) {
-    __shared__ double red[1024];
+__global__ void __launch_bounds__(256) loss_kernel(int64_t n, int B, const T* __restrict__ out,
+                                                   const float* __restrict__ target, float* __restrict__ g,
+                                                   double* __restrict__ part) {
+    __shared__ double red[8];
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const float d = ld_act(out, i) - target[i];
         g[i] = d / B;
         acc += (double)d * d;
     }
-    red[threadIdx.x] = acc;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-        __syncthreads();
-    }
     if (threadIdx.x == 0) {
-        loss[0] = red[0] / (2.0 * B);
-        loss[2] += red[0] / 2.0;
+        double v = 0.0;
+        for (int k = 0; k < 8; ++k) v += red[k];
+        part[blockIdx.x] = v;
+    }
+}
+
+__global__ void loss_sum_kernel(int n, int B, const double* __restrict__ part, double* __restrict__ loss) {
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32) acc += part[i];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0) {
+        loss[0] = acc / (2.0 * B);
+        loss[2] += acc / 2.0;
     }
 }
 
@@ -648,13 +696,13 @@ cudaError_t ensure_buffers(ibem_cnn* c, int B, int H, int W) {
 template <typename TI, typename TO, typename TM>
 void launch_conv(ibem_cnn* c, const TI* in, int B, int Cin, int H, int W, const float* w, const float* bias, int Cout,
                  int relu, int bf, const TM* mask, TO* out) {
-    const int tiles = ((H + TS - 1) / TS) * ((W + TS - 1) / TS);
+    const int tiles = ((H + TY - 1) / TY) * ((W + TX - 1) / TX);
     if (Cout <= 4) {
         dim3 grid(tiles, 1, B);
-        conv_tile_kernel<TI, TO, TM, 4><<<grid, 256, 0, c->stream>>>(in, Cin, H, W, w, bias, Cout, relu, bf, mask, out);
+        conv_tile_kernel<TI, TO, TM, 4><<<grid, CT_T, 0, c->stream>>>(in, Cin, H, W, w, bias, Cout, relu, bf, mask, out);
     } else {
         dim3 grid(tiles, (Cout + 15) / 16, B);
-        conv_tile_kernel<TI, TO, TM, 16><<<grid, 256, 0, c->stream>>>(in, Cin, H, W, w, bias, Cout, relu, bf, mask, out);
+        conv_tile_kernel<TI, TO, TM, 16><<<grid, CT_T, 0, c->stream>>>(in, Cin, H, W, w, bias, Cout, relu, bf, mask, out);
     }
     ++c->launches;
 }
@@ -752,29 +800,32 @@ cudaError_t backward(ibem_cnn* c, const float* target, int B, int H, int W, int 
     float* g1 = c->d_gbuf + per;
     float* g2 = c->d_gbuf;
     const int64_t HW = (int64_t)H * W;
-    const int tiles = ((H + TS - 1) / TS) * ((W + TS - 1) / TS);
+    const int tiles = ((H + TY - 1) / TY) * ((W + GX - 1) / GX);
     const int64_t items = (int64_t)B * tiles;
-    const int nx = (int)std::min<int64_t>(items, WG_ITEMS);
-    const int ipc = (int)((items + nx - 1) / nx);
+    const int ipc = (int)((items + WG_ITEMS - 1) / WG_ITEMS);
+    const int nx = (int)((items + ipc - 1) / ipc);
     cudaError_t e;
     size_t maxw = 0;
-    for (int l = 0; l < c->L; ++l) maxw = std::max(maxw, (size_t)c->cout[l] * c->cin[l] * 9);
+    for (int l = 0; l < c->L; ++l) maxw = std::max(maxw, (size_t)c->cout[l] * (c->cin[l] * 9 + 1));
     size_t pb = c->part_floats * sizeof(float);
     if ((e = grow(reinterpret_cast<void**>(&c->d_part), &pb, (size_t)nx * maxw * sizeof(float)))) return e;
     c->part_floats = pb / sizeof(float);
     if (!gout) {
-        loss_kernel<T><<<1, 1024, 0, c->stream>>>((int64_t)B * 2 * HW, B, act + c->L * per, target, g0, c->d_red);
-        ++c->launches;
+        loss_kernel<T><<<LOSS_CTAS, 256, 0, c->stream>>>((int64_t)B * 2 * HW, B, act + c->L * per, target, g0,
+                                                         c->d_red + 8);
+        loss_sum_kernel<<<1, 32, 0, c->stream>>>(LOSS_CTAS, B, c->d_red + 8, c->d_red);
+        c->launches += 2;
     }
     for (int l = c->L - 1; l >= 0; --l) {
         const int Cin = c->cin[l], Cout = c->cout[l];
         // g0 = dL / d(pre-activation of layer l)
-        dim3 wg(nx, (Cin + CIB - 1) / CIB);
-        conv_wgrad_kernel<T><<<wg, 256, 0, c->stream>>>(g0, act + l * per, B, Cin, H, W, Cout, ipc, c->d_part);
-        const int nw = Cout * Cin * 9;
-        sum_rows_kernel<<<cblk(nw, 256), 256, 0, c->stream>>>(c->d_part, nx, nw, c->d_grad + c->woff[l]);
-        bias_grad_kernel<<<Cout, 256, 0, c->stream>>>(g0, B, Cout, HW, c->d_grad + c->boff[l]);
-        c->launches += 3;
+        const int nw = Cout * Cin * 9, np = nw + Cout;
+        if ((e = cudaFuncSetAttribute(conv_wgrad_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM)))
+            return e;
+        conv_wgrad_kernel<T><<<nx, 256, WG_SMEM, c->stream>>>(g0, act + l * per, B, Cin, H, W, Cout, ipc, c->d_part);
+        sum_rows_kernel<<<cblk(np, 32), 256, 0, c->stream>>>(c->d_part, nx, np, nw, c->d_grad + c->woff[l],
+                                                            c->d_grad + c->boff[l]);
+        c->launches += 2;
         if (l > 0) {
             flip_weights_kernel<<<cblk(nw, 256), 256, 0, c->stream>>>(c->d_param + c->woff[l], Cin, Cout, bf, c->d_wt);
             // dL/d(pre-activation of layer l-1): through the flipped convolution, masked by ReLU'
@@ -1067,7 +1118,7 @@ ibem_status ibem_cnn_create(int channels, unsigned long long seed, void* cuda_st
     }
     if (cudaMalloc(&c->d_param, off * sizeof(float)) || cudaMalloc(&c->d_grad, off * sizeof(float)) ||
         cudaMalloc(&c->d_m, off * sizeof(float)) || cudaMalloc(&c->d_v, off * sizeof(float)) ||
-        cudaMalloc(&c->d_wt, maxw * sizeof(float)) || cudaMalloc(&c->d_red, 8 * sizeof(double)) ||
+        cudaMalloc(&c->d_wt, maxw * sizeof(float)) || cudaMalloc(&c->d_red, (8 + LOSS_CTAS) * sizeof(double)) ||
         cudaMalloc(&c->d_status, sizeof(int))) {
         ibem_cnn_destroy(c);
         return IBEM_ERR_OOM;
