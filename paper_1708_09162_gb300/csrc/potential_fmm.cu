@@ -10,7 +10,7 @@
 // Non-admissible elements are summed with the regular Gauss rule of the direct
 // evaluation.
 //
-// Steps: (1) per point, a depth-first walk of the tree counts its far clusters
+// Steps: (1) per point and patch, a depth-first walk of the tree counts its far clusters
 // and near elements and marks the clusters it uses (one host round trip sizes
 // the lists and numbers the marked clusters); (2) the walk again, writing the
 // lists; (3) the moments of the marked clusters only, by projecting the
@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fp64_eval.cuh"
 #include "ibem_internal.cuh"
 
 namespace ibem {
@@ -41,57 +42,72 @@ struct LevelOffsets {
     int64_t off[12];           // cluster id of (level l, patch, morton) = off[l] + patch 4^l + morton
 };
 
-// One thread per point.  fill == false: cnt[2 i] = far clusters, cnt[2 i + 1] =
-// near elements, used[c] = 1 for every far cluster.  fill == true: writes the
-// lists at far_off[i], near_off[i].
+// One thread per (point, patch): the walk below one root.  fill == false: cnt[2 i] =
+// far clusters, cnt[2 i + 1] = near elements of walk i = point * npatch + patch,
+// used[c] = 1 for every far cluster.  fill == true: writes the lists at far_off[i],
+// near_off[i], so a point's entries are contiguous in the order of the patches.
+// Bound by the latency of a walk (some 100 dependent steps), so the walks are as
+// many and short as they can be: with one thread per point both passes took 0.80 ms
+// for 5000 points at level 6, with one per patch 0.29 ms.
 __global__ void pf_lists_kernel(int64_t npts, const double* __restrict__ pts, int npatch, int m, LevelOffsets lo,
                                 const double* __restrict__ balls, double eta, bool fill, int32_t* __restrict__ cnt,
                                 uint8_t* __restrict__ used, const int64_t* __restrict__ far_off,
                                 const int64_t* __restrict__ near_off, int32_t* __restrict__ far_list,
                                 int32_t* __restrict__ near_list, int* __restrict__ status) {
-    const int64_t ip = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ip >= npts) return;
+    const int64_t iw = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (iw >= npts * npatch) return;
+    const int64_t ip = iw / npatch;
+    const int patch = (int)(iw - ip * npatch);
     const double x0 = pts[3 * ip], x1 = pts[3 * ip + 1], x2 = pts[3 * ip + 2];
     int32_t sid[PF_STACK];
     int8_t slv[PF_STACK];
     int64_t nf = 0, nn = 0;
-    const int64_t fo = fill ? far_off[ip] : 0, no = fill ? near_off[ip] : 0;
-    for (int patch = 0; patch < npatch; ++patch) {
-        int sp = 0;
-        sid[sp] = (int32_t)(lo.off[0] + patch);
-        slv[sp++] = 0;
-        while (sp > 0) {
-            --sp;
-            const int32_t c = sid[sp];
-            const int l = slv[sp];
-            const double* b = balls + 4 * (int64_t)c;
-            const double d0 = x0 - b[0], d1 = x1 - b[1], d2 = x2 - b[2];
-            double dist = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - b[3];
-            if (!(dist > 0.0)) dist = 0.0;
-            if (eta * 2.0 * b[3] < dist) {
-                if (fill) far_list[fo + nf] = c;
-                else used[c] = 1;
-                ++nf;
-            } else if (l == m) {
-                if (fill) near_list[no + nn] = (int32_t)(c - lo.off[m]);
-                ++nn;
-            } else {
-                if (sp + 4 > PF_STACK) {   // unreachable for m <= 10; recorded, never overrun
-                    atomicOr(status, IBEM_DEVICE_OVERFLOW);
-                    return;
-                }
-                const int64_t first = lo.off[l + 1] + 4 * (c - lo.off[l]);
-                for (int k = 0; k < 4; ++k) {
-                    sid[sp] = (int32_t)(first + k);
-                    slv[sp++] = (int8_t)(l + 1);
-                }
+    const int64_t fo = fill ? far_off[iw] : 0, no = fill ? near_off[iw] : 0;
+    int sp = 0;
+    sid[sp] = (int32_t)(lo.off[0] + patch);
+    slv[sp++] = 0;
+    while (sp > 0) {
+        --sp;
+        const int32_t c = sid[sp];
+        const int l = slv[sp];
+        const double* b = balls + 4 * (int64_t)c;
+        const double d0 = x0 - b[0], d1 = x1 - b[1], d2 = x2 - b[2];
+        double dist = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - b[3];
+        if (!(dist > 0.0)) dist = 0.0;
+        if (eta * 2.0 * b[3] < dist) {
+            if (fill) far_list[fo + nf] = c;
+            else used[c] = 1;
+            ++nf;
+        } else if (l == m) {
+            if (fill) near_list[no + nn] = (int32_t)(c - lo.off[m]);
+            ++nn;
+        } else {
+            if (sp + 4 > PF_STACK) {   // unreachable for m <= 10; recorded, never overrun
+                atomicOr(status, IBEM_DEVICE_OVERFLOW);
+                return;
+            }
+            const int64_t first = lo.off[l + 1] + 4 * (c - lo.off[l]);
+            for (int k = 0; k < 4; ++k) {
+                sid[sp] = (int32_t)(first + k);
+                slv[sp++] = (int8_t)(l + 1);
             }
         }
     }
     if (!fill) {
-        cnt[2 * ip] = (int32_t)nf;
-        cnt[2 * ip + 1] = (int32_t)nn;
+        cnt[2 * iw] = (int32_t)nf;
+        cnt[2 * iw + 1] = (int32_t)nn;
     }
+}
+
+// offsets of the walks' lists from their counts: far then near, npts * npatch + 1 each
+std::vector<int64_t> walk_offsets(const std::vector<int32_t>& cnt) {
+    const size_t n = cnt.size() / 2;
+    std::vector<int64_t> off(2 * (n + 1), 0);
+    for (size_t i = 0; i < n; ++i) {
+        off[i + 1] = off[i] + cnt[2 * i];
+        off[n + 1 + i + 1] = off[n + 1 + i] + cnt[2 * i + 1];
+    }
+    return off;
 }
 
 // Moments of the marked clusters: one CTA per (cluster, chunk of PF_MV real
@@ -137,18 +153,13 @@ __global__ void pf_moments_kernel(int n_used, const int32_t* __restrict__ used_i
     }
 }
 
+// u*(x, y) from |x - y|^2 (fp64_eval.cuh): the kernels below are bound by the FP64
+// pipe, and this takes about 30 operations instead of 80 with sqrt, division and
+// sincos (5000 points, 4 densities, level 6: evaluation 5.34 ms instead of 6.04)
 template <bool CPLX>
-__device__ __forceinline__ void pf_kernel_value(double d, double kappa, double* gr, double* gi) {
-    const double inv = 1.0 / (4.0 * IBEM_PI * d);
-    if constexpr (CPLX) {
-        double s, c;
-        sincos(kappa * d, &s, &c);
-        *gr = c * inv;
-        *gi = s * inv;
-    } else {
-        *gr = inv;
-        *gi = 0.0;
-    }
+__device__ __forceinline__ void pf_kernel_value(double d2, double kappa, const double2* __restrict__ trig, double* gr,
+                                                double* gi) {
+    green64<CPLX>(d2, kappa, 1.0 / (4.0 * IBEM_PI), trig, gr, gi);
 }
 
 // One CTA per (point, chunk of PF_RC densities).  Far terms: entries (cluster,
@@ -158,13 +169,13 @@ __device__ __forceinline__ void pf_kernel_value(double d, double kappa, double* 
 // (element, Gauss point); the density at a Gauss point is
 // sum_i phi[g][i] x*_e[i] from the lifted coefficients xs [R][E][nb].
 template <bool CPLX>
-__global__ void __launch_bounds__(PF_T) pf_eval_kernel(
-    int64_t npts, const double* __restrict__ pts, int R, const int64_t* __restrict__ far_off,
+__global__ void __launch_bounds__(PF_T, 2) pf_eval_kernel(
+    int64_t npts, int npatch, const double* __restrict__ pts, int R, const int64_t* __restrict__ far_off,
     const int32_t* __restrict__ far_list, const int64_t* __restrict__ near_off, const int32_t* __restrict__ near_list,
     int q2, int64_t n_used, const int32_t* __restrict__ slot, const double* __restrict__ igeo,
     const double* __restrict__ xh, int QQ, int nb, int64_t E,
     const double* __restrict__ qgeo, const double* __restrict__ phi, const double* __restrict__ xs, double kappa,
-    double* __restrict__ u) {
+    const double2* __restrict__ trig, double* __restrict__ u) {
     constexpr int NA = CPLX ? 2 * PF_RC : PF_RC;
     __shared__ double red[PF_T / 32][NA];
     const int64_t ip = blockIdx.x;
@@ -175,62 +186,74 @@ __global__ void __launch_bounds__(PF_T) pf_eval_kernel(
 #pragma unroll
     for (int j = 0; j < NA; ++j) acc[j] = 0.0;
     const int64_t CW = CPLX ? 2 : 1;
+    // Threads are groups of one thread per interpolation (Gauss) point; a group takes every
+    // G-th cluster (element) of the point's list, so no entry needs a division.  Rules
+    // with more points than threads loop over them.
+    const int t = threadIdx.x;
     // far field
-    const int64_t f0 = far_off[ip], nfe = (far_off[ip + 1] - f0) * q2;
-    for (int64_t idx = threadIdx.x; idx < nfe; idx += PF_T) {
-        const int64_t c = far_list[f0 + idx / q2];
-        const int b = (int)(idx % q2);
-        const double* z = igeo + 4 * (c * q2 + b);
-        const double d0 = x0 - z[0], d1 = x1 - z[1], d2 = x2 - z[2];
-        double gr, gi;
-        pf_kernel_value<CPLX>(sqrt(d0 * d0 + d1 * d1 + d2 * d2), kappa, &gr, &gi);
-        gr *= z[3];
-        gi *= z[3];
-        const int64_t C = n_used;
-        const double* mom = xh + (CW * r0 * C + slot[c]) * q2 + b;
+    {
+        const int64_t f0 = far_off[ip * npatch], f1 = far_off[(ip + 1) * npatch];
+        const int G = PF_T / q2 > 0 ? PF_T / q2 : 1, step = q2 < PF_T ? q2 : PF_T;
+        for (int64_t k = f0 + t / step; t < G * step && k < f1; k += G) {
+            const int64_t c = far_list[k];
+            const double* mom0 = xh + (CW * r0 * n_used + slot[c]) * q2;
+            for (int b = t % step; b < q2; b += step) {
+                const double* z = igeo + 4 * (c * q2 + b);
+                const double d0 = x0 - z[0], d1 = x1 - z[1], d2 = x2 - z[2];
+                double gr, gi;
+                pf_kernel_value<CPLX>(fma(d0, d0, fma(d1, d1, d2 * d2)), kappa, trig, &gr, &gi);
+                gr *= z[3];
+                gi *= z[3];
+                const double* mom = mom0 + b;
 #pragma unroll
-        for (int j = 0; j < PF_RC; ++j) {
-            if (j < nc) {
-                if constexpr (CPLX) {
-                    const double mr = mom[(2 * j) * C * q2], mi = mom[(2 * j + 1) * C * q2];
-                    acc[2 * j] = fma(gr, mr, fma(-gi, mi, acc[2 * j]));
-                    acc[2 * j + 1] = fma(gr, mi, fma(gi, mr, acc[2 * j + 1]));
-                } else {
-                    acc[j] = fma(gr, mom[j * C * q2], acc[j]);
+                for (int j = 0; j < PF_RC; ++j) {
+                    if (j < nc) {
+                        if constexpr (CPLX) {
+                            const double mr = mom[(2 * j) * n_used * q2], mi = mom[(2 * j + 1) * n_used * q2];
+                            acc[2 * j] = fma(gr, mr, fma(-gi, mi, acc[2 * j]));
+                            acc[2 * j + 1] = fma(gr, mi, fma(gi, mr, acc[2 * j + 1]));
+                        } else {
+                            acc[j] = fma(gr, mom[j * n_used * q2], acc[j]);
+                        }
+                    }
                 }
             }
         }
     }
     // near field
-    const int64_t n0 = near_off[ip], nne = (near_off[ip + 1] - n0) * QQ;
-    for (int64_t idx = threadIdx.x; idx < nne; idx += PF_T) {
-        const int64_t e = near_list[n0 + idx / QQ];
-        const int g = (int)(idx % QQ);
-        const double* y = qgeo + 4 * (e * QQ + g);
-        const double d0 = x0 - y[0], d1 = x1 - y[1], d2 = x2 - y[2];
-        double gr, gi;
-        pf_kernel_value<CPLX>(sqrt(d0 * d0 + d1 * d1 + d2 * d2), kappa, &gr, &gi);
-        gr *= y[3];
-        gi *= y[3];
-        const double* ph = phi + (int64_t)g * nb;
+    {
+        const int64_t n0 = near_off[ip * npatch], n1 = near_off[(ip + 1) * npatch];
+        const int G = PF_T / QQ > 0 ? PF_T / QQ : 1, step = QQ < PF_T ? QQ : PF_T;
+        for (int64_t k = n0 + t / step; t < G * step && k < n1; k += G) {
+            const int64_t e = near_list[k];
+            for (int g = t % step; g < QQ; g += step) {
+                const double* y = qgeo + 4 * (e * QQ + g);
+                const double d0 = x0 - y[0], d1 = x1 - y[1], d2 = x2 - y[2];
+                double gr, gi;
+                pf_kernel_value<CPLX>(fma(d0, d0, fma(d1, d1, d2 * d2)), kappa, trig, &gr, &gi);
+                gr *= y[3];
+                gi *= y[3];
+                const double* ph = phi + (int64_t)g * nb;
 #pragma unroll
-        for (int j = 0; j < PF_RC; ++j) {
-            if (j < nc) {
-                if constexpr (CPLX) {
-                    const double* cr = xs + ((2 * (r0 + j)) * E + e) * nb;
-                    const double* ci = xs + ((2 * (r0 + j) + 1) * E + e) * nb;
-                    double dr = 0.0, di = 0.0;
-                    for (int i = 0; i < nb; ++i) {
-                        dr = fma(ph[i], cr[i], dr);
-                        di = fma(ph[i], ci[i], di);
+                for (int j = 0; j < PF_RC; ++j) {
+                    if (j < nc) {
+                        if constexpr (CPLX) {
+                            const double* cr = xs + ((2 * (r0 + j)) * E + e) * nb;
+                            const double* ci = xs + ((2 * (r0 + j) + 1) * E + e) * nb;
+                            double dr = 0.0, di = 0.0;
+                            for (int i = 0; i < nb; ++i) {
+                                dr = fma(ph[i], cr[i], dr);
+                                di = fma(ph[i], ci[i], di);
+                            }
+                            acc[2 * j] = fma(gr, dr, fma(-gi, di, acc[2 * j]));
+                            acc[2 * j + 1] = fma(gr, di, fma(gi, dr, acc[2 * j + 1]));
+                        } else {
+                            const double* cr = xs + ((int64_t)(r0 + j) * E + e) * nb;
+                            double dr = 0.0;
+                            for (int i = 0; i < nb; ++i) dr = fma(ph[i], cr[i], dr);
+                            acc[j] = fma(gr, dr, acc[j]);
+                        }
                     }
-                    acc[2 * j] = fma(gr, dr, fma(-gi, di, acc[2 * j]));
-                    acc[2 * j + 1] = fma(gr, di, fma(gi, dr, acc[2 * j + 1]));
-                } else {
-                    const double* cr = xs + ((int64_t)(r0 + j) * E + e) * nb;
-                    double dr = 0.0;
-                    for (int i = 0; i < nb; ++i) dr = fma(ph[i], cr[i], dr);
-                    acc[j] = fma(gr, dr, acc[j]);
                 }
             }
         }
@@ -338,26 +361,23 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     // (1) count, mark the clusters used
     LevelOffsets lo{};
     for (int l = 0; l <= P.m + 1 && l < 12; ++l) lo.off[l] = P.level_off[l];
+    const int64_t nw = npts * P.npatch;   // walks
     int32_t* d_cnt;
     uint8_t* d_used;
-    if ((e = buf.alloc(&d_cnt, (size_t)2 * npts)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
+    if ((e = buf.alloc(&d_cnt, (size_t)2 * nw)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
         (e = cudaMemsetAsync(d_used, 0, (size_t)P.C, st)))
         return e;
-    pf_lists_kernel<<<nblk(npts, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
                                                       d_used, nullptr, nullptr, nullptr, nullptr, h->d_status);
     h->launches++;
-    std::vector<int32_t> cnt((size_t)2 * npts);
+    std::vector<int32_t> cnt((size_t)2 * nw);
     std::vector<uint8_t> used((size_t)P.C);
     if ((e = cudaMemcpyAsync(cnt.data(), d_cnt, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st)) ||
         (e = cudaMemcpyAsync(used.data(), d_used, used.size(), cudaMemcpyDeviceToHost, st)) ||
         (e = cudaStreamSynchronize(st)))
         return e;
-    std::vector<int64_t> off((size_t)2 * (npts + 1), 0);   // far offsets, then near offsets
-    for (int64_t i = 0; i < npts; ++i) {
-        off[i + 1] = off[i] + cnt[2 * i];
-        off[npts + 1 + i + 1] = off[npts + 1 + i] + cnt[2 * i + 1];
-    }
-    const int64_t nfar = off[npts], nnear = off[2 * npts + 1];
+    const std::vector<int64_t> off = walk_offsets(cnt);   // far, then near
+    const int64_t nfar = off[nw], nnear = off[2 * nw + 1];
     if (n_far_terms) *n_far_terms = nfar;
     if (n_near_terms) *n_near_terms = nnear;
     std::vector<int32_t> ids, slot((size_t)P.C, -1);
@@ -382,8 +402,8 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     if (n_used > 0 && (e = cudaMemcpyAsync(d_ids, ids.data(), ids.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
                                            st)))
         return e;
-    pf_lists_kernel<<<nblk(npts, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
-                                                      nullptr, d_off, d_off + npts + 1, d_lists, d_lists + nfar,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
+                                                      nullptr, d_off, d_off + nw + 1, d_lists, d_lists + nfar,
                                                       h->d_status);
     h->launches++;
     // (3) densities as real vectors, moments of the used clusters, lifted
@@ -415,13 +435,13 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     dim3 grid((unsigned)npts, (unsigned)((nrhs + PF_RC - 1) / PF_RC));
     const int QQ = P.Q * P.Q;
     if (h->helm)
-        pf_eval_kernel<true><<<grid, PF_T, 0, st>>>(npts, pts, nrhs, d_off, d_lists, d_off + npts + 1,
+        pf_eval_kernel<true><<<grid, PF_T, 0, st>>>(npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1,
                                                     d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo, d_xhat, QQ,
-                                                    P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, P.prm.kappa, u);
+                                                    P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, P.prm.kappa, h->d_trig64, u);
     else
-        pf_eval_kernel<false><<<grid, PF_T, 0, st>>>(npts, pts, nrhs, d_off, d_lists, d_off + npts + 1,
+        pf_eval_kernel<false><<<grid, PF_T, 0, st>>>(npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1,
                                                      d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo, d_xhat, QQ,
-                                                     P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, 0.0, u);
+                                                     P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, 0.0, h->d_trig64, u);
     h->launches++;
     return cudaGetLastError();
 }
@@ -455,7 +475,7 @@ template <bool CPLX>
 __global__ void __launch_bounds__(RS_T) rs_far_kernel(
     const int32_t* __restrict__ clusters, const int64_t* __restrict__ cptr, const int32_t* __restrict__ csrc,
     const double* __restrict__ src, const double* __restrict__ charges, int R, int64_t nsrc, int q2, int64_t C,
-    const double* __restrict__ igeo, double kappa, double* __restrict__ yh) {
+    const double* __restrict__ igeo, double kappa, const double2* __restrict__ trig, double* __restrict__ yh) {
     constexpr int CW = CPLX ? 2 : 1;
     constexpr int NV = RS_RC * CW;
     __shared__ double part[NV * RS_T];
@@ -475,7 +495,7 @@ __global__ void __launch_bounds__(RS_T) rs_far_kernel(
             const int64_t j = csrc[k];
             const double d0 = z0 - src[3 * j], d1 = z1 - src[3 * j + 1], d2 = z2 - src[3 * j + 2];
             double gr, gi;
-            pf_kernel_value<CPLX>(sqrt(d0 * d0 + d1 * d1 + d2 * d2), kappa, &gr, &gi);
+            pf_kernel_value<CPLX>(fma(d0, d0, fma(d1, d1, d2 * d2)), kappa, trig, &gr, &gi);
 #pragma unroll
             for (int rr = 0; rr < RS_RC; ++rr) {
                 if (rr < nc) {
@@ -516,7 +536,7 @@ __global__ void __launch_bounds__(RS_T) rs_near_kernel(
     const int32_t* __restrict__ elems, const int64_t* __restrict__ eptr, const int32_t* __restrict__ esrc,
     const double* __restrict__ src, const double* __restrict__ charges, int R, int64_t nsrc, int QQ, int nb,
     int64_t E, const double* __restrict__ qgeo, const double* __restrict__ phi, double kappa,
-    double* __restrict__ ys) {
+    const double2* __restrict__ trig, double* __restrict__ ys) {
     constexpr int CW = CPLX ? 2 : 1;
     constexpr int NV = RS_RC * CW;
     constexpr int MAXO = (25 * NV + RS_T - 1) / RS_T;   // nb <= 25
@@ -540,7 +560,7 @@ __global__ void __launch_bounds__(RS_T) rs_near_kernel(
                 const int64_t j = esrc[k];
                 const double d0 = x0 - src[3 * j], d1 = x1 - src[3 * j + 1], d2 = x2 - src[3 * j + 2];
                 double gr, gi;
-                pf_kernel_value<CPLX>(sqrt(d0 * d0 + d1 * d1 + d2 * d2), kappa, &gr, &gi);
+                pf_kernel_value<CPLX>(fma(d0, d0, fma(d1, d1, d2 * d2)), kappa, trig, &gr, &gi);
                 gr *= w;
                 gi *= w;
 #pragma unroll
@@ -622,24 +642,21 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
     // (1) lists per source (the potential's walk)
     LevelOffsets lo{};
     for (int l = 0; l <= P.m + 1 && l < 12; ++l) lo.off[l] = P.level_off[l];
+    const int64_t nw = nsrc * P.npatch;   // walks
     int32_t* d_cnt;
     uint8_t* d_used;
-    if ((e = buf.alloc(&d_cnt, (size_t)2 * nsrc)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
+    if ((e = buf.alloc(&d_cnt, (size_t)2 * nw)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
         (e = cudaMemsetAsync(d_used, 0, (size_t)P.C, st)))
         return e;
-    pf_lists_kernel<<<nblk(nsrc, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
                                                       d_used, nullptr, nullptr, nullptr, nullptr, h->d_status);
     h->launches++;
-    std::vector<int32_t> cnt((size_t)2 * nsrc);
+    std::vector<int32_t> cnt((size_t)2 * nw);
     if ((e = cudaMemcpyAsync(cnt.data(), d_cnt, cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st)) ||
         (e = cudaStreamSynchronize(st)))
         return e;
-    std::vector<int64_t> off((size_t)2 * (nsrc + 1), 0);   // far offsets, then near offsets
-    for (int64_t i = 0; i < nsrc; ++i) {
-        off[i + 1] = off[i] + cnt[2 * i];
-        off[nsrc + 1 + i + 1] = off[nsrc + 1 + i] + cnt[2 * i + 1];
-    }
-    const int64_t nfar = off[nsrc], nnear = off[2 * nsrc + 1];
+    const std::vector<int64_t> off = walk_offsets(cnt);   // far, then near
+    const int64_t nfar = off[nw], nnear = off[2 * nw + 1];
     if (n_far_terms) *n_far_terms = nfar;
     if (n_near_terms) *n_near_terms = nnear;
     int64_t* d_off;
@@ -647,8 +664,8 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
     if ((e = buf.alloc(&d_off, off.size())) || (e = buf.alloc(&d_lists, (size_t)(nfar + nnear))) ||
         (e = cudaMemcpyAsync(d_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st)))
         return e;
-    pf_lists_kernel<<<nblk(nsrc, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
-                                                      nullptr, d_off, d_off + nsrc + 1, d_lists, d_lists + nfar,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
+                                                      nullptr, d_off, d_off + nw + 1, d_lists, d_lists + nfar,
                                                       h->d_status);
     h->launches++;
     std::vector<int32_t> lists((size_t)(nfar + nnear));
@@ -657,7 +674,11 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
         return e;
     if ((e = cudaStreamSynchronize(st))) return e;
     // (2) lists per cluster and per element, sources ascending
-    std::vector<int64_t> foff(off.begin(), off.begin() + nsrc + 1), noff(off.begin() + nsrc + 1, off.end());
+    std::vector<int64_t> foff((size_t)nsrc + 1), noff((size_t)nsrc + 1);
+    for (int64_t i = 0; i <= nsrc; ++i) {
+        foff[i] = off[i * P.npatch];
+        noff[i] = off[nw + 1 + i * P.npatch];
+    }
     std::vector<int32_t> cl, csrc, el, esrc;
     std::vector<int64_t> cptr, eptr;
     transpose_lists(nsrc, foff, lists, 0, P.C, cl, cptr, csrc);
@@ -688,10 +709,10 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
         dim3 grid((unsigned)cl.size(), nchunk);
         if (h->helm)
             rs_far_kernel<true><<<grid, RS_T, 0, st>>>(d_cl, d_cptr, d_csrc, src, charges, nrhs, nsrc, P.q2, P.C,
-                                                       h->d_igeo, P.prm.kappa, d_yh);
+                                                       h->d_igeo, P.prm.kappa, h->d_trig64, d_yh);
         else
             rs_far_kernel<false><<<grid, RS_T, 0, st>>>(d_cl, d_cptr, d_csrc, src, charges, nrhs, nsrc, P.q2, P.C,
-                                                        h->d_igeo, 0.0, d_yh);
+                                                        h->d_igeo, 0.0, h->d_trig64, d_yh);
         h->launches++;
     }
     for (int L = 0; L < P.m; ++L) {
@@ -708,10 +729,10 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
         const int QQ = P.Q * P.Q;
         if (h->helm)
             rs_near_kernel<true><<<grid, RS_T, 0, st>>>(d_el, d_eptr, d_esrc, src, charges, nrhs, nsrc, QQ, P.nb, P.E,
-                                                        h->d_qgeo, h->d_phi, P.prm.kappa, d_ys);
+                                                        h->d_qgeo, h->d_phi, P.prm.kappa, h->d_trig64, d_ys);
         else
             rs_near_kernel<false><<<grid, RS_T, 0, st>>>(d_el, d_eptr, d_esrc, src, charges, nrhs, nsrc, QQ, P.nb,
-                                                         P.E, h->d_qgeo, h->d_phi, 0.0, d_ys);
+                                                         P.E, h->d_qgeo, h->d_phi, 0.0, h->d_trig64, d_ys);
         h->launches++;
     }
     restrict_kernel<<<nblk((int64_t)R2 * P.N, T), T, 0, st>>>(R2, P.N, P.p, P.ne1, h->d_ext, d_ys, P.E,
