@@ -8,14 +8,15 @@
 //
 // Coupling on tcgen05: one CTA per target cluster sigma.  For every far block
 // the CTA evaluates K_{sigma tau} in FP32 (rsqrt, phase reduced to [-pi, pi],
-// sine and cosine) and writes it as BF16 into a shared-memory A tile, in the
-// real form [[Kr, -Ki], [Ki, Kr]] for Helmholtz, padded to MAP = 128 rows and
-// KAP (multiple of 16) columns.  The B tile - the moments x^_tau as BF16 in the
-// same form, RP (multiple of 16) right-hand sides - is prepared once per
+// sine and cosine) and writes it as BF16 into a shared-memory A tile, for
+// Helmholtz [Kr; Ki], padded to MAP = 128 rows and KAP (multiple of 16) columns.
+// The B tile - the moments x^_tau as BF16, RP (multiple of 16) right-hand sides,
+// for Helmholtz the real then the imaginary parts - is prepared once per
 // application in global memory and fetched with one cp.async.bulk per block.
+// Re y = Kr xr - Ki xi and Im y = Kr xi + Ki xr are joined when a row is done.
 // Both tiles are double-buffered; one thread issues tcgen05.mma (kind::f16,
 // BF16 inputs, FP32 accumulation) into a TMEM accumulator [MAP lanes][RP
-// columns] that persists over the whole far row, and tcgen05.commit signals an
+// (complex: 2 RP) columns] that persists over the whole far row, and tcgen05.commit signals an
 // mbarrier when a buffer may be reused.  Tiles use the no-swizzle K-major
 // layout: 8 x 8 core matrices of 128 contiguous bytes, LBO = 128 bytes along
 // K, SBO = (KAP / 8) * 128 bytes along M or N.  All waits are bounded.
@@ -23,6 +24,7 @@
 
 #include <algorithm>
 
+#include "fp32_eval.cuh"
 #include "ibem_internal.cuh"
 
 namespace ibem {
@@ -78,24 +80,46 @@ __global__ void mr_lift_kernel(int R, int64_t E, int p, int ne1, const double* _
     xs[idx] = acc;
 }
 
-template <bool CPLX>
-__global__ void mr_leaf_kernel(int R, int64_t E, int pp, int q, const float* __restrict__ M,
-                               const typename MrType<CPLX>::T* __restrict__ xs, int64_t leaf_off,
-                               typename MrType<CPLX>::T* __restrict__ xh) {
+// Leaf moments and back-projection hold one right-hand side per thread, consecutive
+// threads consecutive right-hand sides: every value is read (and written) once and
+// coalesced, the sums are separable and stay in registers, M comes from shared memory
+// by broadcast.  Bound: HBM / L2.  Level 5, q = 8, 64 right-hand sides: 35 us for the
+// leaf moments and 51 for the back-projection; 318 and 252 with one thread per
+// moment or coefficient, which read its (p+1)^2 or q^2 inputs through L1 each.
+
+// leaf moments x^[av][au] = sum M[av][iv] M[au][iu] x*[iv][iu]; thread (element, right-hand side)
+template <bool CPLX, int PP>
+__global__ void __launch_bounds__(128) mr_leaf_kernel(int R, int64_t E, int q, const float* __restrict__ M,
+                                                      const typename MrType<CPLX>::T* __restrict__ xs, int64_t leaf_off,
+                                                      typename MrType<CPLX>::T* __restrict__ xh) {
     typedef typename MrType<CPLX>::T T;
-    const int q2 = q * q, nb = pp * pp;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= E * q2 * R) return;
-    int r = (int)(idx % R);
-    int64_t rem = idx / R;
-    int a = (int)(rem % q2);
-    int64_t e = rem / q2;
-    const int au = a % q, av = a / q;
-    T acc = mr_zero(T());
-    for (int iv = 0; iv < pp; ++iv)
-        for (int iu = 0; iu < pp; ++iu)
-            acc = mr_axpy(M[au * pp + iu] * M[av * pp + iv], xs[(e * nb + iv * pp + iu) * R + r], acc);
-    xh[((leaf_off + e) * q2 + a) * R + r] = acc;
+    constexpr int nb = PP * PP;
+    __shared__ float Ms[IBEM_MAX_Q * PP];
+    for (int i = threadIdx.x; i < q * PP; i += blockDim.x) Ms[i] = M[i];
+    __syncthreads();
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= E * R) return;
+    const int r = (int)(idx % R);
+    const int64_t e = idx / R;
+    T x[nb];
+#pragma unroll
+    for (int i = 0; i < nb; ++i) x[i] = xs[(e * nb + i) * R + r];
+    T* out = xh + (leaf_off + e) * q * q * R + r;
+    for (int au = 0; au < q; ++au) {
+        T t[PP];
+#pragma unroll
+        for (int iv = 0; iv < PP; ++iv) {
+            t[iv] = mr_zero(T());
+#pragma unroll
+            for (int iu = 0; iu < PP; ++iu) t[iv] = mr_axpy(Ms[au * PP + iu], x[iv * PP + iu], t[iv]);
+        }
+        for (int av = 0; av < q; ++av) {
+            T acc = mr_zero(T());
+#pragma unroll
+            for (int iv = 0; iv < PP; ++iv) acc = mr_axpy(Ms[av * PP + iv], t[iv], acc);
+            out[(int64_t)(av * q + au) * R] = acc;
+        }
+    }
 }
 
 // Separable M2M, one CTA per (parent, chunk of RC right-hand sides):
@@ -186,28 +210,46 @@ __global__ void mr_l2l_sep_kernel(int R, int64_t offL, int64_t offL1, int q, con
     }
 }
 
-// B tiles: per cluster [RP][KAP] BF16 in the canonical no-swizzle K-major layout;
-// column k < q2 is Re x^[k] (x^[k] for Laplace), q2 <= k < 2 q2 is Im x^[k - q2].
+// B tiles: per cluster [RP] (complex [2 RP]: real, then imaginary parts) rows of KAP
+// columns, BF16 in the canonical no-swizzle K-major layout; columns k >= q2 are
+// zero.  A thread converts 8 columns of one right-hand side (reads are coalesced over
+// the right-hand sides) and stores 16 bytes per row.
 template <bool CPLX>
-__global__ void mr_bpack_kernel(int R, int RP, int KAP, int64_t C, int q2, const typename MrType<CPLX>::T* __restrict__ xh,
-                                __nv_bfloat16* __restrict__ xb) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= C * RP * KAP) return;
-    int k = (int)(idx % KAP);
-    int64_t rem = idx / KAP;
-    int r = (int)(rem % RP);
-    int64_t c = rem / RP;
-    float v = 0.0f;
-    if (r < R) {
-        if constexpr (CPLX) {
-            if (k < q2) v = xh[(c * q2 + k) * R + r].x;
-            else if (k < 2 * q2) v = xh[(c * q2 + k - q2) * R + r].y;
-        } else {
-            if (k < q2) v = xh[(c * q2 + k) * R + r];
+__global__ void mr_bpack_kernel(int R, int r0, int RP, int KAP, int64_t C, int q2,
+                                const typename MrType<CPLX>::T* __restrict__ xh, __nv_bfloat16* __restrict__ xb) {
+    const int K8 = KAP >> 3;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= C * K8 * RP) return;
+    const int r = (int)(idx % RP), k8 = (int)((idx / RP) % K8);
+    const int64_t c = idx / RP / K8;
+    float re[8], im[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int k = 8 * k8 + j;
+        re[j] = im[j] = 0.0f;
+        if (r0 + r < R && k < q2) {
+            const auto v = xh[(c * q2 + k) * R + r0 + r];
+            if constexpr (CPLX) {
+                re[j] = v.x;
+                im[j] = v.y;
+            } else {
+                re[j] = v;
+            }
         }
     }
-    int64_t off = c * (int64_t)RP * KAP + ((int64_t)((r >> 3) * (KAP >> 3) + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7));
-    xb[off] = __float2bfloat16(v);
+    auto store = [&](int row, const float (&v)[8]) {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            w[j] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        const int64_t rows = CPLX ? 2 * RP : RP;
+        *reinterpret_cast<uint4*>(xb + c * rows * KAP + ((int64_t)(row >> 3) * K8 + k8) * 64 + (row & 7) * 8) =
+            make_uint4(w[0], w[1], w[2], w[3]);
+    };
+    store(r, re);
+    if constexpr (CPLX) store(RP + r, im);
 }
 
 // ---- tensor-core coupling ---------------------------------------------------------------
@@ -231,8 +273,76 @@ __device__ inline bool tc_wait(uint64_t* bar, unsigned parity, long long limit) 
     return false;
 }
 
+// Two independent FP32 operations per instruction: the generation below is bound by
+// issue, and a thread has two columns.
+using mr_f2 = unsigned long long;
+__device__ __forceinline__ mr_f2 f2_pack(float a, float b) {
+    mr_f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(mr_f2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ mr_f2 f2_sub(mr_f2 a, mr_f2 b) {
+    mr_f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ mr_f2 f2_mul(mr_f2 a, mr_f2 b) {
+    mr_f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ mr_f2 f2_fma(mr_f2 a, mr_f2 b, mr_f2 c) {
+    mr_f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+struct MrPoint2 {   // two source points as pairs, w = surface measure
+    mr_f2 x, y, z, w;
+};
+__device__ __forceinline__ MrPoint2 mr_point2(const float4 a, const float4 b) {
+    return {f2_pack(a.x, b.x), f2_pack(a.y, b.y), f2_pack(a.z, b.z), f2_pack(a.w, b.w)};
+}
+// K at one target point (coordinates and measure / (4 pi), each twice) and two source
+// points: BF16 pairs of the real and the imaginary part
+template <bool CPLX>
+__device__ __forceinline__ void mr_values(const ulonglong2 xy, const ulonglong2 zw, const MrPoint2& Y, float kappa,
+                                          uint32_t* kr, uint32_t* ki) {
+    const mr_f2 d0 = f2_sub(xy.x, Y.x), d1 = f2_sub(xy.y, Y.y), d2 = f2_sub(zw.x, Y.z);
+    const mr_f2 r2 = f2_fma(d0, d0, f2_fma(d1, d1, f2_mul(d2, d2)));
+    const float2 s = f2_get(r2);
+    const mr_f2 rinv = f2_pack(approx_rsqrt(s.x), approx_rsqrt(s.y));
+    const mr_f2 w = f2_mul(f2_mul(zw.y, Y.w), rinv);
+    if constexpr (CPLX) {
+        // phase reduced to [-pi, pi] first (the hardware sine and cosine are accurate
+        // on that interval only); 1.5 2^23 rounds to the nearest integer
+        const mr_f2 a = f2_mul(f2_pack(kappa, kappa), f2_mul(r2, rinv));
+        const mr_f2 M = f2_pack(12582912.0f, 12582912.0f);
+        const mr_f2 n = f2_sub(f2_fma(a, f2_pack(0.15915494309189535f, 0.15915494309189535f), M), M);
+        const float2 ph = f2_get(f2_fma(f2_pack(-6.283185307179586f, -6.283185307179586f), n, a));
+        const float2 re = f2_get(f2_mul(w, f2_pack(approx_cos(ph.x), approx_cos(ph.y))));
+        const float2 im = f2_get(f2_mul(w, f2_pack(approx_sin(ph.x), approx_sin(ph.y))));
+        const __nv_bfloat162 hr = __floats2bfloat162_rn(re.x, re.y), hi = __floats2bfloat162_rn(im.x, im.y);
+        *kr = *reinterpret_cast<const uint32_t*>(&hr);
+        *ki = *reinterpret_cast<const uint32_t*>(&hi);
+    } else {
+        const float2 re = f2_get(w);
+        const __nv_bfloat162 hr = __floats2bfloat162_rn(re.x, re.y);
+        *kr = *reinterpret_cast<const uint32_t*>(&hr);
+    }
+}
+
 // Q > 0: compiled for q = Q (index arithmetic of the K generation by shifts and
 // constants); Q = 0: q and KAP at run time.
+// Bound: the generation of K, by issue (ncu before this form: about 90% of the issue
+// slots, XU 33%), then by the XU pipe (three operations per complex value, 3.3 ms at
+// level 5, q = 8).  The A tile holds K once ([Kr; Ki], not [[Kr, -Ki], [Ki, Kr]]), two
+// values share packed instructions, and for q = 8 a thread's two source points
+// serve four rows.  Level 5, 16 right-hand sides: 6.63 ms, 7.48 before.
 template <bool CPLX, int Q>
 __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     const int32_t* __restrict__ rows, const int64_t* __restrict__ fptr, const int32_t* __restrict__ fsrc,
@@ -241,7 +351,7 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     int* __restrict__ status) {
     constexpr int MAP = 128;
     const int q = Q > 0 ? Q : q_rt;
-    const int KAP = Q > 0 ? (((CPLX ? 2 * Q * Q : Q * Q) + 15) & ~15) : KAP_rt;
+    const int KAP = Q > 0 ? ((Q * Q + 15) & ~15) : KAP_rt;
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t* bfull = reinterpret_cast<uint64_t*>(smem);        // [2]
     uint64_t* mdone = bfull + 2;                                 // [2]
@@ -249,10 +359,11 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     int* issued_sh = reinterpret_cast<int*>(smem + 76);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + 64);
     int* flag = reinterpret_cast<int*>(smem + 72);
-    float4* Xs = reinterpret_cast<float4*>(smem + 128);
+    ulonglong2* Xs = reinterpret_cast<ulonglong2*>(smem + 128);   // [q2][2]: (x, x, y, y), (z, z, w, w)
     const int q2 = q * q;
-    const size_t abytes = (size_t)MAP * KAP * 2, bbytes = (size_t)RP * KAP * 2;
-    unsigned char* tiles = smem + 1024 * ((128 + (size_t)q2 * 16 + 1023) / 1024);
+    const int NB = CPLX ? 2 * RP : RP;                           // B rows, accumulator columns
+    const size_t abytes = (size_t)MAP * KAP * 2, bbytes = (size_t)NB * KAP * 2;
+    unsigned char* tiles = smem + 1024 * ((128 + (size_t)q2 * 32 + 1023) / 1024);
     // buffer b: A tile at tiles + b * abytes, B tile at tiles + 2 * abytes + b * bbytes
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;   // 544 threads: 16 generating warps + 1
     const int sigma = rows[blockIdx.x];
@@ -277,7 +388,8 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     for (int i = t; i < q2; i += blockDim.x) {
         float4 g = geo[(int64_t)sigma * q2 + i];
         g.w *= 0.07957747154594767f;   // k / (4 pi)
-        Xs[i] = g;
+        Xs[2 * i] = make_ulonglong2(f2_pack(g.x, g.x), f2_pack(g.y, g.y));
+        Xs[2 * i + 1] = make_ulonglong2(f2_pack(g.z, g.z), f2_pack(g.w, g.w));
     }
     // padding rows / columns of both A buffers stay zero
     for (size_t i = t; i < 2 * abytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(tiles)[i] = make_uint4(0, 0, 0, 0);
@@ -286,7 +398,9 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(RP >> 3) << 17) | ((uint32_t)(MAP >> 4) << 24);
+    // N <= 256 per MMA: beyond 128 complex right-hand sides the columns take two MMAs
+    const int NM = NB <= 256 ? NB : NB / 2;
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NM >> 3) << 17) | ((uint32_t)(MAP >> 4) << 24);
     // Warps 0..15 generate the A tiles, warp 16 (lane 0) issues the moments' copy
     // and the MMAs.  No CTA barrier inside the loops: a generating thread waits by
     // itself until the MMAs of block i - 2 have released buffer i & 1, each warp
@@ -307,63 +421,37 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
             }
             const int tau = fsrc[b0 + i];
             // A tile: the coupling block in FP32, stored as BF16.  A warp fills one
-            // 8 x 8 core matrix per step (lane -> row lane / 4, columns 2 (lane % 4)
+            // 8 x 8 core matrix (of Kr and of Ki) per step (lane -> row lane / 4, columns 2 (lane % 4)
             // and +1) with packed 4-byte stores: 128 contiguous bytes, no bank conflicts.
             __nv_bfloat16* A = reinterpret_cast<__nv_bfloat16*>(tiles + buf * abytes);
             const float4* Y = geo + (int64_t)tau * q2;
-            const int q8 = (q2 + 7) >> 3;
-            // quadrant offsets of the real form when q2 is a multiple of 8
-            const int offR = (q2 >> 3) * 64, offD = (q2 >> 3) * K8 * 64;
-            const bool aligned8 = (q2 & 7) == 0;
-            // 512 threads: 16 warps; with q fixed the trip count is known and the
-            // loop unrolls, so a warp keeps several core matrices' SFU work in flight
-    #pragma unroll
-            for (int cm = warp; cm < q8 * q8; cm += 16) {
-                const int ca = cm / q8, cb = cm - ca * q8;
-                const int a = 8 * ca + (lane >> 2), b = 8 * cb + 2 * (lane & 3);
-                if (a >= q2 || b >= q2) continue;   // q2 is even, so b + 1 < q2 as well
-                const float4 X = Xs[a];
-                float wr[2], wi[2];
-    #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const float4 Yb = Y[b + u];
-                    const float d0 = X.x - Yb.x, d1 = X.y - Yb.y, d2 = X.z - Yb.z;
-                    const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-                    const float rinv = rsqrtf(r2);
-                    const float w = X.w * Yb.w * rinv;          // X.w holds k / (4 pi)
-                    if constexpr (CPLX) {
-                        // phase reduced to [-pi, pi] first (the hardware sine and
-                        // cosine are accurate on that interval only)
-                        float ph = kappa * (r2 * rinv);
-                        ph = fmaf(-6.283185307179586f, rintf(ph * 0.15915494309189535f), ph);
-                        float sn, cs;
-                        __sincosf(ph, &sn, &cs);
-                        wr[u] = w * cs;
-                        wi[u] = w * sn;
-                    } else {
-                        wr[u] = w;
-                        wi[u] = 0.0f;
-                    }
+            auto put = [&](int a, int b, uint32_t kr, uint32_t ki) {   // rows a (Kr) and q2 + a (Ki)
+                auto at = [&](int m) {
+                    return reinterpret_cast<uint32_t*>(A + ((m >> 3) * K8 + (b >> 3)) * 64 + (m & 7) * 8 + (b & 7));
+                };
+                *at(a) = kr;
+                if constexpr (CPLX) *at(q2 + a) = ki;
+            };
+            uint32_t kr, ki = 0;
+            if constexpr (Q == 8) {
+                // 64 core matrices: a warp keeps its columns and takes every second row group
+                const int b = 8 * (warp & 7) + 2 * (lane & 3);
+                const MrPoint2 Y2 = mr_point2(Y[b], Y[b + 1]);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int a = 8 * ((warp >> 3) + 2 * k) + (lane >> 2);
+                    mr_values<CPLX>(Xs[2 * a], Xs[2 * a + 1], Y2, kappa, &kr, &ki);
+                    put(a, b, kr, ki);
                 }
-                const int base = (ca * K8 + (b >> 3)) * 64 + (a & 7) * 8 + (b & 7);
-                const __nv_bfloat162 kr = __floats2bfloat162_rn(wr[0], wr[1]);
-                reinterpret_cast<__nv_bfloat162*>(A + base)[0] = kr;
-                if constexpr (CPLX) {
-                    const __nv_bfloat162 mki = __floats2bfloat162_rn(-wi[0], -wi[1]);
-                    const __nv_bfloat162 ki = __floats2bfloat162_rn(wi[0], wi[1]);
-                    if (aligned8) {
-                        reinterpret_cast<__nv_bfloat162*>(A + base + offR)[0] = mki;
-                        reinterpret_cast<__nv_bfloat162*>(A + base + offD)[0] = ki;
-                        reinterpret_cast<__nv_bfloat162*>(A + base + offD + offR)[0] = kr;
-                    } else {
-                        auto at = [&](int m, int k) -> __nv_bfloat162* {
-                            return reinterpret_cast<__nv_bfloat162*>(A + ((m >> 3) * K8 + (k >> 3)) * 64 + (m & 7) * 8 +
-                                                                     (k & 7));
-                        };
-                        *at(a, b + q2) = mki;
-                        *at(a + q2, b) = ki;
-                        *at(a + q2, b + q2) = kr;
-                    }
+            } else {
+                const int q8 = (q2 + 7) >> 3;
+#pragma unroll 2
+                for (int cm = warp; cm < q8 * q8; cm += 16) {
+                    const int ca = cm / q8, cb = cm - ca * q8;
+                    const int a = 8 * ca + (lane >> 2), b = 8 * cb + 2 * (lane & 3);
+                    if (a >= q2 || b >= q2) continue;   // q2 is even, so b + 1 < q2 as well
+                    mr_values<CPLX>(Xs[2 * a], Xs[2 * a + 1], mr_point2(Y[b], Y[b + 1]), kappa, &kr, &ki);
+                    put(a, b, kr, ki);
                 }
             }
             // this warp's part of the A tile is written: make it visible to the
@@ -387,7 +475,7 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
                          : "memory");
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                              tsm(tiles + 2 * abytes + buf * bbytes)),
-                         "l"(xb + (int64_t)tau * RP * KAP), "r"((unsigned)bbytes), "r"(tsm(&bfull[buf]))
+                         "l"(xb + (int64_t)tau * NB * KAP), "r"((unsigned)bbytes), "r"(tsm(&bfull[buf]))
                          : "memory");
             const bool aok = tc_wait(&afull[buf], (unsigned)((i >> 1) & 1), wait_limit);
             const bool bok = aok && tc_wait(&bfull[buf], (unsigned)((i >> 1) & 1), wait_limit);
@@ -400,16 +488,18 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
             }
             __nv_bfloat16* A = reinterpret_cast<__nv_bfloat16*>(tiles + buf * abytes);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int kk = 0; kk < KAP / 16; ++kk) {
-                const uint64_t ad = umma_desc(tsm(A) + kk * 256, 128, K8 * 128);
-                const uint64_t bd = umma_desc(tsm(tiles + 2 * abytes + buf * bbytes) + kk * 256, 128, K8 * 128);
-                const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                    : "memory");
-            }
+            for (int n0 = 0; n0 < NB; n0 += NM)
+                for (int kk = 0; kk < KAP / 16; ++kk) {
+                    const uint64_t ad = umma_desc(tsm(A) + kk * 256, 128, K8 * 128);
+                    const uint64_t bd = umma_desc(tsm(tiles + 2 * abytes + buf * bbytes) + n0 * KAP * 2 + kk * 256, 128,
+                                                  K8 * 128);
+                    const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)n0),
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                        : "memory");
+                }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              tsm(&mdone[buf]))
                          : "memory");
@@ -431,34 +521,45 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     }
     if (__syncthreads_or(!ok || failed)) {
         if (t == 0) atomicOr(status, 1);
-    } else if (warp < 4) {
-        // warps 0..3 own TMEM lane quarters 0..3
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    } else {
+        // warps 0..3 own TMEM lane quarters 0..3; 16 right-hand sides at a time through
+        // shared memory (the tiles are free), where the rows of Kr and Ki meet
+        constexpr int SS = 33;
+        float* S = reinterpret_cast<float*>(tiles);   // [128][SS]: 16 real, 16 imaginary columns
         const int row = 32 * warp + lane;
-        const int mvalid = CPLX ? 2 * q2 : q2;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int c0 = 0; c0 < RP; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < mvalid) {
-                for (int j = 0; j < 16; ++j) {
-                    const int r = c0 + j;
-                    if (r >= R) break;
-                    const float val = __uint_as_float(v[j]);
-                    if constexpr (CPLX) {
-                        float* dst = reinterpret_cast<float*>(yh + ((int64_t)sigma * q2 + (row % q2)) * R + r);
-                        dst[row < q2 ? 0 : 1] = val;
-                    } else {
-                        yh[((int64_t)sigma * q2 + row) * R + r] = val;
-                    }
+            if (warp < 4) {
+#pragma unroll
+                for (int h = 0; h < (CPLX ? 2 : 1); ++h) {
+                    uint32_t v[16];
+                    const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(h * RP + c0);
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                        "[%16];"
+                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+                          "=r"(v[14]), "=r"(v[15])
+                        : "r"(taddr));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) S[row * SS + 16 * h + j] = __uint_as_float(v[j]);
                 }
             }
+            __syncthreads();
+            for (int e = t; e < 16 * q2; e += blockDim.x) {
+                const int j = e & 15, a = e >> 4, r = c0 + j;
+                if (r >= R) continue;
+                const int64_t o = ((int64_t)sigma * q2 + a) * R + r;
+                const float* Sr = S + a * SS;
+                if constexpr (CPLX) {
+                    const float* Si = S + (q2 + a) * SS;
+                    yh[o] = make_float2(Sr[j] - Si[16 + j], Sr[16 + j] + Si[j]);
+                } else {
+                    yh[o] = Sr[j];
+                }
+            }
+            __syncthreads();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -509,27 +610,6 @@ __global__ void mr_store_kernel(int64_t n_far, const int32_t* __restrict__ ftgt,
         T[st_tile_off(a, b)] = __float2bfloat16(w * cs);
         T[st_tile_off(ST_Q2 + a, b)] = __float2bfloat16(w * sn);
     }
-}
-
-// moments x^ [C][64][R] (float2) -> per (chunk, cluster) [2 RQ][64] BF16 tiles
-__global__ void mr_bpack_stored_kernel(int R, int RQ, int nch, int64_t C, const float2* __restrict__ xh,
-                                       __nv_bfloat16* __restrict__ xb) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int N = 2 * RQ;
-    if (idx >= (int64_t)nch * C * N * ST_Q2) return;
-    const int k = (int)(idx % ST_Q2);
-    int64_t rem = idx / ST_Q2;
-    const int n = (int)(rem % N);
-    rem /= N;
-    const int64_t c = rem % C;
-    const int ch = (int)(rem / C);
-    const int r = ch * 64 + (n < RQ ? n : n - RQ);   // RQ <= 64
-    float v = 0.0f;
-    if (r < R) {
-        const float2 x = xh[(c * ST_Q2 + k) * R + r];
-        v = n < RQ ? x.x : x.y;
-    }
-    xb[((int64_t)ch * C + c) * N * ST_Q2 + st_tile_off(n, k)] = __float2bfloat16(v);
 }
 
 template <int ST_NST>
@@ -700,24 +780,41 @@ cudaError_t launch_stored(ibem_handle* h, int nst, unsigned nrows, int nch, cons
 }
 
 // ---- L2L, back-projection, near field, restriction ---------------------------------------
-template <bool CPLX>
-__global__ void mr_back_kernel(int R, int64_t E, int pp, int q, const float* __restrict__ M,
-                               const typename MrType<CPLX>::T* __restrict__ yh, int64_t leaf_off,
-                               typename MrType<CPLX>::T* __restrict__ ys) {
+// y*[iv][iu] = sum M[av][iv] M[au][iu] y^[av][au]; thread (element, right-hand side)
+template <bool CPLX, int PP>
+__global__ void __launch_bounds__(128) mr_back_kernel(int R, int64_t E, int q, const float* __restrict__ M,
+                                                      const typename MrType<CPLX>::T* __restrict__ yh, int64_t leaf_off,
+                                                      typename MrType<CPLX>::T* __restrict__ ys) {
     typedef typename MrType<CPLX>::T T;
-    const int q2 = q * q, nb = pp * pp;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= E * nb * R) return;
-    int r = (int)(idx % R);
-    int64_t rem = idx / R;
-    int i = (int)(rem % nb);
-    int64_t e = rem / nb;
-    const int iu = i % pp, iv = i / pp;
-    T acc = mr_zero(T());
-    for (int av = 0; av < q; ++av)
-        for (int au = 0; au < q; ++au)
-            acc = mr_axpy(M[au * pp + iu] * M[av * pp + iv], yh[((leaf_off + e) * q2 + av * q + au) * R + r], acc);
-    ys[idx] = acc;
+    constexpr int nb = PP * PP;
+    __shared__ float Ms[IBEM_MAX_Q * PP];
+    for (int i = threadIdx.x; i < q * PP; i += blockDim.x) Ms[i] = M[i];
+    __syncthreads();
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= E * R) return;
+    const int r = (int)(idx % R);
+    const int64_t e = idx / R;
+    const T* in = yh + (leaf_off + e) * q * q * R + r;
+    T out[nb];
+#pragma unroll
+    for (int i = 0; i < nb; ++i) out[i] = mr_zero(T());
+    for (int au = 0; au < q; ++au) {
+        T t[PP];
+#pragma unroll
+        for (int iv = 0; iv < PP; ++iv) t[iv] = mr_zero(T());
+#pragma unroll 4
+        for (int av = 0; av < q; ++av) {
+            const T y = in[(int64_t)(av * q + au) * R];
+#pragma unroll
+            for (int iv = 0; iv < PP; ++iv) t[iv] = mr_axpy(Ms[av * PP + iv], y, t[iv]);
+        }
+#pragma unroll
+        for (int iv = 0; iv < PP; ++iv)
+#pragma unroll
+            for (int iu = 0; iu < PP; ++iu) out[iv * PP + iu] = mr_axpy(Ms[au * PP + iu], t[iv], out[iv * PP + iu]);
+    }
+#pragma unroll
+    for (int i = 0; i < nb; ++i) ys[(e * nb + i) * R + r] = out[i];
 }
 
 // one CTA per target element; thread (i, r) over the row's near blocks
@@ -750,13 +847,16 @@ __global__ void mr_near_kernel(int R, int nb, const int64_t* __restrict__ nptr, 
     }
 }
 
-// Same product with one thread per right-hand side holding all NB rows of its
-// element: the element's blocks pass through shared memory in chunks of KC
-// (broadcast reads, 4 FMA per complex entry and load), each source value is
-// loaded once per block (coalesced over the right-hand sides).  The sums run in
-// the same order (blocks, then columns) as in mr_near_kernel.
+// Same product with a thread holding all NB rows of its element for one right-hand
+// side: the element's blocks pass through shared memory in chunks of KC (broadcast
+// reads, 4 FMA per complex entry and load), each source value is loaded once per
+// block (coalesced over the right-hand sides).  The CTA's threads form slices of RT >=
+// R threads; slice q takes every S-th block of a chunk, and the slices are added in
+// order through shared memory.  Bound: FMA and the latency of the source values;
+// without slices 16 right-hand sides kept half a warp per element busy (level 5, p = 2:
+// 1272 us, now 240 us; 64 right-hand sides 942 us, now 430 us).
 template <bool CPLX, int NB>
-__global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, const int64_t* __restrict__ nptr,
+__global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, int RT, const int64_t* __restrict__ nptr,
                                                            const int32_t* __restrict__ nsrc,
                                                            const float* __restrict__ blocks,
                                                            const typename MrType<CPLX>::T* __restrict__ xs,
@@ -764,11 +864,12 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, const int64_t*
     typedef typename MrType<CPLX>::T T;
     constexpr int CW = CPLX ? 2 : 1;
     constexpr int BF = NB * NB * CW;                             // floats per block
-    constexpr int KC = (NB == 9 ? 32 : 8) * (CPLX ? 1 : 2);      // blocks per shared-memory chunk
-    __shared__ float sb[KC * BF];
+    constexpr int KC = (NB == 9 ? 32 : 16) * (CPLX ? 1 : 2);     // blocks per shared-memory chunk
+    static_assert(KC * BF >= 256 * NB * CW, "the slices' sums fit in the chunk");
+    __shared__ __align__(16) float sb[KC * BF];
     __shared__ int ss[KC];
     const int64_t e = blockIdx.x;
-    const int r = threadIdx.x;
+    const int t = threadIdx.x, slice = t / RT, r = t - slice * RT, S = blockDim.x / RT;
     const bool act = r < R;
     float ar[NB], ai[NB];
 #pragma unroll
@@ -776,11 +877,11 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, const int64_t*
     const int64_t k0 = nptr[e], k1 = nptr[e + 1];
     for (int64_t kb = k0; kb < k1; kb += KC) {
         const int kc = (int)(k1 - kb < KC ? k1 - kb : KC);
-        for (int i = threadIdx.x; i < kc * BF; i += blockDim.x) sb[i] = blocks[kb * BF + i];
-        for (int i = threadIdx.x; i < kc; i += blockDim.x) ss[i] = nsrc[kb + i];
+        for (int i = t; i < kc * BF; i += blockDim.x) sb[i] = blocks[kb * BF + i];
+        for (int i = t; i < kc; i += blockDim.x) ss[i] = nsrc[kb + i];
         __syncthreads();
         if (act) {
-            for (int kk = 0; kk < kc; ++kk) {
+            for (int kk = slice; kk < kc; kk += S) {
                 const int64_t s = ss[kk];
                 T xv[NB];
 #pragma unroll
@@ -791,9 +892,9 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, const int64_t*
 #pragma unroll
                     for (int j = 0; j < NB; ++j) {
                         if constexpr (CPLX) {
-                            const float br = B[2 * (i * NB + j)], bi = B[2 * (i * NB + j) + 1];
-                            ar[i] = fmaf(br, xv[j].x, fmaf(-bi, xv[j].y, ar[i]));
-                            ai[i] = fmaf(br, xv[j].y, fmaf(bi, xv[j].x, ai[i]));
+                            const float2 b = *reinterpret_cast<const float2*>(B + 2 * (i * NB + j));
+                            ar[i] = fmaf(b.x, xv[j].x, fmaf(-b.y, xv[j].y, ar[i]));
+                            ai[i] = fmaf(b.x, xv[j].y, fmaf(b.y, xv[j].x, ai[i]));
                         } else {
                             ar[i] = fmaf(B[i * NB + j], xv[j], ar[i]);
                         }
@@ -803,12 +904,25 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, const int64_t*
         }
         __syncthreads();
     }
-    if (!act) return;
+    float* red = sb;                                             // [NB][CW][blockDim]
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        T* out = ys + (e * NB + i) * R + r;
-        if constexpr (CPLX) *out = make_float2(out->x + ar[i], out->y + ai[i]);
-        else *out += ar[i];
+        red[(i * CW) * 256 + t] = ar[i];
+        if constexpr (CPLX) red[(i * CW + 1) * 256 + t] = ai[i];
+    }
+    __syncthreads();
+    for (int o = t; o < NB * RT; o += blockDim.x) {
+        const int i = o / RT, rr = o - i * RT;
+        if (rr >= R) continue;
+        float v[CW];
+#pragma unroll
+        for (int c = 0; c < CW; ++c) {
+            v[c] = 0.0f;
+            for (int q = 0; q < S; ++q) v[c] += red[(i * CW + c) * 256 + q * RT + rr];
+        }
+        T* out = ys + (e * NB + i) * R + rr;
+        if constexpr (CPLX) *out = make_float2(out->x + v[0], out->y + v[CW - 1]);
+        else *out += v[0];
     }
 }
 
@@ -864,14 +978,14 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
     const int T_ = 256;
     const int q2 = P.q2;
     const int RP = (R + 15) & ~15;
-    const int KAP = ((CPLX ? 2 * q2 : q2) + 15) & ~15;
+    const int KAP = (q2 + 15) & ~15, NB = CPLX ? 2 * RP : RP;
     // work space (grown on demand)
     const size_t need_t = (size_t)R * P.N, need_s = (size_t)R * P.Nstar, need_h = (size_t)R * P.C * (q2 > 0 ? q2 : 1);
-    // moments as BF16 tiles: generated coupling [C][RP][KAP]; stored coupling
+    // moments as BF16 tiles: generated coupling [C][NB][KAP]; stored coupling
     // [nch][C][2 RQ][64] with chunks of 64 right-hand sides
     const bool stored = CPLX && h->d_Kbf != nullptr;
     const int RQ = ((R < 64 ? R : 64) + 7) & ~7, nch = (R + 63) / 64;
-    size_t need_b = (size_t)P.C * RP * (KAP > 0 ? KAP : 16);
+    size_t need_b = (size_t)P.C * NB * (KAP > 0 ? KAP : 16);
     if (stored) need_b = std::max(need_b, (size_t)nch * P.C * 2 * RQ * ST_Q2);
     const size_t bytes = sizeof(T) * (need_t + 2 * need_s + 2 * need_h) + 2 * need_b + 1024;
     if (bytes > h->mr_bytes) {
@@ -899,7 +1013,14 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
         const int64_t leaf_off = P.level_off[P.m];
         {
             PhaseTimer pt(h, 1);
-            mr_leaf_kernel<CPLX><<<nblk(P.E * q2 * R, T_), T_, 0, st>>>(R, P.E, P.pp, P.q, h->d_Mf, xs, leaf_off, xh);
+            const unsigned lg = nblk(P.E * R, 128);
+            switch (P.pp) {
+                case 1: mr_leaf_kernel<CPLX, 1><<<lg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, xs, leaf_off, xh); break;
+                case 2: mr_leaf_kernel<CPLX, 2><<<lg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, xs, leaf_off, xh); break;
+                case 3: mr_leaf_kernel<CPLX, 3><<<lg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, xs, leaf_off, xh); break;
+                case 4: mr_leaf_kernel<CPLX, 4><<<lg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, xs, leaf_off, xh); break;
+                default: mr_leaf_kernel<CPLX, 5><<<lg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, xs, leaf_off, xh);
+            }
             h->launches++;
             const size_t smm = (size_t)8 * q2 * MR_RC * sizeof(T) + 2 * q2 * sizeof(float);
             for (int L = P.m - 1; L >= 0; --L) {
@@ -913,9 +1034,11 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
         const unsigned nrows = (unsigned)h->far_rows.size();
         if (nrows > 0 && stored) {
             PhaseTimer pt(h, 2);
-            mr_bpack_stored_kernel<<<nblk((int64_t)nch * P.C * 2 * RQ * ST_Q2, T_), T_, 0, st>>>(
-                R, RQ, nch, P.C, reinterpret_cast<const float2*>(xh), xb);
-            h->launches++;
+            for (int ch = 0; ch < nch; ++ch) {
+                mr_bpack_kernel<CPLX><<<nblk((int64_t)P.C * RQ * (ST_Q2 / 8), T_), T_, 0, st>>>(
+                    R, 64 * ch, RQ, ST_Q2, P.C, ST_Q2, xh, xb + (int64_t)ch * P.C * 2 * RQ * ST_Q2);
+                h->launches++;
+            }
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
             if ((e = cudaStreamIsCapturing(st, &cap))) return e;
             if (h->st_nst == 0 && cap == cudaStreamCaptureStatusNone) {
@@ -953,11 +1076,12 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
             h->launches++;
         } else if (nrows > 0) {
             PhaseTimer pt(h, 2);
-            mr_bpack_kernel<CPLX><<<nblk((int64_t)P.C * RP * KAP, T_), T_, 0, st>>>(R, RP, KAP, P.C, q2, xh, xb);
+            mr_bpack_kernel<CPLX><<<nblk((int64_t)P.C * RP * (KAP / 8), T_), T_, 0, st>>>(R, 0, RP, KAP, P.C, q2, xh, xb);
             int tcols = 32;
-            while (tcols < RP) tcols <<= 1;
-            const size_t sm = 1024 * ((128 + (size_t)q2 * 16 + 1023) / 1024) + 2 * (size_t)128 * KAP * 2 +
-                              2 * (size_t)RP * KAP * 2;
+            while (tcols < NB) tcols <<= 1;
+            // the tiles, or the 128 x 33 floats that the row is joined in
+            const size_t sm = 1024 * ((128 + (size_t)q2 * 32 + 1023) / 1024) +
+                              std::max<size_t>(2 * (size_t)(128 + NB) * KAP * 2, 128 * 33 * sizeof(float));
             auto kern = P.q == 8 ? mr_coupling_tc_kernel<CPLX, 8>
                                  : (P.q == 6 ? mr_coupling_tc_kernel<CPLX, 6> : mr_coupling_tc_kernel<CPLX, 0>);
             if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
@@ -974,18 +1098,26 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
                 R, P.level_off[L], P.level_off[L + 1], P.q, h->d_Sf, yh);
             h->launches++;
         }
-        mr_back_kernel<CPLX><<<nblk(P.E * P.nb * R, T_), T_, 0, st>>>(R, P.E, P.pp, P.q, h->d_Mf, yh, leaf_off, ys);
+        const unsigned bg = nblk(P.E * R, 128);
+        switch (P.pp) {
+            case 1: mr_back_kernel<CPLX, 1><<<bg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, yh, leaf_off, ys); break;
+            case 2: mr_back_kernel<CPLX, 2><<<bg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, yh, leaf_off, ys); break;
+            case 3: mr_back_kernel<CPLX, 3><<<bg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, yh, leaf_off, ys); break;
+            case 4: mr_back_kernel<CPLX, 4><<<bg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, yh, leaf_off, ys); break;
+            default: mr_back_kernel<CPLX, 5><<<bg, 128, 0, st>>>(R, P.E, P.q, h->d_Mf, yh, leaf_off, ys);
+        }
         h->launches++;
     }
     int nthreads = P.nb * R < 512 ? ((P.nb * R + 31) / 32) * 32 : 512;
     {
         PhaseTimer pt(h, 4);
-        const int tr = ((R + 31) / 32) * 32;
+        // slices of 16, 32, ... threads, as many as fit in 256 threads
+        const int RT = R <= 16 ? 16 : ((R + 31) / 32) * 32, tr = RT * std::max(1, std::min(256 / RT, 16));
         if (P.nb == 9)
-            mr_near_rows_kernel<CPLX, 9><<<(unsigned)P.E, tr, 0, st>>>(R, h->d_near_ptr, h->d_near_src, h->d_near32,
+            mr_near_rows_kernel<CPLX, 9><<<(unsigned)P.E, tr, 0, st>>>(R, RT, h->d_near_ptr, h->d_near_src, h->d_near32,
                                                                        xs, ys);
         else if (P.nb == 16)
-            mr_near_rows_kernel<CPLX, 16><<<(unsigned)P.E, tr, 0, st>>>(R, h->d_near_ptr, h->d_near_src, h->d_near32,
+            mr_near_rows_kernel<CPLX, 16><<<(unsigned)P.E, tr, 0, st>>>(R, RT, h->d_near_ptr, h->d_near_src, h->d_near32,
                                                                         xs, ys);
         else
             mr_near_kernel<CPLX><<<(unsigned)P.E, nthreads, 0, st>>>(R, P.nb, h->d_near_ptr, h->d_near_src,
