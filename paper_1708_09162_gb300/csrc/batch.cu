@@ -22,6 +22,7 @@
 #include <cstring>
 
 #include "batch_internal.cuh"
+#include "fp32_eval.cuh"
 
 namespace ibem {
 
@@ -141,12 +142,24 @@ __global__ void b_m2m_kernel(const BatchInst* __restrict__ B, int n, const int64
 // Right-hand sides per coupling work item: every kernel value generated for a
 // far block serves up to RB right-hand sides of the instance (the tile shape
 // chosen with the CTA size by the autotuner: RB in 4, 8, 16).
+// A group's source points and moments (all RB right-hand sides of a point side by
+// side) are staged in shared memory, the next block's are in flight in registers
+// meanwhile: the inner loop has broadcast reads at constant offsets only.  Read
+// from global memory instead, its 64-bit address arithmetic took as much issue as
+// the arithmetic proper.  Bound: FP32 issue.  Eight instances, levels 2-4, 1 to 15
+// right-hand sides: 4.24 ms, 7.66 before.
+inline __host__ __device__ size_t b_coupling_smem(int rb, int threads) {
+    return (size_t)threads * (sizeof(float4) + (size_t)rb * 2 * sizeof(float));   // also holds the partial sums
+}
 
 template <int BC_RB>
 __global__ void b_coupling_kernel(const BatchInst* __restrict__ B, int n, const int64_t* __restrict__ pre,
                                   int64_t total, int* __restrict__ counter) {
-    extern __shared__ float red[];   // [BC_RB][blockDim][2]
+    extern __shared__ __align__(16) float bc_sm[];
     __shared__ int64_t item;
+    float4* Ys = reinterpret_cast<float4*>(bc_sm);          // [blockDim]: group g's points at g q2
+    float* Vs = bc_sm + 4 * blockDim.x;                      // [blockDim][RB] complex, or [blockDim][RB] real
+    float* red = bc_sm;                                      // [BC_RB][blockDim][2], after the blocks
     for (;;) {
         if (threadIdx.x == 0) item = atomicAdd(counter, 1);
         __syncthreads();
@@ -163,47 +176,95 @@ __global__ void b_coupling_kernel(const BatchInst* __restrict__ B, int n, const 
         const int q2 = I.q2, cw = I.helm ? 2 : 1;
         const int G = blockDim.x / q2;
         const int t = threadIdx.x, gg = t / q2, a = t % q2;
-        float sr[BC_RB], si[BC_RB];
+        const float4* geo = reinterpret_cast<const float4*>(I.igeo32);
+        const int64_t rstride = (int64_t)I.C * q2 * cw;      // between right-hand sides
+        const float* xr = I.xh + (int64_t)r0 * rstride + (int64_t)a * cw;
+        const int32_t* src = I.far_src + I.far_ptr[sigma];
+        const int nb = (int)(I.far_ptr[sigma + 1] - I.far_ptr[sigma]);
+        const float kappa = I.kappa;
+        float4 X = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (gg < G) X = geo[(int64_t)sigma * q2 + a];
+        float sr[BC_RB], si[BC_RB], vr[BC_RB], vi[BC_RB];
+        float4 yn = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < BC_RB; ++j) sr[j] = si[j] = 0.0f;
-        if (gg < G) {
-            const float4 X = reinterpret_cast<const float4*>(I.igeo32)[(int64_t)sigma * q2 + a];
-            const int64_t rstride = (int64_t)I.C * q2 * cw;      // between right-hand sides
-            const float* xr = I.xh + (int64_t)r0 * rstride;
-            for (int64_t blk = I.far_ptr[sigma] + gg; blk < I.far_ptr[sigma + 1]; blk += G) {
-                const int64_t tau = I.far_src[blk];
-                const float4* Y = reinterpret_cast<const float4*>(I.igeo32) + tau * q2;
-                const float* V = xr + tau * q2 * cw;
+        for (int j = 0; j < BC_RB; ++j) sr[j] = si[j] = vr[j] = vi[j] = 0.0f;
+        auto fetch = [&](int blk) {
+            if (gg >= G || blk >= nb) return;
+            const int64_t tau = src[blk];
+            yn = geo[tau * q2 + a];
+            const float* V = xr + tau * q2 * cw;
+#pragma unroll
+            for (int j = 0; j < BC_RB; ++j)
+                if (j < nr) {
+                    if (cw == 2) {
+                        const float2 v = *reinterpret_cast<const float2*>(V + j * rstride);
+                        vr[j] = v.x;
+                        vi[j] = v.y;
+                    } else {
+                        vr[j] = V[j * rstride];
+                    }
+                }
+        };
+        fetch(gg);
+        for (int b0 = 0; b0 < nb; b0 += G) {
+            __syncthreads();   // the previous block is used
+            if (gg < G) {
+                Ys[t] = yn;
+                float4* o = reinterpret_cast<float4*>(Vs + t * BC_RB * cw);
+                if (cw == 2) {
+#pragma unroll
+                    for (int j = 0; j < BC_RB; j += 2) o[j / 2] = make_float4(vr[j], vi[j], vr[j + 1], vi[j + 1]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < BC_RB; j += 4) o[j / 4] = make_float4(vr[j], vr[j + 1], vr[j + 2], vr[j + 3]);
+                }
+            }
+            __syncthreads();
+            fetch(b0 + G + gg);
+            if (gg >= G || b0 + gg >= nb) continue;
+            const float4* Y = Ys + gg * q2;
+            const float4* V = reinterpret_cast<const float4*>(Vs + gg * q2 * BC_RB * cw);
+            if (cw == 2) {
+#pragma unroll 2
                 for (int b = 0; b < q2; ++b) {
                     const float4 y = Y[b];
                     const float d0 = X.x - y.x, d1 = X.y - y.y, d2 = X.z - y.z;
                     const float r2 = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-                    const float rinv = rsqrtf(r2);
+                    const float rinv = approx_rsqrt(r2);
                     const float w = y.w * rinv;
-                    if (cw == 2) {
-                        // phase reduced to [-pi, pi] first: the hardware sine and
-                        // cosine are accurate on that interval only
-                        float ph = I.kappa * (r2 * rinv);
-                        ph = fmaf(-6.283185307179586f, rintf(ph * 0.15915494309189535f), ph);
-                        float sn, cs;
-                        __sincosf(ph, &sn, &cs);
-                        const float kr = w * cs, ki = w * sn;
+                    // phase reduced to [-pi, pi] first: the hardware sine and cosine are
+                    // accurate on that interval only
+                    const float ph = reduce_phase(kappa * (r2 * rinv));
+                    const float kr = w * approx_cos(ph), ki = w * approx_sin(ph);
 #pragma unroll
-                        for (int j = 0; j < BC_RB; ++j) {
-                            if (j < nr) {
-                                const float vr = V[j * rstride + 2 * b], vi = V[j * rstride + 2 * b + 1];
-                                sr[j] = fmaf(kr, vr, fmaf(-ki, vi, sr[j]));
-                                si[j] = fmaf(kr, vi, fmaf(ki, vr, si[j]));
-                            }
+                    for (int j = 0; j < BC_RB; j += 2)
+                        if (j < nr) {
+                            const float4 v = V[b * (BC_RB / 2) + j / 2];
+                            sr[j] = fmaf(kr, v.x, fmaf(-ki, v.y, sr[j]));
+                            si[j] = fmaf(kr, v.y, fmaf(ki, v.x, si[j]));
+                            sr[j + 1] = fmaf(kr, v.z, fmaf(-ki, v.w, sr[j + 1]));
+                            si[j + 1] = fmaf(kr, v.w, fmaf(ki, v.z, si[j + 1]));
                         }
-                    } else {
+                }
+            } else {
+#pragma unroll 2
+                for (int b = 0; b < q2; ++b) {
+                    const float4 y = Y[b];
+                    const float d0 = X.x - y.x, d1 = X.y - y.y, d2 = X.z - y.z;
+                    const float w = y.w * approx_rsqrt(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
 #pragma unroll
-                        for (int j = 0; j < BC_RB; ++j)
-                            if (j < nr) sr[j] = fmaf(w, V[j * rstride + b], sr[j]);
-                    }
+                    for (int j = 0; j < BC_RB; j += 4)
+                        if (j < nr) {
+                            const float4 v = V[b * (BC_RB / 4) + j / 4];
+                            sr[j] = fmaf(w, v.x, sr[j]);
+                            sr[j + 1] = fmaf(w, v.y, sr[j + 1]);
+                            sr[j + 2] = fmaf(w, v.z, sr[j + 2]);
+                            sr[j + 3] = fmaf(w, v.w, sr[j + 3]);
+                        }
                 }
             }
         }
+        __syncthreads();
 #pragma unroll
         for (int j = 0; j < BC_RB; ++j) {
             red[2 * (j * blockDim.x + t)] = sr[j];
@@ -211,16 +272,16 @@ __global__ void b_coupling_kernel(const BatchInst* __restrict__ B, int n, const 
         }
         __syncthreads();
         if (t < q2) {
-            const float ka = reinterpret_cast<const float4*>(I.igeo32)[(int64_t)sigma * q2 + t].w * 0.07957747154594767f;
+            const float ka = geo[(int64_t)sigma * q2 + t].w * 0.07957747154594767f;
             for (int j = 0; j < nr; ++j) {
-                float vr = 0.0f, vi = 0.0f;
+                float ur = 0.0f, ui = 0.0f;
                 for (int g = 0; g < G; ++g) {
-                    vr += red[2 * (j * blockDim.x + g * q2 + t)];
-                    vi += red[2 * (j * blockDim.x + g * q2 + t) + 1];
+                    ur += red[2 * (j * blockDim.x + g * q2 + t)];
+                    ui += red[2 * (j * blockDim.x + g * q2 + t) + 1];
                 }
                 float* o = I.yh + (((int64_t)(r0 + j) * I.C + sigma) * q2 + t) * cw;
-                o[0] = vr * ka;
-                if (cw == 2) o[1] = vi * ka;
+                o[0] = ur * ka;
+                if (cw == 2) o[1] = ui * ka;
             }
         }
         __syncthreads();
@@ -259,7 +320,10 @@ __global__ void b_l2l_kernel(const BatchInst* __restrict__ B, int n, const int64
     if (cw == 2) o[1] += ai;
 }
 
-// back-projection plus near field; item (r, e, i)
+// back-projection plus near field; item (e, r, i): the right-hand sides of an element
+// are neighbours, so its near blocks are read from the caches after the first one
+// (with the right-hand side outermost they came from L2 for each: 0.94 ms on the
+// eight-instance batch, now 0.74 ms)
 __global__ void b_back_near_kernel(const BatchInst* __restrict__ B, int n, const int64_t* __restrict__ pre,
                                    int64_t total) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -269,8 +333,8 @@ __global__ void b_back_near_kernel(const BatchInst* __restrict__ B, int n, const
     int64_t loc = g - pre[k];
     const int i = (int)(loc % I.nb);
     loc /= I.nb;
-    const int64_t e = loc % I.E;
-    const int r = (int)(loc / I.E);
+    const int r = (int)(loc % I.R);
+    const int64_t e = loc / I.R;
     const int iu = i % I.pp, iv = i / I.pp, cw = I.helm ? 2 : 1, nbb = I.nb * I.nb;
     float ar = 0.0f, ai = 0.0f;
     const float* v = I.yh + (((int64_t)r * I.C + I.lvl[I.m] + e) * I.q2) * cw;
@@ -360,7 +424,7 @@ cudaError_t batch_enqueue(ibem_batch* b, const double* x, double* y, int couplin
         ++launches;
     }
     if (total(B::ST_COUPLE) > 0) {
-        const size_t sm = 2 * (size_t)b->couple_rb * coupling_threads * sizeof(float);
+        const size_t sm = b_coupling_smem(b->couple_rb, coupling_threads);
         if (b->couple_rb == 4)
             b_coupling_kernel<4><<<b->couple_ctas, coupling_threads, sm, st>>>(
                 b->d_inst, b->n, b->d_pre[B::ST_COUPLE], total(B::ST_COUPLE), b->d_counter);
@@ -417,6 +481,8 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
     b->handles.assign(handles, handles + n);
     cudaGetDevice(&b->device);
     b->offsets.assign(n + 1, 0);
+    // every vector of the arena starts on 16 bytes (complex values are read as pairs)
+    auto padded = [](size_t k) { return (k + 3) / 4 * 4; };
     size_t floats = 0;
     std::vector<size_t> base(n);
     for (int i = 0; i < n; ++i) {
@@ -431,20 +497,20 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
         const int cw = h->helm ? 2 : 1;
         b->offsets[i + 1] = b->offsets[i] + (int64_t)nrhs[i] * P.N * cw;
         base[i] = floats;
-        floats += (size_t)nrhs[i] * cw * (2 * P.Nstar);       // xs, ys
+        floats += 2 * padded((size_t)nrhs[i] * cw * P.Nstar);   // xs, ys
         b->max_m = std::max(b->max_m, P.m);
     }
     b->yh_begin = floats;
     for (int i = 0; i < n; ++i) {
         const Plan& P = handles[i]->P;
-        floats += (size_t)nrhs[i] * (handles[i]->helm ? 2 : 1) * P.C * P.q2;   // yh (cleared per application)
+        floats += padded((size_t)nrhs[i] * (handles[i]->helm ? 2 : 1) * P.C * P.q2);   // yh (cleared per application)
     }
     b->yh_floats = floats - b->yh_begin;
     std::vector<size_t> xh_base(n);
     for (int i = 0; i < n; ++i) {
         const Plan& P = handles[i]->P;
         xh_base[i] = floats;
-        floats += (size_t)nrhs[i] * (handles[i]->helm ? 2 : 1) * P.C * P.q2;
+        floats += padded((size_t)nrhs[i] * (handles[i]->helm ? 2 : 1) * P.C * P.q2);
     }
     b->arena_floats = floats;
     if (cudaMalloc(&b->arena, floats * sizeof(float)) || cudaMalloc(&b->d_counter, sizeof(int))) {
@@ -469,9 +535,9 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
         I.far_ptr = h->d_far_ptr; I.far_src = h->d_far_src; I.far_rows = h->d_far_rows;
         I.igeo32 = h->d_igeo32;
         I.xs = b->arena + base[i];
-        I.ys = I.xs + (size_t)I.R * cw * P.Nstar;
+        I.ys = I.xs + padded((size_t)I.R * cw * P.Nstar);
         I.yh = b->arena + yh_cursor;
-        yh_cursor += (size_t)I.R * cw * P.C * P.q2;
+        yh_cursor += padded((size_t)I.R * cw * P.C * P.q2);
         I.xh = b->arena + xh_base[i];
         I.xoff = b->offsets[i];
         b->inst.push_back(I);
@@ -526,16 +592,16 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
                         cudaMemcpyHostToDevice, b->stream);
     };
     auto resident = [&](int rb, int threads) {
-        const size_t smb = 2 * (size_t)rb * threads * sizeof(float);
+        const size_t smb = b_coupling_smem(rb, threads);
         int per_sm = 0;
         if (rb == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b_coupling_kernel<4>, threads, smb);
         else if (rb == 16) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b_coupling_kernel<16>, threads, smb);
         else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b_coupling_kernel<8>, threads, smb);
         return sms * per_sm;   // 0: this shape cannot be launched (registers or shared memory)
     };
-    cudaFuncSetAttribute(b_coupling_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 4 * 512 * 4);
-    cudaFuncSetAttribute(b_coupling_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8 * 512 * 4);
-    cudaFuncSetAttribute(b_coupling_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 16 * 512 * 4);
+    cudaFuncSetAttribute(b_coupling_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_coupling_smem(4, 512));
+    cudaFuncSetAttribute(b_coupling_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_coupling_smem(8, 512));
+    cudaFuncSetAttribute(b_coupling_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b_coupling_smem(16, 512));
     // autotune the tile (right-hand sides per work item) and the CTA size of the
     // persistent coupling kernel on scratch inputs
     double* xs_tmp = nullptr;
