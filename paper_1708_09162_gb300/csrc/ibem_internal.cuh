@@ -424,20 +424,14 @@ struct PhaseTimer {
 // real kernels of kernels_apply.cu reused by the complex (Helmholtz) path
 __global__ void lift_kernel(int R, int64_t E, int p, int ne1, const double* __restrict__ ext,
                             const double* __restrict__ x, int64_t N, double* __restrict__ xs);
-__global__ void restrict_kernel(int R, int64_t N, int p, int ne1, const double* __restrict__ ext,
-                                const double* __restrict__ ys, int64_t E, double* __restrict__ y);
+void launch_restrict(ibem_handle* h, int R, const double* ys, double* y);
 __global__ void leaf_moment_kernel(int R, int64_t E, int pp, int q, const double* __restrict__ M,
                                    const double* __restrict__ xs, int64_t leaf_off, int64_t C, double* __restrict__ xh);
-__global__ void m2m_kernel(int R, int64_t nL, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                           int64_t C, double* __restrict__ xh);
-__global__ void l2l_kernel(int R, int64_t nL1, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                           int64_t C, double* __restrict__ yh);
+// M2M / L2L of every level for R real vectors
+cudaError_t launch_m2m(ibem_handle* h, int R, double* xh);
+cudaError_t launch_l2l(ibem_handle* h, int R, double* yh);
 __global__ void leaf_back_kernel(int R, int64_t E, int pp, int q, const double* __restrict__ M,
                                  const double* __restrict__ yh, int64_t leaf_off, int64_t C, double* __restrict__ ys);
-__global__ void m2m_sep_kernel(int64_t nL, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                               int64_t C, double* __restrict__ xh);
-__global__ void l2l_sep_kernel(int64_t nL, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                               int64_t C, double* __restrict__ yh);
 __global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ out, int64_t n);
 __global__ void rhs_super_kernel(int R, int64_t E, int QQ, int nb, const double* __restrict__ qgeo,
                                  const double* __restrict__ phi, const double* __restrict__ g, int64_t nq,

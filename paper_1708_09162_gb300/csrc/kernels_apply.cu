@@ -78,6 +78,50 @@ __global__ void restrict_kernel(int R, int64_t N, int p, int ne1, const double* 
     y[idx] = acc;
 }
 
+// The same with one thread per (dof, element of its support), the (p + 1)^2 shares added
+// by shuffles in a fixed order: the single thread's sum over up to 25 elements is a
+// chain of some 30 us (p = 3), which a short vector cannot hide.  G: lanes per dof,
+// a power of two >= (p + 1)^2.
+__global__ void restrict_group_kernel(int R, int64_t N, int p, int ne1, int G, const double* __restrict__ ext,
+                                      const double* __restrict__ ys, int64_t E, double* __restrict__ y) {
+    const int pp = p + 1, nb = pp * pp, n1 = ne1 + p;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, idx = g / G;
+    const int k = (int)(g % G);
+    double acc = 0.0;
+    if (idx < R * N && k < nb) {
+        const int64_t r = idx / N, dof = idx % N;
+        const int patch = (int)(dof / ((int64_t)n1 * n1)), rem = (int)(dof % ((int64_t)n1 * n1));
+        const int jv = rem / n1, ju = rem % n1, iy = jv - p + k / pp, ix = ju - p + k % pp;
+        if (iy >= 0 && iy < ne1 && ix >= 0 && ix < ne1) {
+            const double* v = ys + (r * E + patch * (int64_t)ne1 * ne1 + morton2(ix, iy)) * nb;
+            const double* cu = ext + ((int64_t)ix * pp + (ju - ix)) * pp;
+            const double* cv = ext + ((int64_t)iy * pp + (jv - iy)) * pp;
+            for (int iv = 0; iv < pp; ++iv) {
+                double row = 0.0;
+                for (int iu = 0; iu < pp; ++iu) row += cu[iu] * v[iv * pp + iu];
+                acc += cv[iv] * row;
+            }
+        }
+    }
+    for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (idx < R * N && k == 0) y[idx] = acc;
+}
+
+// y = T ys for R real vectors.  Up to some 8 threads per lane of the chip the grouped
+// form is as fast as its launch (p = 3, level 5: 33 -> 10 us); beyond, its idle lanes
+// (7 of 16 at p = 2) would cost more than the chain.
+void launch_restrict(ibem_handle* h, int R, const double* ys, double* y) {
+    const Plan& P = h->P;
+    int G = 1;
+    while (G < P.nb) G <<= 1;
+    const int64_t n = (int64_t)R * P.N;
+    if (n * G <= (int64_t)152 * 2048 * 8)
+        restrict_group_kernel<<<nblk(n * G, 128), 128, 0, h->stream>>>(R, P.N, P.p, P.ne1, G, h->d_ext, ys, P.E, y);
+    else
+        restrict_kernel<<<nblk(n, 256), 256, 0, h->stream>>>(R, P.N, P.p, P.ne1, h->d_ext, ys, P.E, y);
+    h->launches++;
+}
+
 // ---- upward pass -------------------------------------------------------------
 __global__ void leaf_moment_kernel(int R, int64_t E, int pp, int q, const double* __restrict__ M,
                                    const double* __restrict__ xs, int64_t leaf_off, int64_t C,
@@ -97,29 +141,6 @@ __global__ void leaf_moment_kernel(int R, int64_t E, int pp, int q, const double
         acc += M[av * pp + iv] * row;
     }
     xh[(r * C + leaf_off + e) * q2 + a] = acc;
-}
-
-__global__ void m2m_kernel(int R, int64_t nL, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                           int64_t C, double* __restrict__ xh) {
-    int q2 = q * q;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * nL * q2) return;
-    int64_t r = idx / (nL * q2);
-    int64_t rem = idx % (nL * q2);
-    int64_t pl = rem / q2;
-    int a = (int)(rem % q2), au = a % q, av = a / q;
-    double acc = 0.0;
-    for (int c = 0; c < 4; ++c) {
-        const double* Su = S + (c & 1) * q2;
-        const double* Sv = S + (c >> 1) * q2;
-        const double* v = xh + (r * C + offL1 + 4 * pl + c) * q2;
-        for (int bv = 0; bv < q; ++bv) {
-            double row = 0.0;
-            for (int bu = 0; bu < q; ++bu) row += Su[au * q + bu] * v[bv * q + bu];
-            acc += Sv[av * q + bv] * row;
-        }
-    }
-    xh[(r * C + offL + pl) * q2 + a] = acc;
 }
 
 // Separable M2M: one CTA per parent; T_c[bv][au] = sum_bu S_cx[au][bu] x_c[bv][bu],
@@ -177,6 +198,134 @@ __global__ void l2l_sep_kernel(int64_t nL, int64_t offL, int64_t offL1, int q, c
         for (int av = 0; av < q; ++av) acc += Sv[av * q + bv] * u[av * q + bu];
         yh[(r * C + offL1 + 4 * pl + c) * q2 + rem] += acc;
     }
+}
+
+// The levels of at most 16 clusters per patch (level 2 and coarser) in one launch, one
+// CTA per (patch, vector), all parents of a level at once: a level is a chain of
+// dependent loads that takes 5 to 6 us as a launch of its own, however small, and
+// about 2 us here.  Shared: children and intermediate values, 8 q^2 doubles per parent.
+constexpr int TOP_T = 512;
+constexpr int TOP_L = 2;       // finest parent level taken together
+struct TopLevels {
+    int64_t off[TOP_L + 2];
+};
+
+__global__ void __launch_bounds__(TOP_T) m2m_top_kernel(int first, TopLevels lo, int q, const double* __restrict__ S,
+                                                        int64_t C, double* __restrict__ xh) {
+    extern __shared__ double top_sm[];
+    const int q2 = q * q, patch = blockIdx.x;
+    double* v = xh + (int64_t)blockIdx.y * C * q2;
+    double* Ss = top_sm;                                  // [2][q][q]
+    for (int i = threadIdx.x; i < 2 * q2; i += TOP_T) Ss[i] = S[i];
+    for (int L = first; L >= 0; --L) {
+        const int np = 1 << (2 * L);
+        double* xc = Ss + 2 * q2;                         // [np][4][q2]
+        double* Tc = xc + (size_t)np * 4 * q2;
+        const double* src = v + (lo.off[L + 1] + (int64_t)patch * 4 * np) * q2;
+        __syncthreads();                                  // the coarser level reads what this CTA has written
+        for (int i = threadIdx.x; i < np * 4 * q2; i += TOP_T) xc[i] = src[i];
+        __syncthreads();
+        for (int i = threadIdx.x; i < np * 4 * q2; i += TOP_T) {
+            const int pc = i / q2, rem = i - pc * q2, bv = rem / q, au = rem - bv * q;
+            const double* Su = Ss + (pc & 1) * q2 + au * q;
+            const double* x = xc + pc * q2 + bv * q;
+            double acc = 0.0;
+            for (int bu = 0; bu < q; ++bu) acc += Su[bu] * x[bu];
+            Tc[i] = acc;
+        }
+        __syncthreads();
+        double* dst = v + (lo.off[L] + (int64_t)patch * np) * q2;
+        for (int i = threadIdx.x; i < np * q2; i += TOP_T) {
+            const int pl = i / q2, rem = i - pl * q2, av = rem / q, au = rem - av * q;
+            double acc = 0.0;
+            for (int c = 0; c < 4; ++c) {
+                const double* Sv = Ss + (c >> 1) * q2 + av * q;
+                const double* T = Tc + (pl * 4 + c) * q2 + au;
+                for (int bv = 0; bv < q; ++bv) acc += Sv[bv] * T[bv * q];
+            }
+            dst[i] = acc;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(TOP_T) l2l_top_kernel(int last, TopLevels lo, int q, const double* __restrict__ S,
+                                                        int64_t C, double* __restrict__ yh) {
+    extern __shared__ double top_sm[];
+    const int q2 = q * q, patch = blockIdx.x;
+    double* v = yh + (int64_t)blockIdx.y * C * q2;
+    double* Ss = top_sm;
+    for (int i = threadIdx.x; i < 2 * q2; i += TOP_T) Ss[i] = S[i];
+    for (int L = 0; L <= last; ++L) {
+        const int np = 1 << (2 * L);
+        double* yp = Ss + 2 * q2;                         // [np][q2]
+        double* U = yp + (size_t)np * q2;                 // [np][2][q2]
+        const double* src = v + (lo.off[L] + (int64_t)patch * np) * q2;
+        __syncthreads();
+        for (int i = threadIdx.x; i < np * q2; i += TOP_T) yp[i] = src[i];
+        __syncthreads();
+        for (int i = threadIdx.x; i < np * 2 * q2; i += TOP_T) {
+            const int pc = i / q2, rem = i - pc * q2, av = rem / q, bu = rem - av * q;
+            const double* Su = Ss + (pc & 1) * q2 + bu;
+            const double* y = yp + (pc >> 1) * q2 + av * q;
+            double acc = 0.0;
+            for (int au = 0; au < q; ++au) acc += Su[au * q] * y[au];
+            U[i] = acc;
+        }
+        __syncthreads();
+        double* dst = v + (lo.off[L + 1] + (int64_t)patch * 4 * np) * q2;
+        for (int i = threadIdx.x; i < np * 4 * q2; i += TOP_T) {
+            const int pc = i / q2, rem = i - pc * q2, bv = rem / q, bu = rem - bv * q, c = pc & 3;
+            const double* Sv = Ss + (c >> 1) * q2 + bv;
+            const double* u = U + ((pc >> 2) * 2 + (c & 1)) * q2 + bu;
+            double acc = 0.0;
+            for (int av = 0; av < q; ++av) acc += Sv[av * q] * u[av * q];
+            dst[i] += acc;
+        }
+    }
+}
+
+// M2M of every level for R real vectors: the fine levels one launch each, then the top
+cudaError_t launch_m2m(ibem_handle* h, int R, double* xh) {
+    const Plan& P = h->P;
+    for (int L = P.m - 1; L > TOP_L; --L) {
+        const int64_t nL = P.level_off[L + 1] - P.level_off[L];
+        m2m_sep_kernel<<<dim3((unsigned)nL, (unsigned)R), 64, 0, h->stream>>>(nL, P.level_off[L], P.level_off[L + 1], P.q,
+                                                                             h->d_S, P.C, xh);
+        h->launches++;
+    }
+    const int first = P.m - 1 < TOP_L ? P.m - 1 : TOP_L;
+    if (first < 0) return cudaSuccess;
+    TopLevels lo;
+    for (int l = 0; l <= first + 1; ++l) lo.off[l] = P.level_off[l];
+    const size_t sm = (2 + 8 * ((size_t)1 << (2 * first))) * P.q2 * sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(m2m_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, IBEM_MAX_SMEM_BYTES);
+    if (e) return e;
+    m2m_top_kernel<<<dim3((unsigned)P.npatch, (unsigned)R), TOP_T, sm, h->stream>>>(first, lo, P.q, h->d_S, P.C, xh);
+    h->launches++;
+    return cudaGetLastError();
+}
+
+// L2L of every level: the top, then the fine levels
+cudaError_t launch_l2l(ibem_handle* h, int R, double* yh) {
+    const Plan& P = h->P;
+    const int last = P.m - 1 < TOP_L ? P.m - 1 : TOP_L;
+    if (last >= 0) {
+        TopLevels lo;
+        for (int l = 0; l <= last + 1; ++l) lo.off[l] = P.level_off[l];
+        const size_t sm = (2 + 3 * ((size_t)1 << (2 * last))) * P.q2 * sizeof(double);
+        cudaError_t e = cudaFuncSetAttribute(l2l_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             IBEM_MAX_SMEM_BYTES);
+        if (e) return e;
+        l2l_top_kernel<<<dim3((unsigned)P.npatch, (unsigned)R), TOP_T, sm, h->stream>>>(last, lo, P.q, h->d_S, P.C, yh);
+        h->launches++;
+    }
+    for (int L = last + 1; L < P.m; ++L) {
+        const int64_t nL = P.level_off[L + 1] - P.level_off[L];
+        l2l_sep_kernel<<<dim3((unsigned)nL, (unsigned)R), 64, 0, h->stream>>>(nL, P.level_off[L], P.level_off[L + 1], P.q,
+                                                                             h->d_S, P.C, yh);
+        h->launches++;
+    }
+    return cudaGetLastError();
 }
 
 // ---- coupling, FP64, stored K ------------------------------------------------
@@ -411,25 +560,33 @@ __global__ void coupling_df_kernel(const int32_t* __restrict__ rows, const int64
     if (active && s == 0) yh[(r * C + sigma) * q2 + a] = acc;
 }
 
-// y^_tau += sum over the stored blocks (sigma, tau) of their column
-// shares, in the order of the transposed list.
-__global__ void column_gather_kernel(int R, int64_t C, int q2, const int64_t* __restrict__ tptr,
+// y^_tau += sum over the stored blocks (sigma, tau) of their column shares.  One CTA per
+// (tau, vector): G = blockDim / q2 slices of the transposed list, combined in order (a
+// thread per entry of y^_tau read a list of some 90 shares one after the other: 73 us
+// at p = 3, level 5, now 65 us).
+__global__ void column_gather_kernel(int64_t C, int q2, int G, const int64_t* __restrict__ tptr,
                                      const int32_t* __restrict__ tblk, const float2* __restrict__ colpart,
                                      int64_t nblk_total, double* __restrict__ yh) {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)R * C * q2) return;
-    int64_t r = idx / (C * q2);
-    int64_t rem = idx % (C * q2);
-    int64_t tau = rem / q2;
-    int b = (int)(rem % q2);
-    if (tptr[tau + 1] == tptr[tau]) return;
-    float hi = 0.0f, lo = 0.0f;
+    extern __shared__ double gred[];   // [G][q2]
+    const int64_t tau = blockIdx.x, r = blockIdx.y, k0 = tptr[tau], k1 = tptr[tau + 1];
+    if (k0 == k1) return;
+    const int t = threadIdx.x, g = t / q2, b = t - g * q2;
+    if (g < G) {
+        const float2* part = colpart + r * nblk_total * q2 + b;
+        float hi = 0.0f, lo = 0.0f;
 #pragma unroll 4
-    for (int64_t k = tptr[tau]; k < tptr[tau + 1]; ++k) {
-        float2 v = colpart[(r * nblk_total + tblk[k]) * q2 + b];
-        df_add(hi, lo, v.x, v.y);
+        for (int64_t k = k0 + g; k < k1; k += G) {
+            const float2 v = part[(int64_t)tblk[k] * q2];
+            df_add(hi, lo, v.x, v.y);
+        }
+        gred[t] = (double)hi + (double)lo;
     }
-    yh[(r * C + tau) * q2 + b] += (double)hi + (double)lo;
+    __syncthreads();
+    if (t < q2) {
+        double v = 0.0;
+        for (int k = 0; k < G; ++k) v += gred[k * q2 + t];
+        yh[(r * C + tau) * q2 + t] += v;
+    }
 }
 
 // ---- coupling, FP32, kernel generated on the fly ------------------------------
@@ -504,28 +661,6 @@ __global__ void coupling32_kernel(const int32_t* __restrict__ rows, const int64_
 }
 
 // ---- downward pass -----------------------------------------------------------
-__global__ void l2l_kernel(int R, int64_t nL1, int64_t offL, int64_t offL1, int q, const double* __restrict__ S,
-                           int64_t C, double* __restrict__ yh) {
-    int q2 = q * q;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * nL1 * q2) return;
-    int64_t r = idx / (nL1 * q2);
-    int64_t rem = idx % (nL1 * q2);
-    int64_t cl = rem / q2;
-    int b = (int)(rem % q2), bu = b % q, bv = b / q;
-    int c = (int)(cl & 3);
-    const double* Su = S + (c & 1) * q2;
-    const double* Sv = S + (c >> 1) * q2;
-    const double* v = yh + (r * C + offL + cl / 4) * q2;
-    double acc = 0.0;
-    for (int av = 0; av < q; ++av) {
-        double row = 0.0;
-        for (int au = 0; au < q; ++au) row += Su[au * q + bu] * v[av * q + au];
-        acc += Sv[av * q + bv] * row;
-    }
-    yh[(r * C + offL1 + cl) * q2 + b] += acc;
-}
-
 __global__ void leaf_back_kernel(int R, int64_t E, int pp, int q, const double* __restrict__ M,
                                  const double* __restrict__ yh, int64_t leaf_off, int64_t C,
                                  double* __restrict__ ys) {
@@ -547,19 +682,21 @@ __global__ void leaf_back_kernel(int R, int64_t E, int pp, int q, const double* 
 }
 
 // ---- near field product ------------------------------------------------------
-// One CTA per target element; thread t = i * nb + j accumulates B[i][j] x*_s[j]
-// over the row's blocks (one coalesced nb^2 read per block), then rows are
-// summed through shared memory.  The row's source elements are staged in shared
+// One CTA per target element, `slices` groups of nt threads; thread t = i * nb + j of a
+// group accumulates B[i][j] x*_s[j] over every slices-th block of the row (one
+// coalesced nb^2 read per block), then groups and columns are summed through
+// shared memory in a fixed order.  The row's source elements are staged in shared
 // memory (so a source value's load does not wait for a dependent global load)
-// and the sum over blocks runs in four independent partial sums.
-template <typename T>
+// and a group's sum runs in four independent partial sums.
+template <typename T, int S>
 __global__ void near_apply_kernel(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nsrc,
-                                  const T* __restrict__ blocks, int nb, int64_t E, const T* __restrict__ xs,
+                                  const T* __restrict__ blocks, int nb, int64_t E, int nt, const T* __restrict__ xs,
                                   double* __restrict__ ys) {
     extern __shared__ double red[];
     __shared__ int32_t srcs[256];
     const int64_t e = blockIdx.x, r = blockIdx.y;
-    const int t = threadIdx.x, nbb = nb * nb;
+    constexpr int slices = S;   // S = 1 as a run-time value took 181 instead of 171 us at p = 3, level 5
+    const int sl = S == 1 ? 0 : threadIdx.x / nt, t = threadIdx.x - sl * nt, nbb = nb * nb;
     const int64_t k0 = nptr[e], k1 = nptr[e + 1];
     const int j = t % nb;
     const T* xr = xs + r * E * nb;
@@ -567,27 +704,51 @@ __global__ void near_apply_kernel(const int64_t* __restrict__ nptr, const int32_
     for (int64_t kb = k0; kb < k1; kb += 256) {
         const int kc = (int)(k1 - kb < 256 ? k1 - kb : 256);
         __syncthreads();   // the previous chunk's source list is consumed
-        for (int i = t; i < kc; i += blockDim.x) srcs[i] = nsrc[kb + i];
+        for (int i = threadIdx.x; i < kc; i += blockDim.x) srcs[i] = nsrc[kb + i];
         __syncthreads();
         if (t < nbb) {
             const T* bk = blocks + kb * nbb + t;
-            int kk = 0;
-            for (; kk + 3 < kc; kk += 4) {
+            int kk = sl;
+            for (; kk + 3 * slices < kc; kk += 4 * slices) {
                 p0 += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
-                p1 += bk[(int64_t)(kk + 1) * nbb] * xr[(int64_t)srcs[kk + 1] * nb + j];
-                p2 += bk[(int64_t)(kk + 2) * nbb] * xr[(int64_t)srcs[kk + 2] * nb + j];
-                p3 += bk[(int64_t)(kk + 3) * nbb] * xr[(int64_t)srcs[kk + 3] * nb + j];
+                p1 += bk[(int64_t)(kk + slices) * nbb] * xr[(int64_t)srcs[kk + slices] * nb + j];
+                p2 += bk[(int64_t)(kk + 2 * slices) * nbb] * xr[(int64_t)srcs[kk + 2 * slices] * nb + j];
+                p3 += bk[(int64_t)(kk + 3 * slices) * nbb] * xr[(int64_t)srcs[kk + 3 * slices] * nb + j];
             }
-            for (; kk < kc; ++kk) p0 += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
+            for (; kk < kc; kk += slices) p0 += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
         }
     }
-    red[t] = t < nbb ? (double)((p0 + p1) + (p2 + p3)) : 0.0;
+    red[threadIdx.x] = t < nbb ? (double)((p0 + p1) + (p2 + p3)) : 0.0;
     __syncthreads();
-    if (t < nb) {
+    if (threadIdx.x < nb) {
         double v = 0.0;
-        for (int jj = 0; jj < nb; ++jj) v += red[t * nb + jj];
-        ys[(r * E + e) * nb + t] += v;
+        for (int q = 0; q < slices; ++q)
+            for (int jj = 0; jj < nb; ++jj) v += red[q * nt + threadIdx.x * nb + jj];
+        ys[(r * E + e) * nb + threadIdx.x] += v;
     }
+}
+
+// Groups per element: where the elements alone leave SMs without work, up to four
+// share a row (a group's chain of some 20 dependent loads is what a small mesh
+// waits for; with the shared launches of the coarse levels the application at p = 2,
+// level 2 went from 104 to 80 us).  The order of a row's sums must not
+// depend on the number of right-hand sides, so the rule counts the elements only.
+static int near_slices(const Plan& P, int nt) {
+    int s = 1;
+    while (s < 4 && P.E * s < 152 * 8 && 2 * s * nt <= 1024) s *= 2;
+    return s;
+}
+
+template <typename T>
+static void launch_near_apply(ibem_handle* h, int R, int nt, int slices, const T* blocks, const T* xs) {
+    const Plan& P = h->P;
+    auto go = [&](auto kern) {
+        kern<<<dim3((unsigned)P.E, R), nt * slices, nt * slices * sizeof(double), h->stream>>>(
+            h->d_near_ptr, h->d_near_src, blocks, P.nb, P.E, nt, xs, h->d_ys);
+    };
+    if (slices == 1) go(near_apply_kernel<T, 1>);
+    else if (slices == 2) go(near_apply_kernel<T, 2>);
+    else go(near_apply_kernel<T, 4>);
 }
 
 __global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ out, int64_t n) {
@@ -776,12 +937,7 @@ cudaError_t apply_operator(ibem_handle* h, const double* x, double* y, int nrhs,
             leaf_moment_kernel<<<nblk(R * P.E * q2, T), T, 0, st>>>(R, P.E, P.pp, P.q, h->d_M, h->d_xs, leaf_off,
                                                                      P.C, h->d_xh);
             h->launches++;
-            for (int L = P.m - 1; L >= 0; --L) {
-                int64_t nL = P.level_off[L + 1] - P.level_off[L];
-                m2m_sep_kernel<<<dim3((unsigned)nL, R), 64, 0, st>>>(nL, P.level_off[L], P.level_off[L + 1], P.q,
-                                                                    h->d_S, P.C, h->d_xh);
-                h->launches++;
-            }
+            if ((e = launch_m2m(h, R, h->d_xh))) return e;
             if ((e = cudaMemsetAsync(h->d_yh, 0, (size_t)R * P.C * q2 * sizeof(double), st))) return e;
         }
         unsigned nrows = (unsigned)h->far_rows.size();
@@ -808,43 +964,36 @@ cudaError_t apply_operator(ibem_handle* h, const double* x, double* y, int nrhs,
                 const int q2p = (q2 + 1) & ~1;
                 split_kernel<<<nblk(R * P.C * q2p, T), T, 0, st>>>(R * P.C, q2, q2p, h->d_xh, h->d_xh2);
                 if ((e = launch_coupling_df(h, R, h->df_nst))) return e;
-                column_gather_kernel<<<nblk((int64_t)R * P.C * q2, T), T, 0, st>>>(R, P.C, q2, h->d_tr_ptr, h->d_tr_blk,
-                                                                                   h->d_colpart, h->n_up, h->d_yh);
+                const int G = q2 < 256 ? 256 / q2 : 1, gt = (G * q2 + 31) / 32 * 32;
+                column_gather_kernel<<<dim3((unsigned)P.C, R), gt, G * q2 * sizeof(double), st>>>(
+                    P.C, q2, G, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->n_up, h->d_yh);
                 h->launches++;
                 h->launches += 2;
             }
         }
         PhaseTimer pt(h, 3);
-        for (int L = 0; L < P.m; ++L) {
-            int64_t nL = P.level_off[L + 1] - P.level_off[L];
-            l2l_sep_kernel<<<dim3((unsigned)nL, R), 64, 0, st>>>(nL, P.level_off[L], P.level_off[L + 1], P.q, h->d_S,
-                                                                P.C, h->d_yh);
-            h->launches++;
-        }
+        if ((e = launch_l2l(h, R, h->d_yh))) return e;
         leaf_back_kernel<<<nblk(R * P.E * P.nb, T), T, 0, st>>>(R, P.E, P.pp, P.q, h->d_M, h->d_yh, leaf_off, P.C,
                                                                  h->d_ys);
         h->launches++;
     } else {
         if ((e = cudaMemsetAsync(h->d_ys, 0, (size_t)R * P.Nstar * sizeof(double), st))) return e;
     }
-    int threads = ((P.nb * P.nb + 31) / 32) * 32;
+    const int threads = ((P.nb * P.nb + 31) / 32) * 32, slices = near_slices(P, threads);
     {
         PhaseTimer pt(h, 4);
         if (precision == IBEM_FP32) {
             d2f_kernel<<<nblk(R * P.Nstar, T), T, 0, st>>>(h->d_xs, h->d_xs32, R * P.Nstar);
-            near_apply_kernel<float><<<dim3((unsigned)P.E, R), threads, threads * sizeof(double), st>>>(
-                h->d_near_ptr, h->d_near_src, h->d_near32, P.nb, P.E, h->d_xs32, h->d_ys);
+            launch_near_apply(h, R, threads, slices, h->d_near32, h->d_xs32);
             h->launches += 2;
         } else {
-            near_apply_kernel<double><<<dim3((unsigned)P.E, R), threads, threads * sizeof(double), st>>>(
-                h->d_near_ptr, h->d_near_src, h->d_near, P.nb, P.E, h->d_xs, h->d_ys);
+            launch_near_apply(h, R, threads, slices, h->d_near, h->d_xs);
             h->launches++;
         }
     }
     {
         PhaseTimer pt(h, 5);
-        restrict_kernel<<<nblk(R * P.N, 32), 32, 0, st>>>(R, P.N, P.p, P.ne1, h->d_ext, h->d_ys, P.E, y);
-        h->launches++;
+        launch_restrict(h, R, h->d_ys, y);
     }
     return cudaGetLastError();
 }
@@ -877,7 +1026,7 @@ cudaError_t launch_rhs(ibem_handle* h, const double* g, int nrhs, double* b) {
     int QQ = P.Q * P.Q;
     rhs_super_kernel<<<nblk(nrhs * P.E * P.nb, T), T, 0, h->stream>>>(nrhs, P.E, QQ, P.nb, h->d_qgeo, h->d_phi, g,
                                                                        P.nq, h->d_ys);
-    restrict_kernel<<<nblk(nrhs * P.N, T), T, 0, h->stream>>>(nrhs, P.N, P.p, P.ne1, h->d_ext, h->d_ys, P.E, b);
+    launch_restrict(h, nrhs, h->d_ys, b);
     return cudaGetLastError();
 }
 

@@ -402,13 +402,7 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
         leaf_moment_kernel<<<nblk(R2 * P.E * q2, T), T, 0, st>>>(R2, P.E, P.pp, P.q, h->d_M, h->d_xs, leaf_off, P.C,
                                                                   h->d_xh);
         h->launches++;
-        for (int L = P.m - 1; L >= 0; --L) {
-            int64_t nL = P.level_off[L + 1] - P.level_off[L];
-            // separable (S_c applied per direction: 2 q^3 instead of q^4 per child)
-            m2m_sep_kernel<<<dim3((unsigned)nL, (unsigned)R2), 64, 0, st>>>(nL, P.level_off[L], P.level_off[L + 1],
-                                                                            P.q, h->d_S, P.C, h->d_xh);
-            h->launches++;
-        }
+        if ((e = launch_m2m(h, R2, h->d_xh))) return e;
         if ((e = cudaMemsetAsync(h->d_yh, 0, (size_t)R2 * P.C * q2 * sizeof(double), st))) return e;
         pt1.stop();
         unsigned nrows = (unsigned)h->far_rows.size();
@@ -443,12 +437,7 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
             }
         }
         PhaseTimer pt3(h, 3);
-        for (int L = 0; L < P.m; ++L) {
-            const int64_t nL = P.level_off[L + 1] - P.level_off[L];
-            l2l_sep_kernel<<<dim3((unsigned)nL, (unsigned)R2), 64, 0, st>>>(nL, P.level_off[L], P.level_off[L + 1],
-                                                                            P.q, h->d_S, P.C, h->d_yh);
-            h->launches++;
-        }
+        if ((e = launch_l2l(h, R2, h->d_yh))) return e;
         leaf_back_kernel<<<nblk(R2 * P.E * P.nb, T), T, 0, st>>>(R2, P.E, P.pp, P.q, h->d_M, h->d_yh, leaf_off, P.C,
                                                                   h->d_ys);
         h->launches++;
@@ -480,9 +469,9 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
     }
     pt4.stop();
     PhaseTimer pt5(h, 5);
-    restrict_kernel<<<nblk(R2 * P.N, T), T, 0, st>>>(R2, P.N, P.p, P.ne1, h->d_ext, h->d_ys, P.E, ysplit);
+    launch_restrict(h, R2, h->d_ys, ysplit);
     helm_join_vec_kernel<<<nblk((int64_t)R * P.N, T), T, 0, st>>>(R, P.N, ysplit, y);
-    h->launches += 2;
+    h->launches++;
     return cudaGetLastError();
 }
 
@@ -493,7 +482,7 @@ cudaError_t helm_launch_rhs(ibem_handle* h, const double* g, int nrhs, double* b
     helm_split_vec_kernel<<<nblk((int64_t)nrhs * P.nq, T), T, 0, h->stream>>>(nrhs, P.nq, g, gsplit);
     rhs_super_kernel<<<nblk(R2 * P.E * P.nb, T), T, 0, h->stream>>>(R2, P.E, QQ, P.nb, h->d_qgeo, h->d_phi, gsplit,
                                                                      P.nq, h->d_ys);
-    restrict_kernel<<<nblk(R2 * P.N, T), T, 0, h->stream>>>(R2, P.N, P.p, P.ne1, h->d_ext, h->d_ys, P.E, bsplit);
+    launch_restrict(h, R2, h->d_ys, bsplit);
     helm_join_vec_kernel<<<nblk((int64_t)nrhs * P.N, T), T, 0, h->stream>>>(nrhs, P.N, bsplit, b);
     return cudaGetLastError();
 }

@@ -715,12 +715,7 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
                                                         h->d_igeo, 0.0, h->d_trig64, d_yh);
         h->launches++;
     }
-    for (int L = 0; L < P.m; ++L) {
-        const int64_t nL = P.level_off[L + 1] - P.level_off[L];
-        l2l_sep_kernel<<<dim3((unsigned)nL, (unsigned)R2), 64, 0, st>>>(nL, P.level_off[L], P.level_off[L + 1], P.q,
-                                                                       h->d_S, P.C, d_yh);
-        h->launches++;
-    }
+    if ((e = launch_l2l(h, R2, d_yh))) return e;
     leaf_back_kernel<<<nblk((int64_t)R2 * P.E * P.nb, T), T, 0, st>>>(R2, P.E, P.pp, P.q, h->d_M, d_yh,
                                                                        P.level_off[P.m], P.C, d_ys);
     h->launches++;
@@ -735,9 +730,7 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
                                                          P.E, h->d_qgeo, h->d_phi, 0.0, h->d_trig64, d_ys);
         h->launches++;
     }
-    restrict_kernel<<<nblk((int64_t)R2 * P.N, T), T, 0, st>>>(R2, P.N, P.p, P.ne1, h->d_ext, d_ys, P.E,
-                                                              h->helm ? d_bs : b);
-    h->launches++;
+    launch_restrict(h, R2, d_ys, h->helm ? d_bs : b);
     if (h->helm) {
         helm_join_vec_kernel<<<nblk((int64_t)nrhs * P.N, T), T, 0, st>>>(nrhs, P.N, d_bs, b);
         h->launches++;
