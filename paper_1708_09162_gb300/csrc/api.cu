@@ -99,7 +99,7 @@ void free_handle(ibem_handle* h) {
                     h->d_pairs_by_cls[1], h->d_pairs_by_cls[2], h->d_pairs_by_cls[3], h->d_pairs_by_cls[4],
                     h->d_near, h->d_near32, h->d_far_ptr, h->d_far_src, h->d_far_tgt, h->d_K, h->d_Kdf, h->d_xh2, h->d_far_rows,
                     h->d_xs, h->d_ys, h->d_xh, h->d_yh, h->d_xs32, h->d_ys32, h->d_yh32, h->d_src32, h->d_diag,
-                    h->d_solver, h->d_red, h->d_status, h->d_Kc, h->d_xh4, h->d_hcol, h->d_hsx, h->d_hsy,
+                    h->d_solver, h->d_red, h->d_status, h->d_Kc, h->d_xh4, h->d_xsdf, h->d_hcol, h->d_hsx, h->d_hsy,
                     h->d_bj_ptr, h->d_bj_off, h->d_bj_dofs, h->d_bj_inv, h->d_up_ptr, h->d_up_src,
                     h->d_up_tgt, h->d_up_rows, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->d_mr, h->d_Mf, h->d_Sf,
                     h->d_gen_pts, h->d_gen_trig, h->d_gen_x, h->d_Kbf, h->d_graded_pairs, h->d_graded_tab,

@@ -327,6 +327,7 @@ struct ibem_handle {
     float2* d_xh2 = nullptr;        // forward moments split into (hi, lo) float pairs
     float4* d_Kc = nullptr;         // Helmholtz: double-float complex coupling (re_hi, re_lo, im_hi, im_lo), one of two mirrored blocks
     float4* d_xh4 = nullptr;        // Helmholtz: forward moments as double-float complex, one pass of right-hand sides
+    float4* d_xsdf = nullptr;       // Helmholtz: lifted coefficients as double-float complex [E nb][R]
     float4* d_hcol = nullptr;       // Helmholtz: column shares of the stored blocks, one pass
     int hdf_rhs = 0;                // right-hand sides d_xh4 and d_hcol are sized for
     double* d_hsx = nullptr;        // Helmholtz: split-layout input  [2R][max(N, nq)]

@@ -761,8 +761,9 @@ cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
     if (nrhs <= h->ws_nrhs) return cudaSuccess;
     Plan& P = h->P;
     if (h->helm) {
-        cudaFree(h->d_hsx); cudaFree(h->d_hsy);
+        cudaFree(h->d_hsx); cudaFree(h->d_hsy); cudaFree(h->d_xsdf);
         h->d_hsx = h->d_hsy = nullptr;
+        h->d_xsdf = nullptr;
     }
     cudaFree(h->d_xs); cudaFree(h->d_ys); cudaFree(h->d_xh); cudaFree(h->d_yh);
     cudaFree(h->d_xs32); cudaFree(h->d_src32); cudaFree(h->d_xh2);
@@ -793,6 +794,8 @@ cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
         size_t n = (size_t)(P.N > P.nq ? P.N : P.nq);
         if ((e = cudaMalloc(&h->d_hsx, (size_t)nrhs * n * sizeof(double)))) return e;
         if ((e = cudaMalloc(&h->d_hsy, (size_t)nrhs * P.N * sizeof(double)))) return e;
+        // split lifted coefficients of the double-float near product (4 and more right-hand sides)
+        if (nrhs >= 8 && (e = cudaMalloc(&h->d_xsdf, (size_t)(nrhs / 2) * P.Nstar * sizeof(float4)))) return e;
     }
     h->ws_nrhs = nrhs;
     return cudaSuccess;

@@ -14,6 +14,8 @@
 // re_lo, im_hi, im_lo), layout [n_up][kpt][4 q2] like the Laplace case
 // (kernels_helm_df.cu), or - when they would not fit in the memory budget -
 // generated on the fly.
+#include <algorithm>
+
 #include "fp64_eval.cuh"
 #include "ibem_internal.cuh"
 
@@ -255,6 +257,12 @@ __global__ void helm_near_apply_kernel(const int64_t* __restrict__ nptr, const i
 // (row i, right-hand side r) accumulates sum_j B[i][j] x*_s[j][r] with exact
 // products and TwoSum accumulation (as the coupling's double-float arithmetic);
 // each block is read once for all right-hand sides.  Adds to ys (split layout).
+// The coefficients are split once per application (helm_split_lift_kernel): splitting
+// them again for each of some 50 near blocks kept the FP64 pipe busier than the
+// products the FP32 pipe.  Few right-hand sides leave most of the CTA idle, so its
+// threads form S slices that take S blocks at a time.  Stages are double buffered
+// (one barrier per S blocks).  p = 2: 64 right-hand sides at level 5 5.34 ms instead of
+// 6.18, 8 at level 3 156 us instead of 199.
 constexpr int HN_T = 256;
 
 __device__ __forceinline__ void hn_split(double v, float& h, float& l) {
@@ -272,59 +280,120 @@ __device__ __forceinline__ void hn_mac(float ah, float al, float bh, float bl, f
     lo += err + e;
 }
 
+// lifted coefficients of the split layout [2R][E nb] -> (re_h, re_l, im_h, im_l) [E nb][R]
+__global__ void helm_split_lift_kernel(int R, int64_t n, const double* __restrict__ xs, float4* __restrict__ out) {
+    __shared__ double2 tile[32][33];
+    const int64_t k0 = (int64_t)blockIdx.x * 32;
+    const int r0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int r = ty; r < 32; r += 8)
+        if (r0 + r < R && k0 + tx < n)
+            tile[r][tx] = make_double2(xs[(int64_t)(2 * (r0 + r)) * n + k0 + tx],
+                                       xs[(int64_t)(2 * (r0 + r) + 1) * n + k0 + tx]);
+    __syncthreads();
+    for (int k = ty; k < 32; k += 8)
+        if (r0 + tx < R && k0 + k < n) {
+            const double2 v = tile[tx][k];
+            float4 o;
+            hn_split(v.x, o.x, o.y);
+            hn_split(v.y, o.z, o.w);
+            out[(k0 + k) * R + r0 + tx] = o;
+        }
+}
+
+// nt: threads per slice; dynamic shared memory 2 S (nb^2 + nb R) float4
 __global__ void __launch_bounds__(HN_T) helm_near_df_kernel(const int64_t* __restrict__ nptr,
                                                             const int32_t* __restrict__ nsrc,
-                                                            const double2* __restrict__ blocks, int nb, int R,
-                                                            int64_t E, const double* __restrict__ xs,
+                                                            const double2* __restrict__ blocks, int nb, int R, int S,
+                                                            int nt, int64_t E, const float4* __restrict__ xl,
                                                             double* __restrict__ ys) {
     extern __shared__ float4 hn_sm[];
-    float4* Bs = hn_sm;              // [nb * nb] (re_h, re_l, im_h, im_l)
-    float4* Xs = hn_sm + nb * nb;    // [nb][R]  (re_h, re_l, im_h, im_l)
     const int64_t e = blockIdx.x;
-    const int t = threadIdx.x, nbb = nb * nb, np = nb * R;
+    const int t = threadIdx.x, nbb = nb * nb, np = nb * R, sl = t / nt, ts = t - sl * nt;
+    const int per = S * (nbb + np);  // float4 per stage: S blocks, then S coefficient sets
     constexpr int MAXP = 8;          // (row, right-hand side) pairs per thread: nb R <= 8 HN_T
+    constexpr int MAXB = 3;          // block entries per thread: S nb^2 <= 3 HN_T
     float acc[MAXP][4];
 #pragma unroll
     for (int k = 0; k < MAXP; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0f;
-    for (int64_t k = nptr[e]; k < nptr[e + 1]; ++k) {
-        const int64_t s = nsrc[k];
-        __syncthreads();   // the previous block is consumed
-        for (int q = t; q < nbb; q += HN_T) {
-            const double2 b = blocks[k * nbb + q];
-            float4 v;
-            hn_split(b.x, v.x, v.y);
-            hn_split(b.y, v.z, v.w);
-            Bs[q] = v;
-        }
-        for (int q = t; q < np; q += HN_T) {
-            const int j = q / R, r = q % R;
-            float4 v;
-            hn_split(xs[((int64_t)(2 * r) * E + s) * nb + j], v.x, v.y);
-            hn_split(xs[((int64_t)(2 * r + 1) * E + s) * nb + j], v.z, v.w);
-            Xs[q] = v;
-        }
-        __syncthreads();
+    const int64_t k0 = nptr[e];
+    const int n = (int)(nptr[e + 1] - k0);
+    double2 bn[MAXB];
+    auto fetch = [&](int c) {        // blocks c .. c + S - 1: entries into registers, coefficients into the stage
+        const int live = n - c < S ? n - c : S;
 #pragma unroll
-        for (int m = 0; m < MAXP; ++m) {
-            const int p = t + HN_T * m;
-            if (p < np) {
-                const int i = p / R, r = p % R;
-                for (int j = 0; j < nb; ++j) {
-                    const float4 b = Bs[i * nb + j], x = Xs[j * R + r];
-                    // (Br + i Bi)(xr + i xi) = (Br xr - Bi xi) + i (Br xi + Bi xr)
-                    hn_mac(b.x, b.y, x.x, x.y, acc[m][0], acc[m][1]);
-                    hn_mac(-b.z, -b.w, x.z, x.w, acc[m][0], acc[m][1]);
-                    hn_mac(b.x, b.y, x.z, x.w, acc[m][2], acc[m][3]);
-                    hn_mac(b.z, b.w, x.x, x.y, acc[m][2], acc[m][3]);
+        for (int m = 0; m < MAXB; ++m) {
+            const int q = t + HN_T * m;
+            if (q < live * nbb) bn[m] = blocks[(k0 + c) * nbb + q];
+        }
+        float4* X = hn_sm + ((c / S) & 1) * per + S * nbb;
+        for (int q = t; q < live * np; q += HN_T) {
+            const int b = q / np, o = q - b * np;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(X + q)),
+                         "l"(xl + (int64_t)nsrc[k0 + c + b] * np + o)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (n > 0) fetch(0);
+    for (int c = 0; c < n; c += S) {
+        const int live = n - c < S ? n - c : S;
+        float4* Bs = hn_sm + ((c / S) & 1) * per;
+#pragma unroll
+        for (int m = 0; m < MAXB; ++m) {
+            const int q = t + HN_T * m;
+            if (q < live * nbb) {
+                float4 v;
+                hn_split(bn[m].x, v.x, v.y);
+                hn_split(bn[m].y, v.z, v.w);
+                Bs[q] = v;
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();             // the stage is complete; the other one is used
+        if (c + S < n) fetch(c + S);
+        if (sl < live) {
+            const float4* B = Bs + sl * nbb;
+            const float4* X = Bs + S * nbb + sl * np;
+#pragma unroll
+            for (int m = 0; m < MAXP; ++m) {
+                const int p = ts + nt * m;
+                if (p < np) {
+                    const int i = p / R, r = p - i * R;
+                    for (int j = 0; j < nb; ++j) {
+                        const float4 b = B[i * nb + j], x = X[j * R + r];
+                        // (Br + i Bi)(xr + i xi) = (Br xr - Bi xi) + i (Br xi + Bi xr)
+                        hn_mac(b.x, b.y, x.x, x.y, acc[m][0], acc[m][1]);
+                        hn_mac(-b.z, -b.w, x.z, x.w, acc[m][0], acc[m][1]);
+                        hn_mac(b.x, b.y, x.z, x.w, acc[m][2], acc[m][3]);
+                        hn_mac(b.z, b.w, x.x, x.y, acc[m][2], acc[m][3]);
+                    }
                 }
             }
         }
     }
+    if (S > 1) {                     // nt >= np: one pair per thread; the slices in order
+        __syncthreads();
+        if (sl < S && ts < np) hn_sm[sl * np + ts] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+        __syncthreads();
+        if (t < np) {
+            double vr = 0.0, vi = 0.0;
+            for (int q = 0; q < S; ++q) {
+                const float4 v = hn_sm[q * np + t];
+                vr += (double)v.x + (double)v.y;
+                vi += (double)v.z + (double)v.w;
+            }
+            const int i = t / R, r = t - i * R;
+            ys[((int64_t)(2 * r) * E + e) * nb + i] += vr;
+            ys[((int64_t)(2 * r + 1) * E + e) * nb + i] += vi;
+        }
+        return;
+    }
 #pragma unroll
     for (int m = 0; m < MAXP; ++m) {
-        const int p = t + HN_T * m;
+        const int p = ts + nt * m;
         if (p < np) {
-            const int i = p / R, r = p % R;
+            const int i = p / R, r = p - i * R;
             ys[((int64_t)(2 * r) * E + e) * nb + i] += (double)acc[m][0] + (double)acc[m][1];
             ys[((int64_t)(2 * r + 1) * E + e) * nb + i] += (double)acc[m][2] + (double)acc[m][3];
         }
@@ -453,12 +522,18 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
         h->launches += 2;
     } else {
         if (R >= 4 && P.nb * R <= 8 * HN_T) {
-            const size_t sm = (size_t)(P.nb * P.nb + P.nb * R) * sizeof(float4);
+            const int np = P.nb * R;
+            const int nt = np <= HN_T / 2 ? ((np + 31) / 32) * 32 : HN_T;
+            const int S = std::min(HN_T / nt, std::max(1, 3 * HN_T / (P.nb * P.nb)));
+            const size_t sm = (size_t)2 * S * (P.nb * P.nb + np) * sizeof(float4);
             if ((e = cudaFuncSetAttribute(helm_near_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
                 return e;
+            helm_split_lift_kernel<<<dim3((unsigned)((P.Nstar + 31) / 32), (unsigned)((R + 31) / 32)), 256, 0, st>>>(
+                R, P.Nstar, h->d_xs, h->d_xsdf);
             helm_near_df_kernel<<<(unsigned)P.E, HN_T, sm, st>>>(h->d_near_ptr, h->d_near_src,
                                                                  reinterpret_cast<const double2*>(h->d_near), P.nb,
-                                                                 R, P.E, h->d_xs, h->d_ys);
+                                                                 R, S, nt, P.E, h->d_xsdf, h->d_ys);
+            h->launches++;
         } else {
             helm_near_apply_kernel<double2, double><<<dim3((unsigned)P.E, R), threads, 2 * threads * sizeof(double),
                                                       st>>>(h->d_near_ptr, h->d_near_src,
