@@ -179,18 +179,35 @@ __global__ void __launch_bounds__(CT_T) conv_tile_kernel(const TI* __restrict__ 
 // (core-matrix stride along M = 128 B) and the channel groups are NBP * 16 B
 // apart (stride along K).  Weights per tap: core (co / 8, ci / 8) at
 // ((co / 8) * KG + ci / 8) * 128 B.  A tile is TC_MB blocks of 128 consecutive
-// positions sharing one band of TC_MB * 128 + 2P + 2 rows (copied with cp.async,
-// zero-filled outside the image); each block accumulates in its own 32 TMEM
-// columns (tcgen05.mma kind::f16, M = 128, N = NP, K = 16, BF16 operands, FP32
-// accumulation), and all MMAs of a tile are committed once.  Epilogue: bias,
-// optional ReLU, BF16 store.
+// positions sharing one band of TC_MB * 128 + 2P + 2 rows; each block accumulates
+// in its own 32 TMEM columns (tcgen05.mma kind::f16, M = 128, N = NP, K = 16, BF16
+// operands, FP32 accumulation), and all MMAs of a tile are committed once.
+// Epilogue: bias, optional ReLU, BF16 store.
+//
+// Activations lie by channel group, [B][C / 8][H][W][8]: the part of an image row in
+// a band is then one contiguous run per group, copied by one cp.async.bulk
+// (some 28 of them for a tile of 130-pixel rows instead of 3112 16-byte copies with
+// their index arithmetic), and the epilogue's 16-byte stores of a warp are
+// contiguous too.  One persistent CTA per SM: a producer warp runs up to four
+// bands ahead (the zero padding is stored by its lanes), a warp issues MMAs into
+// two sets of accumulators, eight warps do the epilogue of the tile before.
+// Bound: the MMAs, about 75 cycles each for N = 32 and N = 16 alike (128 rows of A from
+// shared memory at K = 16), 72 per tile; neither the order of the MMAs (blocks
+// innermost: 65 us per layer) nor a row pitch that starts the taps' rows on 128
+// bytes (64 us) changes it.  96 images of 130 x 130: 39 us (2 -> 32), 62 (32 -> 32)
+// and 59 (32 -> 2); with copy, MMAs and epilogue in sequence in two CTAs of 128
+// threads per SM it was 52, 97 and 75.
 //   CGI: channel groups of an input pixel (1: the 2-channel input padded to 8
 //        channels, 4: 32 channels); the band holds KG = max(CGI, 2) groups
 //        (the second group of a 1-group input is zero, and so are its weights).
 //   NP:  MMA width (32, or 16 for the 2-channel output layer); NOUT channels kept.
-//   OUT_PLANAR: output [B][NOUT][H][W] (last layer) instead of pixel-major.
+//   OUT_PLANAR: output [B][NOUT][H][W] (last layer) instead of by channel group.
 constexpr int TC_M = 128;
 constexpr int TC_MB = 4;
+constexpr int TC_STAGES = 4;                  // bands at most
+constexpr int TC_EW = 8;                      // epilogue warps; then the producer, then the MMA warp
+constexpr int TC_T = 32 * (TC_EW + 2);
+constexpr int TC_BARS = 128;                  // bytes for barriers, TMEM address and flag
 
 __device__ inline unsigned cnn_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -199,7 +216,8 @@ __device__ inline uint64_t cnn_desc(unsigned addr, unsigned lbo, unsigned sbo) {
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
-__device__ inline bool cnn_wait(uint64_t* bar, unsigned parity, long long limit) {
+// false after `limit` polls, or once another role has given up
+__device__ inline bool cnn_wait(uint64_t* bar, unsigned parity, long long limit, volatile int* fail) {
     for (long long it = 0; it < limit; ++it) {
         unsigned ok;
         asm volatile(
@@ -208,19 +226,26 @@ __device__ inline bool cnn_wait(uint64_t* bar, unsigned parity, long long limit)
             : "r"(cnn_smem(bar)), "r"(parity)
             : "memory");
         if (ok) return true;
+        if (fail && *fail) return false;
     }
+    if (fail) *fail = 1;
     return false;
 }
 
-// w [Cout][Cin][9] FP32 -> BF16 canonical tiles [9][NP / 8][KG][8][8] (zero padded)
-__global__ void tc_weights_kernel(const float* __restrict__ w, int Cin, int Cout, int NP, int KG,
-                                  __nv_bfloat16* __restrict__ wt) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int CI = 8 * KG;
+struct TcWeights {
+    const float* w[4];
+    __nv_bfloat16* wt[4];
+    int cin[4], cout[4], np[4], kg[4];
+};
+
+// w [Cout][Cin][9] FP32 -> BF16 canonical tiles [9][NP / 8][KG][8][8] (zero padded); layer blockIdx.y
+__global__ void tc_weights_kernel(TcWeights p) {
+    const int l = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int KG = p.kg[l], NP = p.np[l], Cin = p.cin[l], Cout = p.cout[l], CI = 8 * KG;
     if (i >= NP * CI * 9) return;
     const int k = i % 9, ci = (i / 9) % CI, co = i / (9 * CI);
-    const float v = (co < Cout && ci < Cin) ? w[((int64_t)co * Cin + ci) * 9 + k] : 0.0f;
-    wt[(k * (NP / 8) * KG + (co >> 3) * KG + (ci >> 3)) * 64 + (co & 7) * 8 + (ci & 7)] = __float2bfloat16(v);
+    const float v = (co < Cout && ci < Cin) ? p.w[l][((int64_t)co * Cin + ci) * 9 + k] : 0.0f;
+    p.wt[l][(k * (NP / 8) * KG + (co >> 3) * KG + (ci >> 3)) * 64 + (co & 7) * 8 + (ci & 7)] = __float2bfloat16(v);
 }
 
 // FP32 planar [B][2][H][W] -> BF16 pixel-major [B][H][W][8] (channels 2..7 zero)
@@ -232,21 +257,26 @@ __global__ void pack8_kernel(int64_t npx, int64_t HW, const float* __restrict__ 
     *reinterpret_cast<uint4*>(out + i * 8) = make_uint4(*reinterpret_cast<uint32_t*>(&v), 0u, 0u, 0u);
 }
 
-// Persistent CTAs of 128 threads (one output position per thread and block).
 template <int CGI, int NP, int NOUT, bool OUT_PLANAR>
-__global__ void __launch_bounds__(128) conv_tc_kernel(const __nv_bfloat16* __restrict__ in, int B, int H, int W,
-                                                      const __nv_bfloat16* __restrict__ wt,
-                                                      const float* __restrict__ bias, int relu, int nbp,
-                                                      __nv_bfloat16* __restrict__ out, long long wait_limit,
-                                                      int* __restrict__ status) {
+__global__ void __launch_bounds__(TC_T, 1) conv_tc_kernel(const __nv_bfloat16* __restrict__ in, int B, int H, int W,
+                                                          const __nv_bfloat16* __restrict__ wt,
+                                                          const float* __restrict__ bias, int relu, int nbp, int nst,
+                                                          __nv_bfloat16* __restrict__ out, long long wait_limit,
+                                                          int* __restrict__ status) {
     constexpr int KG = CGI < 2 ? 2 : CGI;
     constexpr int WBYTES = 9 * (NP / 8) * KG * 128;
     constexpr int TILE = TC_M * TC_MB;
+    constexpr int ACC = 32 * TC_MB;               // TMEM columns of a tile; two tiles in flight
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* wsm = smem;
-    unsigned char* band = smem + WBYTES;
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(band + KG * nbp * 16);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
+    unsigned char* bands = smem + WBYTES;
+    const int bbytes = KG * nbp * 16;
+    uint64_t* full = reinterpret_cast<uint64_t*>(bands + (size_t)nst * bbytes);
+    uint64_t* empty = full + TC_STAGES;
+    uint64_t* accf = empty + TC_STAGES;
+    uint64_t* acce = accf + 2;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(acce + 2);
+    volatile int* fail = reinterpret_cast<int*>(tslot + 1);
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int P = W + 2;
     const int64_t tiles_img = ((int64_t)H * P + TILE - 1) / TILE;
@@ -255,141 +285,202 @@ __global__ void __launch_bounds__(128) conv_tc_kernel(const __nv_bfloat16* __res
     for (int i = t; i < WBYTES / 16; i += blockDim.x)
         reinterpret_cast<uint4*>(wsm)[i] = reinterpret_cast<const uint4*>(wt)[i];
     if (CGI < KG)   // zero channel group of a 1-group input
-        for (int r = t; r < nbp; r += blockDim.x)
-            *reinterpret_cast<uint4*>(band + ((size_t)1 * nbp + r) * 16) = make_uint4(0u, 0u, 0u, 0u);
-    float bv[NOUT];
-#pragma unroll
-    for (int c = 0; c < NOUT; ++c) bv[c] = bias[c];
+        for (int i = t; i < nst * nbp; i += blockDim.x)
+            *reinterpret_cast<uint4*>(bands + (size_t)(i / nbp) * bbytes + ((size_t)nbp + i % nbp) * 16) =
+                make_uint4(0u, 0u, 0u, 0u);
     if (t == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cnn_smem(mbar)) : "memory");
+        for (int s = 0; s < TC_STAGES; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cnn_smem(full + s)) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cnn_smem(empty + s)) : "memory");
+        }
+        for (int s = 0; s < 2; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cnn_smem(accf + s)) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(cnn_smem(acce + s)), "r"(TC_EW) : "memory");
+        }
+        *fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(cnn_smem(tslot)),
-                     "r"(32 * TC_MB)
+                     "r"(2 * ACC)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tslot;
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NP >> 3) << 17) |
-                           ((uint32_t)(TC_M >> 4) << 24);
-    // descriptors of offset 0; an operand starting k * 16 bytes later is desc + k
-    // (the start-address field counts 16-byte units; all addresses < 256 KB)
-    const uint64_t adesc0 = cnn_desc(cnn_smem(band), nbp * 16, 128);
-    const uint64_t bdesc0 = cnn_desc(cnn_smem(wsm), 128, KG * 128);
-    int it = 0;
-    bool failed = false;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-        const int64_t b = tile / tiles_img;
-        const int o0 = (int)((tile % tiles_img) * TILE);
-        // band of padded rows o0 .. o0 + nb - 1: all 16-byte copies in flight at
-        // once (cp.async), zero-filled outside the image (source size 0)
-        for (int idx = t; idx < nb * CGI; idx += blockDim.x) {
-            const int r = idx / CGI, g = idx % CGI;
-            const int i = o0 + r;
-            const int py = i / P, px = i - py * P;
-            const bool inside = py >= 1 && py <= H && px >= 1 && px <= W;
-            const __nv_bfloat16* s = inside ? in + ((b * H + (py - 1)) * W + (px - 1)) * (8 * CGI) + g * 8 : in;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                             cnn_smem(band + ((size_t)g * nbp + r) * 16)),
-                         "l"(s), "r"(inside ? 16u : 0u)
-                         : "memory");
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (t == 0) {
-#pragma unroll 1
-            for (int mb = 0; mb < TC_MB; ++mb)
-#pragma unroll 1
-                for (int tap = 0; tap < 9; ++tap) {
-                    const int roff = mb * TC_M + (tap / 3) * P + (tap % 3);
-                    for (int s = 0; s < KG / 2; ++s) {
-                        const uint64_t ad = adesc0 + (uint64_t)(2 * s * nbp + roff);
-                        const uint64_t bd = bdesc0 + (uint64_t)(tap * (NP / 8) * KG * 8 + 2 * s * 8);
-                        const uint32_t acc = (tap > 0 || s > 0) ? 1u : 0u;
+    if (warp == TC_EW) {
+        // producer: lanes take (padded row, channel group) pieces of the band o0 .. o0 + nb - 1
+        int it = 0;
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+            const int s = it % nst;
+            if (it >= nst) {
+                const bool ok = cnn_wait(empty + s, (unsigned)((it / nst - 1) & 1), wait_limit, fail);
+                if (!__all_sync(0xffffffffu, ok)) break;
+            }
+            const int64_t b = tile / tiles_img;
+            const int o0 = (int)((tile - b * tiles_img) * TILE);
+            unsigned char* band = bands + (size_t)s * bbytes;
+            const int r0 = o0 / P, nr = (o0 + nb - 1) / P - r0 + 1;
+            for (int i = lane; i < nr * CGI; i += 32) {
+                const int g = i % CGI, py = r0 + i / CGI;
+                const int lo = max(o0, py * P), hi = min(o0 + nb, (py + 1) * P);
+                const int a = max(lo, py * P + 1), e = min(hi, py * P + 1 + W);
+                unsigned char* dst = band + ((size_t)g * nbp + (lo - o0)) * 16;
+                if (py >= 1 && py <= H) {
+                    if (a > lo) *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+                    if (hi > e) *reinterpret_cast<uint4*>(dst + (size_t)(hi - 1 - lo) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    if (e > a) {
+                        const unsigned bytes = (unsigned)(e - a) * 16u;
+                        const __nv_bfloat16* src =
+                            in + (((b * CGI + g) * H + (py - 1)) * (int64_t)W + (a - py * P - 1)) * 8;
+                        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(cnn_smem(full + s)),
+                                     "r"(bytes)
+                                     : "memory");
                         asm volatile(
-                            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + 32u * mb),
-                            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                cnn_smem(dst + (size_t)(a - lo) * 16)),
+                            "l"(src), "r"(bytes), "r"(cnn_smem(full + s))
                             : "memory");
                     }
-                }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             cnn_smem(mbar))
-                         : "memory");
-        }
-        const bool ok = cnn_wait(mbar, (unsigned)(it & 1), wait_limit);
-        if (__syncthreads_or(!ok)) {
-            // the MMAs may still run: wait for them (bounded) before the band is released
-            cnn_wait(mbar, (unsigned)(it & 1), 1LL << 24);
-            failed = true;
-            break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll 1
-        for (int mb = 0; mb < TC_MB; ++mb) {
-            const int o = o0 + mb * TC_M + 32 * warp + lane;
-            const int y = o / P, x = o - y * P;
-            uint32_t v[NP];
-#pragma unroll
-            for (int c0 = 0; c0 < NP; c0 += 16) {
-                const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(32 * mb + c0);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                    "[%16];"
-                    : "=r"(v[c0 + 0]), "=r"(v[c0 + 1]), "=r"(v[c0 + 2]), "=r"(v[c0 + 3]), "=r"(v[c0 + 4]),
-                      "=r"(v[c0 + 5]), "=r"(v[c0 + 6]), "=r"(v[c0 + 7]), "=r"(v[c0 + 8]), "=r"(v[c0 + 9]),
-                      "=r"(v[c0 + 10]), "=r"(v[c0 + 11]), "=r"(v[c0 + 12]), "=r"(v[c0 + 13]), "=r"(v[c0 + 14]),
-                      "=r"(v[c0 + 15])
-                    : "r"(taddr));
-            }
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (y < H && x < W) {
-                if constexpr (OUT_PLANAR) {
-#pragma unroll
-                    for (int co = 0; co < NOUT; ++co) {
-                        float f = __uint_as_float(v[co]) + bv[co];
-                        if (relu) f = fmaxf(f, 0.0f);
-                        out[((b * NOUT + co) * H + y) * (int64_t)W + x] = __float2bfloat16(f);
-                    }
                 } else {
-                    uint4* dst = reinterpret_cast<uint4*>(out + ((b * H + y) * W + x) * NOUT);
+                    for (int k = 0; k < hi - lo; ++k) reinterpret_cast<uint4*>(dst)[k] = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(cnn_smem(full + s)) : "memory");
+        }
+        // the copies in flight land before the CTA gives its memory back
+        for (int k = max(0, it - nst); k < it; ++k)
+            cnn_wait(full + k % nst, (unsigned)((k / nst) & 1), 1LL << 24, nullptr);
+    } else if (warp == TC_EW + 1) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NP >> 3) << 17) |
+                               ((uint32_t)(TC_M >> 4) << 24);
+        // descriptors of offset 0; an operand starting k * 16 bytes later is desc + k
+        // (the start-address field counts 16-byte units; all addresses < 256 KB)
+        const uint64_t adesc0 = cnn_desc(cnn_smem(bands), nbp * 16, 128);
+        const uint64_t bdesc0 = cnn_desc(cnn_smem(wsm), 128, KG * 128);
+        int it = 0;
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+            const int s = it % nst, buf = it & 1;
+            bool ok = cnn_wait(full + s, (unsigned)((it / nst) & 1), wait_limit, fail);
+            if (ok && it >= 2) ok = cnn_wait(acce + buf, (unsigned)(((it >> 1) - 1) & 1), wait_limit, fail);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (lane == 0) {
+                const uint64_t ad0 = adesc0 + (uint64_t)(s * (bbytes >> 4));
+#pragma unroll 1
+                for (int mb = 0; mb < TC_MB; ++mb) {
+                    const uint32_t d = tmem + (uint32_t)(buf * ACC + 32 * mb);
 #pragma unroll
-                    for (int q4 = 0; q4 < NOUT / 8; ++q4) {
-                        uint32_t pk[4];
+                    for (int tap = 0; tap < 9; ++tap) {
+                        const int roff = mb * TC_M + (tap / 3) * P + (tap % 3);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            float f0 = __uint_as_float(v[q4 * 8 + 2 * j]) + bv[q4 * 8 + 2 * j];
-                            float f1 = __uint_as_float(v[q4 * 8 + 2 * j + 1]) + bv[q4 * 8 + 2 * j + 1];
-                            if (relu) {
-                                f0 = fmaxf(f0, 0.0f);
-                                f1 = fmaxf(f1, 0.0f);
-                            }
-                            __nv_bfloat162 h2 = __floats2bfloat162_rn(f0, f1);
-                            pk[j] = *reinterpret_cast<uint32_t*>(&h2);
+                        for (int k = 0; k < KG / 2; ++k) {
+                            const uint64_t ad = ad0 + (uint64_t)(2 * k * nbp + roff);
+                            const uint64_t bd = bdesc0 + (uint64_t)(tap * (NP / 8) * KG * 8 + 2 * k * 8);
+                            const uint32_t acc = (tap > 0 || k > 0) ? 1u : 0u;
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+                                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                                : "memory");
                         }
-                        dst[q4] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    }
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 cnn_smem(empty + s))
+                             : "memory");
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 cnn_smem(accf + buf))
+                             : "memory");
+            }
+            __syncwarp();
+        }
+        // the MMAs issued end before bands and accumulators are given back
+        for (int k = max(0, it - 2); k < it; ++k)
+            cnn_wait(accf + (k & 1), (unsigned)((k >> 1) & 1), 1LL << 24, nullptr);
+    } else {
+        // epilogue: warp quarter of the lanes, two of the four blocks each
+        float bv[NOUT];
+#pragma unroll
+        for (int c = 0; c < NOUT; ++c) bv[c] = bias[c];
+        const int64_t HW = (int64_t)H * W;
+        int it = 0;
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+            const int buf = it & 1;
+            const bool ok = cnn_wait(accf + buf, (unsigned)((it >> 1) & 1), wait_limit, fail);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int64_t b = tile / tiles_img;
+            const int o0 = (int)((tile - b * tiles_img) * TILE);
+#pragma unroll
+            for (int k = 0; k < TC_MB * 4 / TC_EW; ++k) {
+                const int mb = (warp >> 2) * (TC_MB * 4 / TC_EW) + k;
+                const int o = o0 + mb * TC_M + 32 * (warp & 3) + lane;
+                const int y = o / P, x = o - y * P;
+                uint32_t v[NP];
+#pragma unroll
+                for (int c0 = 0; c0 < NP; c0 += 16) {
+                    const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) +
+                                           (uint32_t)(buf * ACC + 32 * mb + c0);
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                        "[%16];"
+                        : "=r"(v[c0 + 0]), "=r"(v[c0 + 1]), "=r"(v[c0 + 2]), "=r"(v[c0 + 3]), "=r"(v[c0 + 4]),
+                          "=r"(v[c0 + 5]), "=r"(v[c0 + 6]), "=r"(v[c0 + 7]), "=r"(v[c0 + 8]), "=r"(v[c0 + 9]),
+                          "=r"(v[c0 + 10]), "=r"(v[c0 + 11]), "=r"(v[c0 + 12]), "=r"(v[c0 + 13]), "=r"(v[c0 + 14]),
+                          "=r"(v[c0 + 15])
+                        : "r"(taddr));
+                }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (k == TC_MB * 4 / TC_EW - 1) {   // the accumulators are read: the next tile but one may use them
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(cnn_smem(acce + buf)) : "memory");
+                }
+                if (y < H && x < W) {
+                    if constexpr (OUT_PLANAR) {
+#pragma unroll
+                        for (int co = 0; co < NOUT; ++co) {
+                            float f = __uint_as_float(v[co]) + bv[co];
+                            if (relu) f = fmaxf(f, 0.0f);
+                            out[(b * NOUT + co) * HW + (int64_t)y * W + x] = __float2bfloat16(f);
+                        }
+                    } else {
+                        uint4* dst = reinterpret_cast<uint4*>(out) + b * (NOUT / 8) * HW + (int64_t)y * W + x;
+#pragma unroll
+                        for (int q4 = 0; q4 < NOUT / 8; ++q4) {
+                            uint32_t pk[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                float f0 = __uint_as_float(v[q4 * 8 + 2 * j]) + bv[q4 * 8 + 2 * j];
+                                float f1 = __uint_as_float(v[q4 * 8 + 2 * j + 1]) + bv[q4 * 8 + 2 * j + 1];
+                                if (relu) {
+                                    f0 = fmaxf(f0, 0.0f);
+                                    f1 = fmaxf(f1, 0.0f);
+                                }
+                                __nv_bfloat162 h2 = __floats2bfloat162_rn(f0, f1);
+                                pk[j] = *reinterpret_cast<uint32_t*>(&h2);
+                            }
+                            dst[q4 * HW] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        }
                     }
                 }
             }
         }
-        // the next tile rewrites the band and the accumulators
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
     }
-    if (failed && t == 0) atomicOr(status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (*fail && t == 0) atomicOr(status, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(32 * TC_MB)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * ACC)
                      : "memory");
 }
 
@@ -724,38 +815,33 @@ cudaError_t forward(ibem_cnn* c, const float* in, int B, int H, int W, int bf) {
 }
 
 // Inference forward in BF16 on the tensor cores (C = 32 and a band that fits in
-// shared memory; otherwise the FMA path).  Slots: 0 the input as BF16 pixel-major
-// 8-channel pixels, 1..3 hidden outputs (pixel-major), 4 the output (planar), so
-// the output sits where forward() leaves it.
+// shared memory; otherwise the FMA path).  Slots: 0 the input as BF16 8-channel
+// pixels, 1..3 hidden outputs (by channel group), 4 the output (planar), so the
+// output sits where forward() leaves it.
 template <int CGI, int NP, int NOUT, bool OUT_PLANAR>
 cudaError_t launch_tc(ibem_cnn* c, const __nv_bfloat16* in, int B, int H, int W, const __nv_bfloat16* wt,
                       const float* bias, int relu, __nv_bfloat16* out, int* status, long long wait_limit) {
     constexpr int KG = CGI < 2 ? 2 : CGI;
     const int P = W + 2, nb = TC_M * TC_MB + 2 * P + 2, nbp = ((nb + 7) & ~7) + 2;
-    const size_t sm = (size_t)9 * (NP / 8) * KG * 128 + (size_t)KG * nbp * 16 + 16;
+    const size_t fixed = (size_t)9 * (NP / 8) * KG * 128 + TC_BARS, band = (size_t)KG * nbp * 16;
+    const int nst = (int)std::min<size_t>(TC_STAGES, (IBEM_MAX_SMEM_BYTES - fixed) / band);   // >= 1: tc_fits
+    const size_t sm = fixed + nst * band;
     auto kern = conv_tc_kernel<CGI, NP, NOUT, OUT_PLANAR>;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, kern))) return e;
     int nsm = 0, dev = 0;
     cudaGetDevice(&dev);
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev))) return e;
-    // resident CTAs per SM from shared memory (1 KB reserved per CTA), registers
-    // and TMEM (512 columns, 32 * TC_MB per CTA)
-    int per_sm = (int)std::min<size_t>(512 / (32 * TC_MB), (size_t)233472 / (sm + 1024));
-    per_sm = std::min(per_sm, 65536 / std::max(1, fa.numRegs * 128));
-    per_sm = std::max(per_sm, 1);
     const int64_t ntiles = (int64_t)B * (((int64_t)H * P + TC_M * TC_MB - 1) / (TC_M * TC_MB));
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)per_sm * nsm));
-    kern<<<grid, 128, sm, c->stream>>>(in, B, H, W, wt, bias, relu, nbp, out, wait_limit, status);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, nsm));
+    kern<<<grid, TC_T, sm, c->stream>>>(in, B, H, W, wt, bias, relu, nbp, nst, out, wait_limit, status);
     ++c->launches;
     return cudaGetLastError();
 }
 
 bool tc_fits(int W) {
     const int P = W + 2, nb = TC_M * TC_MB + 2 * P + 2, nbp = ((nb + 7) & ~7) + 2;
-    return (size_t)9 * 4 * 4 * 128 + (size_t)4 * nbp * 16 + 16 <= 227 * 1024;
+    return (size_t)9 * 4 * 4 * 128 + (size_t)4 * nbp * 16 + TC_BARS <= IBEM_MAX_SMEM_BYTES;
 }
 
 cudaError_t forward_infer(ibem_cnn* c, const float* in, int B, int H, int W, int* status, long long wait_limit) {
@@ -767,17 +853,21 @@ cudaError_t forward_infer(ibem_cnn* c, const float* in, int B, int H, int W, int
     if ((e = grow(&c->d_wtc, &c->wtc_bytes, (w0 + 2 * w1 + w3) * sizeof(__nv_bfloat16)))) return e;
     __nv_bfloat16* wt = reinterpret_cast<__nv_bfloat16*>(c->d_wtc);
     __nv_bfloat16* wl[4] = {wt, wt + w0, wt + w0 + w1, wt + w0 + 2 * w1};
-    const int np[4] = {32, 32, 32, 16}, kg[4] = {2, 4, 4, 4};
+    TcWeights tw;
     for (int l = 0; l < 4; ++l) {
-        const int n = np[l] * 8 * kg[l] * 9;
-        tc_weights_kernel<<<cblk(n, 256), 256, 0, c->stream>>>(c->d_param + c->woff[l], c->cin[l], c->cout[l], np[l],
-                                                              kg[l], wl[l]);
+        tw.w[l] = c->d_param + c->woff[l];
+        tw.wt[l] = wl[l];
+        tw.cin[l] = c->cin[l];
+        tw.cout[l] = c->cout[l];
+        tw.np[l] = l < 3 ? 32 : 16;
+        tw.kg[l] = l > 0 ? 4 : 2;
     }
+    tc_weights_kernel<<<dim3(cblk(32 * 32 * 9, 256), 4), 256, 0, c->stream>>>(tw);
     const size_t per = c->act_slot;
     __nv_bfloat16* act = reinterpret_cast<__nv_bfloat16*>(c->d_act);
     const int64_t npx = (int64_t)B * H * W;
     pack8_kernel<<<cblk(npx, 256), 256, 0, c->stream>>>(npx, (int64_t)H * W, in, act);
-    c->launches += 5;
+    c->launches += 2;
     if ((e = launch_tc<1, 32, 32, false>(c, act, B, H, W, wl[0], c->d_param + c->boff[0], 1, act + per, status,
                                          wait_limit)))
         return e;
