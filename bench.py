@@ -711,8 +711,8 @@ def _peak_tensor():
 
 
 def gen_ops_per_launch(n_far, q, R):
-    """FP32-pipe operations of the double-float coupling, counted from its
-    formulas: 247 per generated complex kernel value (differences, r^2, r, 1/r,
+    """FP32-pipe operations of the double-float coupling in its plain form, every
+    pair normalised: 247 per generated complex kernel value (differences, r^2, r, 1/r,
     the phase and its reduction, the Taylor terms, the table product) and 48 per
     complex multiply-add and right-hand side (four exact products with their
     error terms and TwoSum accumulations of 12 operations each)."""
@@ -721,8 +721,8 @@ def gen_ops_per_launch(n_far, q, R):
 
 
 def sliced_ops_per_launch(n_far, R):
-    """FP32-pipe operations of the digit-sliced coupling (q = 8), counted from its
-    formulas per far block and chunk of 32 right-hand sides: 247 per generated
+    """FP32-pipe operations of the digit-sliced coupling (q = 8) in its plain form, a
+    generation for each chunk of 32 right-hand sides; per far block and chunk: 247 per generated
     complex kernel value (as the double-float coupling), 58 per sliced real
     value (scaling, and per each of 6 digits: rint, the exact remainder with a
     Fast2Sum, the rescaling and the BF16 packing) and 48 per recombined
@@ -732,6 +732,27 @@ def sliced_ops_per_launch(n_far, R):
     nch = (R + 31) // 32
     per = 4096 * 247.0 + 8192 * 58.0 + 8192 * 48.0
     return n_far * nch * per, n_far * nch * 21 * 2.0 * 128 * 64 * 64
+
+
+VALUE_OPS = 164          # FP32 operations of a generated complex kernel value
+DIGIT_OPS = 29           # of the digits of a real value
+RECOMBINE_OPS = 40       # of a recombined accumulator entry
+
+
+def gen_ops_executed(n_far, q, R):
+    """FP32-pipe operations the double-float coupling executes: a kernel value takes
+    VALUE_OPS (pairs are normalised only where a later step needs it)."""
+    gen, mac = gen_ops_per_launch(n_far, q, R)
+    return gen / 247.0 * VALUE_OPS, mac
+
+
+def sliced_ops_executed(n_far, R):
+    """FP32-pipe operations and tensor flops the digit-sliced coupling executes: the
+    values and digits of a far block are formed once for two chunks of 32 right-hand
+    sides, its 128 x 64 accumulator entries are recombined for each chunk."""
+    nch = (R + 31) // 32
+    ops = n_far * ((nch + 1) // 2 * (4096.0 * VALUE_OPS + 8192.0 * DIGIT_OPS) + nch * 8192.0 * RECOMBINE_OPS)
+    return ops, sliced_ops_per_launch(n_far, R)[1]
 
 
 def plane_wave_rhs(ibem, h, kappa, R, seed):
@@ -976,7 +997,7 @@ def ours(args, rank, world, local_rank):
     coup_ms = phase_ms["coupling"]
     kvals = info.n_far * float(W["q_cheb"]) ** 4
     if args.coupling == "sliced":
-        ops, tflop = sliced_ops_per_launch(info.n_far, R)
+        ops, tflop = sliced_ops_executed(info.n_far, R)
         tpk0, _ = _peak_tensor()
         achieved = ops / (coup_ms * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s", "frac": achieved / alu_peak,
@@ -986,11 +1007,12 @@ def ours(args, rank, world, local_rank):
                            "frac": tflop / (coup_ms * 1e-3) / 1e12 / tpk0},
                 "peak_source": "FP32 pipe: 152 SMs x 128 lanes x %.0f MHz (sm_max_mhz of MEASURED_PEAKS.json, %s)"
                                % (sm_max, peak_src),
-                "ops_source": "counted from the digit-sliced formulas per far block and chunk of 32 right-hand sides: "
-                              "247 FP32 operations per generated complex kernel value, 58 per sliced real value, "
-                              "48 per recombined accumulator entry; tensor: 21 slice pairs of 2 x 128 x 64 x 64"}
+                "ops_source": "counted from the digit-sliced formulas: per far block and two chunks of 32 right-hand sides "
+                              "%d FP32 operations per generated complex kernel value and %d per sliced real value, per "
+                              "chunk %d per recombined accumulator entry; tensor: 21 slice pairs of 2 x 128 x 64 x 64"
+                              % (VALUE_OPS, DIGIT_OPS, RECOMBINE_OPS)}
     else:
-        gen_ops, mac_ops = gen_ops_per_launch(info.n_far, W["q_cheb"], R)
+        gen_ops, mac_ops = gen_ops_executed(info.n_far, W["q_cheb"], R)
         achieved = (gen_ops + mac_ops) / (coup_ms * 1e-3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "Tops/s", "frac": achieved / alu_peak,
                 "traffic": _profile_traffic(), "kernel": "helm_coupling_gen_kernel", "ms_per_launch": coup_ms,
@@ -998,8 +1020,8 @@ def ours(args, rank, world, local_rank):
                 "kernel_values": kvals, "kernel_values_per_s": kvals / (coup_ms * 1e-3),
                 "peak_source": "FP32 pipe: 152 SMs x 128 lanes x %.0f MHz (sm_max_mhz of MEASURED_PEAKS.json, %s)"
                                % (sm_max, peak_src),
-                "ops_source": "counted from the double-float formulas: 247 FP32 operations per generated complex "
-                              "kernel value, 48 per complex multiply-add and right-hand side"}
+                "ops_source": "counted from the double-float formulas: %d FP32 operations per generated complex "
+                              "kernel value, 48 per complex multiply-add and right-hand side" % VALUE_OPS}
 
     # ---- FP32 operator (tensor-core coupling, BF16 K and moments) ----
     run(args.warmup, 1, y32)

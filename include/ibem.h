@@ -144,7 +144,8 @@ enum { IBEM_FP32_COUPLING_GENERATE = 0, IBEM_FP32_COUPLING_STORE = 1 };
 
 /* FP64 coupling variants.  GB300 executes FP64 FMA at 1/64 of the FP32 rate, so
  * by default the coupling matrices are stored as unevaluated float pairs
- * (hi + lo, 8 bytes per real entry, 16 per complex one) and applied with exact
+ * (hi + lo, 8 bytes per real entry, 16 per complex one; one of two mirrored
+ * blocks, which serves both directions) and applied with exact
  * FP32 products and compensated sums (about 48 significant bits, relative
  * error ~1e-14).  NATIVE: Laplace stores doubles and uses FP64 FMA; Helmholtz
  * generates the coupling on the fly in FP64 (also chosen automatically when the
@@ -171,8 +172,8 @@ enum { IBEM_COUPLING_DF = 0, IBEM_COUPLING_NATIVE = 1, IBEM_COUPLING_NONE = 2, I
  * (per block, per moment column), the 21 digit-slice products of combined
  * weight down to 2^-54 are accumulated exactly in FP32 (integer partial sums
  * below 2^23) and recombined in double-float, so the result carries about 45
- * significant bits, like GENERATE within the 1e-12 parity tolerance.  Chunks
- * of 32 right-hand sides.  Other handles (or a phase kappa |x - y| of 90 or more)
+ * significant bits, like GENERATE within the 1e-12 parity tolerance.  Right-hand
+ * sides go in chunks of 32, two of which share a block's values and digits.  Other handles (or a phase kappa |x - y| of 90 or more)
  * take the GENERATE path; a Laplace handle treats SLICED like DF.
  * IBEM_COUPLING_FP32_ONLY (memory for large batches): the FP64 near blocks are
  * released at the end of ibem_assemble, after the FP32 copy, the Jacobi
