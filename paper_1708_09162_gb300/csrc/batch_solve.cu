@@ -219,9 +219,7 @@ struct BatchKrylov {
             const BatchInst& I = b->inst[i];
             const int cw = I.helm ? 2 : 1;
             if (precond == IBEM_PRECOND_BLOCK_JACOBI) {
-                for (int r = 0; r < I.R; ++r)
-                    apply_block_jacobi(h, v + b->offsets[i] + (int64_t)r * I.N * cw,
-                                       z + b->offsets[i] + (int64_t)r * I.N * cw);
+                apply_block_jacobi(h, v + b->offsets[i], z + b->offsets[i], I.R);
             } else {
                 inst_jacobi_kernel<<<sblk((int64_t)I.R * I.N, 256), 256, 0, st>>>(
                     v + b->offsets[i], precond == IBEM_PRECOND_JACOBI ? h->d_diag : nullptr, I.N, I.R, cw,

@@ -1099,7 +1099,7 @@ cudaError_t op_batch(ibem_handle* h, ibem_cnn* c, const OpScratch& o, int nb, in
     cudaError_t e;
     const int f = c->coarse, nc = (n1 + f - 1) / f;
     const int64_t nch = (int64_t)nb * npatch * 2;
-    for (int j = 0; j < nb; ++j) apply_block_jacobi(h, o.R + (size_t)j * vec, o.S + (size_t)j * vec);
+    apply_block_jacobi(h, o.R, o.S, nb);
     vec_sumsq_kernel<<<nb, 256, 0, st>>>(vec, o.S, o.ss);
     batch_pack_kernel<<<cblk((int64_t)nb * N, 256), 256, 0, st>>>(nb, N, n1, o.S, o.ss, o.img);
     if (f > 1)

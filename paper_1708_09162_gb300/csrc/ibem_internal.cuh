@@ -488,7 +488,8 @@ bool mr_supported(const ibem_handle* h, int nrhs);
 bool mr_store_possible(const ibem_handle* h);
 cudaError_t mr_store_coupling(ibem_handle* h);
 cudaError_t apply_operator_mrhs(ibem_handle* h, const double* x, double* y, int nrhs);
-void apply_block_jacobi(ibem_handle* h, const double* r, double* z);
+// z = M^-1 r for R vectors stored one after the other
+void apply_block_jacobi(ibem_handle* h, const double* r, double* z, int R = 1);
 // Helmholtz coupling generated in double-float for many right-hand sides (kernels_gen.cu).
 bool gen_supported(const ibem_handle* h);
 cudaError_t launch_coupling_gen(ibem_handle* h, int R);

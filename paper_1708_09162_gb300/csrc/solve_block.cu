@@ -250,13 +250,10 @@ struct Ctx {
     // z = M^-1 v for R columns (fixed preconditioners)
     cudaError_t precondition(const double* v, double* z, int R) {
         if (precond == IBEM_PRECOND_BLOCK_JACOBI || precond == IBEM_PRECOND_LEARNED) {
-            for (int r = 0; r < R; ++r) {
-                if (precond == IBEM_PRECOND_LEARNED) {
-                    cudaError_t e = cnn_precondition(h, h->cnn, v + (size_t)r * m, z + (size_t)r * m);
-                    if (e) return e;
-                } else {
-                    apply_block_jacobi(h, v + (size_t)r * m, z + (size_t)r * m);
-                }
+            if (precond == IBEM_PRECOND_BLOCK_JACOBI) apply_block_jacobi(h, v, z, R);
+            for (int r = 0; precond == IBEM_PRECOND_LEARNED && r < R; ++r) {
+                cudaError_t e = cnn_precondition(h, h->cnn, v + (size_t)r * m, z + (size_t)r * m);
+                if (e) return e;
             }
             return cudaGetLastError();
         }
