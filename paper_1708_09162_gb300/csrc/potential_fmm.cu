@@ -33,6 +33,7 @@ namespace {
 
 constexpr int PF_STACK = 32;   // depth-first stack below one root: at most 3 m + 1 <= 31 entries (m <= 10)
 constexpr int PF_RC = 16;      // densities per CTA of the evaluation
+constexpr int PF_RS = 4;       // the same for few densities
 constexpr int PF_MV = 8;       // real vectors per CTA of the cluster moments
 constexpr int PF_T = 256;
 
@@ -155,32 +156,35 @@ __global__ void pf_moments_kernel(int n_used, const int32_t* __restrict__ used_i
 
 // u*(x, y) from |x - y|^2 (fp64_eval.cuh): the kernels below are bound by the FP64
 // pipe, and this takes about 30 operations instead of 80 with sqrt, division and
-// sincos (5000 points, 4 densities, level 6: evaluation 5.34 ms instead of 6.04)
+// sincos (5000 points, 4 densities, level 6, 16 sums per thread: 5.34 ms instead of 6.04)
 template <bool CPLX>
 __device__ __forceinline__ void pf_kernel_value(double d2, double kappa, const double2* __restrict__ trig, double* gr,
                                                 double* gi) {
     green64<CPLX>(d2, kappa, 1.0 / (4.0 * IBEM_PI), trig, gr, gi);
 }
 
-// One CTA per (point, chunk of PF_RC densities).  Far terms: entries (cluster,
+// One CTA per (point, chunk of RC densities).  Far terms: entries (cluster,
 // interpolation point b) of the point's list, flattened over the CTA's
 // threads; the moments of R densities (complex: 2 R real vectors, real part
 // first) are [R][n_used][q2], cluster c at row slot[c].  Near terms: entries
 // (element, Gauss point); the density at a Gauss point is
 // sum_i phi[g][i] x*_e[i] from the lifted coefficients xs [R][E][nb].
-template <bool CPLX>
-__global__ void __launch_bounds__(PF_T, 2) pf_eval_kernel(
+// RC: PF_RC, or PF_RS where all densities fit into it: the sums of 16 complex densities
+// take 64 registers and 160 additions and 320 shuffles per thread at the end, against
+// some 20 pairs per thread (5000 points, 4 densities, level 6: 2.59 ms, 5.34 with 16).
+template <bool CPLX, int RC>
+__global__ void __launch_bounds__(PF_T, RC <= PF_RS ? 2 : 1) pf_eval_kernel(
     int64_t npts, int npatch, const double* __restrict__ pts, int R, const int64_t* __restrict__ far_off,
     const int32_t* __restrict__ far_list, const int64_t* __restrict__ near_off, const int32_t* __restrict__ near_list,
     int q2, int64_t n_used, const int32_t* __restrict__ slot, const double* __restrict__ igeo,
     const double* __restrict__ xh, int QQ, int nb, int64_t E,
     const double* __restrict__ qgeo, const double* __restrict__ phi, const double* __restrict__ xs, double kappa,
     const double2* __restrict__ trig, double* __restrict__ u) {
-    constexpr int NA = CPLX ? 2 * PF_RC : PF_RC;
+    constexpr int NA = CPLX ? 2 * RC : RC;
     __shared__ double red[PF_T / 32][NA];
     const int64_t ip = blockIdx.x;
-    const int r0 = blockIdx.y * PF_RC;
-    const int nc = R - r0 < PF_RC ? R - r0 : PF_RC;
+    const int r0 = blockIdx.y * RC;
+    const int nc = R - r0 < RC ? R - r0 : RC;
     const double x0 = pts[3 * ip], x1 = pts[3 * ip + 1], x2 = pts[3 * ip + 2];
     double acc[NA];
 #pragma unroll
@@ -206,7 +210,7 @@ __global__ void __launch_bounds__(PF_T, 2) pf_eval_kernel(
                 gi *= z[3];
                 const double* mom = mom0 + b;
 #pragma unroll
-                for (int j = 0; j < PF_RC; ++j) {
+                for (int j = 0; j < RC; ++j) {
                     if (j < nc) {
                         if constexpr (CPLX) {
                             const double mr = mom[(2 * j) * n_used * q2], mi = mom[(2 * j + 1) * n_used * q2];
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(PF_T, 2) pf_eval_kernel(
                 gi *= y[3];
                 const double* ph = phi + (int64_t)g * nb;
 #pragma unroll
-                for (int j = 0; j < PF_RC; ++j) {
+                for (int j = 0; j < RC; ++j) {
                     if (j < nc) {
                         if constexpr (CPLX) {
                             const double* cr = xs + ((2 * (r0 + j)) * E + e) * nb;
@@ -432,16 +436,19 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
         h->launches++;
     }
     // (4) evaluation
-    dim3 grid((unsigned)npts, (unsigned)((nrhs + PF_RC - 1) / PF_RC));
     const int QQ = P.Q * P.Q;
-    if (h->helm)
-        pf_eval_kernel<true><<<grid, PF_T, 0, st>>>(npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1,
-                                                    d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo, d_xhat, QQ,
-                                                    P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, P.prm.kappa, h->d_trig64, u);
-    else
-        pf_eval_kernel<false><<<grid, PF_T, 0, st>>>(npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1,
-                                                     d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo, d_xhat, QQ,
-                                                     P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, 0.0, h->d_trig64, u);
+    auto eval = [&](auto kern, int rc) {
+        kern<<<dim3((unsigned)npts, (unsigned)((nrhs + rc - 1) / rc)), PF_T, 0, st>>>(
+            npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1, d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo,
+            d_xhat, QQ, P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, P.prm.kappa, h->d_trig64, u);
+    };
+    if (h->helm) {
+        if (nrhs <= PF_RS) eval(pf_eval_kernel<true, PF_RS>, PF_RS);
+        else eval(pf_eval_kernel<true, PF_RC>, PF_RC);
+    } else {
+        if (nrhs <= PF_RS) eval(pf_eval_kernel<false, PF_RS>, PF_RS);
+        else eval(pf_eval_kernel<false, PF_RC>, PF_RC);
+    }
     h->launches++;
     return cudaGetLastError();
 }
