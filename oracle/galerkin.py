@@ -138,7 +138,7 @@ class Discretisation:
         if len(matches) == 1:
             ka, kb = singular.canonical_orientation(self.corners[eA], self.corners[eB], "vertex", tol)
             return "vertex", ka, kb
-        d = np.sqrt(np.sum((cA - cB) ** 2)) - rA - rB
+        d = np.sqrt(np.sum((cA - cB) ** 2)) - (rA + rB)
         dist = d if d > 0.0 else 0.0
         if dist < 0.5 * diam:
             return "nearsing", 0, 0
@@ -152,7 +152,7 @@ class Discretisation:
             return self.n_singular
         (cA, rA), (cB, rB) = self.balls[eA], self.balls[eB]
         diam = 2.0 * (rA if rA > rB else rB)
-        d = np.sqrt(np.sum((cA - cB) ** 2)) - rA - rB
+        d = np.sqrt(np.sum((cA - cB) ** 2)) - (rA + rB)
         return graded_order(self.n_regular, self.grading, d if d > 0.0 else 0.0, diam)
 
     # ---- element-pair block --------------------------------------------------

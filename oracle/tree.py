@@ -9,9 +9,10 @@ Readings (the printed definition uses 0 < mu < 1 with max diam < mu dist, and
 its far/near sentence is garbled):
 * admissible  iff  eta * max(diam_s, diam_t) < dist(s, t), eta = 1/mu (eta = 1.6
   in the workloads);
-* diam = 2 r and dist = max(0, |c_s - c_t| - r_s - r_t), with c = F(midpoint) and
+* diam = 2 r and dist = max(0, |c_s - c_t| - (r_s + r_t)), with c = F(midpoint) and
   r = max |F(x) - c| over a 5 x 5 uniform grid of parameter points including
-  the corners;
+  the corners; the radii are added first, so that dist is the same for (s, t) and
+  (t, s) in floating point too and the block tree is symmetric;
 * the block tree starts from all patch pairs at level 0; an admissible block is
   far field, a non-admissible block at the leaf level (elements) is near field,
   any other block is split into its 4 x 4 child pairs.
@@ -58,7 +59,7 @@ class ClusterGeometry:
         the printed max diam < mu dist)."""
         cs, rs = self.ball(s)
         ct, rt = self.ball(t)
-        d = np.sqrt(np.sum((cs - ct) ** 2)) - rs - rt
+        d = np.sqrt(np.sum((cs - ct) ** 2)) - (rs + rt)
         dist = d if d > 0.0 else 0.0
         diam = 2.0 * (rs if rs > rt else rt)
         if reading == "eta_dist":

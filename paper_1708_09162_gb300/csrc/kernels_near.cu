@@ -88,7 +88,7 @@ __device__ __forceinline__ void bernstein_at(double t, double (&b)[PP]) {
     }
 }
 
-// index of the pair (s, t) in the lists, given that (t, s) is one
+// index of the pair (s, t) in the lists, -1 if it is not there (the plan refuses such lists)
 __device__ inline int64_t mirror_of(int64_t t, int64_t s, const int64_t* __restrict__ nptr,
                                     const int32_t* __restrict__ nsrc) {
     int64_t lo = nptr[s], hi = nptr[s + 1];
@@ -97,7 +97,7 @@ __device__ inline int64_t mirror_of(int64_t t, int64_t s, const int64_t* __restr
         if (nsrc[mid] < t) lo = mid + 1;
         else hi = mid;
     }
-    return lo;
+    return lo < nptr[s + 1] && nsrc[lo] == t ? lo : -1;
 }
 
 // ---- regular and subdivided pairs ------------------------------------------------
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(NT) near_product_kernel(GeomView g, const int3
 #pragma unroll
             for (int c = 0; c < CW; ++c) {
                 blocks[(k * nb * nb + e) * CW + c] = acc[n][c];
-                blocks[(k2 * nb * nb + j * nb + i) * CW + c] = acc[n][c];
+                if (k2 >= 0) blocks[(k2 * nb * nb + j * nb + i) * CW + c] = acc[n][c];
             }
         }
     }
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(NT) near_touch_kernel(GeomView g, int cls, con
             blocks[k * nb * nb * CW + e] = v + vt;
         } else {
             blocks[k * nb * nb * CW + e] = v;
-            blocks[k2 * nb * nb * CW + e] = vt;
+            if (k2 >= 0) blocks[k2 * nb * nb * CW + e] = vt;
         }
     }
 }

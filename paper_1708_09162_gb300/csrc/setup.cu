@@ -127,9 +127,13 @@ Ball ball_of(const GeomView& g, int patch, int level, int ix, int iy) {
     return b;
 }
 
+// Symmetric to the last bit (the radii are added first), so that (a, b) and (b, a)
+// get the same admissibility, class and Gauss order: one of two mirrored blocks is
+// formed and stored for both.  With (d - a.r) - b.r a tie on an axis-parallel cube went
+// either way.
 double ball_dist(const Ball& a, const Ball& b) {
     double d0 = a.c[0] - b.c[0], d1 = a.c[1] - b.c[1], d2 = a.c[2] - b.c[2];
-    double d = std::sqrt(d0 * d0 + d1 * d1 + d2 * d2) - a.r - b.r;
+    double d = std::sqrt(d0 * d0 + d1 * d1 + d2 * d2) - (a.r + b.r);
     return d > 0.0 ? d : 0.0;
 }
 
@@ -157,6 +161,20 @@ int dihedral_corner(int k, int s, int t) {
     if (ix == 1 && iy == 0) return 1;
     if (ix == 1 && iy == 1) return 2;
     return 3;
+}
+
+// true if a list of rows (sources ascending) holds the mirror (s, t) of every entry (t, s)
+// and same(k, k2) holds for both: going through the rows in order, the mirrors of row
+// s's entries come by in the order of row s
+template <typename Same>
+bool mirrored(const std::vector<int64_t>& ptr, const std::vector<int32_t>& src, Same same) {
+    std::vector<int64_t> next(ptr.begin(), ptr.end() - 1);
+    for (int64_t t = 0; t + 1 < (int64_t)ptr.size(); ++t)
+        for (int64_t k = ptr[t]; k < ptr[t + 1]; ++k) {
+            const int64_t s = src[k], k2 = next[s]++;
+            if (k2 >= ptr[s + 1] || src[k2] != t || !same(k, k2)) return false;
+        }
+    return true;
 }
 
 double corner_gap(const double* a, const double* b) {
@@ -387,6 +405,12 @@ std::string build_plan(const ibem_patch* patches, int npatch, const ibem_params*
         P.far_src[k] = far[k].second;
     }
     for (int64_t c = 0; c < P.C; ++c) P.far_ptr[c + 1] += P.far_ptr[c];
+    // what the near assembly and the symmetric couplings rely on
+    if (!mirrored(P.near_ptr, P.near_src, [&](int64_t k, int64_t k2) {
+            return P.near_cls[k] == P.near_cls[k2] && P.near_order[k] == P.near_order[k2];
+        }) ||
+        !mirrored(P.far_ptr, P.far_src, [](int64_t, int64_t) { return true; }))
+        return "degenerate patch geometry: block lists are not symmetric";
     return "";
 }
 

@@ -78,3 +78,20 @@ def fichera():
         e1, e2 = np.eye(3)[(axis + 1) % 3], np.eye(3)[(axis + 2) % 3]
         patches.append(_square(np.zeros(3), e1, e2))
     return patches
+
+
+def cube(side=1.0, centre=(0.0, 0.0, 0.0), turn=0.0):
+    """Six bilinear faces of an axis-parallel cube, turned by `turn` about z and
+    shifted; many of its cluster pairs sit exactly on a threshold of distance over
+    diameter, so rounding decides them."""
+    c, s = np.cos(turn), np.sin(turn)
+    rot = np.array([[c, -s, 0.0], [s, c, 0.0], [0.0, 0.0, 1.0]])
+    patches = []
+    for axis in range(3):
+        for sign in (1.0, -1.0):
+            e1, e2 = np.eye(3)[(axis + 1) % 3], np.eye(3)[(axis + 2) % 3]
+            if sign < 0:
+                e1, e2 = e2, e1
+            deg_u, deg_v, ku, kv, ctrl, w = _square(sign * np.eye(3)[axis] - e1 - e2, 2.0 * e1, 2.0 * e2)
+            patches.append((deg_u, deg_v, ku, kv, 0.5 * side * ctrl @ rot.T + np.asarray(centre), w))
+    return patches
