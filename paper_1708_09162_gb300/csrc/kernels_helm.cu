@@ -389,6 +389,7 @@ __global__ void __launch_bounds__(HN_T) helm_near_df_kernel(const int64_t* __res
         }
         return;
     }
+    if (sl > 0) return;              // one slice: nt < HN_T leaves threads without a pair
 #pragma unroll
     for (int m = 0; m < MAXP; ++m) {
         const int p = ts + nt * m;
