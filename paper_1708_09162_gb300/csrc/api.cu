@@ -534,6 +534,9 @@ ibem_status ibem_assemble(ibem_handle* h) {
             }
         }
     }
+    // work vectors sized before the coupling was stored (by ibem_rhs, for instance) lack
+    // its column shares: the next application sizes them again
+    if (h->d_Kdf && !h->d_colpart) h->ws_nrhs = 0;
     if (h->helm) {
         if ((e = helm_launch_near_assembly(h))) return cuda_fail(h, e, "near assembly");
         if ((e = helm_launch_far_assembly(h))) return cuda_fail(h, e, "far assembly");
