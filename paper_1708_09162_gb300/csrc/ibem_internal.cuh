@@ -497,6 +497,7 @@ cudaError_t launch_coupling_gen(ibem_handle* h, int R);
 bool sliced_supported(const ibem_handle* h);
 cudaError_t launch_coupling_sliced(ibem_handle* h, int R);
 // Helmholtz coupling from stored double-float matrices (kernels_helm_df.cu).
+cudaError_t ensure_helm_df(ibem_handle* h, int R);
 cudaError_t launch_helm_coupling_df(ibem_handle* h, int R);
 // Double-float coupling launcher and the autotuner of its ring depth (kernels_apply.cu).
 cudaError_t launch_coupling_df(ibem_handle* h, int R, int nst);

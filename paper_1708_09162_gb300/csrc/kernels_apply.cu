@@ -758,6 +758,8 @@ __global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ ou
 
 cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
     // nrhs counts real right-hand sides (a complex one counts twice)
+    cudaError_t e;
+    if (h->d_Kc && (e = ensure_helm_df(h, (nrhs + 1) / 2))) return e;
     if (nrhs <= h->ws_nrhs) return cudaSuccess;
     Plan& P = h->P;
     if (h->helm) {
@@ -772,7 +774,6 @@ cudaError_t ensure_workspace(ibem_handle* h, int nrhs) {
     h->d_xs32 = nullptr;
     h->d_src32 = nullptr;
     h->ws_nrhs = 0;
-    cudaError_t e;
     size_t ns = (size_t)nrhs * P.Nstar, nh = (size_t)nrhs * P.C * (P.q2 > 0 ? P.q2 : 1);
     if ((e = cudaMalloc(&h->d_xs, ns * sizeof(double)))) return e;
     if ((e = cudaMalloc(&h->d_ys, ns * sizeof(double)))) return e;

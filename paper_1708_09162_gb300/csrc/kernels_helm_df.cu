@@ -294,7 +294,8 @@ cudaError_t launch_sym_rb(ibem_handle* h, int r0, int rc, int ng, int RB) {
 }  // namespace
 
 // Work space of the stored coupling for R complex right-hand sides: moments and
-// column shares of one pass.
+// column shares of one pass.  Sized with the other work vectors (ensure_workspace), not
+// in the application, which a program may record into a graph.
 cudaError_t ensure_helm_df(ibem_handle* h, int R) {
     const int rc = R < HS_RC ? R : HS_RC;
     if (rc <= h->hdf_rhs) return cudaSuccess;
@@ -316,7 +317,6 @@ cudaError_t launch_helm_coupling_df(ibem_handle* h, int R) {
     const Plan& P = h->P;
     cudaStream_t st = h->stream;
     cudaError_t e;
-    if ((e = ensure_helm_df(h, R))) return e;
     const int q2 = P.q2, q2p = (q2 + 1) & ~1, T = 256;
     if (h->up_rows.empty()) return cudaSuccess;
     for (int r0 = 0; r0 < R; r0 += HS_RC) {

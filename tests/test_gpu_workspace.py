@@ -31,3 +31,40 @@ def test_right_hand_side_before_assembly(kernel, R):
         assert rel_err(a[0].cpu().numpy(), a[1].cpu().numpy()) < 1e-13
     for h in hs:
         ibem.ibem_destroy(h)
+
+
+@pytest.mark.parametrize("first", ["rhs", "fp32"])
+def test_application_recorded_after_another_call_of_its_width(first):
+    # the stored Helmholtz coupling's work space is sized with the rest: after any call of as
+    # many vectors an FP64 application allocates nothing, so it can be recorded (thread-local
+    # capture fails on an allocation)
+    import torch
+    ibem = lib()
+    stream = torch.cuda.Stream()
+    prm = ibem.make_params(1, 2, q_cheb=5, eta=1.6, kernel=1, kappa=3.0)
+    hs = [ibem.ibem_create(ibem.sphere_patches(), prm, stream) for _ in range(2)]
+    info = ibem.ibem_get_info(hs[0])
+    rng = np.random.default_rng(1602)
+    x = torch.from_numpy(rng.normal(size=(3, info.ndof, 2))).cuda()
+    g = torch.from_numpy(rng.normal(size=(3, info.n_quad_points, 2))).cuda()
+    ref, y = torch.full_like(x, np.nan), torch.full_like(x, np.nan)
+    torch.cuda.synchronize()
+    for h in hs:
+        ibem.ibem_assemble(h)
+    ibem.ibem_matvec(hs[0], x, ref, 3)             # loads every kernel
+    if first == "rhs":
+        ibem.ibem_rhs(hs[1], g, 3, y)
+    else:
+        ibem.ibem_matvec(hs[1], x, y, 3, ibem.IBEM_FP32)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        ibem.ibem_matvec(hs[1], x, y, 3)
+    y.fill_(float("nan"))
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, ref)
+    del graph
+    for h in hs:
+        ibem.ibem_destroy(h)
