@@ -734,7 +734,7 @@ def sliced_ops_per_launch(n_far, R):
     return n_far * nch * per, n_far * nch * 21 * 2.0 * 128 * 64 * 64
 
 
-VALUE_OPS = 164          # FP32 operations of a generated complex kernel value
+VALUE_OPS = 176          # FP32 operations of a generated complex kernel value
 DIGIT_OPS = 29           # of the digits of a real value
 RECOMBINE_OPS = 40       # of a recombined accumulator entry
 
