@@ -50,75 +50,84 @@ __global__ void lift_kernel(int R, int64_t E, int p, int ne1, const double* __re
     xs[idx] = acc;
 }
 
-__global__ void restrict_kernel(int R, int64_t N, int p, int ne1, const double* __restrict__ ext,
-                                const double* __restrict__ ys, int64_t E, double* __restrict__ y) {
-    int pp = p + 1, nb = pp * pp, n1 = ne1 + p;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * N) return;
-    int64_t r = idx / N, dof = idx % N;
-    int patch = (int)(dof / ((int64_t)n1 * n1));
-    int rem = (int)(dof % ((int64_t)n1 * n1));
-    int jv = rem / n1, ju = rem % n1;
-    int64_t per = (int64_t)ne1 * ne1;
+// y = T ys: a dof adds the shares of the (p + 1)^2 elements under it.  The sum is a tree
+// over the elements (halves, quarters, ...; zero for an element beyond the patch), the
+// same whether a thread takes all of them or a group of G lanes one each, so the bits
+// of a vector do not depend on how many are restricted with it.
+template <int PP>
+__device__ __forceinline__ double restrict_share(int k, int ju, int jv, int64_t row, int ne1,
+                                                 const double* __restrict__ ext, const double* __restrict__ ys) {
+    const int iy = jv - (PP - 1) + k / PP, ix = ju - (PP - 1) + k % PP;
+    if (k >= PP * PP || iy < 0 || iy >= ne1 || ix < 0 || ix >= ne1) return 0.0;
+    const double* v = ys + (row + morton2(ix, iy)) * (PP * PP);
+    const double* cu = ext + ((int64_t)ix * PP + (ju - ix)) * PP;
+    const double* cv = ext + ((int64_t)iy * PP + (jv - iy)) * PP;
     double acc = 0.0;
-    for (int iy = jv - p; iy <= jv; ++iy) {
-        if (iy < 0 || iy >= ne1) continue;
-        for (int ix = ju - p; ix <= ju; ++ix) {
-            if (ix < 0 || ix >= ne1) continue;
-            const double* v = ys + (r * E + patch * per + morton2(ix, iy)) * nb;
-            const double* cu = ext + ((int64_t)ix * pp + (ju - ix)) * pp;
-            const double* cv = ext + ((int64_t)iy * pp + (jv - iy)) * pp;
-            for (int iv = 0; iv < pp; ++iv) {
-                double row = 0.0;
-                for (int iu = 0; iu < pp; ++iu) row += cu[iu] * v[iv * pp + iu];
-                acc += cv[iv] * row;
-            }
-        }
+#pragma unroll
+    for (int iv = 0; iv < PP; ++iv) {
+        double part = 0.0;
+#pragma unroll
+        for (int iu = 0; iu < PP; ++iu) part = fma(cu[iu], v[iv * PP + iu], part);
+        acc = fma(cv[iv], part, acc);
     }
-    y[idx] = acc;
+    return acc;
 }
 
-// The same with one thread per (dof, element of its support), the (p + 1)^2 shares added
-// by shuffles in a fixed order: the single thread's sum over up to 25 elements is a
-// chain of some 30 us (p = 3), which a short vector cannot hide.  G: lanes per dof,
-// a power of two >= (p + 1)^2.
-__global__ void restrict_group_kernel(int R, int64_t N, int p, int ne1, int G, const double* __restrict__ ext,
-                                      const double* __restrict__ ys, int64_t E, double* __restrict__ y) {
-    const int pp = p + 1, nb = pp * pp, n1 = ne1 + p;
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, idx = g / G;
-    const int k = (int)(g % G);
-    double acc = 0.0;
-    if (idx < R * N && k < nb) {
-        const int64_t r = idx / N, dof = idx % N;
-        const int patch = (int)(dof / ((int64_t)n1 * n1)), rem = (int)(dof % ((int64_t)n1 * n1));
-        const int jv = rem / n1, ju = rem % n1, iy = jv - p + k / pp, ix = ju - p + k % pp;
-        if (iy >= 0 && iy < ne1 && ix >= 0 && ix < ne1) {
-            const double* v = ys + (r * E + patch * (int64_t)ne1 * ne1 + morton2(ix, iy)) * nb;
-            const double* cu = ext + ((int64_t)ix * pp + (ju - ix)) * pp;
-            const double* cv = ext + ((int64_t)iy * pp + (jv - iy)) * pp;
-            for (int iv = 0; iv < pp; ++iv) {
-                double row = 0.0;
-                for (int iu = 0; iu < pp; ++iu) row += cu[iu] * v[iv * pp + iu];
-                acc += cv[iv] * row;
-            }
-        }
+__host__ __device__ constexpr int restrict_lanes(int nb) { return nb <= 1 ? 1 : (nb <= 4 ? 4 : (nb <= 16 ? 16 : 32)); }
+
+// GROUP: G lanes per dof, added by shuffles (lane 0 forms the tree's root).  A single
+// thread's chain over up to 25 elements takes some 30 us (p = 3), which a short vector
+// cannot hide.
+template <int PP, bool GROUP>
+__global__ void __launch_bounds__(128) restrict_kernel(int64_t n, int64_t N, int ne1, const double* __restrict__ ext,
+                                                       const double* __restrict__ ys, int64_t E, double* __restrict__ y) {
+    constexpr int G = restrict_lanes(PP * PP);
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, idx = GROUP ? g / G : g;
+    const int n1 = ne1 + PP - 1;
+    const int64_t at = idx < n ? idx : n - 1, r = at / N, dof = at % N;
+    const int patch = (int)(dof / ((int64_t)n1 * n1)), rem = (int)(dof % ((int64_t)n1 * n1));
+    const int jv = rem / n1, ju = rem % n1;
+    const int64_t row = r * E + patch * (int64_t)ne1 * ne1;
+    double acc;
+    if constexpr (GROUP) {
+        acc = restrict_share<PP>((int)(g % G), ju, jv, row, ne1, ext, ys);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    } else {
+        double s[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) s[k] = restrict_share<PP>(k, ju, jv, row, ne1, ext, ys);
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < o; ++k) s[k] += s[k + o];
+        acc = s[0];
     }
-    for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (idx < R * N && k == 0) y[idx] = acc;
+    if (idx < n && (!GROUP || g % G == 0)) y[idx] = acc;
 }
 
-// y = T ys for R real vectors.  Up to some 8 threads per lane of the chip the grouped
-// form is as fast as its launch (p = 3, level 5: 33 -> 10 us); beyond, its idle lanes
-// (7 of 16 at p = 2) would cost more than the chain.
-void launch_restrict(ibem_handle* h, int R, const double* ys, double* y) {
+template <int PP>
+static void launch_restrict_pp(ibem_handle* h, int64_t n, const double* ys, double* y) {
     const Plan& P = h->P;
-    int G = 1;
-    while (G < P.nb) G <<= 1;
-    const int64_t n = (int64_t)R * P.N;
-    if (n * G <= (int64_t)152 * 2048 * 8)
-        restrict_group_kernel<<<nblk(n * G, 128), 128, 0, h->stream>>>(R, P.N, P.p, P.ne1, G, h->d_ext, ys, P.E, y);
+    constexpr int G = restrict_lanes(PP * PP);
+    // groups while one wave of the chip's threads holds them; beyond, the idle lanes (7 of 16
+    // at p = 2) cost more than the chain
+    if (n * G <= (int64_t)152 * 2048)
+        restrict_kernel<PP, true><<<nblk(n * G, 128), 128, 0, h->stream>>>(n, P.N, P.ne1, h->d_ext, ys, P.E, y);
     else
-        restrict_kernel<<<nblk(n, 256), 256, 0, h->stream>>>(R, P.N, P.p, P.ne1, h->d_ext, ys, P.E, y);
+        restrict_kernel<PP, false><<<nblk(n, 128), 128, 0, h->stream>>>(n, P.N, P.ne1, h->d_ext, ys, P.E, y);
+}
+
+// y = T ys for R real vectors
+void launch_restrict(ibem_handle* h, int R, const double* ys, double* y) {
+    const int64_t n = (int64_t)R * h->P.N;
+    switch (h->P.pp) {
+        case 1: launch_restrict_pp<1>(h, n, ys, y); break;
+        case 2: launch_restrict_pp<2>(h, n, ys, y); break;
+        case 3: launch_restrict_pp<3>(h, n, ys, y); break;
+        case 4: launch_restrict_pp<4>(h, n, ys, y); break;
+        default: launch_restrict_pp<5>(h, n, ys, y);
+    }
     h->launches++;
 }
 
