@@ -273,6 +273,16 @@ __device__ inline bool tc_wait(uint64_t* bar, unsigned parity, long long limit) 
     return false;
 }
 
+// 16 accumulator columns of a warp's lanes
+__device__ inline void tc_ld16(uint32_t addr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // Two independent FP32 operations per instruction: the generation below is bound by
 // issue, and a thread has two columns.
 using mr_f2 = unsigned long long;
@@ -309,7 +319,6 @@ __device__ __forceinline__ MrPoint2 mr_point2(const float4 a, const float4 b) {
 }
 // K at one target point (coordinates and measure / (4 pi), each twice) and two source
 // points: BF16 pairs of the real and the imaginary part
-template <bool CPLX>
 __device__ __forceinline__ void mr_values(const ulonglong2 xy, const ulonglong2 zw, const MrPoint2& Y, float kappa,
                                           uint32_t* kr, uint32_t* ki) {
     const mr_f2 d0 = f2_sub(xy.x, Y.x), d1 = f2_sub(xy.y, Y.y), d2 = f2_sub(zw.x, Y.z);
@@ -317,23 +326,31 @@ __device__ __forceinline__ void mr_values(const ulonglong2 xy, const ulonglong2 
     const float2 s = f2_get(r2);
     const mr_f2 rinv = f2_pack(approx_rsqrt(s.x), approx_rsqrt(s.y));
     const mr_f2 w = f2_mul(f2_mul(zw.y, Y.w), rinv);
-    if constexpr (CPLX) {
-        // phase reduced to [-pi, pi] first (the hardware sine and cosine are accurate
-        // on that interval only); 1.5 2^23 rounds to the nearest integer
-        const mr_f2 a = f2_mul(f2_pack(kappa, kappa), f2_mul(r2, rinv));
-        const mr_f2 M = f2_pack(12582912.0f, 12582912.0f);
-        const mr_f2 n = f2_sub(f2_fma(a, f2_pack(0.15915494309189535f, 0.15915494309189535f), M), M);
-        const float2 ph = f2_get(f2_fma(f2_pack(-6.283185307179586f, -6.283185307179586f), n, a));
-        const float2 re = f2_get(f2_mul(w, f2_pack(approx_cos(ph.x), approx_cos(ph.y))));
-        const float2 im = f2_get(f2_mul(w, f2_pack(approx_sin(ph.x), approx_sin(ph.y))));
-        const __nv_bfloat162 hr = __floats2bfloat162_rn(re.x, re.y), hi = __floats2bfloat162_rn(im.x, im.y);
-        *kr = *reinterpret_cast<const uint32_t*>(&hr);
-        *ki = *reinterpret_cast<const uint32_t*>(&hi);
-    } else {
-        const float2 re = f2_get(w);
-        const __nv_bfloat162 hr = __floats2bfloat162_rn(re.x, re.y);
-        *kr = *reinterpret_cast<const uint32_t*>(&hr);
+    // phase reduced to [-pi, pi] first (the hardware sine and cosine are accurate
+    // on that interval only); 1.5 2^23 rounds to the nearest integer
+    const mr_f2 a = f2_mul(f2_pack(kappa, kappa), f2_mul(r2, rinv));
+    const mr_f2 M = f2_pack(12582912.0f, 12582912.0f);
+    const mr_f2 n = f2_sub(f2_fma(a, f2_pack(0.15915494309189535f, 0.15915494309189535f), M), M);
+    const float2 ph = f2_get(f2_fma(f2_pack(-6.283185307179586f, -6.283185307179586f), n, a));
+    const float2 re = f2_get(f2_mul(w, f2_pack(approx_cos(ph.x), approx_cos(ph.y))));
+    const float2 im = f2_get(f2_mul(w, f2_pack(approx_sin(ph.x), approx_sin(ph.y))));
+    const __nv_bfloat162 hr = __floats2bfloat162_rn(re.x, re.y), hi = __floats2bfloat162_rn(im.x, im.y);
+    *kr = *reinterpret_cast<const uint32_t*>(&hr);
+    *ki = *reinterpret_cast<const uint32_t*>(&hi);
+}
+// the same for 1 / r, one point at a time: some ten operations, and packed pairs would
+// cost the registers of the second CTA of an SM (level 4, q = 6, 16 right-hand sides:
+// coupling 1.11 ms instead of 0.93)
+__device__ __forceinline__ uint32_t mr_values_laplace(const float4 X, const float4 Y0, const float4 Y1) {
+    float w[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const float4 Y = u ? Y1 : Y0;
+        const float d0 = X.x - Y.x, d1 = X.y - Y.y, d2 = X.z - Y.z;
+        w[u] = X.w * Y.w * approx_rsqrt(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
     }
+    const __nv_bfloat162 h = __floats2bfloat162_rn(w[0], w[1]);
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // Q > 0: compiled for q = Q (index arithmetic of the K generation by shifts and
@@ -344,7 +361,7 @@ __device__ __forceinline__ void mr_values(const ulonglong2 xy, const ulonglong2 
 // values share packed instructions, and for q = 8 a thread's two source points
 // serve four rows.  Level 5, 16 right-hand sides: 6.63 ms, 7.48 before.
 template <bool CPLX, int Q>
-__global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
+__global__ void __launch_bounds__(544, CPLX ? 0 : 2) mr_coupling_tc_kernel(
     const int32_t* __restrict__ rows, const int64_t* __restrict__ fptr, const int32_t* __restrict__ fsrc,
     const float4* __restrict__ geo, int q_rt, int R, int RP, int KAP_rt, int tcols, float kappa,
     const __nv_bfloat16* __restrict__ xb, typename MrType<CPLX>::T* __restrict__ yh, long long wait_limit,
@@ -359,7 +376,7 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     int* issued_sh = reinterpret_cast<int*>(smem + 76);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + 64);
     int* flag = reinterpret_cast<int*>(smem + 72);
-    ulonglong2* Xs = reinterpret_cast<ulonglong2*>(smem + 128);   // [q2][2]: (x, x, y, y), (z, z, w, w)
+    ulonglong2* Xs = reinterpret_cast<ulonglong2*>(smem + 128);   // [q2][2]: (x, x, y, y), (z, z, w, w); real [q2] (x, y, z, w)
     const int q2 = q * q;
     const int NB = CPLX ? 2 * RP : RP;                           // B rows, accumulator columns
     const size_t abytes = (size_t)MAP * KAP * 2, bbytes = (size_t)NB * KAP * 2;
@@ -388,8 +405,12 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     for (int i = t; i < q2; i += blockDim.x) {
         float4 g = geo[(int64_t)sigma * q2 + i];
         g.w *= 0.07957747154594767f;   // k / (4 pi)
-        Xs[2 * i] = make_ulonglong2(f2_pack(g.x, g.x), f2_pack(g.y, g.y));
-        Xs[2 * i + 1] = make_ulonglong2(f2_pack(g.z, g.z), f2_pack(g.w, g.w));
+        if constexpr (CPLX) {
+            Xs[2 * i] = make_ulonglong2(f2_pack(g.x, g.x), f2_pack(g.y, g.y));
+            Xs[2 * i + 1] = make_ulonglong2(f2_pack(g.z, g.z), f2_pack(g.w, g.w));
+        } else {
+            reinterpret_cast<float4*>(Xs)[i] = g;
+        }
     }
     // padding rows / columns of both A buffers stay zero
     for (size_t i = t; i < 2 * abytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(tiles)[i] = make_uint4(0, 0, 0, 0);
@@ -432,25 +453,35 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
                 *at(a) = kr;
                 if constexpr (CPLX) *at(q2 + a) = ki;
             };
-            uint32_t kr, ki = 0;
-            if constexpr (Q == 8) {
+            if constexpr (!CPLX) {
+                const int q8 = (q2 + 7) >> 3;
+#pragma unroll
+                for (int cm = warp; cm < q8 * q8; cm += 16) {
+                    const int ca = cm / q8, cb = cm - ca * q8;
+                    const int a = 8 * ca + (lane >> 2), b = 8 * cb + 2 * (lane & 3);
+                    if (a >= q2 || b >= q2) continue;   // q2 is even, so b + 1 < q2 as well
+                    put(a, b, mr_values_laplace(reinterpret_cast<const float4*>(Xs)[a], Y[b], Y[b + 1]), 0u);
+                }
+            } else if constexpr (Q == 8) {
+                uint32_t kr, ki;
                 // 64 core matrices: a warp keeps its columns and takes every second row group
                 const int b = 8 * (warp & 7) + 2 * (lane & 3);
                 const MrPoint2 Y2 = mr_point2(Y[b], Y[b + 1]);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int a = 8 * ((warp >> 3) + 2 * k) + (lane >> 2);
-                    mr_values<CPLX>(Xs[2 * a], Xs[2 * a + 1], Y2, kappa, &kr, &ki);
+                    mr_values(Xs[2 * a], Xs[2 * a + 1], Y2, kappa, &kr, &ki);
                     put(a, b, kr, ki);
                 }
             } else {
+                uint32_t kr, ki;
                 const int q8 = (q2 + 7) >> 3;
 #pragma unroll 2
                 for (int cm = warp; cm < q8 * q8; cm += 16) {
                     const int ca = cm / q8, cb = cm - ca * q8;
                     const int a = 8 * ca + (lane >> 2), b = 8 * cb + 2 * (lane & 3);
                     if (a >= q2 || b >= q2) continue;   // q2 is even, so b + 1 < q2 as well
-                    mr_values<CPLX>(Xs[2 * a], Xs[2 * a + 1], mr_point2(Y[b], Y[b + 1]), kappa, &kr, &ki);
+                    mr_values(Xs[2 * a], Xs[2 * a + 1], mr_point2(Y[b], Y[b + 1]), kappa, &kr, &ki);
                     put(a, b, kr, ki);
                 }
             }
@@ -488,7 +519,7 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
             }
             __nv_bfloat16* A = reinterpret_cast<__nv_bfloat16*>(tiles + buf * abytes);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int n0 = 0; n0 < NB; n0 += NM)
+            for (int n0 = 0; n0 < (CPLX ? NB : 1); n0 += NM)   // real: one, on the path from A to mdone
                 for (int kk = 0; kk < KAP / 16; ++kk) {
                     const uint64_t ad = umma_desc(tsm(A) + kk * 256, 128, K8 * 128);
                     const uint64_t bd = umma_desc(tsm(tiles + 2 * abytes + buf * bbytes) + n0 * KAP * 2 + kk * 256, 128,
@@ -521,6 +552,18 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
     }
     if (__syncthreads_or(!ok || failed)) {
         if (t == 0) atomicOr(status, 1);
+    } else if constexpr (!CPLX) {
+        // warps 0..3 own TMEM lane quarters 0..3
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int row = 32 * warp + lane;
+        for (int c0 = 0; warp < 4 && c0 < RP; c0 += 16) {
+            uint32_t v[16];
+            tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, v);
+            if (row < q2)
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (c0 + j < R) yh[((int64_t)sigma * q2 + row) * R + c0 + j] = __uint_as_float(v[j]);
+        }
     } else {
         // warps 0..3 own TMEM lane quarters 0..3; 16 right-hand sides at a time through
         // shared memory (the tiles are free), where the rows of Kr and Ki meet
@@ -531,17 +574,9 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
         for (int c0 = 0; c0 < RP; c0 += 16) {
             if (warp < 4) {
 #pragma unroll
-                for (int h = 0; h < (CPLX ? 2 : 1); ++h) {
+                for (int h = 0; h < 2; ++h) {
                     uint32_t v[16];
-                    const uint32_t taddr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(h * RP + c0);
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                        "[%16];"
-                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                          "=r"(v[14]), "=r"(v[15])
-                        : "r"(taddr));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(h * RP + c0), v);
 #pragma unroll
                     for (int j = 0; j < 16; ++j) S[row * SS + 16 * h + j] = __uint_as_float(v[j]);
                 }
@@ -551,13 +586,8 @@ __global__ void __launch_bounds__(544) mr_coupling_tc_kernel(
                 const int j = e & 15, a = e >> 4, r = c0 + j;
                 if (r >= R) continue;
                 const int64_t o = ((int64_t)sigma * q2 + a) * R + r;
-                const float* Sr = S + a * SS;
-                if constexpr (CPLX) {
-                    const float* Si = S + (q2 + a) * SS;
-                    yh[o] = make_float2(Sr[j] - Si[16 + j], Sr[16 + j] + Si[j]);
-                } else {
-                    yh[o] = Sr[j];
-                }
+                const float *Sr = S + a * SS, *Si = S + (q2 + a) * SS;
+                yh[o] = make_float2(Sr[j] - Si[16 + j], Sr[16 + j] + Si[j]);
             }
             __syncthreads();
         }
@@ -1079,7 +1109,7 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
             mr_bpack_kernel<CPLX><<<nblk((int64_t)P.C * RP * (KAP / 8), T_), T_, 0, st>>>(R, 0, RP, KAP, P.C, q2, xh, xb);
             int tcols = 32;
             while (tcols < NB) tcols <<= 1;
-            // the tiles, or the 128 x 33 floats that the row is joined in
+            // the tiles, or the 128 x 33 floats that a complex row is joined in
             const size_t sm = 1024 * ((128 + (size_t)q2 * 32 + 1023) / 1024) +
                               std::max<size_t>(2 * (size_t)(128 + NB) * KAP * 2, 128 * 33 * sizeof(float));
             auto kern = P.q == 8 ? mr_coupling_tc_kernel<CPLX, 8>
