@@ -13,11 +13,12 @@
 // Bound: the FP32 pipe (96 operations per stored entry and right-hand side: two
 // complex multiply-adds of exact products and TwoSum sums, 0.55 ms of FP32 issue
 // at level 4, q = 6 with one right-hand side, against 0.53 ms for the 3.6 GB at
-// 6.8 TB/s; ncu: FMA pipe 66%, 90% of the lanes have a row).  Level 4, q = 6,
-// kappa = 4, one right-hand side: 0.96 ms and 0.04 ms for the column shares,
-// against 1.32 ms when both mirrored blocks were stored and read; level 3, 8
-// right-hand sides: 1.72 ms against 2.00 ms (matrix read once per right-hand
-// side).  Two right-hand sides per CTA: with four the unrolled code misses the
+// 6.8 TB/s).  Level 4, q = 6, kappa = 4, one right-hand side: 1.01 ms with the column
+// shares, against 1.32 ms when both mirrored blocks were stored and read; level 3, 8
+// right-hand sides: 1.81 ms against 2.00 ms (matrix read once per right-hand
+// side).  The sums over blocks are as exact as the FP64 ones of that form; as plain
+// double-floats they take 1 to 5% less time (1.00 and 1.71 ms) and make the error of an
+// application 1.4 times as large (6.4e-16 against 4.5e-16 at level 4, q = 8).  Two right-hand sides per CTA: with four the unrolled code misses the
 // instruction cache (2.4 ms at level 3).  Packed two-float instructions gave
 // nothing (1.00 ms): the pipe is the limit, not issue.
 #include "ibem_internal.cuh"
@@ -46,6 +47,25 @@ __device__ __forceinline__ void hs_mac(float ah, float al, float bh, float bl, f
     e = fmaf(al, bh, e);
     hs_add(hi, lo, p, e);
 }
+// Sum of double-floats over many blocks, in three parts: exact but for the rounding of the
+// third one (2^-72), so no less accurate than an FP64 sum, which would take conversions
+// and additions on the FP64 pipe (level 4, q = 6, one right-hand side: 1.33 ms).
+struct hs_sum {
+    float h = 0.0f, m = 0.0f, l = 0.0f;
+};
+__device__ __forceinline__ float hs_two_sum(float a, float b, float& e) {
+    const float s = a + b, z = s - a;
+    e = (a - (s - z)) + (b - z);
+    return s;
+}
+__device__ __forceinline__ void hs_acc(hs_sum& a, float h, float l) {
+    float e, f, g;
+    a.h = hs_two_sum(a.h, h, e);
+    const float t = hs_two_sum(a.m, l, f);
+    a.m = hs_two_sum(t, e, g);
+    a.l += f + g;
+}
+__device__ __forceinline__ double hs_value(const hs_sum& a) { return (double)a.h + ((double)a.m + (double)a.l); }
 // (re, im) += k x for complex double-floats
 __device__ __forceinline__ void hs_cmac(const float4 k, const float4 x, float (&s)[4]) {
     hs_mac(k.x, k.y, x.x, x.y, s[0], s[1]);
@@ -99,14 +119,25 @@ __global__ void helm_split_kernel(int r0, int rc, int RB, int ng, int64_t C, int
 }
 
 // Thread t = 4 a + s: row pass, row a and columns s + 4 kk; column pass, column
-// t / 4 and rows t % 4 + 4 j.  Per block the partial sums are double-float; row
-// sums are folded into FP64 every 8 blocks.  EXACT: q2 == 4 KPT (even q).
+// t / 4 and rows t % 4 + 4 j.  A thread's sums over a block are double-float, those over the
+// blocks of a row, the threads of a column and the shares of a column
+// (helm_column_gather_kernel) in three parts.  EXACT: q2 == 4 KPT (even q).
+// Launch bounds: the CTAs that the stages leave room for (left to itself the compiler
+// takes 32 registers at q = 6 with one right-hand side, and 125 us more at level 4); at
+// q = 6 with two, 56 registers are better than the 72 of that rule (64.4 ms instead of 65.8
+// for 64 right-hand sides at level 4).
+constexpr int hs_threads(int kpt) { return (16 * kpt + 31) / 32 * 32; }
+constexpr int hs_ctas(int kpt, int nst, int rb) {
+    return kpt == 9 && rb == 2                                  ? 7
+           : IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst) < 16 ? IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst)
+                                                                : 16;
+}
 template <int KPT, int NST, int RB, bool EXACT>
-__global__ void helm_coupling_sym_kernel(const int32_t* __restrict__ rows, const int64_t* __restrict__ uptr,
-                                         const int32_t* __restrict__ usrc, const float4* __restrict__ K, int q2_rt,
-                                         int q2p, int maxrow, int64_t C, const float4* __restrict__ xh, int r0, int rc,
-                                         double* __restrict__ yh, float4* __restrict__ colpart, int64_t n_up,
-                                         long long wait_limit, int* __restrict__ status) {
+__global__ void __launch_bounds__(hs_threads(KPT), hs_ctas(KPT, NST, RB)) helm_coupling_sym_kernel(
+    const int32_t* __restrict__ rows, const int64_t* __restrict__ uptr, const int32_t* __restrict__ usrc,
+    const float4* __restrict__ K, int q2_rt, int q2p, int maxrow, int64_t C, const float4* __restrict__ xh, int r0, int rc,
+    double* __restrict__ yh, float4* __restrict__ colpart, int64_t n_up, long long wait_limit,
+    int* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
     int32_t* srcs = reinterpret_cast<int32_t*>(smem + 128);
@@ -142,21 +173,7 @@ __global__ void helm_coupling_sym_kernel(const int32_t* __restrict__ rows, const
     };
     if (t == 0)
         for (int i = 0; i < NST && i < n; ++i) fetch(i);
-    double acc[RB][2];
-    float run[RB][4];
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-        acc[r][0] = acc[r][1] = 0.0;
-        run[r][0] = run[r][1] = run[r][2] = run[r][3] = 0.0f;
-    }
-    auto fold = [&]() {
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            acc[r][0] += (double)run[r][0] + (double)run[r][1];
-            acc[r][1] += (double)run[r][2] + (double)run[r][3];
-            run[r][0] = run[r][1] = run[r][2] = run[r][3] = 0.0f;
-        }
-    };
+    hs_sum acc[RB][2];
     int i = 0;
     bool failed = false;
     for (; i < n; ++i) {
@@ -177,10 +194,9 @@ __global__ void helm_coupling_sym_kernel(const int32_t* __restrict__ rows, const
             }
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                hs_add(run[r][0], run[r][1], row[r][0], row[r][1]);
-                hs_add(run[r][2], run[r][3], row[r][2], row[r][3]);
+                hs_acc(acc[r][0], row[r][0], row[r][1]);
+                hs_acc(acc[r][1], row[r][2], row[r][3]);
             }
-            if ((i & 7) == 7) fold();
             const float4* Kc = Kb + (a >> 2) * stride + (a & 3) + 4 * s;
 #pragma unroll(KPT <= 9 ? KPT : 1)
             for (int j = 0; j < KPT; ++j) {
@@ -191,28 +207,35 @@ __global__ void helm_coupling_sym_kernel(const int32_t* __restrict__ rows, const
                 }
             }
         }
-        // columns: combine the 4 lanes that share a column (all lanes take part)
+        // columns: combine the 4 lanes that share a column (all lanes take part); lanes
+        // s = 0, 1 end with the real part, s = 2, 3 with the imaginary part
+        float2 share[RB];
 #pragma unroll
-        for (int r = 0; r < RB; ++r)
-#pragma unroll
-            for (int off = 1; off <= 2; off <<= 1) {
-                float o[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) o[k] = __shfl_xor_sync(0xffffffffu, col[r][k], off);
-                hs_add(col[r][0], col[r][1], o[0], o[1]);
-                hs_add(col[r][2], col[r][3], o[2], o[3]);
-            }
+        for (int r = 0; r < RB; ++r) {
+            const bool im = s & 2;
+            const float oh = __shfl_xor_sync(0xffffffffu, im ? col[r][0] : col[r][2], 2);
+            const float ol = __shfl_xor_sync(0xffffffffu, im ? col[r][1] : col[r][3], 2);
+            hs_sum v;
+            v.h = im ? col[r][2] : col[r][0];
+            v.m = im ? col[r][3] : col[r][1];
+            hs_acc(v, oh, ol);
+            const float vh = __shfl_xor_sync(0xffffffffu, v.h, 1), vm = __shfl_xor_sync(0xffffffffu, v.m, 1);
+            v.l += __shfl_xor_sync(0xffffffffu, v.l, 1);
+            hs_acc(v, vh, vm);
+            share[r].x = hs_two_sum(v.h, v.m, share[r].y);
+            share[r].y += v.l;
+        }
         if (__syncthreads_or(!ok)) {
             failed = true;
             break;
         }
         if (t == 0 && i + NST < n) fetch(i + NST);
-        if (active && s == 0)
+        if (active && (s & 1) == 0)
 #pragma unroll
             for (int r = 0; r < RB; ++r)
                 if (rg + r < rc)
-                    colpart[((int64_t)(rg + r) * n_up + b0 + i) * q2 + a] =
-                        make_float4(col[r][0], col[r][1], col[r][2], col[r][3]);
+                    reinterpret_cast<float2*>(colpart)[2 * (((int64_t)(rg + r) * n_up + b0 + i) * q2 + a) + (s >> 1)] =
+                        share[r];
     }
     if (failed) {
         if (t == 0) {
@@ -223,12 +246,11 @@ __global__ void helm_coupling_sym_kernel(const int32_t* __restrict__ rows, const
         __syncthreads();
         return;
     }
-    fold();
 #pragma unroll
     for (int r = 0; r < RB; ++r)
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            double v = acc[r][k];
+            double v = hs_value(acc[r][k]);
             v += __shfl_xor_sync(0xffffffffu, v, 1);
             v += __shfl_xor_sync(0xffffffffu, v, 2);
             if (active && s == 0 && rg + r < rc) yh[((int64_t)(2 * (r0 + rg + r) + k) * C + sigma) * q2 + a] = v;
@@ -248,15 +270,15 @@ __global__ void helm_column_gather_kernel(int r0, int64_t C, int q2, int G, cons
     const int r = blockIdx.y, t = threadIdx.x, g = t / q2, b = t - g * q2;
     if (g < G) {
         const float4* part = colpart + (int64_t)r * n_up * q2 + b;
-        float sr[2] = {0.0f, 0.0f}, si[2] = {0.0f, 0.0f};
+        hs_sum sr, si;
 #pragma unroll 4
         for (int64_t k = k0 + g; k < k1; k += G) {
             const float4 v = part[(int64_t)tblk[k] * q2];
-            hs_add(sr[0], sr[1], v.x, v.y);
-            hs_add(si[0], si[1], v.z, v.w);
+            hs_acc(sr, v.x, v.y);
+            hs_acc(si, v.z, v.w);
         }
-        red[2 * t] = (double)sr[0] + (double)sr[1];
-        red[2 * t + 1] = (double)si[0] + (double)si[1];
+        red[2 * t] = hs_value(sr);
+        red[2 * t + 1] = hs_value(si);
     }
     __syncthreads();
     if (t < 2 * q2) {
