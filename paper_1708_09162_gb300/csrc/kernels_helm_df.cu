@@ -21,6 +21,8 @@
 // application 1.4 times as large (6.4e-16 against 4.5e-16 at level 4, q = 8).  Two right-hand sides per CTA: with four the unrolled code misses the
 // instruction cache (2.4 ms at level 3).  Packed two-float instructions gave
 // nothing (1.00 ms): the pipe is the limit, not issue.
+#include <algorithm>
+
 #include "ibem_internal.cuh"
 
 namespace ibem {
@@ -29,8 +31,23 @@ namespace {
 
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-constexpr int HS_RC = 8;     // right-hand sides per pass (bounds the column shares)
+constexpr int HS_RC = 8;     // right-hand sides per pass at least
 constexpr int HS_RB = 2;     // right-hand sides per CTA at most
+constexpr int64_t HS_SHARES = (int64_t)256 << 20;   // bytes of column shares beyond which a pass takes no more than HS_RC
+
+// Most right-hand sides per pass.  A pass holds the column shares of its right-hand
+// sides (q^2 float4 per stored block and right-hand side), so on large trees eight;
+// on small ones, which eight do not fill (level 2, q = 4, 64 right-hand sides: 8
+// passes took 435 us, one 256), all that fit.
+int hs_most(const ibem_handle* h) {
+    const int64_t per = (h->n_up > 0 ? h->n_up : 1) * (int64_t)h->P.q2 * (int64_t)sizeof(float4);
+    return (int)std::min<int64_t>(1 << 20, std::max<int64_t>(HS_RC, HS_SHARES / per / 2 * 2));
+}
+// passes of equal size up to a pair
+int hs_pass(const ibem_handle* h, int R) {
+    const int n = (R + hs_most(h) - 1) / hs_most(h);
+    return std::min(R, ((R + n - 1) / n + 1) / 2 * 2);
+}
 
 __device__ __forceinline__ void hs_add(float& hi, float& lo, float h2, float l2) {
     const float s = hi + h2;
@@ -123,17 +140,13 @@ __global__ void helm_split_kernel(int r0, int rc, int RB, int ng, int64_t C, int
 // blocks of a row, the threads of a column and the shares of a column
 // (helm_column_gather_kernel) in three parts.  EXACT: q2 == 4 KPT (even q).
 // Launch bounds: the CTAs that the stages leave room for (left to itself the compiler
-// takes 32 registers at q = 6 with one right-hand side, and 125 us more at level 4); at
-// q = 6 with two, 56 registers are better than the 72 of that rule (64.4 ms instead of 65.8
-// for 64 right-hand sides at level 4).
+// takes 32 registers at q = 6 with one right-hand side, and 125 us more at level 4).
 constexpr int hs_threads(int kpt) { return (16 * kpt + 31) / 32 * 32; }
-constexpr int hs_ctas(int kpt, int nst, int rb) {
-    return kpt == 9 && rb == 2                                  ? 7
-           : IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst) < 16 ? IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst)
-                                                                : 16;
+constexpr int hs_ctas(int kpt, int nst) {
+    return IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst) < 16 ? IBEM_MAX_SMEM_BYTES / (256 * kpt * kpt * nst) : 16;
 }
 template <int KPT, int NST, int RB, bool EXACT>
-__global__ void __launch_bounds__(hs_threads(KPT), hs_ctas(KPT, NST, RB)) helm_coupling_sym_kernel(
+__global__ void __launch_bounds__(hs_threads(KPT), hs_ctas(KPT, NST)) helm_coupling_sym_kernel(
     const int32_t* __restrict__ rows, const int64_t* __restrict__ uptr, const int32_t* __restrict__ usrc,
     const float4* __restrict__ K, int q2_rt, int q2p, int maxrow, int64_t C, const float4* __restrict__ xh, int r0, int rc,
     double* __restrict__ yh, float4* __restrict__ colpart, int64_t n_up, long long wait_limit,
@@ -290,7 +303,7 @@ __global__ void helm_column_gather_kernel(int r0, int64_t C, int q2, int G, cons
 }
 
 template <int KPT, int NST, int RB>
-cudaError_t launch_sym(ibem_handle* h, int r0, int rc, int ng) {
+cudaError_t launch_sym(ibem_handle* h, int r0, int rc, int ng, const float4* xh, float4* col) {
     constexpr bool EXACT = KPT == 1 || KPT == 4 || KPT == 9 || KPT == 16 || KPT == 25;
     const Plan& P = h->P;
     const int q2 = P.q2, q2p = (q2 + 1) & ~1;
@@ -302,15 +315,38 @@ cudaError_t launch_sym(ibem_handle* h, int r0, int rc, int ng) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
     kern<<<dim3((unsigned)h->up_rows.size(), (unsigned)ng), threads, sm, h->stream>>>(
-        h->d_up_rows, h->d_up_ptr, h->d_up_src, h->d_Kc, q2, q2p, h->max_up_row, P.C, h->d_xh4, r0, rc, h->d_yh,
-        h->d_hcol, h->n_up, h->wait_limit, h->d_status);
+        h->d_up_rows, h->d_up_ptr, h->d_up_src, h->d_Kc, q2, q2p, h->max_up_row, P.C, xh, r0, rc, h->d_yh, col,
+        h->n_up, h->wait_limit, h->d_status);
     h->launches++;
     return cudaGetLastError();
 }
 
 template <int KPT, int NST>
-cudaError_t launch_sym_rb(ibem_handle* h, int r0, int rc, int ng, int RB) {
-    return RB == 1 ? launch_sym<KPT, NST, 1>(h, r0, rc, ng) : launch_sym<KPT, NST, 2>(h, r0, rc, ng);
+cudaError_t launch_sym_rb(ibem_handle* h, int r0, int rc, int RB, const float4* xh, float4* col) {
+    return RB == 1 ? launch_sym<KPT, NST, 1>(h, r0, rc, rc, xh, col)
+                   : launch_sym<KPT, NST, 2>(h, r0, rc, (rc + 1) / 2, xh, col);
+}
+
+// rc right-hand sides from r0 in groups of RB (the last one padded): moments to xh, row
+// sums, column shares to col
+cudaError_t launch_groups(ibem_handle* h, int r0, int rc, int RB, float4* xh, float4* col) {
+    const Plan& P = h->P;
+    const int q2p = (P.q2 + 1) & ~1, ng = (rc + RB - 1) / RB, T = 256;
+    helm_split_kernel<<<nblk((int64_t)ng * P.C * RB * q2p, T), T, 0, h->stream>>>(r0, rc, RB, ng, P.C, P.q2, q2p,
+                                                                                  h->d_xh, xh);
+    h->launches++;
+    switch (h->kpt) {
+        case 1: return launch_sym_rb<1, 8>(h, r0, rc, RB, xh, col);
+        case 3: return launch_sym_rb<3, 6>(h, r0, rc, RB, xh, col);
+        case 4: return launch_sym_rb<4, 4>(h, r0, rc, RB, xh, col);
+        case 7: return launch_sym_rb<7, 3>(h, r0, rc, RB, xh, col);
+        case 9: return launch_sym_rb<9, 2>(h, r0, rc, RB, xh, col);
+        case 13: return launch_sym_rb<13, 2>(h, r0, rc, RB, xh, col);
+        case 16: return launch_sym_rb<16, 2>(h, r0, rc, RB, xh, col);
+        case 21: return launch_sym_rb<21, 1>(h, r0, rc, RB, xh, col);
+        case 25: return launch_sym_rb<25, 1>(h, r0, rc, RB, xh, col);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace
@@ -319,7 +355,7 @@ cudaError_t launch_sym_rb(ibem_handle* h, int r0, int rc, int ng, int RB) {
 // column shares of one pass.  Sized with the other work vectors (ensure_workspace), not
 // in the application, which a program may record into a graph.
 cudaError_t ensure_helm_df(ibem_handle* h, int R) {
-    const int rc = R < HS_RC ? R : HS_RC;
+    const int rc = std::min(R, hs_most(h));
     if (rc <= h->hdf_rhs) return cudaSuccess;
     const Plan& P = h->P;
     cudaFree(h->d_xh4);
@@ -328,8 +364,7 @@ cudaError_t ensure_helm_df(ibem_handle* h, int R) {
     h->d_hcol = nullptr;
     h->hdf_rhs = 0;
     cudaError_t e;
-    // groups of RB right-hand sides pad a pass by at most one group
-    if ((e = cudaMalloc(&h->d_xh4, (size_t)(rc + HS_RB) * P.C * ((P.q2 + 1) & ~1) * sizeof(float4)))) return e;
+    if ((e = cudaMalloc(&h->d_xh4, (size_t)(rc + 1) * P.C * ((P.q2 + 1) & ~1) * sizeof(float4)))) return e;
     if ((e = cudaMalloc(&h->d_hcol, (size_t)rc * (h->n_up > 0 ? h->n_up : 1) * P.q2 * sizeof(float4)))) return e;
     h->hdf_rhs = rc;
     return cudaSuccess;
@@ -339,28 +374,19 @@ cudaError_t launch_helm_coupling_df(ibem_handle* h, int R) {
     const Plan& P = h->P;
     cudaStream_t st = h->stream;
     cudaError_t e;
-    const int q2 = P.q2, q2p = (q2 + 1) & ~1, T = 256;
+    const int q2 = P.q2, q2p = (q2 + 1) & ~1, pass = hs_pass(h, R);
     if (h->up_rows.empty()) return cudaSuccess;
-    for (int r0 = 0; r0 < R; r0 += HS_RC) {
-        const int rc = R - r0 < HS_RC ? R - r0 : HS_RC;
-        // groups of equal size: at most one padded right-hand side each
-        const int ng = (rc + HS_RB - 1) / HS_RB, RB = (rc + ng - 1) / ng;
-        helm_split_kernel<<<nblk((int64_t)ng * P.C * RB * q2p, T), T, 0, st>>>(r0, rc, RB, ng, P.C, q2, q2p, h->d_xh,
-                                                                               h->d_xh4);
-        h->launches++;
-        switch (h->kpt) {
-            case 1: e = launch_sym_rb<1, 8>(h, r0, rc, ng, RB); break;
-            case 3: e = launch_sym_rb<3, 6>(h, r0, rc, ng, RB); break;
-            case 4: e = launch_sym_rb<4, 4>(h, r0, rc, ng, RB); break;
-            case 7: e = launch_sym_rb<7, 3>(h, r0, rc, ng, RB); break;
-            case 9: e = launch_sym_rb<9, 2>(h, r0, rc, ng, RB); break;
-            case 13: e = launch_sym_rb<13, 2>(h, r0, rc, ng, RB); break;
-            case 16: e = launch_sym_rb<16, 2>(h, r0, rc, ng, RB); break;
-            case 21: e = launch_sym_rb<21, 1>(h, r0, rc, ng, RB); break;
-            case 25: e = launch_sym_rb<25, 1>(h, r0, rc, ng, RB); break;
-            default: e = cudaErrorInvalidValue;
-        }
-        if (e) return e;
+    for (int r0 = 0; r0 < R; r0 += pass) {
+        const int rc = R - r0 < pass ? R - r0 : pass;
+        // pairs, and an odd one by itself (as half of a pair it takes twice the time: level 4, q = 6,
+        // three right-hand sides 4.27 ms, now 3.48), unless the launch is too small to fill
+        // the chip and one more costs more
+        const bool tiny = (int64_t)h->up_rows.size() * ((rc + 1) / 2) <= 2 * 152;
+        const int two = tiny && rc > 1 ? rc : rc / HS_RB * HS_RB;
+        if (two > 0 && (e = launch_groups(h, r0, two, HS_RB, h->d_xh4, h->d_hcol))) return e;
+        if (two < rc && (e = launch_groups(h, r0 + two, 1, 1, h->d_xh4 + (size_t)two * P.C * q2p,
+                                           h->d_hcol + (size_t)two * h->n_up * q2)))
+            return e;
         const int G = 256 / q2 > 0 ? 256 / q2 : 1;
         const int threads = ((G * q2 > 2 * q2 ? G * q2 : 2 * q2) + 31) / 32 * 32;
         helm_column_gather_kernel<<<dim3((unsigned)P.C, (unsigned)rc), threads, (size_t)2 * threads * sizeof(double), st>>>(

@@ -61,3 +61,20 @@ def test_right_hand_sides(kernel):
     for r0, n in ((0, 1), (5, 3), (23, 1)):
         assert torch.equal(rhs(g[r0:r0 + n].contiguous()), b[r0:r0 + n]), (r0, n)
     ibem.ibem_destroy(h)
+
+
+# passes of the stored Helmholtz coupling: one pass of all, pairs with one left over, and a
+# launch too small for that; fewer than four columns take another near product
+@pytest.mark.parametrize("p,m,q,R", [(1, 2, 4, 63), (0, 3, 6, 15)])
+def test_helmholtz_stored_far_field(p, m, q, R):
+    import torch
+    h = _handle(p, m, q, 1)
+    x = _vectors(1820 + R, R, lib().ibem_get_info(h).ndof, 2)
+    for n in (3, 2):
+        y = _apply(h, x[:n].contiguous())
+        for r in range(n):
+            assert torch.equal(_apply(h, x[r:r + 1].contiguous())[0], y[r]), (n, r)
+    y = _apply(h, x)
+    assert torch.equal(_apply(h, x), y)
+    assert float((_apply(h, x[:3].contiguous()) - y[:3]).abs().max()) < 1e-12 * float(y.abs().max())
+    lib().ibem_destroy(h)
