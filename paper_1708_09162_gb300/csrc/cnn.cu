@@ -561,15 +561,17 @@ __global__ void flip_weights_kernel(const float* __restrict__ w, int Cin, int Co
 // the FMA pipe bounds it (9 FMA per four reads before: 458 us for the four layers of
 // 96 images of 34 x 34, and 484 us for the bias sums in kernels of their own; now
 // 274 us for both).  part: [rows][Cout * Cin * 9 + Cout].
-template <typename T>
+// LOW: tiles of gh < TY rows, and no columns beyond the image
+template <typename T, bool LOW>
 __global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict__ g, const T* __restrict__ in, int B,
-                                                         int Cin, int H, int W, int Cout, int items_per_cta,
+                                                         int Cin, int H, int W, int Cout, int low, int items_per_cta,
                                                          float* __restrict__ part) {
     extern __shared__ __align__(16) float wg_sm[];
     float4* s_g = reinterpret_cast<float4*>(wg_sm);                    // [GP][8]: 4 channels each
     float* s_in = wg_sm + GP * 32;                                     // [32][TY + 2][GX + 2]
     constexpr int RW = GX + 2, PL = (TY + 2) * RW + 1;                 // odd plane stride: no bank conflicts over ci
-    const int tiles_x = (W + GX - 1) / GX, tiles = tiles_x * ((H + TY - 1) / TY);
+    const int gh = LOW ? low : TY;
+    const int tiles_x = (W + GX - 1) / GX, tiles = tiles_x * ((H + gh - 1) / gh);
     const int64_t HW = (int64_t)H * W;
     const int t = threadIdx.x, cq = t & 7, ci = t >> 3;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
@@ -585,14 +587,16 @@ __global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict
     for (int64_t item = it0; item < it1; ++item) {
         const int64_t b = item / tiles;
         const int tile = (int)(item % tiles);
-        const int ty0 = (tile / tiles_x) * TY, tx0 = (tile % tiles_x) * GX;
-        for (int i = t; i < 32 * GP; i += 256) {
-            const int o = i / GP, pix = i - o * GP, yy = ty0 + pix / GX, xx = tx0 + pix % GX;
+        const int ty0 = (tile / tiles_x) * gh, tx0 = (tile % tiles_x) * GX;
+        const int ny = LOW ? min(gh, H - ty0) : TY, nx = LOW ? min(GX, W - tx0) : GX, np = gh * GX;
+        for (int i = t; i < 32 * np; i += 256) {
+            const int o = i / np, pix = i - o * np, yy = ty0 + pix / GX, xx = tx0 + pix % GX;
             reinterpret_cast<float*>(s_g)[pix * 32 + o] =
                 (o < Cout && yy < H && xx < W) ? g[(b * Cout + o) * HW + (int64_t)yy * W + xx] : 0.0f;
         }
-        for (int i = t; i < Cin * (TY + 2) * RW; i += 256) {
-            const int c = i / ((TY + 2) * RW), r = i - c * (TY + 2) * RW;
+        const int rows = (gh + 2) * RW;
+        for (int i = t; i < Cin * rows; i += 256) {
+            const int c = i / rows, r = i - c * rows;
             const int yy = ty0 - 1 + r / RW, xx = tx0 - 1 + r % RW;
             float v = 0.0f;
             if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = ld_act(in, (b * Cin + c) * HW + (int64_t)yy * W + xx);
@@ -601,7 +605,7 @@ __global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict
         __syncthreads();
         if (wact) {
             const float* base = s_in + ci * PL;
-            for (int py = 0; py < TY; ++py) {
+            for (int py = 0; py < ny; ++py) {
                 // 3 x 3 window slid along the row: three new values per pixel
                 float w0[3], w1[3];
 #pragma unroll
@@ -610,7 +614,7 @@ __global__ void __launch_bounds__(256) conv_wgrad_kernel(const float* __restrict
                     w1[dy] = base[(py + dy) * RW + 1];
                 }
 #pragma unroll 6
-                for (int px = 0; px < GX; ++px) {
+                for (int px = 0; px < nx; ++px) {
                     const float4 gv = s_g[(py * GX + px) * 8 + cq];
                     const float gc[4] = {gv.x, gv.y, gv.z, gv.w};
 #pragma unroll
@@ -961,8 +965,13 @@ cudaError_t backward(ibem_cnn* c, const float* target, int B, int H, int W, int 
     float* g1 = c->d_gbuf + per;
     float* g2 = c->d_gbuf;
     const int64_t HW = (int64_t)H * W;
-    const int tiles = ((H + TY - 1) / TY) * ((W + GX - 1) / GX);
-    const int64_t items = (int64_t)B * tiles;
+    // rows of a weight-gradient tile: all TY where the tiles keep every SM busy, else fewer,
+    // so that a CTA's chain of pixels is shorter (six images of 18 x 18, 32 channels:
+    // 101 us for the four layers with 12 rows)
+    int gh = TY;
+    auto wg_items = [&](int rows) { return (int64_t)B * ((H + rows - 1) / rows) * ((W + GX - 1) / GX); };
+    while (gh > 1 && wg_items(gh) < WG_ITEMS) gh /= 2;   // 12, 6, 3, 1
+    const int64_t items = wg_items(gh);
     const int ipc = (int)((items + WG_ITEMS - 1) / WG_ITEMS);
     const int nx = (int)((items + ipc - 1) / ipc);
     cudaError_t e;
@@ -981,9 +990,9 @@ cudaError_t backward(ibem_cnn* c, const float* target, int B, int H, int W, int 
         const int Cin = c->cin[l], Cout = c->cout[l];
         // g0 = dL / d(pre-activation of layer l)
         const int nw = Cout * Cin * 9, np = nw + Cout;
-        if ((e = cudaFuncSetAttribute(conv_wgrad_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM)))
-            return e;
-        conv_wgrad_kernel<T><<<nx, 256, WG_SMEM, c->stream>>>(g0, act + l * per, B, Cin, H, W, Cout, ipc, c->d_part);
+        auto wgrad = gh < TY ? conv_wgrad_kernel<T, true> : conv_wgrad_kernel<T, false>;
+        if ((e = cudaFuncSetAttribute(wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM))) return e;
+        wgrad<<<nx, 256, WG_SMEM, c->stream>>>(g0, act + l * per, B, Cin, H, W, Cout, gh, ipc, c->d_part);
         sum_rows_kernel<<<cblk(np, 32), 256, 0, c->stream>>>(c->d_part, nx, np, nw, c->d_grad + c->woff[l],
                                                             c->d_grad + c->boff[l]);
         c->launches += 2;
