@@ -43,54 +43,54 @@ struct LevelOffsets {
     int64_t off[12];           // cluster id of (level l, patch, morton) = off[l] + patch 4^l + morton
 };
 
-// One thread per (point, patch): the walk below one root.  fill == false: cnt[2 i] =
-// far clusters, cnt[2 i + 1] = near elements of walk i = point * npatch + patch,
-// used[c] = 1 for every far cluster.  fill == true: writes the lists at far_off[i],
-// near_off[i], so a point's entries are contiguous in the order of the patches.
-// Bound by the latency of a walk (some 100 dependent steps), so the walks are as
-// many and short as they can be: with one thread per point both passes took 0.80 ms
-// for 5000 points at level 6, with one per patch 0.29 ms.
-__global__ void pf_lists_kernel(int64_t npts, const double* __restrict__ pts, int npatch, int m, LevelOffsets lo,
+// One thread per walk, G of them per point: all roots (G = 1) or one each (G = npatch).
+// fill == false: cnt[2 i] = far clusters, cnt[2 i + 1] = near elements of walk i =
+// point * G + g, used[c] = 1 for every far cluster.  fill == true: writes the lists at
+// far_off[i], near_off[i], so a point's entries are contiguous in the order of the
+// patches.
+__global__ void pf_lists_kernel(int64_t npts, const double* __restrict__ pts, int npatch, int G, int m, LevelOffsets lo,
                                 const double* __restrict__ balls, double eta, bool fill, int32_t* __restrict__ cnt,
                                 uint8_t* __restrict__ used, const int64_t* __restrict__ far_off,
                                 const int64_t* __restrict__ near_off, int32_t* __restrict__ far_list,
                                 int32_t* __restrict__ near_list, int* __restrict__ status) {
     const int64_t iw = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (iw >= npts * npatch) return;
-    const int64_t ip = iw / npatch;
-    const int patch = (int)(iw - ip * npatch);
+    if (iw >= npts * G) return;
+    const int64_t ip = iw / G;
+    const int g = (int)(iw - ip * G);
     const double x0 = pts[3 * ip], x1 = pts[3 * ip + 1], x2 = pts[3 * ip + 2];
     int32_t sid[PF_STACK];
     int8_t slv[PF_STACK];
     int64_t nf = 0, nn = 0;
     const int64_t fo = fill ? far_off[iw] : 0, no = fill ? near_off[iw] : 0;
-    int sp = 0;
-    sid[sp] = (int32_t)(lo.off[0] + patch);
-    slv[sp++] = 0;
-    while (sp > 0) {
-        --sp;
-        const int32_t c = sid[sp];
-        const int l = slv[sp];
-        const double* b = balls + 4 * (int64_t)c;
-        const double d0 = x0 - b[0], d1 = x1 - b[1], d2 = x2 - b[2];
-        double dist = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - b[3];
-        if (!(dist > 0.0)) dist = 0.0;
-        if (eta * 2.0 * b[3] < dist) {
-            if (fill) far_list[fo + nf] = c;
-            else used[c] = 1;
-            ++nf;
-        } else if (l == m) {
-            if (fill) near_list[no + nn] = (int32_t)(c - lo.off[m]);
-            ++nn;
-        } else {
-            if (sp + 4 > PF_STACK) {   // unreachable for m <= 10; recorded, never overrun
-                atomicOr(status, IBEM_DEVICE_OVERFLOW);
-                return;
-            }
-            const int64_t first = lo.off[l + 1] + 4 * (c - lo.off[l]);
-            for (int k = 0; k < 4; ++k) {
-                sid[sp] = (int32_t)(first + k);
-                slv[sp++] = (int8_t)(l + 1);
+    for (int patch = G == 1 ? 0 : g, end = G == 1 ? npatch : g + 1; patch < end; ++patch) {
+        int sp = 0;
+        sid[sp] = (int32_t)(lo.off[0] + patch);
+        slv[sp++] = 0;
+        while (sp > 0) {
+            --sp;
+            const int32_t c = sid[sp];
+            const int l = slv[sp];
+            const double* b = balls + 4 * (int64_t)c;
+            const double d0 = x0 - b[0], d1 = x1 - b[1], d2 = x2 - b[2];
+            double dist = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - b[3];
+            if (!(dist > 0.0)) dist = 0.0;
+            if (eta * 2.0 * b[3] < dist) {
+                if (fill) far_list[fo + nf] = c;
+                else used[c] = 1;
+                ++nf;
+            } else if (l == m) {
+                if (fill) near_list[no + nn] = (int32_t)(c - lo.off[m]);
+                ++nn;
+            } else {
+                if (sp + 4 > PF_STACK) {   // unreachable for m <= 10; recorded, never overrun
+                    atomicOr(status, IBEM_DEVICE_OVERFLOW);
+                    return;
+                }
+                const int64_t first = lo.off[l + 1] + 4 * (c - lo.off[l]);
+                for (int k = 0; k < 4; ++k) {
+                    sid[sp] = (int32_t)(first + k);
+                    slv[sp++] = (int8_t)(l + 1);
+                }
             }
         }
     }
@@ -100,7 +100,14 @@ __global__ void pf_lists_kernel(int64_t npts, const double* __restrict__ pts, in
     }
 }
 
-// offsets of the walks' lists from their counts: far then near, npts * npatch + 1 each
+// Walks per point.  A walk is a chain of some 100 dependent steps per root, so few
+// points take one per root (5000 points at level 6: both passes 0.29 ms, 0.80 with one
+// per point).  The host adds up and sends the offsets of every walk, so from 5000 to 10000
+// points on one per point is quicker, for 6 and for 16 roots (whole call, q = 6, one
+// density: 16 roots 2.6 and 2.0 ms at 5000 points, 14.2 and 16.7 at 50000).
+int walks_per_point(int64_t npts, int npatch) { return npts <= 8192 ? npatch : 1; }
+
+// offsets of the walks' lists from their counts: far then near, npts * G + 1 each
 std::vector<int64_t> walk_offsets(const std::vector<int32_t>& cnt) {
     const size_t n = cnt.size() / 2;
     std::vector<int64_t> off(2 * (n + 1), 0);
@@ -174,7 +181,7 @@ __device__ __forceinline__ void pf_kernel_value(double d2, double kappa, const d
 // some 20 pairs per thread (5000 points, 4 densities, level 6: 2.59 ms, 5.34 with 16).
 template <bool CPLX, int RC>
 __global__ void __launch_bounds__(PF_T, RC <= PF_RS ? 2 : 1) pf_eval_kernel(
-    int64_t npts, int npatch, const double* __restrict__ pts, int R, const int64_t* __restrict__ far_off,
+    int64_t npts, int walks, const double* __restrict__ pts, int R, const int64_t* __restrict__ far_off,
     const int32_t* __restrict__ far_list, const int64_t* __restrict__ near_off, const int32_t* __restrict__ near_list,
     int q2, int64_t n_used, const int32_t* __restrict__ slot, const double* __restrict__ igeo,
     const double* __restrict__ xh, int QQ, int nb, int64_t E,
@@ -196,7 +203,7 @@ __global__ void __launch_bounds__(PF_T, RC <= PF_RS ? 2 : 1) pf_eval_kernel(
     const int t = threadIdx.x;
     // far field
     {
-        const int64_t f0 = far_off[ip * npatch], f1 = far_off[(ip + 1) * npatch];
+        const int64_t f0 = far_off[ip * walks], f1 = far_off[(ip + 1) * walks];
         const int G = PF_T / q2 > 0 ? PF_T / q2 : 1, step = q2 < PF_T ? q2 : PF_T;
         for (int64_t k = f0 + t / step; t < G * step && k < f1; k += G) {
             const int64_t c = far_list[k];
@@ -226,7 +233,7 @@ __global__ void __launch_bounds__(PF_T, RC <= PF_RS ? 2 : 1) pf_eval_kernel(
     }
     // near field
     {
-        const int64_t n0 = near_off[ip * npatch], n1 = near_off[(ip + 1) * npatch];
+        const int64_t n0 = near_off[ip * walks], n1 = near_off[(ip + 1) * walks];
         const int G = PF_T / QQ > 0 ? PF_T / QQ : 1, step = QQ < PF_T ? QQ : PF_T;
         for (int64_t k = n0 + t / step; t < G * step && k < n1; k += G) {
             const int64_t e = near_list[k];
@@ -365,13 +372,14 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     // (1) count, mark the clusters used
     LevelOffsets lo{};
     for (int l = 0; l <= P.m + 1 && l < 12; ++l) lo.off[l] = P.level_off[l];
-    const int64_t nw = npts * P.npatch;   // walks
+    const int G = walks_per_point(npts, P.npatch);
+    const int64_t nw = npts * G;
     int32_t* d_cnt;
     uint8_t* d_used;
     if ((e = buf.alloc(&d_cnt, (size_t)2 * nw)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
         (e = cudaMemsetAsync(d_used, 0, (size_t)P.C, st)))
         return e;
-    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, G, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
                                                       d_used, nullptr, nullptr, nullptr, nullptr, h->d_status);
     h->launches++;
     std::vector<int32_t> cnt((size_t)2 * nw);
@@ -406,7 +414,7 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     if (n_used > 0 && (e = cudaMemcpyAsync(d_ids, ids.data(), ids.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
                                            st)))
         return e;
-    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(npts, pts, P.npatch, G, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
                                                       nullptr, d_off, d_off + nw + 1, d_lists, d_lists + nfar,
                                                       h->d_status);
     h->launches++;
@@ -439,7 +447,7 @@ cudaError_t launch_potential_fmm(ibem_handle* h, const double* w, int nrhs, cons
     const int QQ = P.Q * P.Q;
     auto eval = [&](auto kern, int rc) {
         kern<<<dim3((unsigned)npts, (unsigned)((nrhs + rc - 1) / rc)), PF_T, 0, st>>>(
-            npts, P.npatch, pts, nrhs, d_off, d_lists, d_off + nw + 1, d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo,
+            npts, G, pts, nrhs, d_off, d_lists, d_off + nw + 1, d_lists + nfar, P.q2, n_used, d_slot, h->d_igeo,
             d_xhat, QQ, P.nb, P.E, h->d_qgeo, h->d_phi, d_xs, P.prm.kappa, h->d_trig64, u);
     };
     if (h->helm) {
@@ -649,13 +657,14 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
     // (1) lists per source (the potential's walk)
     LevelOffsets lo{};
     for (int l = 0; l <= P.m + 1 && l < 12; ++l) lo.off[l] = P.level_off[l];
-    const int64_t nw = nsrc * P.npatch;   // walks
+    const int G = walks_per_point(nsrc, P.npatch);
+    const int64_t nw = nsrc * G;
     int32_t* d_cnt;
     uint8_t* d_used;
     if ((e = buf.alloc(&d_cnt, (size_t)2 * nw)) || (e = buf.alloc(&d_used, (size_t)P.C)) ||
         (e = cudaMemsetAsync(d_used, 0, (size_t)P.C, st)))
         return e;
-    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, G, P.m, lo, h->d_balls, P.prm.eta, false, d_cnt,
                                                       d_used, nullptr, nullptr, nullptr, nullptr, h->d_status);
     h->launches++;
     std::vector<int32_t> cnt((size_t)2 * nw);
@@ -671,7 +680,7 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
     if ((e = buf.alloc(&d_off, off.size())) || (e = buf.alloc(&d_lists, (size_t)(nfar + nnear))) ||
         (e = cudaMemcpyAsync(d_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st)))
         return e;
-    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
+    pf_lists_kernel<<<nblk(nw, 128), 128, 0, st>>>(nsrc, src, P.npatch, G, P.m, lo, h->d_balls, P.prm.eta, true, d_cnt,
                                                       nullptr, d_off, d_off + nw + 1, d_lists, d_lists + nfar,
                                                       h->d_status);
     h->launches++;
@@ -683,8 +692,8 @@ cudaError_t launch_rhs_sources(ibem_handle* h, const double* src, const double* 
     // (2) lists per cluster and per element, sources ascending
     std::vector<int64_t> foff((size_t)nsrc + 1), noff((size_t)nsrc + 1);
     for (int64_t i = 0; i <= nsrc; ++i) {
-        foff[i] = off[i * P.npatch];
-        noff[i] = off[nw + 1 + i * P.npatch];
+        foff[i] = off[i * G];
+        noff[i] = off[nw + 1 + i * G];
     }
     std::vector<int32_t> cl, csrc, el, esrc;
     std::vector<int64_t> cptr, eptr;
