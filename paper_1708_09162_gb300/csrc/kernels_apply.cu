@@ -691,25 +691,28 @@ __global__ void leaf_back_kernel(int R, int64_t E, int pp, int q, const double* 
 }
 
 // ---- near field product ------------------------------------------------------
-// One CTA per target element, `slices` groups of nt threads; thread t = i * nb + j of a
-// group accumulates B[i][j] x*_s[j] over every slices-th block of the row (one
-// coalesced nb^2 read per block), then groups and columns are summed through
-// shared memory in a fixed order.  The row's source elements are staged in shared
+// One CTA per target element; thread t = i * nb + j accumulates B[i][j] x*_s[j] over the
+// blocks of the row in S slices, every S-th block each (one coalesced nb^2 read per
+// block), then slices and columns are summed through shared memory in a fixed
+// order.  P groups of nt threads take the slices: one group each (P = S), or one
+// group all of them in turn (P = 1).  The row's source elements are staged in shared
 // memory (so a source value's load does not wait for a dependent global load)
-// and a group's sum runs in four independent partial sums.
-template <typename T, int S>
+// and a slice's sum runs in four independent partial sums.
+template <typename T, int S, int P>
 __global__ void near_apply_kernel(const int64_t* __restrict__ nptr, const int32_t* __restrict__ nsrc,
                                   const T* __restrict__ blocks, int nb, int64_t E, int nt, const T* __restrict__ xs,
                                   double* __restrict__ ys) {
-    extern __shared__ double red[];
+    extern __shared__ double red[];   // [S][nt]
     __shared__ int32_t srcs[256];
     const int64_t e = blockIdx.x, r = blockIdx.y;
-    constexpr int slices = S;   // S = 1 as a run-time value took 181 instead of 171 us at p = 3, level 5
-    const int sl = S == 1 ? 0 : threadIdx.x / nt, t = threadIdx.x - sl * nt, nbb = nb * nb;
+    constexpr int SETS = S / P;
+    const int grp = P == 1 ? 0 : threadIdx.x / nt, t = threadIdx.x - grp * nt, nbb = nb * nb;
     const int64_t k0 = nptr[e], k1 = nptr[e + 1];
     const int j = t % nb;
     const T* xr = xs + r * E * nb;
-    T p0 = (T)0, p1 = (T)0, p2 = (T)0, p3 = (T)0;
+    T p[SETS][4];
+#pragma unroll
+    for (int q = 0; q < SETS; ++q) p[q][0] = p[q][1] = p[q][2] = p[q][3] = (T)0;
     for (int64_t kb = k0; kb < k1; kb += 256) {
         const int kc = (int)(k1 - kb < 256 ? k1 - kb : 256);
         __syncthreads();   // the previous chunk's source list is consumed
@@ -717,31 +720,36 @@ __global__ void near_apply_kernel(const int64_t* __restrict__ nptr, const int32_
         __syncthreads();
         if (t < nbb) {
             const T* bk = blocks + kb * nbb + t;
-            int kk = sl;
-            for (; kk + 3 * slices < kc; kk += 4 * slices) {
-                p0 += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
-                p1 += bk[(int64_t)(kk + slices) * nbb] * xr[(int64_t)srcs[kk + slices] * nb + j];
-                p2 += bk[(int64_t)(kk + 2 * slices) * nbb] * xr[(int64_t)srcs[kk + 2 * slices] * nb + j];
-                p3 += bk[(int64_t)(kk + 3 * slices) * nbb] * xr[(int64_t)srcs[kk + 3 * slices] * nb + j];
+#pragma unroll
+            for (int q = 0; q < SETS; ++q) {
+                int kk = grp + P * q;
+                for (; kk + 3 * S < kc; kk += 4 * S) {
+                    p[q][0] += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
+                    p[q][1] += bk[(int64_t)(kk + S) * nbb] * xr[(int64_t)srcs[kk + S] * nb + j];
+                    p[q][2] += bk[(int64_t)(kk + 2 * S) * nbb] * xr[(int64_t)srcs[kk + 2 * S] * nb + j];
+                    p[q][3] += bk[(int64_t)(kk + 3 * S) * nbb] * xr[(int64_t)srcs[kk + 3 * S] * nb + j];
+                }
+                for (; kk < kc; kk += S) p[q][0] += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
             }
-            for (; kk < kc; kk += slices) p0 += bk[(int64_t)kk * nbb] * xr[(int64_t)srcs[kk] * nb + j];
         }
     }
-    red[threadIdx.x] = t < nbb ? (double)((p0 + p1) + (p2 + p3)) : 0.0;
+#pragma unroll
+    for (int q = 0; q < SETS; ++q)
+        red[(grp + P * q) * nt + t] = t < nbb ? (double)((p[q][0] + p[q][1]) + (p[q][2] + p[q][3])) : 0.0;
     __syncthreads();
     if (threadIdx.x < nb) {
         double v = 0.0;
-        for (int q = 0; q < slices; ++q)
+        for (int q = 0; q < S; ++q)
             for (int jj = 0; jj < nb; ++jj) v += red[q * nt + threadIdx.x * nb + jj];
         ys[(r * E + e) * nb + threadIdx.x] += v;
     }
 }
 
-// Groups per element: where the elements alone leave SMs without work, up to four
-// share a row (a group's chain of some 20 dependent loads is what a small mesh
-// waits for; with the shared launches of the coarse levels the application at p = 2,
-// level 2 went from 104 to 80 us).  The order of a row's sums must not
-// depend on the number of right-hand sides, so the rule counts the elements only.
+// Slices per row: up to four where the elements alone leave SMs without work (a
+// slice's chain of some 20 dependent loads is what a small mesh waits for; with
+// the shared launches of the coarse levels the application at p = 2, level 2 went
+// from 104 to 80 us).  The order of a row's sums must not depend on the number of
+// right-hand sides, so this rule counts the elements only.
 static int near_slices(const Plan& P, int nt) {
     int s = 1;
     while (s < 4 && P.E * s < 152 * 8 && 2 * s * nt <= 1024) s *= 2;
@@ -751,13 +759,17 @@ static int near_slices(const Plan& P, int nt) {
 template <typename T>
 static void launch_near_apply(ibem_handle* h, int R, int nt, int slices, const T* blocks, const T* xs) {
     const Plan& P = h->P;
-    auto go = [&](auto kern) {
-        kern<<<dim3((unsigned)P.E, R), nt * slices, nt * slices * sizeof(double), h->stream>>>(
+    auto go = [&](auto kern, int groups) {
+        kern<<<dim3((unsigned)P.E, R), nt * groups, nt * slices * sizeof(double), h->stream>>>(
             h->d_near_ptr, h->d_near_src, blocks, P.nb, P.E, nt, xs, h->d_ys);
     };
-    if (slices == 1) go(near_apply_kernel<T, 1>);
-    else if (slices == 2) go(near_apply_kernel<T, 2>);
-    else go(near_apply_kernel<T, 4>);
+    // a group per slice while the CTAs do not fill the chip, else one group, with the same
+    // sums (level 3, p = 2, dense, eight right-hand sides: 250 us, 259 with four groups; four
+    // right-hand sides are still better off with four, 383 us against 392 at p = 1)
+    const bool one = P.E * R >= 152 * 16;
+    if (slices == 1) go(near_apply_kernel<T, 1, 1>, 1);
+    else if (slices == 2) one ? go(near_apply_kernel<T, 2, 1>, 1) : go(near_apply_kernel<T, 2, 2>, 2);
+    else one ? go(near_apply_kernel<T, 4, 1>, 1) : go(near_apply_kernel<T, 4, 4>, 4);
 }
 
 __global__ void d2f_kernel(const double* __restrict__ in, float* __restrict__ out, int64_t n) {
