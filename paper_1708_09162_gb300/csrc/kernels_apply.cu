@@ -219,6 +219,19 @@ struct TopLevels {
     int64_t off[TOP_L + 2];
 };
 
+// finest parent level that the shared launch takes, -1 for none: a single level (m = 1) is as
+// quick, and cheaper to launch, by itself
+static int top_levels(const Plan& P) { return P.m < 2 ? -1 : (P.m - 1 < TOP_L ? P.m - 1 : TOP_L); }
+
+// the opt-in for more than 48 KB of shared memory, where it is needed (a host call of
+// about a microsecond)
+template <typename K>
+static cudaError_t allow_smem(K kern, size_t bytes) {
+    return bytes <= 48 * 1024 ? cudaSuccess
+                              : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     IBEM_MAX_SMEM_BYTES);
+}
+
 __global__ void __launch_bounds__(TOP_T) m2m_top_kernel(int first, TopLevels lo, int q, const double* __restrict__ S,
                                                         int64_t C, double* __restrict__ xh) {
     extern __shared__ double top_sm[];
@@ -296,18 +309,18 @@ __global__ void __launch_bounds__(TOP_T) l2l_top_kernel(int last, TopLevels lo, 
 // M2M of every level for R real vectors: the fine levels one launch each, then the top
 cudaError_t launch_m2m(ibem_handle* h, int R, double* xh) {
     const Plan& P = h->P;
-    for (int L = P.m - 1; L > TOP_L; --L) {
+    const int first = top_levels(P);
+    for (int L = P.m - 1; L > first; --L) {
         const int64_t nL = P.level_off[L + 1] - P.level_off[L];
         m2m_sep_kernel<<<dim3((unsigned)nL, (unsigned)R), 64, 0, h->stream>>>(nL, P.level_off[L], P.level_off[L + 1], P.q,
                                                                              h->d_S, P.C, xh);
         h->launches++;
     }
-    const int first = P.m - 1 < TOP_L ? P.m - 1 : TOP_L;
-    if (first < 0) return cudaSuccess;
+    if (first < 0) return cudaGetLastError();
     TopLevels lo;
     for (int l = 0; l <= first + 1; ++l) lo.off[l] = P.level_off[l];
     const size_t sm = (2 + 8 * ((size_t)1 << (2 * first))) * P.q2 * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(m2m_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, IBEM_MAX_SMEM_BYTES);
+    cudaError_t e = allow_smem(m2m_top_kernel, sm);
     if (e) return e;
     m2m_top_kernel<<<dim3((unsigned)P.npatch, (unsigned)R), TOP_T, sm, h->stream>>>(first, lo, P.q, h->d_S, P.C, xh);
     h->launches++;
@@ -317,13 +330,12 @@ cudaError_t launch_m2m(ibem_handle* h, int R, double* xh) {
 // L2L of every level: the top, then the fine levels
 cudaError_t launch_l2l(ibem_handle* h, int R, double* yh) {
     const Plan& P = h->P;
-    const int last = P.m - 1 < TOP_L ? P.m - 1 : TOP_L;
+    const int last = top_levels(P);
     if (last >= 0) {
         TopLevels lo;
         for (int l = 0; l <= last + 1; ++l) lo.off[l] = P.level_off[l];
         const size_t sm = (2 + 3 * ((size_t)1 << (2 * last))) * P.q2 * sizeof(double);
-        cudaError_t e = cudaFuncSetAttribute(l2l_top_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             IBEM_MAX_SMEM_BYTES);
+        cudaError_t e = allow_smem(l2l_top_kernel, sm);
         if (e) return e;
         l2l_top_kernel<<<dim3((unsigned)P.npatch, (unsigned)R), TOP_T, sm, h->stream>>>(last, lo, P.q, h->d_S, P.C, yh);
         h->launches++;
