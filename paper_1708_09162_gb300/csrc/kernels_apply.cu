@@ -584,7 +584,10 @@ __global__ void coupling_df_kernel(const int32_t* __restrict__ rows, const int64
 // y^_tau += sum over the stored blocks (sigma, tau) of their column shares.  One CTA per
 // (tau, vector): G = blockDim / q2 slices of the transposed list, combined in order (a
 // thread per entry of y^_tau read a list of some 90 shares one after the other: 73 us
-// at p = 3, level 5, now 65 us).
+// at p = 3, level 5, now 65 us).  For q <= 4 the slices are too many and too short
+// (level 5, q = 4, 64 vectors: 2.5 ms against 1.15), so there a thread per entry
+// (column_gather_entry_kernel); by q only, so that a vector's bits do not depend on how many
+// there are.
 __global__ void column_gather_kernel(int64_t C, int q2, int G, const int64_t* __restrict__ tptr,
                                      const int32_t* __restrict__ tblk, const float2* __restrict__ colpart,
                                      int64_t nblk_total, double* __restrict__ yh) {
@@ -608,6 +611,23 @@ __global__ void column_gather_kernel(int64_t C, int q2, int G, const int64_t* __
         for (int k = 0; k < G; ++k) v += gred[k * q2 + t];
         yh[(r * C + tau) * q2 + t] += v;
     }
+}
+
+__global__ void column_gather_entry_kernel(int64_t n, int64_t C, int q2, const int64_t* __restrict__ tptr,
+                                           const int32_t* __restrict__ tblk, const float2* __restrict__ colpart,
+                                           int64_t nblk_total, double* __restrict__ yh) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;   // (vector, tau, entry)
+    if (idx >= n) return;
+    const int64_t rt = idx / q2, r = rt / C, tau = rt - r * C, k1 = tptr[tau + 1];
+    if (tptr[tau] == k1) return;
+    const float2* part = colpart + r * nblk_total * q2 + (idx - rt * q2);
+    float hi = 0.0f, lo = 0.0f;
+#pragma unroll 4
+    for (int64_t k = tptr[tau]; k < k1; ++k) {
+        const float2 v = part[(int64_t)tblk[k] * q2];
+        df_add(hi, lo, v.x, v.y);
+    }
+    yh[idx] += (double)hi + (double)lo;
 }
 
 // ---- coupling, FP32, kernel generated on the fly ------------------------------
@@ -1001,9 +1021,14 @@ cudaError_t apply_operator(ibem_handle* h, const double* x, double* y, int nrhs,
                 const int q2p = (q2 + 1) & ~1;
                 split_kernel<<<nblk(R * P.C * q2p, T), T, 0, st>>>(R * P.C, q2, q2p, h->d_xh, h->d_xh2);
                 if ((e = launch_coupling_df(h, R, h->df_nst))) return e;
-                const int G = q2 < 256 ? 256 / q2 : 1, gt = (G * q2 + 31) / 32 * 32;
-                column_gather_kernel<<<dim3((unsigned)P.C, R), gt, G * q2 * sizeof(double), st>>>(
-                    P.C, q2, G, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->n_up, h->d_yh);
+                if (P.q <= 4) {
+                    column_gather_entry_kernel<<<nblk((int64_t)R * P.C * q2, T), T, 0, st>>>(
+                        (int64_t)R * P.C * q2, P.C, q2, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->n_up, h->d_yh);
+                } else {
+                    const int G = q2 < 256 ? 256 / q2 : 1, gt = (G * q2 + 31) / 32 * 32;
+                    column_gather_kernel<<<dim3((unsigned)P.C, R), gt, G * q2 * sizeof(double), st>>>(
+                        P.C, q2, G, h->d_tr_ptr, h->d_tr_blk, h->d_colpart, h->n_up, h->d_yh);
+                }
                 h->launches++;
                 h->launches += 2;
             }
