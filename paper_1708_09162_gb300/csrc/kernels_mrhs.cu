@@ -880,27 +880,33 @@ __global__ void mr_near_kernel(int R, int nb, const int64_t* __restrict__ nptr, 
 // Same product with a thread holding all NB rows of its element for one right-hand
 // side: the element's blocks pass through shared memory in chunks of KC (broadcast
 // reads, 4 FMA per complex entry and load), each source value is loaded once per
-// block (coalesced over the right-hand sides).  The CTA's threads form slices of RT >=
-// R threads; slice q takes every S-th block of a chunk, and the slices are added in
-// order through shared memory.  Bound: FMA and the latency of the source values;
-// without slices 16 right-hand sides kept half a warp per element busy (level 5, p = 2:
-// 1272 us, now 240 us; 64 right-hand sides 942 us, now 430 us).
+// block (coalesced over the right-hand sides).  The CTA's threads form S slices of RT
+// threads, each for up to 64 right-hand sides (blockIdx.y: further ones); slice q takes
+// every S-th block of a chunk, and the slices are added in order through shared
+// memory.  S depends on the degree only, so a column's bits do not depend on how many
+// are applied with it.  Bound: FMA and the latency of the source values; without slices
+// 16 right-hand sides kept half a warp per element busy (level 5, p = 2: 1272 us, now 260;
+// 64 right-hand sides 942 us, now 465).
+// Launch bounds: three CTAs of eight slices per SM (two, with 57 registers: 33 to 115 us more
+// at 64 right-hand sides), two of four.
+constexpr int mr_near_slices(int nb) { return nb == 9 ? 8 : 4; }
 template <bool CPLX, int NB>
-__global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, int RT, const int64_t* __restrict__ nptr,
-                                                           const int32_t* __restrict__ nsrc,
-                                                           const float* __restrict__ blocks,
-                                                           const typename MrType<CPLX>::T* __restrict__ xs,
-                                                           typename MrType<CPLX>::T* __restrict__ ys) {
+__global__ void __launch_bounds__(64 * mr_near_slices(NB), NB == 9 ? 3 : 2) mr_near_rows_kernel(
+    int R, int RC, int RT, const int64_t* __restrict__ nptr, const int32_t* __restrict__ nsrc,
+    const float* __restrict__ blocks, const typename MrType<CPLX>::T* __restrict__ xs,
+    typename MrType<CPLX>::T* __restrict__ ys) {
     typedef typename MrType<CPLX>::T T;
-    constexpr int CW = CPLX ? 2 : 1;
+    constexpr int CW = CPLX ? 2 : 1, S = NB == 9 ? 8 : 4;
     constexpr int BF = NB * NB * CW;                             // floats per block
     constexpr int KC = (NB == 9 ? 32 : 16) * (CPLX ? 1 : 2);     // blocks per shared-memory chunk
-    static_assert(KC * BF >= 256 * NB * CW, "the slices' sums fit in the chunk");
+    constexpr int HB = KC * BF / (CW * 64 * S) < NB ? KC * BF / (CW * 64 * S) : NB;   // rows combined at a time
+    static_assert(HB > 0, "a row of the slices' sums fits in the chunk");
     __shared__ __align__(16) float sb[KC * BF];
     __shared__ int ss[KC];
     const int64_t e = blockIdx.x;
-    const int t = threadIdx.x, slice = t / RT, r = t - slice * RT, S = blockDim.x / RT;
-    const bool act = r < R;
+    const int t = threadIdx.x, slice = t / RT, r = t - slice * RT, r0 = blockIdx.y * RC;
+    const int cols = R - r0 < RC ? R - r0 : RC;
+    const bool act = r < cols;
     float ar[NB], ai[NB];
 #pragma unroll
     for (int i = 0; i < NB; ++i) ar[i] = ai[i] = 0.0f;
@@ -915,7 +921,7 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, int RT, const 
                 const int64_t s = ss[kk];
                 T xv[NB];
 #pragma unroll
-                for (int j = 0; j < NB; ++j) xv[j] = xs[(s * NB + j) * R + r];
+                for (int j = 0; j < NB; ++j) xv[j] = xs[(s * NB + j) * R + r0 + r];
                 const float* B = sb + kk * BF;
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
@@ -934,25 +940,31 @@ __global__ void __launch_bounds__(256) mr_near_rows_kernel(int R, int RT, const 
         }
         __syncthreads();
     }
-    float* red = sb;                                             // [NB][CW][blockDim]
+    float* red = sb;                                             // [HB][CW][64 S]
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
-        red[(i * CW) * 256 + t] = ar[i];
-        if constexpr (CPLX) red[(i * CW + 1) * 256 + t] = ai[i];
-    }
-    __syncthreads();
-    for (int o = t; o < NB * RT; o += blockDim.x) {
-        const int i = o / RT, rr = o - i * RT;
-        if (rr >= R) continue;
-        float v[CW];
+    for (int i0 = 0; i0 < NB; i0 += HB) {
+        if (i0 > 0) __syncthreads();
 #pragma unroll
-        for (int c = 0; c < CW; ++c) {
-            v[c] = 0.0f;
-            for (int q = 0; q < S; ++q) v[c] += red[(i * CW + c) * 256 + q * RT + rr];
+        for (int i = i0; i < i0 + HB && i < NB; ++i) {
+            red[(i - i0) * CW * 64 * S + t] = ar[i];
+            if constexpr (CPLX) red[((i - i0) * CW + 1) * 64 * S + t] = ai[i];
         }
-        T* out = ys + (e * NB + i) * R + rr;
-        if constexpr (CPLX) *out = make_float2(out->x + v[0], out->y + v[CW - 1]);
-        else *out += v[0];
+        __syncthreads();
+        for (int o = t; o < HB * RT; o += blockDim.x) {
+            const int i = i0 + o / RT, rr = o % RT;
+            if (i >= NB || rr >= cols) continue;
+            T* out = ys + (e * NB + i) * R + r0 + rr;
+            const T was = *out;
+            float v[CW];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) {
+                v[c] = 0.0f;
+#pragma unroll
+                for (int q = 0; q < S; ++q) v[c] += red[((i - i0) * CW + c) * 64 * S + q * RT + rr];
+            }
+            if constexpr (CPLX) *out = make_float2(was.x + v[0], was.y + v[CW - 1]);
+            else *out = was + v[0];
+        }
     }
 }
 
@@ -1141,14 +1153,15 @@ static cudaError_t mr_apply(ibem_handle* h, const double* x, double* y, int R) {
     int nthreads = P.nb * R < 512 ? ((P.nb * R + 31) / 32) * 32 : 512;
     {
         PhaseTimer pt(h, 4);
-        // slices of 16, 32, ... threads, as many as fit in 256 threads
-        const int RT = R <= 16 ? 16 : ((R + 31) / 32) * 32, tr = RT * std::max(1, std::min(256 / RT, 16));
+        // equal groups of at most 64 right-hand sides, a slice of 16, 32 or 64 threads each
+        const int groups = (R + 63) / 64, RC = (R + groups - 1) / groups, RT = RC <= 16 ? 16 : (RC <= 32 ? 32 : 64);
+        const dim3 ng((unsigned)P.E, (unsigned)groups);
         if (P.nb == 9)
-            mr_near_rows_kernel<CPLX, 9><<<(unsigned)P.E, tr, 0, st>>>(R, RT, h->d_near_ptr, h->d_near_src, h->d_near32,
-                                                                       xs, ys);
+            mr_near_rows_kernel<CPLX, 9><<<ng, RT * mr_near_slices(9), 0, st>>>(R, RC, RT, h->d_near_ptr, h->d_near_src,
+                                                                                h->d_near32, xs, ys);
         else if (P.nb == 16)
-            mr_near_rows_kernel<CPLX, 16><<<(unsigned)P.E, tr, 0, st>>>(R, RT, h->d_near_ptr, h->d_near_src, h->d_near32,
-                                                                        xs, ys);
+            mr_near_rows_kernel<CPLX, 16><<<ng, RT * mr_near_slices(16), 0, st>>>(
+                R, RC, RT, h->d_near_ptr, h->d_near_src, h->d_near32, xs, ys);
         else
             mr_near_kernel<CPLX><<<(unsigned)P.E, nthreads, 0, st>>>(R, P.nb, h->d_near_ptr, h->d_near_src,
                                                                      h->d_near32, xs, ys);

@@ -78,3 +78,15 @@ def test_helmholtz_stored_far_field(p, m, q, R):
     assert torch.equal(_apply(h, x), y)
     assert float((_apply(h, x[:3].contiguous()) - y[:3]).abs().max()) < 1e-12 * float(y.abs().max())
     lib().ibem_destroy(h)
+
+
+# FP32 operator of 16 and more columns: 16 to 64 per group of the near product, one to four groups
+@pytest.mark.parametrize("kernel,p,m,q", [(0, 2, 3, 4), (0, 3, 2, 6), (1, 2, 3, 4), (1, 3, 2, 8), (1, 1, 3, 4)])
+def test_fp32_many(kernel, p, m, q):
+    import torch
+    h = _handle(p, m, q, kernel)
+    x = _vectors(1830 + p, 200, lib().ibem_get_info(h).ndof, *((2,) if kernel else ()))
+    y = _apply(h, x, 1)
+    for r0, n in ((0, 16), (3, 17), (100, 40), (136, 64), (60, 65), (72, 128)):
+        assert torch.equal(_apply(h, x[r0:r0 + n].contiguous(), 1), y[r0:r0 + n]), (r0, n)
+    lib().ibem_destroy(h)
