@@ -259,10 +259,13 @@ __global__ void helm_near_apply_kernel(const int64_t* __restrict__ nptr, const i
 // each block is read once for all right-hand sides.  Adds to ys (split layout).
 // The coefficients are split once per application (helm_split_lift_kernel): splitting
 // them again for each of some 50 near blocks kept the FP64 pipe busier than the
-// products the FP32 pipe.  Few right-hand sides leave most of the CTA idle, so its
-// threads form S slices that take S blocks at a time.  Stages are double buffered
-// (one barrier per S blocks).  p = 2: 64 right-hand sides at level 5 5.34 ms instead of
-// 6.18, 8 at level 3 156 us instead of 199.
+// products the FP32 pipe.  The sums are those of S slices, every S-th block each, added in
+// FP64 in order.  S depends on the degree only, so a column's bits do not depend on
+// how many are applied with it: two slices where two blocks fit a CTA's registers
+// (p <= 3), else one.  The slices are groups of threads that take S blocks at a time, or,
+// where a slice's (row, right-hand side) pairs would exceed its threads eightfold, sets of
+// sums that all threads fill in turn.  Stages are double buffered (one barrier per
+// stage).
 constexpr int HN_T = 256;
 
 __device__ __forceinline__ void hn_split(double v, float& h, float& l) {
@@ -300,32 +303,35 @@ __global__ void helm_split_lift_kernel(int R, int64_t n, const double* __restric
         }
 }
 
-// nt: threads per slice; dynamic shared memory 2 S (nb^2 + nb R) float4
+// S slices, P of them side by side (P = S or 1); MAXP pairs (row, right-hand side) per
+// thread: nb R <= MAXP HN_T / P.  Dynamic shared memory 2 P (nb^2 + nb R) float4.
+template <int S, int P, int MAXP>
 __global__ void __launch_bounds__(HN_T) helm_near_df_kernel(const int64_t* __restrict__ nptr,
                                                             const int32_t* __restrict__ nsrc,
-                                                            const double2* __restrict__ blocks, int nb, int R, int S,
-                                                            int nt, int64_t E, const float4* __restrict__ xl,
-                                                            double* __restrict__ ys) {
+                                                            const double2* __restrict__ blocks, int nb, int R, int64_t E,
+                                                            const float4* __restrict__ xl, double* __restrict__ ys) {
     extern __shared__ float4 hn_sm[];
+    constexpr int SETS = S / P, NTH = HN_T / P;
+    constexpr int MAXB = 3;          // block entries per thread: P nb^2 <= 3 HN_T
     const int64_t e = blockIdx.x;
-    const int t = threadIdx.x, nbb = nb * nb, np = nb * R, sl = t / nt, ts = t - sl * nt;
-    const int per = S * (nbb + np);  // float4 per stage: S blocks, then S coefficient sets
-    constexpr int MAXP = 8;          // (row, right-hand side) pairs per thread: nb R <= 8 HN_T
-    constexpr int MAXB = 3;          // block entries per thread: S nb^2 <= 3 HN_T
-    float acc[MAXP][4];
+    const int t = threadIdx.x, nbb = nb * nb, np = nb * R, sl = t / NTH, ts = t - sl * NTH;
+    const int per = P * (nbb + np);  // float4 per stage: P blocks, then P coefficient sets
+    float acc[SETS][MAXP][4];
 #pragma unroll
-    for (int k = 0; k < MAXP; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0f;
+    for (int q = 0; q < SETS; ++q)
+#pragma unroll
+        for (int k = 0; k < MAXP; ++k) acc[q][k][0] = acc[q][k][1] = acc[q][k][2] = acc[q][k][3] = 0.0f;
     const int64_t k0 = nptr[e];
     const int n = (int)(nptr[e + 1] - k0);
     double2 bn[MAXB];
-    auto fetch = [&](int c) {        // blocks c .. c + S - 1: entries into registers, coefficients into the stage
-        const int live = n - c < S ? n - c : S;
+    auto fetch = [&](int c) {        // blocks c .. c + P - 1: entries into registers, coefficients into the stage
+        const int live = n - c < P ? n - c : P;
 #pragma unroll
         for (int m = 0; m < MAXB; ++m) {
             const int q = t + HN_T * m;
             if (q < live * nbb) bn[m] = blocks[(k0 + c) * nbb + q];
         }
-        float4* X = hn_sm + ((c / S) & 1) * per + S * nbb;
+        float4* X = hn_sm + ((c / P) & 1) * per + P * nbb;
         for (int q = t; q < live * np; q += HN_T) {
             const int b = q / np, o = q - b * np;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
@@ -336,69 +342,106 @@ __global__ void __launch_bounds__(HN_T) helm_near_df_kernel(const int64_t* __res
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     if (n > 0) fetch(0);
-    for (int c = 0; c < n; c += S) {
-        const int live = n - c < S ? n - c : S;
-        float4* Bs = hn_sm + ((c / S) & 1) * per;
+    for (int c0 = 0; c0 < n; c0 += S) {
 #pragma unroll
-        for (int m = 0; m < MAXB; ++m) {
-            const int q = t + HN_T * m;
-            if (q < live * nbb) {
-                float4 v;
-                hn_split(bn[m].x, v.x, v.y);
-                hn_split(bn[m].y, v.z, v.w);
-                Bs[q] = v;
+        for (int set = 0; set < SETS; ++set) {
+            const int c = c0 + set * P;
+            if (c >= n) break;
+            const int live = n - c < P ? n - c : P;
+            float4* Bs = hn_sm + ((c / P) & 1) * per;
+#pragma unroll
+            for (int m = 0; m < MAXB; ++m) {
+                const int q = t + HN_T * m;
+                if (q < live * nbb) {
+                    float4 v;
+                    hn_split(bn[m].x, v.x, v.y);
+                    hn_split(bn[m].y, v.z, v.w);
+                    Bs[q] = v;
+                }
             }
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();             // the stage is complete; the other one is used
-        if (c + S < n) fetch(c + S);
-        if (sl < live) {
-            const float4* B = Bs + sl * nbb;
-            const float4* X = Bs + S * nbb + sl * np;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();         // the stage is complete; the other one is used
+            if (c + P < n) fetch(c + P);
+            if (sl < live) {
+                const float4* B = Bs + sl * nbb;
+                const float4* X = Bs + P * nbb + sl * np;
 #pragma unroll
-            for (int m = 0; m < MAXP; ++m) {
-                const int p = ts + nt * m;
-                if (p < np) {
-                    const int i = p / R, r = p - i * R;
-                    for (int j = 0; j < nb; ++j) {
-                        const float4 b = B[i * nb + j], x = X[j * R + r];
-                        // (Br + i Bi)(xr + i xi) = (Br xr - Bi xi) + i (Br xi + Bi xr)
-                        hn_mac(b.x, b.y, x.x, x.y, acc[m][0], acc[m][1]);
-                        hn_mac(-b.z, -b.w, x.z, x.w, acc[m][0], acc[m][1]);
-                        hn_mac(b.x, b.y, x.z, x.w, acc[m][2], acc[m][3]);
-                        hn_mac(b.z, b.w, x.x, x.y, acc[m][2], acc[m][3]);
+                for (int m = 0; m < MAXP; ++m) {
+                    const int p = ts + NTH * m;
+                    if (p < np) {
+                        const int i = p / R, r = p - i * R;
+                        float(&a)[4] = acc[set][m];
+                        for (int j = 0; j < nb; ++j) {
+                            const float4 b = B[i * nb + j], x = X[j * R + r];
+                            // (Br + i Bi)(xr + i xi) = (Br xr - Bi xi) + i (Br xi + Bi xr)
+                            hn_mac(b.x, b.y, x.x, x.y, a[0], a[1]);
+                            hn_mac(-b.z, -b.w, x.z, x.w, a[0], a[1]);
+                            hn_mac(b.x, b.y, x.z, x.w, a[2], a[3]);
+                            hn_mac(b.z, b.w, x.x, x.y, a[2], a[3]);
+                        }
                     }
                 }
             }
         }
     }
-    if (S > 1) {                     // nt >= np: one pair per thread; the slices in order
+    if (P > 1) {                     // the later slices' sums through shared memory
         __syncthreads();
-        if (sl < S && ts < np) hn_sm[sl * np + ts] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+#pragma unroll
+        for (int m = 0; m < MAXP; ++m) {
+            const int p = ts + NTH * m;
+            if (sl > 0 && p < np)
+                hn_sm[(sl - 1) * np + p] = make_float4(acc[0][m][0], acc[0][m][1], acc[0][m][2], acc[0][m][3]);
+        }
         __syncthreads();
-        if (t < np) {
-            double vr = 0.0, vi = 0.0;
-            for (int q = 0; q < S; ++q) {
-                const float4 v = hn_sm[q * np + t];
+        if (sl > 0) return;
+    }
+#pragma unroll
+    for (int m = 0; m < MAXP; ++m) {
+        const int p = ts + NTH * m;
+        if (p < np) {
+            const int i = p / R, r = p - i * R;
+            double vr = (double)acc[0][m][0] + (double)acc[0][m][1], vi = (double)acc[0][m][2] + (double)acc[0][m][3];
+#pragma unroll
+            for (int q = 1; q < S; ++q) {
+                float4 v;
+                if constexpr (P > 1) v = hn_sm[(q - 1) * np + p];
+                else v = make_float4(acc[q % SETS][m][0], acc[q % SETS][m][1], acc[q % SETS][m][2], acc[q % SETS][m][3]);
                 vr += (double)v.x + (double)v.y;
                 vi += (double)v.z + (double)v.w;
             }
-            const int i = t / R, r = t - i * R;
             ys[((int64_t)(2 * r) * E + e) * nb + i] += vr;
             ys[((int64_t)(2 * r + 1) * E + e) * nb + i] += vi;
         }
-        return;
     }
-    if (sl > 0) return;              // one slice: nt < HN_T leaves threads without a pair
-#pragma unroll
-    for (int m = 0; m < MAXP; ++m) {
-        const int p = ts + nt * m;
-        if (p < np) {
-            const int i = p / R, r = p - i * R;
-            ys[((int64_t)(2 * r) * E + e) * nb + i] += (double)acc[m][0] + (double)acc[m][1];
-            ys[((int64_t)(2 * r + 1) * E + e) * nb + i] += (double)acc[m][2] + (double)acc[m][3];
-        }
+}
+
+// near product of R >= 4 columns, nb R <= 8 HN_T
+static cudaError_t launch_helm_near_df(ibem_handle* h, int R) {
+    const Plan& P = h->P;
+    const int np = P.nb * R;
+    auto go = [&](auto kern, int side) -> cudaError_t {
+        const size_t sm = (size_t)2 * side * (P.nb * P.nb + np) * sizeof(float4);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e) return e;
+        kern<<<(unsigned)P.E, HN_T, sm, h->stream>>>(h->d_near_ptr, h->d_near_src,
+                                                     reinterpret_cast<const double2*>(h->d_near), P.nb, R, P.E,
+                                                     h->d_xsdf, h->d_ys);
+        h->launches++;
+        return cudaGetLastError();
+    };
+    if (P.nb <= 16) {
+        const int per = (np + HN_T / 2 - 1) / (HN_T / 2);
+        if (per <= 1) return go(helm_near_df_kernel<2, 2, 1>, 2);
+        if (per <= 2) return go(helm_near_df_kernel<2, 2, 2>, 2);
+        if (per <= 4) return go(helm_near_df_kernel<2, 2, 4>, 2);
+        if (per <= 8) return go(helm_near_df_kernel<2, 2, 8>, 2);
+        return go(helm_near_df_kernel<2, 1, 8>, 1);
     }
+    const int per = (np + HN_T - 1) / HN_T;
+    if (per <= 1) return go(helm_near_df_kernel<1, 1, 1>, 1);
+    if (per <= 2) return go(helm_near_df_kernel<1, 1, 2>, 1);
+    if (per <= 4) return go(helm_near_df_kernel<1, 1, 4>, 1);
+    return go(helm_near_df_kernel<1, 1, 8>, 1);
 }
 
 // ---- layout conversion ---------------------------------------------------------------
@@ -523,18 +566,9 @@ cudaError_t helm_apply_operator(ibem_handle* h, const double* x, double* y, int 
         h->launches += 2;
     } else {
         if (R >= 4 && P.nb * R <= 8 * HN_T) {
-            const int np = P.nb * R;
-            const int nt = np <= HN_T / 2 ? ((np + 31) / 32) * 32 : HN_T;
-            const int S = std::min(HN_T / nt, std::max(1, 3 * HN_T / (P.nb * P.nb)));
-            const size_t sm = (size_t)2 * S * (P.nb * P.nb + np) * sizeof(float4);
-            if ((e = cudaFuncSetAttribute(helm_near_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
-                return e;
             helm_split_lift_kernel<<<dim3((unsigned)((P.Nstar + 31) / 32), (unsigned)((R + 31) / 32)), 256, 0, st>>>(
                 R, P.Nstar, h->d_xs, h->d_xsdf);
-            helm_near_df_kernel<<<(unsigned)P.E, HN_T, sm, st>>>(h->d_near_ptr, h->d_near_src,
-                                                                 reinterpret_cast<const double2*>(h->d_near), P.nb,
-                                                                 R, S, nt, P.E, h->d_xsdf, h->d_ys);
-            h->launches++;
+            if ((e = launch_helm_near_df(h, R))) return e;
         } else {
             helm_near_apply_kernel<double2, double><<<dim3((unsigned)P.E, R), threads, 2 * threads * sizeof(double),
                                                       st>>>(h->d_near_ptr, h->d_near_src,

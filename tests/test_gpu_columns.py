@@ -90,3 +90,16 @@ def test_fp32_many(kernel, p, m, q):
     for r0, n in ((0, 16), (3, 17), (100, 40), (136, 64), (60, 65), (72, 128)):
         assert torch.equal(_apply(h, x[r0:r0 + n].contiguous(), 1), y[r0:r0 + n]), (r0, n)
     lib().ibem_destroy(h)
+
+
+# FP64 Helmholtz of four and more columns: one to eight pairs (row, column) per thread, slices side by
+# side and (from some 64 columns at p = 3, 113 at p = 2) in turn
+@pytest.mark.parametrize("p,m,q,R", [(0, 3, 0, 300), (1, 3, 4, 70), (2, 3, 4, 120), (3, 2, 4, 100), (4, 2, 4, 40)])
+def test_helmholtz(p, m, q, R):
+    import torch
+    h = _handle(p, m, q, 1)
+    x = _vectors(1840 + p, R, lib().ibem_get_info(h).ndof, 2)
+    y = _apply(h, x)
+    for r0, n in ((0, 4), (1, 5), (2, 9), (0, 16), (R - 33, 33)):
+        assert torch.equal(_apply(h, x[r0:r0 + n].contiguous()), y[r0:r0 + n]), (r0, n)
+    lib().ibem_destroy(h)
