@@ -24,6 +24,7 @@ ibem_status fail(ibem_handle* h, ibem_status s, const std::string& msg) {
 
 ibem_status cuda_fail(ibem_handle* h, cudaError_t e, const char* where) {
     std::string msg = std::string(where) + ": " + cudaGetErrorString(e);
+    cudaGetLastError();   // reported here: the next call's launches do not find it again
     return fail(h, e == cudaErrorMemoryAllocation ? IBEM_ERR_OOM : IBEM_ERR_CUDA, msg);
 }
 
@@ -675,7 +676,10 @@ ibem_status ibem_solve(ibem_handle* h, const double* b_dev, double* w_dev, int n
     s = solve_impl(h, b_dev, w_dev, nrhs, rtol, maxit, precond, precision, info);
     if (s == IBEM_ERR_NOCONV) h->err = "solver did not reach rtol within maxit";
     else if (s == IBEM_ERR_BREAKDOWN) h->err = "solver breakdown";
-    else if (s != IBEM_OK) h->err = "solver failed (CUDA error)";
+    else if (s != IBEM_OK) {
+        h->err = "solver failed (CUDA error)";
+        cudaGetLastError();   // as in cuda_fail
+    }
     return s;
 }
 
@@ -712,7 +716,10 @@ ibem_status ibem_solver_pairs(ibem_handle* h, const double* b_dev, int nrhs, dou
     *n_pairs = 0;
     s = solver_pairs_impl(h, b_dev, nrhs, rtol, maxit, stride, max_pairs, in_img_dev, tgt_img_dev, n_pairs, info);
     if (s == IBEM_ERR_NOCONV) h->err = "a solve of the pair generation did not reach rtol (pairs kept)";
-    else if (s != IBEM_OK) h->err = "pair generation failed";
+    else if (s != IBEM_OK) {
+        h->err = "pair generation failed";
+        cudaGetLastError();   // as in cuda_fail
+    }
     return s;
 }
 
@@ -729,7 +736,10 @@ ibem_status ibem_solver_residuals(ibem_handle* h, const double* b_dev, int nrhs,
     *n_out = 0;
     s = solver_residuals_impl(h, b_dev, nrhs, rtol, maxit, stride, max_vecs, r_out_dev, n_out, info);
     if (s == IBEM_ERR_NOCONV) h->err = "a solve of the residual generation did not reach rtol (vectors kept)";
-    else if (s != IBEM_OK) h->err = "residual generation failed";
+    else if (s != IBEM_OK) {
+        h->err = "residual generation failed";
+        cudaGetLastError();   // as in cuda_fail
+    }
     return s;
 }
 
