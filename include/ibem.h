@@ -169,7 +169,7 @@ enum { IBEM_COUPLING_DF = 0, IBEM_COUPLING_NATIVE = 1, IBEM_COUPLING_NONE = 2, I
  * contraction runs on the tensor cores: each far block's double-float kernel
  * values and each cluster's moments are split into 6 signed integer digits
  * (|d| <= 128, weights 2^-7, 2^-15, ..., 2^-47) under a power-of-two scale
- * (per block, per moment column), the 21 digit-slice products of combined
+ * (per row of a block, per moment column), the 21 digit-slice products of combined
  * weight down to 2^-54 are accumulated exactly in FP32 (integer partial sums
  * below 2^23) and recombined in double-float, so the result carries about 45
  * significant bits, like GENERATE within the 1e-12 parity tolerance.  Right-hand

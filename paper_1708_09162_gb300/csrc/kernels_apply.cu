@@ -781,7 +781,8 @@ __global__ void near_apply_kernel(const int64_t* __restrict__ nptr, const int32_
 // slice's chain of some 20 dependent loads is what a small mesh waits for; with
 // the shared launches of the coarse levels the application at p = 2, level 2 went
 // from 104 to 80 us).  The order of a row's sums must not depend on the number of
-// right-hand sides, so this rule counts the elements only.
+// right-hand sides, so this rule counts the elements only; nor on the device, so the
+// chip's 152 SMs are a constant here.
 static int near_slices(const Plan& P, int nt) {
     int s = 1;
     while (s < 4 && P.E * s < 152 * 8 && 2 * s * nt <= 1024) s *= 2;

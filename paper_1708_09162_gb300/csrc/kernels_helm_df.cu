@@ -18,9 +18,10 @@
 // right-hand sides: 1.81 ms against 2.00 ms (matrix read once per right-hand
 // side).  The sums over blocks are as exact as the FP64 ones of that form; as plain
 // double-floats they take 1 to 5% less time (1.00 and 1.71 ms) and make the error of an
-// application 1.4 times as large (6.4e-16 against 4.5e-16 at level 4, q = 8).  Two right-hand sides per CTA: with four the unrolled code misses the
-// instruction cache (2.4 ms at level 3).  Packed two-float instructions gave
-// nothing (1.00 ms): the pipe is the limit, not issue.
+// application 1.4 times as large (6.4e-16 against 4.5e-16 at level 4, q = 8).  Two
+// right-hand sides per CTA: with four the unrolled code misses the instruction cache
+// (2.4 ms at level 3).  Packed two-float instructions gave nothing (1.00 ms): the pipe is
+// the limit (64 to 66% active at level 3), not issue.
 #include <algorithm>
 
 #include "ibem_internal.cuh"

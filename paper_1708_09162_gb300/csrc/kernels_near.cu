@@ -466,8 +466,11 @@ cudaError_t launch_cplx(ibem_handle* h, double kappa, double* blocks) {
 
 // The product rules form the regular and subdivided pairs up to the order whose
 // Q^2 x Q^2 kernel matrix would fit in a CTA's shared memory (12 for Laplace, 10 for
-// Helmholtz at p = 2); the streaming kernel takes the higher ones, where the two
-// have not been compared.
+// Helmholtz at p = 2); the streaming kernel, whose shared memory grows with Q^2 only,
+// takes the higher ones.  The line is not where the two are level: assembly of the
+// sphere at p = 2, level 2 takes 15.2 ms with order 12 and 48.9 with 13 for Laplace, 19.1
+// with order 10, 74.7 with 12 and 97.4 with 13 for Helmholtz, and the kernel values alone
+// would account for factors of 1.4 and 2.1.
 bool near_streamed(int Q, int nb, bool cplx, bool subdiv) {
     const size_t QQ = (size_t)Q * Q, cw = cplx ? 2 : 1;
     return (subdiv ? 32 * QQ + cw * QQ * QQ + cw * QQ * nb + cw * nb * nb : 8 * QQ + cw * QQ * QQ + cw * QQ * nb) *

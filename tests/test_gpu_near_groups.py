@@ -1,6 +1,7 @@
-"""FP64 Helmholtz near product of several right-hand sides where its CTA has one
-slice of half its threads (degree 4, four and five columns) and the widths around
-it: every column against the same column alone (another kernel) at 1e-12."""
+"""FP64 Helmholtz near product of several right-hand sides where they take fewer
+threads than a CTA has (degree 4, four and five columns: 100 and 125 of 256) and the
+widths around it: every column against the same column alone (another kernel) at
+1e-12."""
 import numpy as np
 import pytest
 
