@@ -265,7 +265,10 @@ __global__ void helm_near_apply_kernel(const int64_t* __restrict__ nptr, const i
 // (p <= 3), else one.  The slices are groups of threads that take S blocks at a time, or,
 // where a slice's (row, right-hand side) pairs would exceed its threads eightfold, sets of
 // sums that all threads fill in turn.  Stages are double buffered (one barrier per
-// stage).
+// stage).  Bound: FP32 issue beside the FP64 splits of the blocks; with few columns
+// latency (level 3, 8 columns: both pipes 40% busy).  p = 2, with the split: level 5, 64
+// columns 4.0 ms (6.18 with the coefficients split per block); level 3, 8 columns 0.10 ms
+// (0.20).
 constexpr int HN_T = 256;
 
 __device__ __forceinline__ void hn_split(double v, float& h, float& l) {
