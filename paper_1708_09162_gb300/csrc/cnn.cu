@@ -830,6 +830,13 @@ cudaError_t grow(void** p, size_t* have, size_t need_bytes) {
     *have = 0;
     cudaError_t e = cudaMalloc(p, need_bytes);
     if (!e) *have = need_bytes;
+    else cudaGetLastError();   // reported here: the next call's launches do not find it again
+    return e;
+}
+cudaError_t grow_floats(float** p, size_t* have, size_t need) {
+    size_t bytes = *have * sizeof(float);
+    cudaError_t e = grow(reinterpret_cast<void**>(p), &bytes, need * sizeof(float));
+    *have = bytes / sizeof(float);   // after a refusal too: nothing is left
     return e;
 }
 
@@ -838,14 +845,9 @@ cudaError_t ensure_buffers(ibem_cnn* c, int B, int H, int W) {
     for (int l = 0; l < c->L; ++l) mc = std::max(mc, std::max(c->cin[l], c->cout[l]));
     const size_t slot = (size_t)B * mc * H * W;
     cudaError_t e;
-    size_t ab = c->act_bytes;
-    if ((e = grow(&c->d_act, &ab, slot * (c->L + 1) * sizeof(float)))) return e;
-    c->act_bytes = ab;
+    if ((e = grow(&c->d_act, &c->act_bytes, slot * (c->L + 1) * sizeof(float)))) return e;
     c->act_slot = slot;
-    size_t gb = c->gbuf_floats * sizeof(float);
-    if ((e = grow(reinterpret_cast<void**>(&c->d_gbuf), &gb, 2 * slot * sizeof(float)))) return e;
-    c->gbuf_floats = gb / sizeof(float);
-    return cudaSuccess;
+    return grow_floats(&c->d_gbuf, &c->gbuf_floats, 2 * slot);
 }
 
 template <typename TI, typename TO, typename TM, int COB>
@@ -977,9 +979,7 @@ cudaError_t backward(ibem_cnn* c, const float* target, int B, int H, int W, int 
     cudaError_t e;
     size_t maxw = 0;
     for (int l = 0; l < c->L; ++l) maxw = std::max(maxw, (size_t)c->cout[l] * (c->cin[l] * 9 + 1));
-    size_t pb = c->part_floats * sizeof(float);
-    if ((e = grow(reinterpret_cast<void**>(&c->d_part), &pb, (size_t)nx * maxw * sizeof(float)))) return e;
-    c->part_floats = pb / sizeof(float);
+    if ((e = grow_floats(&c->d_part, &c->part_floats, (size_t)nx * maxw))) return e;
     if (!gout) {
         loss_kernel<T><<<LOSS_CTAS, 256, 0, c->stream>>>((int64_t)B * 2 * HW, B, act + c->L * per, target, g0,
                                                          c->d_red + 8);
@@ -1222,20 +1222,16 @@ cudaError_t cnn_precondition(ibem_handle* h, ibem_cnn* c, const double* v, doubl
     c->stream = h->stream;
     const int B = P.npatch, n1 = P.n1;
     cudaError_t e = cudaSuccess;
-    size_t ib = c->img_floats * sizeof(float);
-    if ((e = grow(reinterpret_cast<void**>(&c->d_img), &ib, (size_t)B * 2 * n1 * n1 * sizeof(float)))) {
+    if ((e = grow_floats(&c->d_img, &c->img_floats, (size_t)B * 2 * n1 * n1))) {
         c->stream = keep;
         return e;
     }
-    c->img_floats = ib / sizeof(float);
     const int f = c->coarse, nc = (n1 + f - 1) / f;
     if (f > 1) {
-        size_t cb = c->cimg_floats * sizeof(float);
-        if ((e = grow(reinterpret_cast<void**>(&c->d_cimg), &cb, (size_t)B * 2 * nc * nc * sizeof(float)))) {
+        if ((e = grow_floats(&c->d_cimg, &c->cimg_floats, (size_t)B * 2 * nc * nc))) {
             c->stream = keep;
             return e;
         }
-        c->cimg_floats = cb / sizeof(float);
     }
     apply_block_jacobi(h, v, z);
     sumsq_kernel<<<1, 1024, 0, h->stream>>>(2 * P.N, z, c->d_red + 1);
@@ -1422,10 +1418,7 @@ ibem_status ibem_cnn_train(ibem_cnn* c, const float* in_dev, const float* target
     if ((augment & IBEM_AUGMENT_DIHEDRAL) && H != W) return IBEM_ERR_ARG;
     const int nb_max = std::min(batch, n_images);
     cudaError_t e;
-    size_t ib = c->img_floats * sizeof(float);
-    if ((e = grow(reinterpret_cast<void**>(&c->d_img), &ib, (size_t)2 * nb_max * 2 * H * W * sizeof(float))))
-        return IBEM_ERR_OOM;
-    c->img_floats = ib / sizeof(float);
+    if ((e = grow_floats(&c->d_img, &c->img_floats, (size_t)2 * nb_max * 2 * H * W))) return IBEM_ERR_OOM;
     if ((e = grow(&c->d_items, &c->items_bytes, (size_t)n_images * sizeof(TrainItem)))) return IBEM_ERR_OOM;
     float* bin = c->d_img;
     float* btgt = c->d_img + (size_t)nb_max * 2 * H * W;

@@ -1,4 +1,4 @@
-"""Work space of the operator, whatever was called before it."""
+"""Work space of the operator and the network, whatever was called before."""
 import numpy as np
 import pytest
 
@@ -68,3 +68,31 @@ def test_application_recorded_after_another_call_of_its_width(first):
     del graph
     for h in hs:
         ibem.ibem_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_network_after_a_refused_allocation(precision):
+    # the activations of 65535 images of 4096 x 4096 (hundreds of TB) cannot be allocated; the
+    # call fails before it touches its images, and neither the network nor a handle finds
+    # the old buffers' sizes or the old error afterwards
+    import ctypes
+    import torch
+    ibem = lib()
+    prec = ibem.IBEM_FP32 if precision == "fp32" else ibem.IBEM_BF16
+    c = ibem.ibem_cnn_create(8, seed=3)
+    h = ibem.ibem_create(ibem.sphere_patches(), ibem.make_params(1, 2, q_cheb=4, eta=1.6))
+    ibem.ibem_assemble(h)
+    v = torch.from_numpy(np.random.default_rng(1604).normal(size=(1, ibem.ibem_get_info(h).ndof))).cuda()
+    x = torch.from_numpy(np.random.default_rng(1603).normal(size=(3, 2, 20, 24)).astype(np.float32)).cuda()
+    out, mv = [torch.full_like(x, np.nan) for _ in range(2)], [torch.full_like(v, np.nan) for _ in range(2)]
+    for k in range(2):
+        ibem.ibem_matvec(h, v, mv[k], 1)
+        ibem.ibem_cnn_forward(c, x, out[k], prec)
+        torch.cuda.synchronize()
+        if k == 0:
+            p = ctypes.c_void_p(x.data_ptr())
+            status = ibem._lib.ibem_cnn_forward(c, p, 65535, 4096, 4096, p, prec)
+            assert ibem._lib.ibem_status_string(status) == b"IBEM_ERR_OOM"
+    assert torch.equal(out[0], out[1]) and torch.equal(mv[0], mv[1])
+    ibem.ibem_destroy(h)
+    ibem.ibem_cnn_destroy(c)
