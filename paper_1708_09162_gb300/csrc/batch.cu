@@ -515,6 +515,7 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
     b->arena_floats = floats;
     if (cudaMalloc(&b->arena, floats * sizeof(float)) || cudaMalloc(&b->d_counter, sizeof(int))) {
         ibem_batch_destroy(b);
+        cudaGetLastError();   // reported here: the next call's launches do not find it again
         return IBEM_ERR_OOM;
     }
     size_t yh_cursor = b->yh_begin;
@@ -574,6 +575,7 @@ ibem_status ibem_batch_create(ibem_handle* const* handles, int n, const int* nrh
     }
     if (fail) {
         ibem_batch_destroy(b);
+        cudaGetLastError();   // reported here: the next call's launches do not find it again
         return IBEM_ERR_OOM;
     }
     int sms = 152;

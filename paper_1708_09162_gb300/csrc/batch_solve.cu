@@ -179,6 +179,11 @@ struct BatchKrylov {
         owned.push_back(*p);
         return true;
     }
+    // a refused allocation: reported by this call, not found again by the next one's launches
+    ibem_status refused() {
+        cudaGetLastError();
+        return IBEM_ERR_OOM;
+    }
     cudaError_t read(size_t count, std::vector<double>& out) {
         cudaError_t e;
         if ((e = cudaMemcpyAsync(h_red, d_red, count * sizeof(double), cudaMemcpyDeviceToHost, st))) return e;
@@ -272,14 +277,16 @@ extern "C" ibem_status ibem_batch_solve(ibem_batch* b, const double* b_dev, doub
     const int nc = K.ncol;
     const int64_t T = K.T;
     K.red = (size_t)6 * (restart + 2) * nc + 64;
-    if (cudaMallocHost(&K.h_red, 2 * K.red * sizeof(double)) != cudaSuccess) return IBEM_ERR_OOM;
+    if (cudaMallocHost(&K.h_red, 2 * K.red * sizeof(double)) != cudaSuccess) return K.refused();
     double *V = nullptr, *w = nullptr, *tmp = nullptr, *r = nullptr, *d = nullptr, *dh = nullptr;
     if (!K.alloc(&K.d_cols, nc) || !K.alloc(&K.d_eoff, nc) || !K.alloc(&K.d_red, K.red) ||
         !K.alloc(&V, (size_t)(restart + 1) * T) || !K.alloc(&w, T) || !K.alloc(&tmp, T) || !K.alloc(&r, T) ||
         !K.alloc(&d, T) || !K.alloc(&dh, (size_t)6 * (restart + 2) * nc))
-        return IBEM_ERR_OOM;
-    if (!b->solve_x && (cudaMalloc(&b->solve_x, T * sizeof(double)) || cudaMalloc(&b->solve_y, T * sizeof(double))))
-        return IBEM_ERR_OOM;
+        return K.refused();
+    // each by itself: one of them may be left of a call that could not get the other
+    if ((!b->solve_x && cudaMalloc(&b->solve_x, T * sizeof(double))) ||
+        (!b->solve_y && cudaMalloc(&b->solve_y, T * sizeof(double))))
+        return K.refused();
     cudaStream_t st = K.st;
     if (cudaMemcpyAsync(K.d_cols, K.cols.data(), nc * sizeof(SegCol), cudaMemcpyHostToDevice, st) ||
         cudaMemcpyAsync(K.d_eoff, eoff.data(), nc * sizeof(int64_t), cudaMemcpyHostToDevice, st))

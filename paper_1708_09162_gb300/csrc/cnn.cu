@@ -1287,6 +1287,7 @@ ibem_status ibem_cnn_create(int channels, unsigned long long seed, void* cuda_st
         cudaMalloc(&c->d_wt, maxw * sizeof(float)) || cudaMalloc(&c->d_red, (8 + LOSS_CTAS) * sizeof(double)) ||
         cudaMalloc(&c->d_status, sizeof(int))) {
         ibem_cnn_destroy(c);
+        cudaGetLastError();   // as in grow
         return IBEM_ERR_OOM;
     }
     if (cudaMemcpyAsync(c->d_param, p.data(), off * sizeof(float), cudaMemcpyHostToDevice, c->stream) ||

@@ -96,3 +96,22 @@ def test_network_after_a_refused_allocation(precision):
     assert torch.equal(out[0], out[1]) and torch.equal(mv[0], mv[1])
     ibem.ibem_destroy(h)
     ibem.ibem_cnn_destroy(c)
+
+
+def test_handle_after_a_refused_batch():
+    # vectors of 256 right-hand sides for each of 8000 instances (some 700 GB) cannot be
+    # allocated; the handle's next application does not find the old error
+    import torch
+    ibem = lib()
+    h = ibem.ibem_create(ibem.sphere_patches(), ibem.make_params(2, 4, q_cheb=4, eta=1.6))
+    ibem.ibem_assemble(h)
+    v = torch.from_numpy(np.random.default_rng(1605).normal(size=(1, ibem.ibem_get_info(h).ndof))).cuda()
+    y = [torch.full_like(v, np.nan) for _ in range(2)]
+    ibem.ibem_matvec(h, v, y[0], 1)
+    with pytest.raises(ibem.IbemError) as e:
+        ibem.ibem_batch_create([h] * 8000, [256] * 8000)
+    assert e.value.status == "IBEM_ERR_OOM"
+    ibem.ibem_matvec(h, v, y[1], 1)
+    torch.cuda.synchronize()
+    assert torch.equal(y[0], y[1])
+    ibem.ibem_destroy(h)
